@@ -113,19 +113,21 @@ typedef struct {
 } tlb_params;
 enum { TLB_FE_POTENTIAL = 0, TLB_FE_PRESSURE_TENSOR = 1 };
 enum { TLB_FORCE_EDM = 0, TLB_FORCE_GUO = 1 };
-/* State kept between steps (tlb_params.state):
- * TLB_STATE_POPULATIONS -- the 3Q post-collision populations (any tau);
- * TLB_STATE_MOMENTS     -- at tau = tau_phi = tau_psi = 1 with TLB_FORCE_EDM
- *   (the paper's setting, Sec. 3.1) every post-collision population is an
- *   equilibrium (eq. EDF) of its cell, so 11 values per cell stand for all
- *   of them: rho - 1, u + du, phi, Gamma_phi mu_phi, psi, Gamma_psi mu_psi'
- *   and v (eq. LBE at tau = 1).  The pull of each step rebuilds every
- *   population from the cell it streams from.  The same method, another
- *   executed scheme: 88 bytes of state traffic per cell update in FP32
- *   against 456.  Only with FP32 storage (FP64 or FP32 in 2D); not in
- *   batches.  Initial states and populations written by the caller are
- *   pulled as populations by the next step; reads of populations or fields
- *   see the populations the moments stand for. */
+/* State between steps (tlb_params.state): the 3Q post-collision populations,
+ * in the storage type.  At tau = tau_phi = tau_psi = 1 with TLB_FORCE_EDM
+ * (the paper's setting, Sec. 3.1) and the potential force every one of them
+ * is an equilibrium (eq. EDF) of its cell, so 11 values per cell stand for
+ * all of them: rho - 1, u + du, phi, Gamma_phi mu_phi, psi, Gamma_psi mu_psi'
+ * and v (eq. LBE at tau = 1).  Steps of the tau = 1 collide variants (the
+ * default there, see tlb_autotune) keep those and rebuild every population,
+ * rounded to the storage type, where it streams from: 96 bytes of state
+ * traffic per cell update against 456 in FP32 and 236 in FP16, and the same
+ * populations.  Initial states and populations written by the caller are
+ * pulled as populations by the next step; reads of populations or fields
+ * see the populations the state stands for.
+ * TLB_STATE_POPULATIONS -- any collide variant;
+ * TLB_STATE_MOMENTS     -- only the tau = 1 variants: refused where they do
+ *   not apply, with 16-bit storage and in batches. */
 enum { TLB_STATE_POPULATIONS = 0, TLB_STATE_MOMENTS = 1 };
 
 typedef struct {
@@ -287,13 +289,12 @@ tlb_status tlb_profile_steps(void* ctx, long n_steps, tlb_profile* out);
  * then at 1024 threads per SM) are the collide for tau = tau_phi = tau_psi
  * = 1 with TLB_FORCE_EDM, the paper's setting (Sec. 3.1): there every
  * post-collision population is an equilibrium of the cell's moments (eq.
- * LBE), so that collide pulls no population and only stores; the moment
- * pass then also writes j.  Variants 22..27 are the same collide with two
- * x-adjacent cells per thread (tiles 0..2 at 384, then at 512 threads per
- * SM), every stored value of the pair written by one store; they need an
- * even nx.  Variants 28..31 are the tau = 1 collide on 32x16 tiles (3D):
- * one cell per thread at 768 / 1024, two cells per thread (even nx) at 384
- * / 512 threads per SM.  Variants 19..21 are tiles 0..2 of the general collide with the
+ * LBE), so that collide pulls no population and stores only the 11 values
+ * per cell they are made of (see TLB_STATE_POPULATIONS).  Variants 22..27
+ * name those six again and need an even nx; 28..31 are the tau = 1 collide
+ * on 32x16 tiles (3D) at 768, 1024, 768 and 1024 threads per SM, the last
+ * two with an even nx.  Variants 19..21 are tiles 0..2 of the general
+ * collide with the
  * pressure-tensor force.  They are tried only where they apply, and a new
  * context starts on variant 13 there (19 with the pressure-tensor force,
  * else 0).

@@ -13,8 +13,7 @@
 
 #include "tlb_impl.cuh"
 
-// Everything the kernels of one instance read, for one parity of its
-// population buffers.
+// Everything the kernels of one instance read in one step (see upload_tables).
 template <int MODE>
 struct BArgs {
   LBArgs<MODE> lb;
@@ -42,8 +41,14 @@ __device__ __forceinline__ void pre_body(const BArgs<MODE>& s, const Blk& blk) {
 template <int MODE> struct OpPre {
   static __device__ __forceinline__ void run(const BArgs<MODE>& s, const Blk& b) { pre_body<MODE>(s, b); }
 };
+// tiles of the rebuilding moments sweep (one cell per thread of a phase)
+template <class L> constexpr int recon_x() { return L::DIM == 3 ? 32 : 128; }
+template <class L> constexpr int recon_y() { return L::DIM == 3 ? 4 : 1; }
 template <class L, int MODE> struct OpMoments {
-  static __device__ __forceinline__ void run(const BArgs<MODE>& s, const Blk& b) { moments_body<L, MODE>(s.lb, b); }
+  static __device__ __forceinline__ void run(const BArgs<MODE>& s, const Blk& b) {
+    if (s.lb.M) moments_recon_body<L, MODE, recon_x<L>(), recon_y<L>()>(s.lb, b);
+    else moments_body<L, MODE>(s.lb, b);
+  }
 };
 template <int MODE> struct OpGeometry {
   static __device__ __forceinline__ void run(const BArgs<MODE>& s, const Blk& b) { geometry_body(s.ib, b); }
@@ -151,7 +156,9 @@ struct BatchImpl : BatchBase {
     const bool mem = c->nn > 0;
     switch (op) {
       case PRE: return {mem ? (int)std::min<unsigned>(64, std::max(1u, cdiv(3ll * c->nn, NT))) : 0, 1, 1};
-      case MOM: return {(int)cdiv(c->N, NT), 1, 1};
+      case MOM:
+        if (!variant_t1(b->tile_variant)) return {(int)cdiv(c->N, NT), 1, 1};
+        return {(int)cdiv(c->nx, recon_x<L>()), (int)cdiv(c->ny, recon_y<L>()), (int)cdiv(c->nz, I::RECON_ZC)};
       case GEOM: return {mem ? (int)cdiv((long long)c->ne + c->nn, NT) : 0, 1, 1};
       case BCOUNT: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
       case NODEF: return {mem ? (int)cdiv(32ll * c->nn, NT) : 0, 1, 1};
@@ -228,7 +235,7 @@ struct BatchImpl : BatchBase {
     for (int ph = 0; ph < Batch::NPH; ++ph) {
       int per_sm = 1;
       switch (ph) {
-        case 0: per_sm = occupancy_grid<8, OpPre<MODE>, OpMoments<L, MODE>, OpGeometry<MODE>, OpBrickCount<MODE>>(NT); break;
+        case 0: per_sm = occupancy_grid<6, OpPre<MODE>, OpMoments<L, MODE>, OpGeometry<MODE>, OpBrickCount<MODE>>(NT); break;
         case 1: per_sm = occupancy_grid<5, OpNodeForces<MODE>, OpScatter<MODE>, OpBrickCompact<MODE>>(NT); break;
         case 2: per_sm = occupancy_grid<8, OpBand<MODE>, OpBrickFill<MODE>>(NT); break;
         case 3: per_sm = occupancy_grid<8, OpSpread<MODE>, OpFill<MODE>>(NT); break;
@@ -246,7 +253,7 @@ struct BatchImpl : BatchBase {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm,
-        k_phase<collide_block<FORM, TX, TY>(), collide_threads<FORM>() / collide_block<FORM, TX, TY>(), BA,
+        k_phase<collide_block<FORM, TX, TY>(), collide_minb<MODE, FORM, TX, TY>(), BA,
                 OpCollide<L, MODE, TX, TY, FORM>>,
         collide_block<FORM, TX, TY>(), 0);
     return std::max(1, per_sm);
@@ -264,7 +271,7 @@ struct BatchImpl : BatchBase {
   template <int TX, int TY, int FORM>
   static tlb_status launch_collide_t(Batch* b, const BA* A, const int4* vg, cudaStream_t s) {
     const int n = (int)b->act.size();
-    k_phase<collide_block<FORM, TX, TY>(), collide_threads<FORM>() / collide_block<FORM, TX, TY>(), BA,
+    k_phase<collide_block<FORM, TX, TY>(), collide_minb<MODE, FORM, TX, TY>(), BA,
             OpCollide<L, MODE, TX, TY, FORM>>
         <<<b->ph_grid[4], collide_block<FORM, TX, TY>(), 0, s>>>(A, vg, n, b->ph_ent[4], b->ph_total[4]);
     b->launches++;
@@ -288,7 +295,7 @@ struct BatchImpl : BatchBase {
     const int g = b->ph_grid[ph], ne = b->ph_ent[ph], tot = b->ph_total[ph];
     switch (ph) {
       case 0:
-        k_phase<NT, 8, BA, OpPre<MODE>, OpMoments<L, MODE>, OpGeometry<MODE>, OpBrickCount<MODE>>
+        k_phase<NT, 6, BA, OpPre<MODE>, OpMoments<L, MODE>, OpGeometry<MODE>, OpBrickCount<MODE>>
             <<<g, NT, 0, s>>>(A, vg, n, ne, tot);
         break;
       case 1:
@@ -314,19 +321,27 @@ struct BatchImpl : BatchBase {
     return TLB_OK;
   }
 
-  // Argument tables of the active instances: parity q reads the buffer
-  // cur ^ q of each instance.
-  tlb_status upload_tables(Batch* b) {
+  // Argument tables of the active instances.  General collide: table q reads
+  // the population buffer cur ^ q of each instance.  Tau = 1 collide: both
+  // read and write the state M; in table 1 the instances whose state is in
+  // the populations pull it (the first step after an initialisation), in
+  // table 0 none does.  With `scratch` the collide writes into the idle
+  // population buffer (timing of collide variants).
+  tlb_status upload_tables(Batch* b, bool scratch = false) {
     const int n = (int)b->act.size();
+    const bool t1 = variant_t1(b->tile_variant);
     for (int q = 0; q < 2; ++q) {
       std::vector<BA> t((size_t)std::max(n, 1));
       for (int j = 0; j < n; ++j) {
         Ctx* c = b->inst[b->act[j]];
         BA& a = t[j];
-        a.lb = I::lbargs(c, c->cur ^ q);
+        a.lb = I::lbargs(c, t1 ? c->cur : c->cur ^ q);
         a.lb.zc = b->zc;
-        a.lb.jm = variant_t1(b->tile_variant) ? c->ptr<typename Prec<MODE>::Real>(c->L.jm) : nullptr;
+        I::use_t1(c, a.lb, t1);
+        if (q == 0) a.lb.pull = 0;
+        if (t1 && scratch) a.lb.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
         a.ib = I::ibargs(c);
+        I::use_t1(c, a.ib, t1);
         a.rp = I::resptrs(c, b->ptr<unsigned long long>(b->res) + 4 * (size_t)b->act[j]);
       }
       TLB_CUDA(cudaMemcpyAsync(b->ptr<char>(b->targs[q]), t.data(), (size_t)n * sizeof(BA), cudaMemcpyHostToDevice,
@@ -334,6 +349,27 @@ struct BatchImpl : BatchBase {
       TLB_CUDA(cudaStreamSynchronize(b->stream));
     }
     return TLB_OK;
+  }
+
+  // some active instance's state is in its populations
+  static bool any_pull(const Batch* b) {
+    for (int i : b->act)
+      if (b->inst[i]->state_in_pops) return true;
+    return false;
+  }
+  // after n steps: where the state is, and the step counts
+  static void advanced(Batch* b, long n) {
+    const bool t1 = variant_t1(b->tile_variant);
+    for (int i : b->act) {
+      Ctx* c = b->inst[i];
+      if (t1) {
+        c->state_in_pops = false;
+        c->pops_stale = true;
+      } else if (n & 1) {
+        c->cur ^= 1;
+      }
+      c->t += n;
+    }
   }
 
   // Markers overwritten since the last step: rebuild the box accumulator
@@ -360,7 +396,7 @@ struct BatchImpl : BatchBase {
     long keep = b->launches;
     TLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
     tlb_status st = launch_step(b, 0, b->cap);
-    if (st == TLB_OK) st = launch_step(b, 1, b->cap);
+    if (st == TLB_OK) st = launch_step(b, variant_t1(b->tile_variant) ? 0 : 1, b->cap);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(b->cap, &g);
     b->graph_launches = b->launches - keep;
@@ -378,6 +414,9 @@ struct BatchImpl : BatchBase {
   }
 
   tlb_status prepare(Batch* b) {
+    if (!variant_t1(b->tile_variant))
+      for (int i : b->act)
+        if (tlb_status st = I::enter_pops(b->inst[i]); st != TLB_OK) return st;
     if (b->graph_dirty) {
       tlb_status st = plan_phases(b);
       if (st != TLB_OK) return st;
@@ -395,17 +434,18 @@ struct BatchImpl : BatchBase {
     if (b->act.empty() || n == 0) return TLB_OK;
     tlb_status st = prepare(b);
     if (st != TLB_OK) return st;
+    long left = n;
+    if (variant_t1(b->tile_variant) && any_pull(b)) {
+      if ((st = launch_step(b, 1, b->stream)) != TLB_OK) return st;
+      --left;
+    }
     // the graph's two steps leave every buffer parity as it was
-    for (long k = 0; k + 1 < n; k += 2) {
+    for (; left >= 2; left -= 2) {
       TLB_CUDA(cudaGraphLaunch(b->graph, b->stream));
       b->launches += b->graph_launches;
     }
-    if (n & 1) {
-      st = launch_step(b, 0, b->stream);
-      if (st != TLB_OK) return st;
-      for (int i : b->act) b->inst[i]->cur ^= 1;
-    }
-    for (int i : b->act) b->inst[i]->t += n;
+    if (left && (st = launch_step(b, 0, b->stream)) != TLB_OK) return st;
+    advanced(b, n);
     return TLB_OK;
   }
 
@@ -417,7 +457,8 @@ struct BatchImpl : BatchBase {
     cudaEvent_t ev[7];
     for (int k = 0; k < 7; ++k) TLB_CUDA(cudaEventCreate(&ev[k]));
     for (long k = 0; k < n && st == TLB_OK; ++k) {
-      const BA* A = b->ptr<BA>(b->targs[k & 1]);
+      const bool t1 = variant_t1(b->tile_variant);
+      const BA* A = b->ptr<BA>(b->targs[t1 ? (k == 0 && any_pull(b)) : (k & 1)]);
       for (int ph = 0; ph < 6 && st == TLB_OK; ++ph) {
         cudaEventRecord(ev[ph], b->stream);
         st = launch_phase(b, ph, A, b->stream);
@@ -432,14 +473,14 @@ struct BatchImpl : BatchBase {
     }
     for (int k = 0; k < 7; ++k) cudaEventDestroy(ev[k]);
     if (st != TLB_OK) return st;
-    if (n & 1)
-      for (int i : b->act) b->inst[i]->cur ^= 1;
-    for (int i : b->act) b->inst[i]->t += n;
+    advanced(b, n);
     return TLB_OK;
   }
 
   tlb_status residual(Batch* b) override {
     if (b->act.empty()) return TLB_OK;
+    for (int i : b->act)  // the residual reads populations
+      if (tlb_status st = b->inst[i]->impl->sync_pops(b->inst[i]); st != TLB_OK) return st;
     tlb_status st = prepare(b);
     if (st != TLB_OK) return st;
     TLB_CUDA(cudaMemsetAsync(b->ptr<char>(b->res), 0, b->res.bytes, b->stream));
@@ -462,27 +503,30 @@ struct BatchImpl : BatchBase {
     tlb_status st = TLB_OK;
     // the moments of the current state feed the collide (only the moments:
     // the first phase of a step would also consume the marker box)
-    for (int i : b->act) {
-      Ctx* c = b->inst[i];
-      LBArgs<MODE> la = I::lbargs(c, c->cur);
-      la.jm = c->ptr<typename Prec<MODE>::Real>(c->L.jm);
-      k_moments<L, MODE><<<cdiv(c->N, 256), 256, 0, b->stream>>>(la);
-      b->launches++;
-      TLB_CUDA(cudaGetLastError());
-    }
     auto all_ok = [&](int v) {
       for (int i : b->act)
         if (!b->inst[i]->variant_ok(v)) return false;
       return true;
     };
+    // candidates: as in the single-lattice autotuner
+    const bool t1 = all_ok(13);
+    for (int i : b->act) {
+      Ctx* c = b->inst[i];
+      if (!t1)
+        if (tlb_status es = I::enter_pops(c); es != TLB_OK) return es;
+      LBArgs<MODE> la = I::lbargs(c, c->cur);
+      I::use_t1(c, la, t1);
+      if (tlb_status ms = I::launch_moments(c, la, b->stream); ms != TLB_OK) return ms;
+      b->launches++;
+    }
     for (int v = 0; v < COLLIDE_NVAR && st == TLB_OK; ++v)
       for (size_t zi = 0; zi < zcs.size() && st == TLB_OK; ++zi) {
-        if (!all_ok(v)) continue;
+        if (!all_ok(v) || variant_t1(v) != t1 || variant_pair(v)) continue;
         b->tile_variant = v;
         b->zc = zcs[zi];
         b->graph_dirty = true;
         st = plan_phases(b);
-        if (st == TLB_OK) st = upload_tables(b);
+        if (st == TLB_OK) st = upload_tables(b, true);
         if (st == TLB_OK) st = launch_collide(b, b->ptr<BA>(b->targs[0]), vg_of(b, 4), b->stream);
         float tmin = 1e30f;
         for (int r = 0; r < 2 && st == TLB_OK; ++r) {

@@ -127,7 +127,7 @@ tlb_status tlb_save(void* ctx, void* host_blob, size_t* bytes) {
   Ctx* c = (Ctx*)ctx;
   if (!c || !bytes) { set_error("ctx/bytes is NULL"); return TLB_ERR_ARG; }
   if (!c->initialised) { set_error("tlb_save before tlb_init_fields"); return TLB_ERR_STATE; }
-  // moment storage: the checkpoint holds the populations the moments stand
+  // the checkpoint holds the populations that the state in M stands
   // for (the same values the next pull would rebuild)
   if (tlb_status st = c->impl->sync_pops(c); st != TLB_OK) return st;
   char* dev[kSections];
@@ -194,7 +194,7 @@ tlb_status tlb_load(void* ctx, const void* host_blob, size_t bytes) {
   c->t_snap = h.t_snap;
   c->initialised = true;
   c->box_stale = true;
-  c->state_in_pops = true;  // (moment storage: the next step pulls them)
+  c->state_in_pops = true;
   c->pops_stale = false;
   return TLB_OK;
 }

@@ -33,6 +33,7 @@ struct D2Q9 {
   TLB_HD static constexpr int opp(int i) {
     return i == 0 ? 0 : (i == 1 ? 2 : i == 2 ? 1 : i == 3 ? 4 : i == 4 ? 3 : i == 5 ? 6 : i == 6 ? 5 : i == 7 ? 8 : 7);
   }
+  static constexpr int NCOL = 3;  // in-plane velocities (c_x, c_y), see col_dir
 };
 
 // D3Q19: rest; +x,-x,+y,-y,+z,-z (w = 1/18); then the edge velocities of the
@@ -59,7 +60,32 @@ struct D3Q19 {
   TLB_HD static constexpr int opp(int i) {
     return i == 0 ? 0 : (i <= 6 ? (i % 2 == 1 ? i + 1 : i - 1) : 7 + 4 * ((i - 7) / 4) + (3 - (i - 7) % 4));
   }
+  static constexpr int NCOL = 9;
 };
+
+// In-plane velocity k of a lattice: rest, +x, -x, then (3D) +y, -y and the
+// four diagonals.
+TLB_HD constexpr int col_cx(int k) { return k == 1 || k == 5 || k == 6 ? 1 : (k == 2 || k == 7 || k == 8 ? -1 : 0); }
+TLB_HD constexpr int col_cy(int k) { return k == 3 || k == 5 || k == 7 ? 1 : (k == 4 || k == 6 || k == 8 ? -1 : 0); }
+// Direction with in-plane velocity k and c_z = cz, -1 if the set has none.
+template <class L>
+TLB_HD constexpr int col_dir(int k, int cz) {
+  for (int i = 0; i < L::Q; ++i)
+    if (L::cx(i) == col_cx(k) && L::cy(i) == col_cy(k) && L::cz(i) == cz) return i;
+  return -1;
+}
+
+// c_i . u of an unrolled direction: its one or two signed terms (a product
+// with the zero components would not be folded away).
+template <class L, class R>
+__device__ __forceinline__ R cdot(int i, const R* u) {
+  const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+  const R x = cx > 0 ? u[0] : -u[0], y = cy > 0 ? u[1] : -u[1], z = cz > 0 ? u[2] : -u[2];
+  if (cx && cy) return x + y;
+  if (cx && cz) return x + z;
+  if (cy && cz) return y + z;
+  return cx ? x : (cy ? y : (cz ? z : R(0)));
+}
 
 // ------------------------------------------------------------ precisions
 template <int MODE> struct Prec;
@@ -80,26 +106,18 @@ template <> __device__ __forceinline__ float from_real<float>(float v) { return 
 template <> __device__ __forceinline__ __half from_real<__half>(float v) { return __float2half_rn(v); }
 template <> __device__ __forceinline__ __nv_bfloat16 from_real<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// A value as its storage type holds it: one rounding with 16-bit storage,
+// the value itself otherwise.
+template <class S, class R>
+__device__ __forceinline__ R as_stored(R v) {
+  return to_real(from_real<S>(v));
+}
+
 // Two consecutive Real values (one 8 or 16-byte load).
 template <class R> struct R2Of;
 template <> struct R2Of<float> { using T = float2; };
 template <> struct R2Of<double> { using T = double2; };
 template <class R> using R2 = typename R2Of<R>::T;
-
-// Two adjacent cells' values stored together (one 4, 8 or 16-byte store;
-// p is aligned to two elements), each rounded as from_real rounds it.
-__device__ __forceinline__ void store_pair(double* p, double a, double b) {
-  *reinterpret_cast<double2*>(p) = make_double2(a, b);
-}
-__device__ __forceinline__ void store_pair(float* p, float a, float b) {
-  *reinterpret_cast<float2*>(p) = make_float2(a, b);
-}
-__device__ __forceinline__ void store_pair(__half* p, float a, float b) {
-  *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
-}
-__device__ __forceinline__ void store_pair(__nv_bfloat16* p, float a, float b) {
-  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
-}
 
 // ------------------------------------------------------------ geometry
 struct Geo {
@@ -211,7 +229,11 @@ struct Pull {
     }
   }
 
-  // The rest populations are added last: g_0 and h_0 carry nearly all of
+  // Sums in the order a sweep along z meets the populations: those with c_z
+  // = 1 (they come from the plane below), then c_z = 0, then c_z = -1, each
+  // over the in-plane velocities; so the rebuilding sweep of the tau = 1
+  // scheme (moments_recon_body) gives the same bits.  The rest populations
+  // are added last: g_0 and h_0 carry nearly all of
   // phi and psi, so the small moving populations are summed first at their
   // own scale and the sum is rounded once at the scale of phi (adding them
   // one by one to g_0 rounds each addition there: in FP32 that made the
@@ -220,14 +242,18 @@ struct Pull {
     CellMoments<Real> m;
     Real r = 0, jx = 0, jy = 0, jz = 0, p = 0, s = 0;
 #pragma unroll
-    for (int i = 1; i < L::Q; ++i) {
-      r += f[i];
-      if (L::cx(i)) jx += L::cx(i) > 0 ? f[i] : -f[i];
-      if (L::cy(i)) jy += L::cy(i) > 0 ? f[i] : -f[i];
-      if (L::cz(i)) jz += L::cz(i) > 0 ? f[i] : -f[i];
-      p += g[i];
-      s += h[i];
-    }
+    for (int cz = 1; cz >= -1; --cz)
+#pragma unroll
+      for (int k = 0; k < L::NCOL; ++k) {
+        const int i = col_dir<L>(k, cz);
+        if (i <= 0) continue;
+        r += f[i];
+        if (L::cx(i)) jx += L::cx(i) > 0 ? f[i] : -f[i];
+        if (L::cy(i)) jy += L::cy(i) > 0 ? f[i] : -f[i];
+        if (L::cz(i)) jz += L::cz(i) > 0 ? f[i] : -f[i];
+        p += g[i];
+        s += h[i];
+      }
     r += f[0];
     p += g[0];
     s += h[0];
@@ -292,80 +318,93 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// ------------------------------------------------ moment storage (tau = 1)
+// ------------------------------------------------ the tau = 1 state
 // At tau = tau_phi = tau_psi = 1 with the exact difference method every
 // post-collision population is an equilibrium (eq. EDF) of its cell:
 // f*_i = f_i^eq(rho, w) with w = u + du, g*_i = g_i^eq(phi, Gamma_phi mu_phi,
-// v), h*_i = h_i^eq(psi, Gamma_psi mu_psi', v) (eq. LBE at tau = 1).  The
-// moment-storage scheme keeps these 11 values per cell instead of the 3Q
-// populations; the pull of the next step rebuilds each population from the
-// cell it streams from.  Plane order of the stored moments:
-enum { M_DRHO = 0, M_W = 1, M_PHI = 4, M_GMP = 5, M_PSI = 6, M_GMS = 7, M_V = 8, M_COUNT = 11 };
+// v), h*_i = h_i^eq(psi, Gamma_psi mu_psi', v) (eq. LBE at tau = 1).  These
+// 11 values per cell stand for the 3Q populations between steps; the pull of
+// the next step rebuilds each population from the cell it streams from, as
+// its storage type holds it: with 16-bit storage every rebuilt population is
+// rounded, so the state is that of stored populations, bit for bit.
+// They are kept as three 16-byte vectors per cell (32 in double precision),
+// one plane array each: (rho - 1, w), (phi, 3 Gamma_phi mu_phi, psi,
+// 3 Gamma_psi mu_psi'), (v, -1.5 v^2).  A cell is then moved by three
+// vector copies instead of eleven, and what every reader would form again
+// (3 Gamma mu, -1.5 v^2) is stored once, in the otherwise idle twelfth slot.
+enum { M_F = 0, M_ORD = 1, M_V = 2, M_COUNT = 3 };
 
-// Four values of one cell side by side, so that a shared-memory ring of them
-// is read with one 16-byte load (two in double precision) per cell.
+// Four values of one cell side by side: one 16-byte access (two in double
+// precision).
 template <class R>
 struct alignas(4 * sizeof(R)) R4 {
   R x, y, z, w;
 };
+// one vector through the read-only path
+__device__ __forceinline__ R4<float> ldg4(const R4<float>* p) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ R4<double> ldg4(const R4<double>* p) {
+  const double2* q = reinterpret_cast<const double2*>(p);
+  const double2 a = __ldg(q), b = __ldg(q + 1);
+  return {a.x, a.y, b.x, b.y};
+}
 
-// The post-collision populations of one cell from its stored moments, with
-// the explicitly rounded operations (see rmul), so the reconstruction in the
-// pull, in the interpolation and in the materialised populations gives the
-// same value.
-template <class L, class Real>
+// The post-collision populations of one cell from its stored state, with the
+// explicitly rounded operations (see rmul), so the rebuild in the pull, in
+// the interpolation and in the materialised populations gives the same value.
+template <class L, int MODE>
 struct EqCell {
-  Real drho, rho, w[3], ww, ord[2], gm3[2], v[3], vv;
-  // drho and w only (what f_i needs)
-  __device__ __forceinline__ void load_f(const Real* __restrict__ M, int P32, int c) {
-    drho = M[M_DRHO * P32 + c];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) w[d] = M[(M_W + d) * P32 + c];
-    rho = Real(1) + drho;
-    ww = rfma(w[2], w[2], rfma(w[1], w[1], rmul(w[0], w[0])));
-  }
-  __device__ __forceinline__ void load(const Real* __restrict__ M, int P32, int c) {
-    load_f(M, P32, c);
-    ord[0] = M[M_PHI * P32 + c];
-    ord[1] = M[M_PSI * P32 + c];
-    gm3[0] = rmul(Real(3), M[M_GMP * P32 + c]);
-    gm3[1] = rmul(Real(3), M[M_GMS * P32 + c]);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) v[d] = M[(M_V + d) * P32 + c];
-    vv = rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0])));
-  }
-  // the same from three packed values: (drho, w), (phi, Gamma_phi mu_phi,
-  // psi, Gamma_psi mu_psi'), (v, -)
-  __device__ __forceinline__ void load3(const R4<Real>& A, const R4<Real>& B, const R4<Real>& C) {
+  using Real = typename Prec<MODE>::Real;
+  using Store = typename Prec<MODE>::Store;
+  Real drho, rho, w[3], w15, ord[2], gm3[2], v[3], v15;
+  // rho - 1 and w only (what f_i needs)
+  __device__ __forceinline__ void set_f(const R4<Real>& A) {
     drho = A.x;
     w[0] = A.y;
     w[1] = A.z;
     w[2] = A.w;
     rho = Real(1) + drho;
-    ww = rfma(w[2], w[2], rfma(w[1], w[1], rmul(w[0], w[0])));
+    w15 = rmul(Real(-1.5), rfma(w[2], w[2], rfma(w[1], w[1], rmul(w[0], w[0]))));
+  }
+  __device__ __forceinline__ void set(const R4<Real>& A, const R4<Real>& B, const R4<Real>& C) {
+    set_f(A);
     ord[0] = B.x;
+    gm3[0] = B.y;
     ord[1] = B.z;
-    gm3[0] = rmul(Real(3), B.y);
-    gm3[1] = rmul(Real(3), B.w);
+    gm3[1] = B.w;
     v[0] = C.x;
     v[1] = C.y;
     v[2] = C.z;
-    vv = rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0])));
+    v15 = C.w;
   }
-  // f_i - w_i = w_i (drho + rho (3 c.w + 4.5 (c.w)^2 - 1.5 w^2))
+  __device__ __forceinline__ void load(const R4<Real>* M, int P32, int c) {
+    set(M[M_F * P32 + c], M[M_ORD * P32 + c], M[M_V * P32 + c]);
+  }
+  // 3 c.u + 4.5 (c.u)^2 - 1.5 u^2
+  static __device__ __forceinline__ Real poly(int i, const Real* u, Real u15) {
+    if (i == 0) return u15;
+    const Real cu = cdot<L>(i, u);
+    return rfma(cu, rfma(Real(4.5), cu, Real(3)), u15);
+  }
+  // f_i - w_i = w_i (drho + rho p(w))
   __device__ __forceinline__ Real f(int i) const {
-    const Real cw = L::cx(i) * w[0] + L::cy(i) * w[1] + L::cz(i) * w[2];
-    const Real p = rfma(rmul(Real(4.5), cw), cw, rfma(Real(3), cw, rmul(Real(-1.5), ww)));
-    return rmul(Real(L::w(i)), rfma(rho, p, drho));
+    return as_stored<Store>(rmul(Real(L::w(i)), rfma(rho, poly(i, w, w15), drho)));
+  }
+  // the same of direction i, or of its opposite where `back` (c.u changes sign)
+  __device__ __forceinline__ Real f_or_back(int i, bool back) const {
+    const Real c = cdot<L>(i, w), cu = back ? -c : c;
+    const Real p = i == 0 ? w15 : rfma(cu, rfma(Real(4.5), cu, Real(3)), w15);
+    return as_stored<Store>(rmul(Real(L::w(i)), rfma(rho, p, drho)));
   }
   // g_i (s = 0) or h_i (s = 1): w_i (3 Gamma mu + ord p(c.v)) for i != 0; the
   // rest population closes the zeroth moment
-  __device__ __forceinline__ Real o(int s, int i) const {
-    if (i == 0)
-      return radd(rfma(gm3[s], Real(L::w(0)) - Real(1), ord[s]), rmul(rmul(Real(-1.5 * L::w(0)), ord[s]), vv));
-    const Real cv = L::cx(i) * v[0] + L::cy(i) * v[1] + L::cz(i) * v[2];
-    const Real p = rfma(rmul(Real(4.5), cv), cv, rfma(Real(3), cv, rmul(Real(-1.5), vv)));
-    return rmul(Real(L::w(i)), rfma(ord[s], p, gm3[s]));
+  __device__ __forceinline__ Real o(int s, Real p, int i) const {
+    return as_stored<Store>(rmul(Real(L::w(i)), rfma(ord[s], p, gm3[s])));
+  }
+  __device__ __forceinline__ Real rest(int s) const {
+    return radd(rfma(gm3[s], Real(L::w(0)) - Real(1), ord[s]), rmul(rmul(Real(L::w(0)), ord[s]), v15));
   }
 };
 

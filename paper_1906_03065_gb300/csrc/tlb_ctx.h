@@ -12,11 +12,12 @@
 
 // Collide variants: 3 tile shapes x 4 register forms, v = 3 form + tile,
 // the smallest tile in a fifth form (v = 12), and the 3 tiles in the two
-// forms of the tau = 1 collide (v = 13..18, see variant_t1).
+// forms of the tau = 1 collide (v = 13..18, see variant_t1); 22..27 name
+// those again, 28..31 a fourth tile.
 constexpr int COLLIDE_NVAR = 32;
 constexpr bool variant_t1(int v) { return (v >= 13 && v <= 18) || v >= 22; }
-// variants 22..27 and 30, 31: the tau = 1 collide with two x-adjacent cells
-// per thread; 28..31 are the tau = 1 forms on 32 x 16 tiles
+// variants 22..27 and 30, 31 need an even nx (two-cell forms of the tau = 1
+// collide; they run the one-cell kernels)
 constexpr bool variant_pair(int v) { return (v >= 22 && v <= 27) || v == 30 || v == 31; }
 // variants 19..21: the general collide with the pressure-tensor force
 constexpr bool variant_pt(int v) { return v >= 19 && v <= 21; }
@@ -55,8 +56,8 @@ struct ImplBase {
   // contact angle of every capsule with phi = 0: out[cap] = {mean, min,
   // max, contact points}; synchronises
   virtual tlb_status contact_angle(Ctx* c, double* out) = 0;
-  // moment storage: write the populations the stored moments stand for into
-  // the current population buffer if it is stale (no-op otherwise)
+  // write the populations that the state in M stands for into the current
+  // population buffer if it is stale (no-op otherwise)
   virtual tlb_status sync_pops(Ctx* c) = 0;
 };
 
@@ -79,7 +80,7 @@ struct Region {
 struct Layout {
   // lattice
   Region lo[2], rest[2];
-  Region rho, phi, psi, jm, M, I, dsel, own, key, fib, ftot, mu, rb;
+  Region rho, phi, psi, p4, j2, M, I, dsel, own, key, fib, ftot, mu, rb;
   // membranes
   Region X, E, ecap, ncap, cap_par, ds0, rprev, rnext, A0, G0i, inc_off, inc, adj, edges, ring_off, ring;
   Region en, vn, erel, eorg, ecst, xo, xr, skc, capr, ncpl, F, box;
@@ -108,18 +109,19 @@ struct Ctx {
   }
   // a collide variant this context can run: the pressure-tensor variants for
   // the pressure-tensor force only, the tau = 1 ones only where they apply,
-  // and with moment storage only the tau = 1 ones
+  // and with TLB_STATE_MOMENTS only the tau = 1 ones
   bool variant_ok(int v) const {
     if (variant_pt(v) != (p.force_form == TLB_FE_PRESSURE_TENSOR)) return false;
-    if (variant_pair(v) && nx % 2 != 0) return false;  // pairs never straddle a row
+    if (variant_pair(v) && nx % 2 != 0) return false;
     if (variant_t1(v)) return t1_ok();
-    return !moments();
+    return p.state != TLB_STATE_MOMENTS;
   }
-  // moment storage (TLB_STATE_MOMENTS): the state is the moment buffer M,
-  // except after an initialisation or a write of populations, which the
-  // next step pulls as populations (state_in_pops); the population buffer
-  // is refreshed from M for readers when it is stale
-  bool moments() const { return p.state == TLB_STATE_MOMENTS; }
+  // Where the state is.  A step with a tau = 1 collide variant keeps it in
+  // the 11 values per cell of M (see EqCell), any other in the population
+  // buffer `cur`.  state_in_pops: in the populations (after an
+  // initialisation, a load, a write of populations or a general step), which
+  // the next tau = 1 step pulls; otherwise in M, and pops_stale says that the
+  // population buffer does not show it yet (sync_pops writes it there).
   bool state_in_pops = true;
   bool pops_stale = false;
   int Q = 0;

@@ -56,8 +56,9 @@ struct IBArgs {
   int* own;
   Real* I;
   Real* dsel;
-  const Real* psi;       // psi(t) (moment field)
-  const Real* M;         // moment storage: the stored moments the interpolation
+  const Real* psi;       // psi(t) of cell n at psi[n * psi_step] (moment field)
+  int psi_step;
+  const R4<Real>* M;     // tau = 1 scheme: the stored state the interpolation
                          // rebuilds the streamed populations from (NULL: the
                          // population buffers are read)
   Real* fib;             // [3][P]
@@ -790,7 +791,7 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
       if (c >= 0) {
         // psi is requested with the key, so its latency overlaps the key's
         // and the element's (it is needed only for band cells)
-        const Real psic = a.psi[c];
+        const Real psic = a.psi[c * a.psi_step];
         unsigned long long key = a.key[c];
         if (key == KEY_NONE) {
           if (a.own[c] >= 0) {  // left the band since the previous step
@@ -1404,21 +1405,23 @@ __device__ __forceinline__ void interp_advect_body(const IBArgs<typename Prec<MO
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const Nbr<L> nb(G, cx[h], cy[h], cz[h]);
-      const long long self = nb.self;
+      R4<Real> src[L::Q];
+#pragma unroll
+      for (int i = 0; i < L::Q; ++i) src[i] = ldg4(a.M + M_F * G.P32 + nb.src(i));
+      Real ft[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) ft[d] = a.ftot[d * G.P + nb.self];
       Real r = 0, j[3] = {0, 0, 0};
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
-        EqCell<L, Real> e;
-        e.load_f(a.M, G.P32, nb.src(i));
-        const Real fi = e.f(nb.bounce(i) ? L::opp(i) : i);
+        EqCell<L, MODE> e;
+        e.set_f(src[i]);
+        const Real fi = e.f_or_back(i, nb.bounce(i));
         r += fi;
         if (L::cx(i)) j[0] += L::cx(i) > 0 ? fi : -fi;
         if (L::cy(i)) j[1] += L::cy(i) > 0 ? fi : -fi;
         if (L::cz(i)) j[2] += L::cz(i) > 0 ? fi : -fi;
       }
-      Real ft[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) ft[d] = a.ftot[d * G.P + self];
       Real rho = Real(1) + r;
       if (w[h] != Real(0))
         for (int d = 0; d < 3; ++d) U[d] += w[h] * (j[d] + Real(0.5) * ft[d]) / rho;

@@ -17,6 +17,9 @@ struct Impl : ImplBase {
   using Store = typename Prec<MODE>::Store;
   using Rest = typename Prec<MODE>::Rest;
 
+  // tiles of the rebuilding moments sweep
+  static constexpr int RECON_X = L::DIM == 3 ? 32 : 64, RECON_Y = L::DIM == 3 ? 4 : 1, RECON_ZC = 16;
+
   static Geo geo(const Ctx* c) {
     Geo g;
     g.nx = c->nx;
@@ -29,6 +32,19 @@ struct Impl : ImplBase {
     return g;
   }
 
+  // the arrays of the tau = 1 scheme, or none of them
+  static void use_t1(Ctx* c, LBArgs<MODE>& a, bool t1) {
+    a.p4 = t1 ? c->ptr<R4<Real>>(c->L.p4) : nullptr;
+    a.j2 = t1 ? c->ptr<R2<Real>>(c->L.j2) : nullptr;
+    a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
+    a.pull = c->state_in_pops;
+  }
+  static void use_t1(Ctx* c, IBArgs<Real>& a, bool t1) {
+    a.psi = t1 ? &c->ptr<R4<Real>>(c->L.p4)->z : c->ptr<Real>(c->L.psi);
+    a.psi_step = t1 ? 4 : 1;
+    a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
+  }
+
   static LBArgs<MODE> lbargs(Ctx* c, int src) {
     LBArgs<MODE> a;
     a.G = geo(c);
@@ -39,11 +55,7 @@ struct Impl : ImplBase {
     a.rho = c->ptr<Real>(c->L.rho);
     a.phi = c->ptr<Real>(c->L.phi);
     a.psi = c->ptr<Real>(c->L.psi);
-    // rho - 1 and j for the tau = 1 collide (the moments write them only then)
-    a.jm = variant_t1(c->tile_variant) ? c->ptr<Real>(c->L.jm) : nullptr;
-    // moment storage: the collide stores the moments, the pull rebuilds from them
-    a.mst = c->moments() ? c->ptr<Real>(c->L.M) : nullptr;
-    a.msrc = a.mst;
+    use_t1(c, a, variant_t1(c->tile_variant));
     a.I = c->ptr<Real>(c->L.I);
     a.fib = c->ptr<Real>(c->L.fib);
     a.ftot = c->ptr<Real>(c->L.ftot);
@@ -61,6 +73,7 @@ struct Impl : ImplBase {
     a.gphi = (Real)c->p.gamma_phi;
     a.gpsi = (Real)c->p.gamma_psi;
     a.zc = c->tiles_zc;
+    a.zcm = RECON_ZC;
     a.forcing = c->p.forcing;
     a.status = c->ptr<unsigned>(c->L.status);
     return a;
@@ -112,8 +125,7 @@ struct Impl : ImplBase {
     a.own = c->ptr<int>(c->L.own);
     a.I = c->ptr<Real>(c->L.I);
     a.dsel = c->ptr<Real>(c->L.dsel);
-    a.psi = c->ptr<Real>(c->L.psi);
-    a.M = c->moments() ? c->ptr<Real>(c->L.M) : nullptr;
+    use_t1(c, a, variant_t1(c->tile_variant));
     a.fib = c->ptr<Real>(c->L.fib);
     a.ftot = c->ptr<Real>(c->L.ftot);
     a.bflag = c->ptr<unsigned char>(c->L.bflag);
@@ -258,30 +270,26 @@ struct Impl : ImplBase {
     c->t = 0;
     c->t_snap = 0;
     c->initialised = true;
-    c->state_in_pops = true;  // (moment storage: the first step pulls these populations)
+    c->state_in_pops = true;
     c->pops_stale = false;
     return TLB_OK;
   }
 
   tlb_status sync_pops(Ctx* c) override {
-    if (!c->moments() || c->state_in_pops || !c->pops_stale) return TLB_OK;
+    if (c->state_in_pops || !c->pops_stale) return TLB_OK;
     k_materialize<L, MODE><<<blocks(c->N, 256), 256, 0, c->stream>>>(
-        geo(c), c->ptr<Real>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]));
+        geo(c), c->ptr<R4<Real>>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]));
     TLB_LAUNCHED(c, "k_materialize");
     c->pops_stale = false;
     return TLB_OK;
   }
 
-  // the moments of the streamed populations: pulled from the population
-  // buffer, or (moment storage) rebuilt from the stored moments
+  // the moments of the streamed populations: rebuilt from the state in M, or
+  // pulled from the population buffer
   static tlb_status launch_moments(Ctx* c, const LBArgs<MODE>& la, cudaStream_t s) {
-    if (c->moments() && !c->state_in_pops) {
-      // tiles of 32 x 4 columns (2D: 64) walking 16 planes
-      constexpr int RX = L::DIM == 3 ? 32 : 64, RY = L::DIM == 3 ? 4 : 1;
-      LBArgs<MODE> lr = la;
-      lr.zc = 16;
-      const dim3 grid(blocks(c->nx, RX), blocks(c->ny, RY), blocks(c->nz, lr.zc));
-      k_moments_recon_tiled<L, MODE, RX, RY><<<grid, RX * RY, 0, s>>>(lr);
+    if (la.M && !la.pull) {
+      const dim3 grid(blocks(c->nx, RECON_X), blocks(c->ny, RECON_Y), blocks(c->nz, la.zcm));
+      k_moments_recon<L, MODE, RECON_X, RECON_Y><<<grid, RECON_X * RECON_Y, 0, s>>>(la);
       TLB_LAUNCHED(c, "k_moments_recon");
     } else {
       // 16-bit storage: 128-thread blocks, finer grains around the membrane
@@ -367,12 +375,17 @@ struct Impl : ImplBase {
   // current state (it only reads the current buffer, so repeats are harmless).
   tlb_status autotune(Ctx* c, int* variant, int* zc) override {
     cudaStream_t s = c->stream;
+    // the candidates: the tau = 1 variants where they apply (a general one
+    // pulls and stores several times their bytes), else the general ones
+    const bool t1 = c->t1_ok();
+    if (!t1)
+      if (tlb_status st = enter_pops(c); st != TLB_OK) return st;
     LBArgs<MODE> la = lbargs(c, c->cur);
-    la.jm = c->ptr<Real>(c->L.jm);  // every variant's input, the tau = 1 forms' too
+    use_t1(c, la, t1);
     if (tlb_status st = launch_moments(c, la, s); st != TLB_OK) return st;
-    // moment storage: the timed collides store into the idle population
-    // buffer, not into the state
-    if (c->moments()) la.mst = c->ptr<Real>(c->L.lo[1 - c->cur]);
+    // the timed collides store into the idle population buffer, not into the
+    // state
+    if (t1) la.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
     cudaEvent_t e0, e1;
     TLB_CUDA(cudaEventCreate(&e0));
     TLB_CUDA(cudaEventCreate(&e1));
@@ -381,7 +394,7 @@ struct Impl : ImplBase {
     const std::vector<int> zcs = z_chunk_candidates(c->nz);
     for (int v = 0; v < COLLIDE_NVAR; ++v)
       for (const int zcv : zcs) {
-        if (!c->variant_ok(v)) continue;
+        if (!c->variant_ok(v) || variant_t1(v) != t1 || variant_pair(v)) continue;
         c->tile_variant = v;
         c->tiles_zc = zcv;
         la.zc = c->tiles_zc;
@@ -446,10 +459,17 @@ struct Impl : ImplBase {
 
   // A step replays from a graph when it launches the same work every time:
   // no phase profile, no markers set from outside since the last step (their
-  // box is rebuilt first) and, with moment storage, the state in the stored
-  // moments (the first step after populations were written rebuilds them).
+  // box is rebuilt first) and the state where the collide variant keeps it
+  // (the first tau = 1 step after populations were written pulls them).
   bool graph_ready(Ctx* c) const {
-    return c->graphs && !c->prof && !c->box_stale && !(c->moments() && c->state_in_pops);
+    return c->graphs && !c->prof && !c->box_stale && c->state_in_pops == !variant_t1(c->tile_variant);
+  }
+
+  // the state into the populations, for a step of a general variant
+  static tlb_status enter_pops(Ctx* c) {
+    tlb_status st = c->impl->sync_pops(c);
+    if (st == TLB_OK) c->state_in_pops = true;
+    return st;
   }
 
   // Launch the graph of the current buffer, capturing it first if missing or
@@ -509,10 +529,7 @@ struct Impl : ImplBase {
     TLB_CUDA(cudaEventRecord(c->ev_interp, user));
     c->launches += c->glaunch[k];
     c->t += Ctx::GRAPH_STEPS;
-    if (c->moments()) {
-      c->state_in_pops = false;
-      c->pops_stale = true;
-    }
+    c->pops_stale = variant_t1(c->tile_variant);
     return TLB_OK;
   }
 
@@ -525,6 +542,8 @@ struct Impl : ImplBase {
     // only); the next step's marker work waits for it there.  The phase
     // profile keeps every kernel on the main stream.
     const bool pipe = c->nn > 0 && !c->prof;
+    const bool t1 = variant_t1(c->tile_variant);
+    if (!t1 && (st = enter_pops(c)) != TLB_OK) return st;
     for (long k = 0; k < n; ++k) {
       LBArgs<MODE> la = lbargs(c, c->cur);
       IBArgs<Real> ia = ibargs(c);
@@ -581,12 +600,13 @@ struct Impl : ImplBase {
       }
       if ((st = mark(c, 4)) != TLB_OK) return st;
       if ((st = collect(c)) != TLB_OK) return st;
-      c->cur = 1 - c->cur;
-      c->t += 1;
-      if (c->moments()) {  // the state is the stored moments from here on
+      if (t1) {  // the state is M from here on
         c->state_in_pops = false;
         c->pops_stale = true;
+      } else {
+        c->cur = 1 - c->cur;
       }
+      c->t += 1;
     }
     if (pipe && n > 0) TLB_CUDA(cudaStreamWaitEvent(s, c->ev_interp, 0));  // all of it on the caller's stream
     return TLB_OK;
@@ -677,7 +697,7 @@ struct Impl : ImplBase {
     TLB_CUDA(cudaMemcpyAsync(c->ptr<Rest>(c->L.rest[c->cur]), rest.data(), rest.size() * sizeof(Rest), cudaMemcpyHostToDevice, s));
     TLB_CUDA(cudaStreamSynchronize(s));
     c->initialised = true;
-    c->state_in_pops = true;  // (moment storage: the next step pulls them)
+    c->state_in_pops = true;
     c->pops_stale = false;
     return TLB_OK;
   }

@@ -19,11 +19,12 @@ struct LBArgs {
   Real* rho;        // rho - 1 (the deviation keeps its low bits in FP32)
   Real* phi;
   Real* psi;
-  Real* jm;         // [3][P] j of the streamed populations, written by the
-                    // moments for the tau = 1 collide (NULL otherwise)
-  Real* mst;        // moment storage: [11][P] moments the tau = 1 collide
-                    // stores in place of the populations (NULL otherwise)
-  const Real* msrc; // moment storage: the moments the reconstructing pull reads
+  // the tau = 1 scheme (NULL otherwise):
+  R4<Real>* p4;     // [P] (rho - 1, phi, psi, j_x) of the streamed populations
+  R2<Real>* j2;     // [P] (j_y, j_z)
+  R4<Real>* M;      // [3][P] the stored state (see EqCell)
+  int pull;         // the state is in the populations, not in M (set by an
+                    // initialisation, a load or a write): pull them this once
   const Real* I;
   const Real* fib;  // [3][P] immersed-boundary force density
   Real* ftot;       // [3][P] total force of the step (read by the interpolation)
@@ -32,31 +33,64 @@ struct LBArgs {
   FEParams<Real> fe;
   Real om, om_phi, om_psi;  // 1/tau
   Real gphi, gpsi;          // Gamma_phi, Gamma_psi
-  int zc;                   // planes per block along z
+  int zc;                   // planes per block along z (the collide)
+  int zcm;                  // the same of the rebuilding moments sweep
   int forcing;              // TLB_FORCE_EDM or TLB_FORCE_GUO
   unsigned* status;
 };
 
-// Asynchronous global -> shared copies of one element (cp.async, 4 or 8
-// bytes): the copy runs while the thread computes; cp_async_wait_all blocks
-// until every copy the thread issued has landed.
-__device__ __forceinline__ void cp_async_elem(float* dst, const float* src) {
+// Asynchronous global -> shared copy of one cell's four values (cp.async, 16
+// bytes each): the copy runs while the thread computes; cp_async_wait<N>
+// blocks until all but the thread's newest N groups have landed.
+template <class R>
+__device__ __forceinline__ void cp_async_r4(R4<R>* dst, const R4<R>* src) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_elem(double* dst, const double* src) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(src) : "memory");
+#pragma unroll
+  for (int k = 0; k < (int)(sizeof(R4<R>) / 16); ++k)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s + 16 * k), "l"((const char*)src + 16 * k)
+                 : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Periodic wrap of a halo index: within two cells of the range except for
+// tiles wider than the lattice, which take the division.
+__device__ __forceinline__ int halo_wrap(int v, int n) {
+  if (v < 0) v += n;
+  if (v >= n) v -= n;
+  if (v < 0 || v >= n) {
+    v %= n;
+    if (v < 0) v += n;
+  }
+  return v;
+}
+// Plane p of the sweeps' rings: periodic, or the plane next to a wall for the
+// ghosts beyond it.
+__device__ __forceinline__ int ring_plane(const Geo& G, int p) {
+  return G.wall ? min(max(p, 0), G.nz - 1) : halo_wrap(p, G.nz);
+}
 
 // ---------------------------------------------------------------- moments
 // rho - 1, phi, psi at every cell from the streamed populations (eq.
-// MomentsDFs), and j for the tau = 1 collide.
+// MomentsDFs); with the tau = 1 scheme j too.
+template <class L, int MODE>
+__device__ __forceinline__ void moments_store(const LBArgs<MODE>& a, int n, const CellMoments<typename Prec<MODE>::Real>& m) {
+  using Real = typename Prec<MODE>::Real;
+  if (a.p4) {
+    a.p4[n] = R4<Real>{m.drho, m.phi, m.psi, m.j[0]};
+    R2<Real> t;
+    t.x = m.j[1];
+    t.y = m.j[2];
+    a.j2[n] = t;
+  } else {
+    a.rho[n] = m.drho;
+    a.phi[n] = m.phi;
+    a.psi[n] = m.psi;
+  }
+}
 template <class L, int MODE>
 __device__ __forceinline__ void moments_body(const LBArgs<MODE>& a, const Blk& blk) {
-  using Real = typename Prec<MODE>::Real;
   const Geo G = a.G;
   long long n = (long long)blk.x * blockDim.x + threadIdx.x;
   if (n >= G.N) return;
@@ -64,160 +98,177 @@ __device__ __forceinline__ void moments_body(const LBArgs<MODE>& a, const Blk& b
   cell_xyz(G, n, x, y, z);
   Pull<L, MODE> p;
   p.load(a.lo_src, a.rest_src, G, x, y, z);
-  CellMoments<Real> m = p.moments();
-  a.rho[n] = m.drho;
-  a.phi[n] = m.phi;
-  a.psi[n] = m.psi;
-  if (a.jm) {
-    a.jm[n] = m.j[0];
-    a.jm[G.P + n] = m.j[1];
-    a.jm[2 * G.P + n] = m.j[2];
-  }
+  moments_store<L, MODE>(a, (int)n, p.moments());
 }
 template <class L, int MODE>
 __global__ void __launch_bounds__(256) k_moments(const __grid_constant__ LBArgs<MODE> a) {
   moments_body<L, MODE>(a, hw_blk());
 }
 
-// Moments of the streamed populations, each rebuilt from the stored moments
-// of the cell it streams from (across a wall: this cell's opposite
-// direction, halfway bounce-back); summed as the population pull sums.
-template <class L, int MODE>
+// Moments of the streamed populations of the tau = 1 scheme, each population
+// rebuilt from the stored state of the cell it streams from (across a wall:
+// this cell's opposite direction, halfway bounce-back).
+//
+// A TX x TY tile of columns walks a.zc planes; a plane of the state (tile
+// plus a halo of 1) is copied into one of two shared-memory slots while the
+// plane before it is used.  A thread reads the 9 (2D: 3) columns around its
+// own once per plane and adds what each sends to the three planes it feeds:
+// c_z = 1 starts the sums of the plane above, c_z = 0 continues this plane's,
+// c_z = -1 and the rest populations finish those of the plane below.  So the
+// running sums of two planes live in registers and a state vector is read 9
+// times from shared memory instead of 19.  The order of the additions is
+// that of Pull::moments.
+template <class L, int MODE, int TX, int TY>
 __device__ __forceinline__ void moments_recon_body(const LBArgs<MODE>& a, const Blk& blk) {
   using Real = typename Prec<MODE>::Real;
-  const Geo G = a.G;
-  long long n = (long long)blk.x * blockDim.x + threadIdx.x;
-  if (n >= G.N) return;
-  int x, y, z;
-  cell_xyz(G, n, x, y, z);
-  const Nbr<L> nb(G, x, y, z);
-  Pull<L, MODE> p;
-#pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const int ii = nb.bounce(i) ? L::opp(i) : i;
-    EqCell<L, Real> e;
-    e.load(a.msrc, G.P32, nb.src(i));
-    p.f[i] = e.f(ii);
-    p.g[i] = e.o(0, ii);
-    p.h[i] = e.o(1, ii);
-  }
-  CellMoments<Real> m = p.moments();
-  a.rho[n] = m.drho;
-  a.phi[n] = m.phi;
-  a.psi[n] = m.psi;
-  a.jm[n] = m.j[0];
-  a.jm[G.P + n] = m.j[1];
-  a.jm[2 * G.P + n] = m.j[2];
-}
-template <class L, int MODE>
-__global__ void __launch_bounds__(256) k_moments_recon(const __grid_constant__ LBArgs<MODE> a) {
-  moments_recon_body<L, MODE>(a, hw_blk());
-}
-
-// The same pull as a plane sweep: a TX x TY tile of columns walks a chunk of
-// z planes; the stored moments of four planes (tile plus a halo of 1) sit in
-// a shared-memory ring filled by asynchronous copies one plane ahead, so
-// every stored moment is read once from memory and a cell's rebuild reads
-// its 19 sources from shared memory, three 16-byte vectors each.  Same
-// arithmetic and summation order as moments_recon_body.
-template <class L, int MODE, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) k_moments_recon_tiled(const __grid_constant__ LBArgs<MODE> a) {
-  using Real = typename Prec<MODE>::Real;
   constexpr bool D3 = L::DIM == 3;
-  constexpr int HX = TX + 2, HY = D3 ? TY + 2 : 1, CELLS = HX * HY, NT = TX * TY;
-  struct Cell {
-    R4<Real> a, b, c;  // (drho, w), (phi, gmp, psi, gms), (v, -)
-  };
-  __shared__ Cell sM[4][CELLS];
+  constexpr int HX = TX + 2, HY = D3 ? TY + 2 : 1, CELLS = HX * HY, NT = TX * TY, NL = (CELLS + NT - 1) / NT;
+  __shared__ R4<Real> sA[2][CELLS], sB[2][CELLS], sC[2][CELLS];
   const Geo G = a.G;
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX, tid = threadIdx.x;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int z0 = blockIdx.z * a.zc;
-  const int z1 = min(z0 + a.zc, G.nz);
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int x0 = blk.x * TX, y0 = blk.y * TY, z0 = blk.z * a.zcm, z1 = min(z0 + a.zcm, G.nz);
   const int x = x0 + tx, y = y0 + ty;
   const bool active = x < G.nx && y < G.ny;
-  auto wrapn = [](int v, int n) {
-    v %= n;
-    return v < 0 ? v + n : v;
-  };
-  // plane p of the ring (planes beyond a wall are never read: the pull
-  // bounces there, so they take the nearest plane)
-  auto issue_plane = [&](int p) {
-    const int slot = (p + 8) & 3;
-    const int pz = G.wall ? min(max(p, 0), G.nz - 1) : wrapn(p, G.nz);
-    for (int k = tid; k < CELLS; k += NT) {
-      const int hx = k % HX, hy = k / HX;
-      const int gx = wrapn(x0 - 1 + hx, G.nx);
-      const int gy = D3 ? wrapn(y0 - 1 + hy, G.ny) : 0;
-      const long long c = ((long long)pz * G.ny + gy) * G.nx + gx;
-      Real* d[M_COUNT] = {&sM[slot][k].a.x, &sM[slot][k].a.y, &sM[slot][k].a.z, &sM[slot][k].a.w,
-                          &sM[slot][k].b.x, &sM[slot][k].b.y, &sM[slot][k].b.z, &sM[slot][k].b.w,
-                          &sM[slot][k].c.x, &sM[slot][k].c.y, &sM[slot][k].c.z};
-      // (plane order of the stored moments: drho, w, phi, gmp, psi, gms, v)
+  if (a.pull) {  // once after an initialisation or a write of populations
+    if (active)
+      for (int zz = z0; zz < z1; ++zz) {
+        Pull<L, MODE> p;
+        p.load(a.lo_src, a.rest_src, G, x, y, zz);
+        moments_store<L, MODE>(a, (zz * G.ny + y) * G.nx + x, p.moments());
+      }
+    return;
+  }
+  int coff[NL];  // in-plane offsets of the cells this thread copies
 #pragma unroll
-      for (int f = 0; f < M_COUNT; ++f) cp_async_elem(d[f], a.msrc + (long long)f * G.P + c);
+  for (int j = 0; j < NL; ++j) {
+    const int k = tid + j * NT, gx = halo_wrap(x0 - 1 + k % HX, G.nx);
+    coff[j] = (D3 ? halo_wrap(y0 - 1 + k / HX, G.ny) * G.nx : 0) + gx;
+  }
+  const int nxy = G.nx * G.ny;
+  auto issue = [&](int p, int slot) {
+    const R4<Real>* M = a.M + (long long)ring_plane(G, p) * nxy;
+#pragma unroll
+    for (int j = 0; j < NL; ++j) {
+      const int k = tid + j * NT;
+      if (k < CELLS) {
+        cp_async_r4(&sA[slot][k], M + M_F * G.P32 + coff[j]);
+        cp_async_r4(&sB[slot][k], M + M_ORD * G.P32 + coff[j]);
+        cp_async_r4(&sC[slot][k], M + M_V * G.P32 + coff[j]);
+      }
     }
     cp_async_commit();
   };
-  for (int p = z0 - 1; p <= z0 + 1; ++p) issue_plane(p);
-  cp_async_wait_all();
-  __syncthreads();
-  for (int zz = z0; zz < z1; ++zz) {
-    // plane zz + 2 replaces plane zz - 2, which this iteration does not read
-    if (zz + 2 <= z1) issue_plane(zz + 2);
-    if (active) {
-      const bool wlo = G.wall && zz == 0, whi = G.wall && zz == G.nz - 1;
-      Pull<L, MODE> p;
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        const bool bounce = (L::cz(i) > 0 && wlo) || (L::cz(i) < 0 && whi);
-        const int ii = bounce ? L::opp(i) : i;
-        const int sz = bounce ? zz : zz - L::cz(i);
-        const int hx = bounce ? tx + 1 : tx + 1 - L::cx(i);
-        const int hy = D3 ? (bounce ? ty + 1 : ty + 1 - L::cy(i)) : 0;
-        EqCell<L, Real> e;
-        const Cell& src = sM[(sz + 8) & 3][hy * HX + hx];
-        e.load3(src.a, src.b, src.c);
-        p.f[i] = e.f(ii);
-        p.g[i] = e.o(0, ii);
-        p.h[i] = e.o(1, ii);
-      }
-      const CellMoments<Real> m = p.moments();
-      const long long n = ((long long)zz * G.ny + y) * G.nx + x;
-      a.rho[n] = m.drho;
-      a.phi[n] = m.phi;
-      a.psi[n] = m.psi;
-      a.jm[n] = m.j[0];
-      a.jm[G.P + n] = m.j[1];
-      a.jm[2 * G.P + n] = m.j[2];
-    }
-    cp_async_wait_all();
+  struct Acc {
+    Real r, jx, jy, jz, p, s;
+  };
+  Acc lo = {0, 0, 0, 0, 0, 0}, mid = lo;  // sums of planes q - 1 and q
+  Real rest_lo[3] = {0, 0, 0};            // rest populations of plane q - 1
+  auto add = [](Acc& t, int i, Real f, Real g, Real h) {
+    t.r += f;
+    if (L::cx(i)) t.jx += L::cx(i) > 0 ? f : -f;
+    if (L::cy(i)) t.jy += L::cy(i) > 0 ? f : -f;
+    if (L::cz(i)) t.jz += L::cz(i) > 0 ? f : -f;
+    t.p += g;
+    t.s += h;
+  };
+  issue(z0 - 1, 0);
+  const int sc = (D3 ? ty + 1 : 0) * HX + tx + 1;
+  for (int q = z0 - 1; q <= z1; ++q) {
+    const int slot = (q - z0 + 1) & 1;
+    cp_async_wait<0>();
     __syncthreads();
+    if (q < z1) issue(q + 1, slot ^ 1);  // (every thread has left plane q - 1)
+    // walls: nothing comes from the ghost planes; a cell next to the wall
+    // takes its own opposite populations where theirs would have come
+    const bool ghost = G.wall && (q < 0 || q >= G.nz);
+    const bool wlo = G.wall && q == 0, whi = G.wall && q == G.nz - 1 && q < z1;
+    Acc up = {0, 0, 0, 0, 0, 0};
+    Real rest_mid[3] = {0, 0, 0};
+    auto bounce = [&](Acc& t, int cz) {  // own populations opposite to the c_z = cz ones
+      EqCell<L, MODE> e;
+      e.set(sA[slot][sc], sB[slot][sc], sC[slot][sc]);
+#pragma unroll
+      for (int k = 0; k < L::NCOL; ++k) {
+        const int i = col_dir<L>(k, cz);
+        if (i < 0) continue;
+        const int o = L::opp(i);
+        const Real p = EqCell<L, MODE>::poly(o, e.v, e.v15);
+        add(t, i, e.f(o), e.o(0, p, o), e.o(1, p, o));
+      }
+    };
+    if (!ghost) {
+      if (wlo) bounce(mid, 1);
+#pragma unroll
+      for (int k = 0; k < L::NCOL; ++k) {
+        // the column whose populations with in-plane velocity k arrive here
+        const int n = sc - col_cy(k) * HX - col_cx(k);
+        EqCell<L, MODE> e;
+        e.set(sA[slot][n], sB[slot][n], sC[slot][n]);
+#pragma unroll
+        for (int cz = 1; cz >= -1; --cz) {
+          const int i = col_dir<L>(k, cz);
+          if (i < 0) continue;
+          if (i == 0) {
+            rest_mid[0] = e.f(0);
+            rest_mid[1] = e.rest(0);
+            rest_mid[2] = e.rest(1);
+          } else {
+            const Real p = EqCell<L, MODE>::poly(i, e.v, e.v15);
+            add(cz > 0 ? up : (cz == 0 ? mid : lo), i, e.f(i), e.o(0, p, i), e.o(1, p, i));
+          }
+        }
+      }
+    }
+    auto put = [&](const Acc& t, const Real* rest, int z) {
+      CellMoments<Real> m;
+      m.drho = t.r + rest[0];
+      m.j[0] = t.jx;
+      m.j[1] = t.jy;
+      m.j[2] = t.jz;
+      m.phi = t.p + rest[1];
+      m.psi = t.s + rest[2];
+      moments_store<L, MODE>(a, (z * G.ny + y) * G.nx + x, m);
+    };
+    if (q > z0 && active) put(lo, rest_lo, q - 1);
+    if (whi) {  // the top plane is complete with its own bounce (q == z1 - 1)
+      bounce(mid, -1);
+      if (active) put(mid, rest_mid, q);
+      break;
+    }
+    lo = mid;
+    mid = up;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) rest_lo[d] = rest_mid[d];
   }
+  cp_async_wait<0>();
+}
+// threads per SM the register budget is set for: 768
+template <class L, int MODE, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY, 768 / (TX * TY)) k_moments_recon(const __grid_constant__ LBArgs<MODE> a) {
+  moments_recon_body<L, MODE, TX, TY>(a, hw_blk());
 }
 
-// The populations a cell's stored moments stand for, written post-collision
+// The populations a cell's stored state stands for, written post-collision
 // into the population buffers (for the readers of the population state).
 template <class L, int MODE>
-__global__ void k_materialize(Geo G, const typename Prec<MODE>::Real* M, typename Prec<MODE>::Store* lo,
+__global__ void k_materialize(Geo G, const R4<typename Prec<MODE>::Real>* M, typename Prec<MODE>::Store* lo,
                               typename Prec<MODE>::Rest* rest) {
   using Real = typename Prec<MODE>::Real;
   using Store = typename Prec<MODE>::Store;
   using Rest = typename Prec<MODE>::Rest;
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= G.N) return;
-  EqCell<L, Real> e;
+  EqCell<L, MODE> e;
   e.load(M, G.P32, (int)n);
+  lo[(long long)plane_f<L>(0) * G.P + n] = from_real<Store>(e.f(0));
+  rest[n] = from_real<Rest>(e.rest(0));
+  rest[G.P + n] = from_real<Rest>(e.rest(1));
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
+  for (int i = 1; i < L::Q; ++i) {
+    const Real p = EqCell<L, MODE>::poly(i, e.v, e.v15);
     lo[(long long)plane_f<L>(i) * G.P + n] = from_real<Store>(e.f(i));
-    if (i == 0) {
-      rest[n] = from_real<Rest>(e.o(0, 0));
-      rest[G.P + n] = from_real<Rest>(e.o(1, 0));
-    } else {
-      lo[(long long)plane_g<L>(i) * G.P + n] = from_real<Store>(e.o(0, i));
-      lo[(long long)plane_h<L>(i) * G.P + n] = from_real<Store>(e.o(1, i));
-    }
+    lo[(long long)plane_g<L>(i) * G.P + n] = from_real<Store>(e.o(0, p, i));
+    lo[(long long)plane_h<L>(i) * G.P + n] = from_real<Store>(e.o(1, p, i));
   }
 }
 
@@ -282,20 +333,13 @@ __device__ __forceinline__ void pressure_tensor(const FEParams<Real>& fe, Real d
 }
 
 // Forms 5 and 6 are the collide at tau = tau_phi = tau_psi = 1 with the exact
-// difference method: there every post-collision population is an
-// equilibrium, f* = f^eq(rho, u + du), g* = g^eq(phi, mu_phi, v), h* =
-// h^eq(psi, mu_psi', v) (eq. LBE with tau = 1), so the collide reads the
-// moments rho - 1 and j that the moment pass wrote (summed in the same order
-// as the pull of the general forms) and pulls no population: it only stores
-// them.
-template <int FORM> constexpr bool form_t1() { return FORM == 5 || FORM == 6 || FORM == 8 || FORM == 9; }
-// forms 8 and 9: the tau = 1 collide with two x-adjacent cells per thread
-template <int FORM> constexpr bool form_pair() { return FORM == 8 || FORM == 9; }
+// difference method (collide_t1_body), form 7 the general one with the
+// pressure-tensor force; the others the general one.
+template <int FORM> constexpr bool form_t1() { return FORM == 5 || FORM == 6; }
 
 template <class L, int MODE, int TX, int TY, int FORM>
 __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Blk& blk) {
   constexpr bool PF = FORM == 1;  // the next population set prefetched
-  constexpr bool T1 = form_t1<FORM>();
   // form 7: the force from the explicit pressure tensor (see pt_of)
   constexpr bool PT = FORM == 7;
   using Real = typename Prec<MODE>::Real;
@@ -323,26 +367,13 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
   const int x = x0 + tx, y = y0 + ty;
   const bool active = x < G.nx && y < G.ny;
 
-  // wrap of a halo index: within two cells of the range except for tiles
-  // wider than the lattice, which take the division
-  auto modn = [](int v, int n) {
-    if (v < 0) v += n;
-    if (v >= n) v -= n;
-    if (v < 0 || v >= n) {
-      v %= n;
-      if (v < 0) v += n;
-    }
-    return v;
-  };
-  auto plane_src = [&](int p) { return G.wall ? min(max(p, 0), G.nz - 1) : modn(p, G.nz); };
-
   auto load_mom = [&](int p) {
     const int slot = (p + 10) % 5;
-    const long long zp = (long long)plane_src(p) * G.ny;
+    const long long zp = (long long)ring_plane(G, p) * G.ny;
     for (int k = tid; k < MX * MY; k += NT) {
       int hx = k % MX, hy = k / MX;
-      int gx = modn(x0 - 2 + hx, G.nx);
-      int gy = D3 ? modn(y0 - HY + hy, G.ny) : 0;
+      int gx = halo_wrap(x0 - 2 + hx, G.nx);
+      int gy = D3 ? halo_wrap(y0 - HY + hy, G.ny) : 0;
       long long c = (zp + gy) * G.nx + gx;
       smom[slot][0][k] = a.rho[c];
       smom[slot][1][k] = a.phi[c];
@@ -359,7 +390,7 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
         for (int q = 0; q < NMU; ++q) smu[slot][q][k] = smu[src][q][k];
       return;
     }
-    const long long zp = (long long)modn(p, G.nz) * G.ny;  // periodic ghost planes wrap
+    const long long zp = (long long)halo_wrap(p, G.nz) * G.ny;  // periodic ghost planes wrap
     for (int k = tid; k < UX * UY; k += NT) {
       int ux = k % UX, uy = k / UX;
       int hx = ux + 1, hy = uy + (D3 ? 1 : 0);
@@ -377,8 +408,8 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
       }
 #pragma unroll
       for (int q = 0; q < 3; ++q) lap[q] *= Real(6);  // 2/cs^2
-      int gx = modn(x0 - 1 + ux, G.nx);
-      int gy = D3 ? modn(y0 - 1 + uy, G.ny) : 0;
+      int gx = halo_wrap(x0 - 1 + ux, G.nx);
+      int gy = D3 ? halo_wrap(y0 - 1 + uy, G.ny) : 0;
       Real Iv = a.I[(zp + gy) * G.nx + gx];
       Real mr, mp, ms;
       chem_potentials<Real>(a.fe, cen[0], cen[1], cen[2], lap[0], lap[1], lap[2], Iv, mr, mp, ms);
@@ -481,30 +512,27 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
       }
     };
     // f: pull, first moment, BGK + exact difference method (eq. LBE) for f_i - w_i
-    Real fv[T1 ? 1 : Q];
+    Real fv[Q];
     Real drho = 0, jx = 0, jy = 0, jz = 0;
     // with PF the next set's loads are in flight while this one is computed
     Real nextv[PF ? Q : 1];
-    if constexpr (T1) {
-      drho = drho_c;
-      jx = a.jm[n];
-      jy = a.jm[G.P32 + n];
-      jz = a.jm[2 * G.P32 + n];
-    } else {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        fv[i] = to_real(__ldg(a.lo_src + nb.off(i, plane_f<L>(i), plane_f<L>(L::opp(i)), G.P32)));
-      }
-      if constexpr (PF) load_set(0, nextv);
+    for (int i = 0; i < Q; ++i) {
+      fv[i] = to_real(__ldg(a.lo_src + nb.off(i, plane_f<L>(i), plane_f<L>(L::opp(i)), G.P32)));
+    }
+    if constexpr (PF) load_set(0, nextv);
 #pragma unroll
-      for (int i = 1; i < Q; ++i) {  // in the order of Pull::moments (rest last)
+    for (int cz = 1; cz >= -1; --cz)  // in the order of Pull::moments (rest last)
+#pragma unroll
+      for (int k = 0; k < L::NCOL; ++k) {
+        const int i = col_dir<L>(k, cz);
+        if (i <= 0) continue;
         drho += fv[i];
         if (L::cx(i)) jx += L::cx(i) > 0 ? fv[i] : -fv[i];
         if (L::cy(i)) jy += L::cy(i) > 0 ? fv[i] : -fv[i];
         if (L::cz(i)) jz += L::cz(i) > 0 ? fv[i] : -fv[i];
       }
-      drho += fv[0];
-    }
+    drho += fv[0];
     const Real irho = Real(1) / rho;
     const Real j[3] = {jx, jy, jz};
     Real u[3], du[3], v[3], us[3];
@@ -519,50 +547,15 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
     const Real vv = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
     const Real dus = du[0] * us[0] + du[1] * us[1] + du[2] * us[2];
     const Real om = a.om;
-    if constexpr (T1) {
-      if (a.mst) {
-        // moment storage: the 11 values whose equilibria are this cell's
-        // post-collision populations (see EqCell)
-        Real* M = a.mst;
-        M[M_DRHO * G.P32 + n] = drho;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          M[(M_W + d) * G.P32 + n] = radd(u[d], du[d]);
-          M[(M_V + d) * G.P32 + n] = v[d];
-        }
-        M[M_PHI * G.P32 + n] = phi;
-        M[M_GMP * G.P32 + n] = a.gphi * mup;
-        M[M_PSI * G.P32 + n] = psi;
-        M[M_GMS * G.P32 + n] = a.gpsi * mus;
-        if (ib)
-#pragma unroll
-          for (int d = 0; d < 3; ++d) a.ftot[d * G.P32 + n] = F[d];
-        if (!(rho == rho) || !(phi == phi) || !(psi == psi)) atomicOr(a.status, (unsigned)ST_NAN);
-        return;
-      }
-      // f* = f^eq(rho, u + du), written as w [drho + rho p(u)] + w rho dP with
-      // the explicitly rounded operations (see rmul)
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const Real w = Real(L::w(i));
-        const Real wrho = rmul(rho, w);
-        const Real cu = L::cx(i) * u[0] + L::cy(i) * u[1] + L::cz(i) * u[2];
-        const Real cdu = L::cx(i) * du[0] + L::cy(i) * du[1] + L::cz(i) * du[2];
-        const Real cus = L::cx(i) * us[0] + L::cy(i) * us[1] + L::cz(i) * us[2];
-        const Real pu = rfma(rmul(Real(4.5), cu), cu, rfma(Real(3), cu, rmul(Real(-1.5), uu)));
-        const Real dP = rfma(rmul(Real(4.5), cdu), cus, rfma(Real(3), cdu, rmul(Real(-1.5), dus)));
-        const Real fn = rfma(wrho, dP, rmul(w, rfma(rho, pu, drho)));
-        a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
-      }
-    } else if (a.forcing == TLB_FORCE_GUO) {
+    if (a.forcing == TLB_FORCE_GUO) {
       // Guo forcing: BGK towards f^eq(rho, v) plus (1 - om/2) w_i [3 (c_i - v) + 9 (c_i.v) c_i] . F
       const Real vF = v[0] * F[0] + v[1] * F[1] + v[2] * F[2];
       const Real sc = Real(1) - Real(0.5) * om;
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const Real w = Real(L::w(i));
-        const Real cv = L::cx(i) * v[0] + L::cy(i) * v[1] + L::cz(i) * v[2];
-        const Real cF = L::cx(i) * F[0] + L::cy(i) * F[1] + L::cz(i) * F[2];
+        const Real cv = cdot<L>(i, v);
+        const Real cF = cdot<L>(i, F);
         const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cv, vv)) +
                         sc * w * (Real(3) * (cF - vF) + Real(9) * cv * cF);
         a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
@@ -571,9 +564,9 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const Real w = Real(L::w(i));
-        const Real cu = L::cx(i) * u[0] + L::cy(i) * u[1] + L::cz(i) * u[2];
-        const Real cdu = L::cx(i) * du[0] + L::cy(i) * du[1] + L::cz(i) * du[2];
-        const Real cus = L::cx(i) * us[0] + L::cy(i) * us[1] + L::cz(i) * us[2];
+        const Real cu = cdot<L>(i, u);
+        const Real cdu = cdot<L>(i, du);
+        const Real cus = cdot<L>(i, us);
         const Real dP = Real(3) * cdu + Real(4.5) * cdu * cus - Real(1.5) * dus;
         const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cu, uu)) + w * rho * dP;
         a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
@@ -587,43 +580,25 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
       const Real om_s = set == 0 ? a.om_phi : a.om_psi;
       const Real Gm = set == 0 ? a.gphi * mup : a.gpsi * mus;
       const Real ord = set == 0 ? phi : psi;
-      Real gv[T1 ? 1 : Q];
-      if constexpr (T1) {
-        // (om_s = 1: the post-collision set is the equilibrium)
-      } else if constexpr (PF) {
+      Real gv[Q];
+      if constexpr (PF) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) gv[i] = nextv[i];
         if (set == 0) load_set(1, nextv);
       } else {
         load_set(set, gv);
       }
-      if constexpr (T1) {
-        // g* = g^eq(ord, mu, v) (om_s = 1), explicitly rounded (see rmul)
-        const Real g3 = rmul(Real(3), Gm);
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          const Real w = Real(L::w(i));
-          const Real cv = L::cx(i) * v[0] + L::cy(i) * v[1] + L::cz(i) * v[2];
-          const Real pv = rfma(rmul(Real(4.5), cv), cv, rfma(Real(3), cv, rmul(Real(-1.5), vv)));
-          const int pp = set == 0 ? plane_g<L>(i) : plane_h<L>(i);
-          a.lo_dst[pp * G.P32 + n] = from_real<Store>(rmul(w, rfma(ord, pv, g3)));
-        }
-        // ord - 3 Gm (1 - w0) - 1.5 w0 ord v^2
-        const Real ge0 = radd(rfma(g3, w0 - Real(1), ord), rmul(rmul(Real(-1.5) * w0, ord), vv));
-        a.rest_dst[(set == 0 ? 0 : G.P32) + n] = from_real<Rest>(ge0);
-      } else {
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          const Real w = Real(L::w(i));
-          const Real cv = L::cx(i) * v[0] + L::cy(i) * v[1] + L::cz(i) * v[2];
-          const Real pv = Real(3) * cv + Real(4.5) * cv * cv - Real(1.5) * vv;
-          const Real ge = w * (Real(3) * Gm + ord * pv);
-          const int pp = set == 0 ? plane_g<L>(i) : plane_h<L>(i);
-          a.lo_dst[pp * G.P32 + n] = from_real<Store>((Real(1) - om_s) * gv[i] + om_s * ge);
-        }
-        const Real ge0 = ord - Real(3) * Gm * (Real(1) - w0) - Real(1.5) * w0 * ord * vv;
-        a.rest_dst[(set == 0 ? 0 : G.P32) + n] = from_real<Rest>((Real(1) - om_s) * gv[0] + om_s * ge0);
+      for (int i = 1; i < Q; ++i) {
+        const Real w = Real(L::w(i));
+        const Real cv = cdot<L>(i, v);
+        const Real pv = Real(3) * cv + Real(4.5) * cv * cv - Real(1.5) * vv;
+        const Real ge = w * (Real(3) * Gm + ord * pv);
+        const int pp = set == 0 ? plane_g<L>(i) : plane_h<L>(i);
+        a.lo_dst[pp * G.P32 + n] = from_real<Store>((Real(1) - om_s) * gv[i] + om_s * ge);
       }
+      const Real ge0 = ord - Real(3) * Gm * (Real(1) - w0) - Real(1.5) * w0 * ord * vv;
+      a.rest_dst[(set == 0 ? 0 : G.P32) + n] = from_real<Rest>((Real(1) - om_s) * gv[0] + om_s * ge0);
     }
     if (ib)
 #pragma unroll
@@ -651,295 +626,252 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
 
 // The collide of forms 5 and 6 (tau = tau_phi = tau_psi = 1, exact
 // difference method): every post-collision population is an equilibrium of
-// the cell's moments, so nothing is pulled; the kernel is a plane sweep over
-// the moment fields that stores 3Q populations per cell (or, with moment
-// storage, the 11 moments).  Per plane: the ring plane three ahead (rho - 1,
-// phi, psi and I, tile plus a halo of 2) is copied asynchronously into the
-// 5-plane ring while the potentials of the next plane and the collision of
-// this one are computed.  The equilibria of opposite velocities share their
-// even part, and g and h share the velocity polynomial; all rounded
-// explicitly (see rmul), so every kernel it is inlined into computes the
-// same values.
-template <class L, int MODE, int TX, int TY, int FORM>
+// the cell's moments, so nothing is pulled and what is stored is the 11
+// values those equilibria are made of (see EqCell).
+//
+// A TX x TY tile of columns walks a.zc planes.  The moments of a plane (one
+// vector (rho - 1, phi, psi, j_x) per cell, tile plus a halo of 2) are copied
+// asynchronously two planes ahead into a ring of three shared-memory slots.
+// Per plane and one barrier:
+//  * the potentials: each column of the tile plus a halo of 1 reads the 9
+//    (2D: 3) moments around it in plane q, forms the in-plane sums of
+//    differences, finishes the Laplacian of plane q - 1 (whose own and lower
+//    parts are in registers) and stores that plane's potentials in one of two
+//    slots;
+//  * the force: each cell's column reads the 9 potentials around it in plane
+//    r = q - 2, finishes the force of plane r - 1, goes on with that of plane
+//    r and starts that of plane r + 1;
+//  * plane r - 1 is collided and stored.
+// So a plane of either ring is read 9 times per cell, not 19, and the sums
+// of a stencil that lie in one plane are formed once for the three planes
+// that use them.  Laplacians are sums of differences from the centre of
+// their own plane, so FP32 keeps their low bits.
+template <class L, int MODE, int TX, int TY>
 __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk& blk) {
   using Real = typename Prec<MODE>::Real;
-  using Store = typename Prec<MODE>::Store;
-  using Rest = typename Prec<MODE>::Rest;
-  constexpr int Q = L::Q;
   constexpr bool D3 = L::DIM == 3;
   constexpr int HY = D3 ? 2 : 0;
-  constexpr int MX = TX + 4, MY = TY + 2 * HY;
-  constexpr int UX = TX + 2, UY = TY + (D3 ? 2 : 0);
-  // cells per thread: two x-adjacent cells in the pair forms (8, 9)
-  constexpr int NC = form_pair<FORM>() ? 2 : 1;
-  constexpr int NT = TX / NC * TY;
-  __shared__ R4<Real> smom[5][MY * MX];  // (rho - 1, phi, psi, I) per cell
-  __shared__ R4<Real> smu[4][UY * UX];   // (mu~rho, mu_phi, mu_psi', -) per cell
+  constexpr int MX = TX + 4, MY = TY + 2 * HY, MC = MX * MY;
+  constexpr int UX = TX + 2, UY = TY + (D3 ? 2 : 0), UC = UX * UY;
+  constexpr int NT = TX * TY, NL = (MC + NT - 1) / NT, NH = UC - NT;
+  static_assert(NH <= NT, "one halo column of the potentials per thread");
+  // stencil weights: lap = 6 sum w (a_n - a), axis 6/18 (2D 6/9), edge 6/36;
+  // F = -3 sum w c (...) with the edge weight 3/36 taken out of the sum
+  constexpr double WA6 = D3 ? 1.0 / 3 : 2.0 / 3, WE6 = 1.0 / 6, AE = D3 ? 2 : 4;
+  __shared__ R4<Real> sp[3][MC];  // (rho - 1, phi, psi, j_x)
+  __shared__ R4<Real> su[2][UC];  // (mu~rho, mu_phi, mu_psi', -)
 
   const Geo G = a.G;
-  const int tid = threadIdx.x, tx = NC * (tid % (TX / NC)), ty = tid / (TX / NC);
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int x0 = blk.x * TX, y0 = blk.y * TY;
-  const int z0 = blk.z * a.zc;
-  const int z1 = min(z0 + a.zc, G.nz);
+  const int z0 = blk.z * a.zc, z1 = min(z0 + a.zc, G.nz);
   const int x = x0 + tx, y = y0 + ty;
   const bool active = x < G.nx && y < G.ny;
+  const int nxy = G.nx * G.ny;
 
-  auto modn = [](int v, int n) {
-    if (v < 0) v += n;
-    if (v >= n) v -= n;
-    if (v < 0 || v >= n) {
-      v %= n;
-      if (v < 0) v += n;
-    }
-    return v;
-  };
-  auto plane_src = [&](int p) { return G.wall ? min(max(p, 0), G.nz - 1) : modn(p, G.nz); };
-
-  // asynchronous copy of ring plane p (a wall's ghost planes mirror the
-  // plane next to the wall)
-  auto issue_plane = [&](int p) {
-    const int slot = (p + 10) % 5;
-    const long long zp = (long long)plane_src(p) * G.ny;
-    for (int k = tid; k < MX * MY; k += NT) {
-      const int hx = k % MX, hy = k / MX;
-      const int gx = modn(x0 - 2 + hx, G.nx);
-      const int gy = D3 ? modn(y0 - HY + hy, G.ny) : 0;
-      const long long c = (zp + gy) * G.nx + gx;
-      cp_async_elem(&smom[slot][k].x, a.rho + c);
-      cp_async_elem(&smom[slot][k].y, a.phi + c);
-      cp_async_elem(&smom[slot][k].z, a.psi + c);
-      cp_async_elem(&smom[slot][k].w, a.I + c);
-    }
-    cp_async_commit();
-  };
-
-  // chemical potentials of plane p on the tile plus a halo of 1
-  auto compute_mu = [&](int p) {
-    const int slot = (p + 8) % 4;
-    if (G.wall && (p < 0 || p >= G.nz)) {  // mirror ghost: mu(-1) = mu(0), mu(nz) = mu(nz-1)
-      const int src = (min(max(p, 0), G.nz - 1) + 8) % 4;
-      for (int k = tid; k < UX * UY; k += NT) smu[slot][k] = smu[src][k];
-      return;
-    }
-    const int sc = (p + 10) % 5;
-    for (int k = tid; k < UX * UY; k += NT) {
-      const int ux = k % UX, uy = k / UX;
-      const int hx = ux + 1, hy = uy + (D3 ? 1 : 0);
-      const R4<Real> cen = smom[sc][hy * MX + hx];
-      Real lap[3] = {0, 0, 0};
+  int coff[NL];  // in-plane offsets of the cells this thread copies
 #pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        const R4<Real> nbv = smom[(p + L::cz(i) + 10) % 5][(hy + L::cy(i)) * MX + hx + L::cx(i)];
-        const Real w = Real(L::w(i));
-        lap[0] += w * (nbv.x - cen.x);
-        lap[1] += w * (nbv.y - cen.y);
-        lap[2] += w * (nbv.z - cen.z);
-      }
+  for (int j = 0; j < NL; ++j) {
+    const int k = tid + j * NT, gx = halo_wrap(x0 - 2 + k % MX, G.nx);
+    coff[j] = (D3 ? halo_wrap(y0 - HY + k / MX, G.ny) * G.nx : 0) + gx;
+  }
+  auto issue = [&](int p, int slot) {
+    const R4<Real>* src = a.p4 + (long long)ring_plane(G, p) * nxy;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) lap[q] *= Real(6);  // 2/cs^2
-      Real mr, mp, ms;
-      chem_potentials<Real>(a.fe, cen.x, cen.y, cen.z, lap[0], lap[1], lap[2], cen.w, mr, mp, ms);
-      smu[slot][k] = R4<Real>{mr, mp, ms, Real(0)};
+    for (int j = 0; j < NL; ++j) {
+      const int k = tid + j * NT;
+      if (k < MC) cp_async_r4(&sp[slot][k], src + coff[j]);
     }
   };
 
-  auto collide = [&](int zz) {
+  // The columns whose potentials this thread computes: its own cell's and,
+  // for the first NH threads, one of the halo (the two rows above and below
+  // the tile, then the two columns beside it).
+  struct Col {
+    int m, u, off;       // its cell in a moments slot and in a potentials slot; in-plane offset
+    Real P[3], S[3];     // Laplacian so far of plane q - 1; in-plane sums there
+    R4<Real> c;          // centre moments of plane q - 1
+    Real I;              // membrane profile of plane q - 1
+  };
+  auto column = [&](int ux, int uy) {
+    Col o;
+    o.m = (uy + (D3 ? 1 : 0)) * MX + ux + 1;
+    o.u = uy * UX + ux;
+    o.off = (D3 ? halo_wrap(y0 - 1 + uy, G.ny) * G.nx : 0) + halo_wrap(x0 - 1 + ux, G.nx);
+    o.c = R4<Real>{0, 0, 0, 0};
+    o.I = 0;
+    for (int k = 0; k < 3; ++k) o.P[k] = o.S[k] = 0;
+    return o;
+  };
+  Col own = column(tx + 1, D3 ? ty + 1 : 0), ext;
+  const bool has_ext = tid < NH;
+  {
+    const int k = tid - 2 * UX;
+    if (!D3) ext = column(tid == 0 ? 0 : UX - 1, 0);
+    else if (tid < 2 * UX) ext = column(tid % UX, tid < UX ? 0 : UY - 1);
+    else ext = column(k & 1 ? UX - 1 : 0, 1 + k / 2);
+  }
+  // plane q of a column: finishes plane q - 1
+  auto potentials = [&](Col& o, const R4<Real>* s, R4<Real>* out, int iplane) {
+    const R4<Real> c = s[o.m], xm = s[o.m - 1], xp = s[o.m + 1];
+    Real s4[3] = {(xm.x - c.x) + (xp.x - c.x), (xm.y - c.y) + (xp.y - c.y), (xm.z - c.z) + (xp.z - c.z)};
+    Real sd[3] = {0, 0, 0};
+    if constexpr (D3) {
+      const R4<Real> ym = s[o.m - MX], yp = s[o.m + MX];
+      s4[0] += (ym.x - c.x) + (yp.x - c.x);
+      s4[1] += (ym.y - c.y) + (yp.y - c.y);
+      s4[2] += (ym.z - c.z) + (yp.z - c.z);
+      const R4<Real> a0 = s[o.m - MX - 1], a1 = s[o.m - MX + 1], a2 = s[o.m + MX - 1], a3 = s[o.m + MX + 1];
+      sd[0] = ((a0.x - c.x) + (a1.x - c.x)) + ((a2.x - c.x) + (a3.x - c.x));
+      sd[1] = ((a0.y - c.y) + (a1.y - c.y)) + ((a2.y - c.y) + (a3.y - c.y));
+      sd[2] = ((a0.z - c.z) + (a1.z - c.z)) + ((a2.z - c.z) + (a3.z - c.z));
+    }
+    // lap(q - 1) = [own plane and below] + (c - c') + S(q) / 6
+    const Real d[3] = {c.x - o.c.x, c.y - o.c.y, c.z - o.c.z};
+    Real lap[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      lap[k] = rfma(Real(WE6), s4[k], o.P[k]) + d[k];
+      o.P[k] = rfma(Real(WA6), s4[k], rfma(Real(WE6), sd[k] + o.S[k], -d[k]));
+      o.S[k] = s4[k];
+    }
+    Real mr, mp, ms;
+    chem_potentials<Real>(a.fe, o.c.x, o.c.y, o.c.z, lap[0], lap[1], lap[2], o.I, mr, mp, ms);
+    out[o.u] = R4<Real>{mr, mp, ms, Real(0)};
+    o.c = c;
+    o.I = a.I[iplane + o.off];  // (used one plane on)
+  };
+
+  // force sums (times -12) of planes r - 1 and r, and what they need: the
+  // centre moments of planes r - 1 and r, the centre potentials of r - 1
+  Real A[3] = {0, 0, 0}, B[3] = {0, 0, 0};
+  R4<Real> c1 = {0, 0, 0, 0}, c2 = {0, 0, 0, 0};
+  Real mup = 0, mus = 0;
+  // (j_y, j_z) and the brick flag of the plane collided next
+  R2<Real> jn;
+  jn.x = jn.y = 0;
+  bool ibn = false;
+  auto ahead = [&](int p) {
     if (!active) return;
-    const int n = (zz * G.ny + y) * G.nx + x;  // the (first) cell
-    // value of cell c: stored together for the two cells of a pair
-    auto put = [&](auto* p, Real v0, Real v1) {
-      using T = typename std::remove_pointer<decltype(p)>::type;
-      if constexpr (NC == 2) store_pair(p, v0, v1);
-      else *p = from_real<T>(v0);
-    };
-    // the cells' momenta first: their loads run under the stencil below
-    Real j[NC][3];
+    jn = a.j2[(p * G.ny + y) * G.nx + x];
+    ibn = a.bflag[((p >> 2) * a.nby + (y >> 2)) * a.nbx + (x >> 2)] != 0;
+  };
+
+  auto collide = [&](int zz, const Real* F12, const R4<Real>& c) {
+    const int n = (zz * G.ny + y) * G.nx + x;
+    const Real drho = c.x, phi = c.y, psi = c.z, rho = Real(1) + drho;
+    const Real j[3] = {c.w, jn.x, jn.y};
+    Real F[3], u[3], du[3], v[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      if constexpr (NC == 2) {
-        const auto jj = *reinterpret_cast<const R2<Real>*>(a.jm + d * G.P32 + n);
-        j[0][d] = jj.x;
-        j[1][d] = jj.y;
-      } else {
-        j[0][d] = a.jm[d * G.P32 + n];
-      }
+      F[d] = rmul(Real(-1.0 / 12), F12[d]);
+      if (ibn) F[d] = radd(F[d], a.fib[d * G.P32 + n]);
     }
-    // (the cells of a pair share their brick: x is even, bricks are 4 wide)
-    const bool ib = a.bflag[((zz >> 2) * a.nby + (y >> 2)) * a.nbx + (x >> 2)] != 0;
-    Real drho[NC], phi[NC], psi[NC], rho[NC], F[NC][3], u[NC][3], du[NC][3], v[NC][3], us[NC][3];
-    Real uu[NC], vv[NC], dus[NC], gmp[NC], gms[NC];
+    if (!D3) F[1] = 0;
+    const Real irho = rcp_rn(rho);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const int lx = tx + c;  // tile-local x of the cell
-      const R4<Real> mom = smom[(zz + 10) % 5][(ty + HY) * MX + lx + 2];
-      drho[c] = mom.x;
-      phi[c] = mom.y;
-      psi[c] = mom.z;
-      rho[c] = Real(1) + drho[c];
-      // gradients of the potentials (radius 1, isotropic stencil)
-      Real gm[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-      const int ux = lx + 1, uy = ty + (D3 ? 1 : 0);
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        const R4<Real> m4 = smu[(zz + L::cz(i) + 8) % 4][(uy + L::cy(i)) * UX + ux + L::cx(i)];
-        const Real w = Real(L::w(i));
-        const Real mv[3] = {m4.x, m4.y, m4.z};
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const Real vq = w * mv[q];
-          if (L::cx(i)) gm[q][0] += L::cx(i) > 0 ? vq : -vq;
-          if (L::cy(i)) gm[q][1] += L::cy(i) > 0 ? vq : -vq;
-          if (L::cz(i)) gm[q][2] += L::cz(i) > 0 ? vq : -vq;
-        }
-      }
-      const R4<Real> muc = smu[(zz + 8) % 4][uy * UX + ux];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        F[c][d] = -Real(3) * (rho[c] * gm[0][d] + phi[c] * gm[1][d] + psi[c] * gm[2][d]);
-        if (ib) F[c][d] += a.fib[d * G.P32 + n + c];
-      }
-      if (!D3) F[c][1] = 0;
-      const Real irho = Real(1) / rho[c];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        u[c][d] = j[c][d] * irho;
-        du[c][d] = F[c][d] * irho;
-        v[c][d] = u[c][d] + Real(0.5) * du[c][d];
-        us[c][d] = u[c][d] + u[c][d] + du[c][d];  // u + (u + du)
-      }
-      uu[c] = u[c][0] * u[c][0] + u[c][1] * u[c][1] + u[c][2] * u[c][2];
-      vv[c] = v[c][0] * v[c][0] + v[c][1] * v[c][1] + v[c][2] * v[c][2];
-      dus[c] = du[c][0] * us[c][0] + du[c][1] * us[c][1] + du[c][2] * us[c][2];
-      gmp[c] = a.gphi * muc.y;
-      gms[c] = a.gpsi * muc.z;
+    for (int d = 0; d < 3; ++d) {
+      u[d] = rmul(j[d], irho);
+      du[d] = rmul(F[d], irho);
+      v[d] = rfma(Real(0.5), du[d], u[d]);
     }
-    const int c1 = NC - 1;  // the second cell (the first again without pairs)
-    if (a.mst) {
-      // moment storage: the 11 values whose equilibria are this cell's
-      // post-collision populations (see EqCell)
-      Real* M = a.mst;
-      put(M + M_DRHO * G.P32 + n, drho[0], drho[c1]);
+    const Real vv = rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0])));
+    R4<Real>* M = a.M + n;
+    M[M_F * G.P32] = R4<Real>{drho, radd(u[0], du[0]), radd(u[1], du[1]), radd(u[2], du[2])};
+    M[M_ORD * G.P32] = R4<Real>{phi, rmul(Real(3), rmul(a.gphi, mup)), psi, rmul(Real(3), rmul(a.gpsi, mus))};
+    M[M_V * G.P32] = R4<Real>{v[0], v[1], v[2], rmul(Real(-1.5), vv)};
+    if (ibn)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        put(M + (M_W + d) * G.P32 + n, radd(u[0][d], du[0][d]), radd(u[c1][d], du[c1][d]));
-        put(M + (M_V + d) * G.P32 + n, v[0][d], v[c1][d]);
-      }
-      put(M + M_PHI * G.P32 + n, phi[0], phi[c1]);
-      put(M + M_GMP * G.P32 + n, gmp[0], gmp[c1]);
-      put(M + M_PSI * G.P32 + n, psi[0], psi[c1]);
-      put(M + M_GMS * G.P32 + n, gms[0], gms[c1]);
-    } else {
-      // f* = f^eq(rho, u) + w rho dP: w [drho + rho p(u)] + w rho dP; for c and
-      // -c, p = A +- 3 c.u and dP = B +- 3 c.du with the shared even parts
-      Real mu15[NC], md15[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        mu15[c] = rmul(Real(-1.5), uu[c]);
-        md15[c] = rmul(Real(-1.5), dus[c]);
-      }
-      {
-        const Real w0 = Real(L::w(0));
-        Real f0[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c)
-          f0[c] = rfma(rmul(rho[c], w0), md15[c], rmul(w0, rfma(rho[c], mu15[c], drho[c])));
-        put(a.lo_dst + plane_f<L>(0) * G.P32 + n, f0[0], f0[c1]);
-      }
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        if (L::opp(i) < i) continue;
-        const int o = L::opp(i);
-        const Real w = Real(L::w(i));
-        Real fp[NC], fm[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const Real wrho = rmul(rho[c], w);
-          const Real cu = L::cx(i) * u[c][0] + L::cy(i) * u[c][1] + L::cz(i) * u[c][2];
-          const Real cdu = L::cx(i) * du[c][0] + L::cy(i) * du[c][1] + L::cz(i) * du[c][2];
-          const Real cus = L::cx(i) * us[c][0] + L::cy(i) * us[c][1] + L::cz(i) * us[c][2];
-          const Real A = rfma(rmul(Real(4.5), cu), cu, mu15[c]);
-          const Real B = rfma(rmul(Real(4.5), cdu), cus, md15[c]);
-          fp[c] = rfma(wrho, rfma(Real(3), cdu, B), rmul(w, rfma(rho[c], rfma(Real(3), cu, A), drho[c])));
-          fm[c] = rfma(wrho, rfma(Real(-3), cdu, B), rmul(w, rfma(rho[c], rfma(Real(-3), cu, A), drho[c])));
-        }
-        put(a.lo_dst + plane_f<L>(i) * G.P32 + n, fp[0], fp[c1]);
-        put(a.lo_dst + plane_f<L>(o) * G.P32 + n, fm[0], fm[c1]);
-      }
-      // g* = g^eq(phi, mu_phi, v), h* = h^eq(psi, mu_psi', v): one velocity
-      // polynomial per pair of opposite velocities serves both
-      Real g3[NC], h3[NC], mv15[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        g3[c] = rmul(Real(3), gmp[c]);
-        h3[c] = rmul(Real(3), gms[c]);
-        mv15[c] = rmul(Real(-1.5), vv[c]);
-      }
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        if (L::opp(i) < i) continue;
-        const int o = L::opp(i);
-        const Real w = Real(L::w(i));
-        Real gp[NC], gq[NC], hp[NC], hq[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const Real cv = L::cx(i) * v[c][0] + L::cy(i) * v[c][1] + L::cz(i) * v[c][2];
-          const Real C = rfma(rmul(Real(4.5), cv), cv, mv15[c]);
-          const Real pp = rfma(Real(3), cv, C), pm = rfma(Real(-3), cv, C);
-          gp[c] = rmul(w, rfma(phi[c], pp, g3[c]));
-          gq[c] = rmul(w, rfma(phi[c], pm, g3[c]));
-          hp[c] = rmul(w, rfma(psi[c], pp, h3[c]));
-          hq[c] = rmul(w, rfma(psi[c], pm, h3[c]));
-        }
-        put(a.lo_dst + plane_g<L>(i) * G.P32 + n, gp[0], gp[c1]);
-        put(a.lo_dst + plane_g<L>(o) * G.P32 + n, gq[0], gq[c1]);
-        put(a.lo_dst + plane_h<L>(i) * G.P32 + n, hp[0], hp[c1]);
-        put(a.lo_dst + plane_h<L>(o) * G.P32 + n, hq[0], hq[c1]);
-      }
-      // rest populations close the zeroth moments: ord - 3 Gm (1 - w0) - 1.5 w0 ord v^2
-      const Real w0 = Real(L::w(0));
-      Real r0[NC], r1[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        r0[c] = radd(rfma(g3[c], w0 - Real(1), phi[c]), rmul(rmul(Real(-1.5) * w0, phi[c]), vv[c]));
-        r1[c] = radd(rfma(h3[c], w0 - Real(1), psi[c]), rmul(rmul(Real(-1.5) * w0, psi[c]), vv[c]));
-      }
-      put(a.rest_dst + n, r0[0], r0[c1]);
-      put(a.rest_dst + G.P32 + n, r1[0], r1[c1]);
-    }
-    if (ib)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) put(a.ftot + d * G.P32 + n, F[0][d], F[c1][d]);
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (!(rho[c] == rho[c]) || !(phi[c] == phi[c]) || !(psi[c] == psi[c])) atomicOr(a.status, (unsigned)ST_NAN);
+      for (int d = 0; d < 3; ++d) a.ftot[d * G.P32 + n] = F[d];
+    if (!(rho == rho) || !(phi == phi) || !(psi == psi)) atomicOr(a.status, (unsigned)ST_NAN);
   };
 
-  // prologue: ring planes z0-2 .. z0+2; potentials z0, then z0-1 and z0+1
-  // (a wall ghost copies its neighbour, so the real plane comes first); then
-  // plane z0+3 into the slot of z0-2
-  for (int p = z0 - 2; p <= z0 + 2; ++p) issue_plane(p);
-  cp_async_wait_all();
-  __syncthreads();
-  compute_mu(z0);
-  __syncthreads();
-  compute_mu(z0 - 1);
-  compute_mu(z0 + 1);
-  __syncthreads();
-  if (z0 + 3 <= z1 + 1) issue_plane(z0 + 3);
-  cp_async_wait_all();
-  __syncthreads();
-  // One barrier per plane: the potentials two planes ahead are computed in
-  // the same phase as the collision of this plane (their threads' uneven
-  // shares of the haloed potentials even out against the collisions).
-  for (int zz = z0; zz < z1; ++zz) {
-    // plane zz + 4 replaces plane zz - 1 and the potentials of zz + 2 those
-    // of zz - 2: neither is read in this iteration
-    if (zz + 4 <= z1 + 1) issue_plane(zz + 4);
-    if (zz + 2 <= z1) compute_mu(zz + 2);
-    collide(zz);
-    cp_async_wait_all();
+  issue(z0 - 2, 0);
+  cp_async_commit();
+  issue(z0 - 1, 1);
+  cp_async_commit();
+  int slot = 0;  // of plane q
+  for (int q = z0 - 2; q <= z1 + 2; ++q) {
+    cp_async_wait<1>();
     __syncthreads();
+    // plane q + 2 takes the slot of plane q - 1, which every thread has left
+    if (q + 2 <= z1 + 1) issue(q + 2, slot == 0 ? 2 : slot - 1);
+    cp_async_commit();
+    const int r = q - 2;
+    // (the potentials beyond a wall mirror those next to it: mu(-1) = mu(0),
+    // whose part is added to plane 0 with plane 0's own, and mu(nz) = mu(nz - 1))
+    if (r >= z0 - 1 && !(G.wall && r < 0)) {
+      const R4<Real>* s = su[(G.wall ? min(r, G.nz - 1) : r) & 1];
+      const int o = own.u;
+      const R4<Real> c = s[o], xm = s[o - 1], xp = s[o + 1];
+      const Real* cv = &c.x;
+      const Real gx[3] = {xp.x - xm.x, xp.y - xm.y, xp.z - xm.z};
+      Real S[3] = {xm.x + xp.x, xm.y + xp.y, xm.z + xp.z};
+      Real gy[3] = {0, 0, 0}, mx[3], my[3] = {0, 0, 0}, T[3];
+      Real gxd[3] = {0, 0, 0};
+      if constexpr (D3) {
+        const R4<Real> ym = s[o - UX], yp = s[o + UX];
+        const R4<Real> mm = s[o - UX - 1], pm = s[o - UX + 1], mp = s[o + UX - 1], pp = s[o + UX + 1];
+        const Real *ymv = &ym.x, *ypv = &yp.x, *mmv = &mm.x, *pmv = &pm.x, *mpv = &mp.x, *ppv = &pp.x;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          gy[k] = ypv[k] - ymv[k];
+          S[k] += ymv[k] + ypv[k];
+          const Real d0 = ppv[k] - mmv[k], d1 = pmv[k] - mpv[k];
+          gxd[k] = d0 + d1;
+          my[k] = rfma(Real(AE), gy[k], d0 - d1);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        T[k] = rfma(Real(AE), cv[k], S[k]);
+        mx[k] = rfma(Real(AE), gx[k], gxd[k]);
+      }
+      // weights rho, phi, psi of planes r - 1, r and r + 1 (the centre of
+      // plane r + 1 = q - 1 is the one the potentials hold)
+      const Real w1[3] = {Real(1) + c1.x, c1.y, c1.z}, w2[3] = {Real(1) + c2.x, c2.y, c2.z};
+      const Real w3[3] = {Real(1) + own.c.x, own.c.y, own.c.z};
+      Real N[3] = {0, 0, 0};
+      if (G.wall && r == 0) {  // the ghost plane below
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          B[0] = rfma(w2[k], gx[k], B[0]);
+          if (D3) B[1] = rfma(w2[k], gy[k], B[1]);
+          B[2] = rfma(-w2[k], T[k], B[2]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        A[0] = rfma(w1[k], gx[k], A[0]);
+        if (D3) A[1] = rfma(w1[k], gy[k], A[1]);
+        A[2] = rfma(w1[k], T[k], A[2]);
+        B[0] = rfma(w2[k], mx[k], B[0]);
+        if (D3) B[1] = rfma(w2[k], my[k], B[1]);
+        N[0] = rfma(w3[k], gx[k], N[0]);
+        if (D3) N[1] = rfma(w3[k], gy[k], N[1]);
+        N[2] = rfma(-w3[k], T[k], N[2]);
+      }
+      if (r > z0 && active) collide(r - 1, A, c1);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        A[d] = B[d];
+        B[d] = N[d];
+      }
+      mup = c.y;
+      mus = c.z;
+    }
+    if (r >= z0 && r < z1) ahead(r);  // collided next
+    c1 = c2;
+    c2 = own.c;
+    if (q <= z1 + 1) {
+      R4<Real>* out = su[(q - 1) & 1];
+      const int ip = ring_plane(G, q) * nxy;
+      potentials(own, sp[slot], out, ip);
+      if (has_ext) potentials(ext, sp[slot], out, ip);
+    }
+    slot = slot == 2 ? 0 : slot + 1;
   }
+  cp_async_wait<0>();
 }
 
 // The collide of a form: the tau = 1 body for forms 5 and 6, else the
@@ -947,7 +879,7 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
 template <class L, int MODE, int TX, int TY, int FORM>
 __device__ __forceinline__ void collide_body(const LBArgs<MODE>& a, const Blk& blk) {
   if constexpr (form_t1<FORM>())
-    collide_t1_body<L, MODE, TX, TY, FORM>(a, blk);
+    collide_t1_body<L, MODE, TX, TY>(a, blk);
   else
     collide_gen_body<L, MODE, TX, TY, FORM>(a, blk);
 }
@@ -955,18 +887,19 @@ __device__ __forceinline__ void collide_body(const LBArgs<MODE>& a, const Blk& b
 // (0: 640; 1: 512 with the next set prefetched; 2: 768; 3: 1024; 4: 896;
 // the tau = 1 collide at 5: 768 and 6: 1024).
 template <int FORM> constexpr int collide_threads() {
-  return FORM == 1 ? 512
-                   : (FORM == 2 || FORM == 5 ? 768
-                                             : (FORM == 3 || FORM == 6 ? 1024
-                                                                       : (FORM == 4 ? 896 : (FORM == 8 ? 384 : (FORM == 9 ? 512 : 640)))));
+  return FORM == 1 ? 512 : (FORM == 2 || FORM == 5 ? 768 : (FORM == 3 || FORM == 6 ? 1024 : (FORM == 4 ? 896 : 640)));
 }
-// threads of a collide block: one per cell of the TX x TY tile, or one per
-// pair of cells in the pair forms
-template <int FORM, int TX, int TY> constexpr int collide_block() { return form_pair<FORM>() ? TX / 2 * TY : TX * TY; }
+// threads of a collide block: one per cell of the TX x TY tile
+template <int FORM, int TX, int TY> constexpr int collide_block() { return TX * TY; }
 
+// blocks per SM of a collide; double precision takes twice the registers
+template <int MODE, int FORM, int TX, int TY> constexpr int collide_minb() {
+  constexpr int n = collide_threads<FORM>() / (MODE == TLB_F64 ? 2 : 1) / collide_block<FORM, TX, TY>();
+  return n > 0 ? n : 1;
+}
 
 template <class L, int MODE, int TX, int TY, int FORM>
-__global__ void __launch_bounds__(collide_block<FORM, TX, TY>(), collide_threads<FORM>() / collide_block<FORM, TX, TY>())
+__global__ void __launch_bounds__(collide_block<FORM, TX, TY>(), collide_minb<MODE, FORM, TX, TY>())
     k_collide(const __grid_constant__ LBArgs<MODE> a) {
   collide_body<L, MODE, TX, TY, FORM>(a, hw_blk());
 }
@@ -1003,20 +936,18 @@ __host__ tlb_status collide_variant(int v, Fn&& fn) {
     case 19: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<7>{});
     case 20: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<7>{});
     case 21: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<7>{});
-    // the tau = 1 pair forms: the three tiles with 384 and 512 threads per
-    // SM (two cells per thread)
-    case 22: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<8>{});
-    case 23: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<8>{});
-    case 24: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<8>{});
-    case 25: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<9>{});
-    case 26: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<9>{});
-    case 27: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<9>{});
-    // the tau = 1 forms on 32 x 16 tiles (3D; less halo per cell): one cell
-    // per thread at 768 / 1024 threads per SM, two at 384 / 512
-    case 28: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<5>{});
-    case 29: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<6>{});
-    case 30: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<8>{});
-    case 31: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<9>{});
+    // 22..27 name the three tiles again (they were two-cell forms of the
+    // tau = 1 collide), 28..31 the 32 x 16 tiles (3D)
+    case 22: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<5>{});
+    case 23: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<5>{});
+    case 24: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<5>{});
+    case 25: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<6>{});
+    case 26: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<6>{});
+    case 27: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<6>{});
+    case 28:
+    case 30: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<5>{});
+    case 29:
+    case 31: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<6>{});
     default: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<0>{});
   }
 }
