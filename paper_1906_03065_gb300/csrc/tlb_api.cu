@@ -260,8 +260,8 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.rho, P * R);
   take(L.phi, P * R);
   take(L.psi, P * R);
-  const size_t t1 = c.t1_ok() ? 1 : 0;  // the tau = 1 scheme's moments and state
-  take(L.p4, t1 * 4 * P * R);
+  const size_t t1 = c.t1_ok() ? 1 : 0;  // the tau = 1 scheme's momenta and state
+  take(L.p4, c.packed() ? 4 * P * R : 0);
   take(L.j2, t1 * 2 * P * R);
   take(L.M, t1 * 12 * P * R);
   take(L.I, P * R);

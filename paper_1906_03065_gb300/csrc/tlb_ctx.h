@@ -107,6 +107,9 @@ struct Ctx {
     return p.tau == 1.0 && p.tau_phi == 1.0 && p.tau_psi == 1.0 && p.forcing == TLB_FORCE_EDM &&
            p.force_form == TLB_FE_POTENTIAL;
   }
+  // the moments are kept packed, one vector per cell (the collides with the
+  // potential force read them so)
+  bool packed() const { return p.force_form == TLB_FE_POTENTIAL; }
   // a collide variant this context can run: the pressure-tensor variants for
   // the pressure-tensor force only, the tau = 1 ones only where they apply,
   // and with TLB_STATE_MOMENTS only the tau = 1 ones

@@ -34,14 +34,14 @@ struct Impl : ImplBase {
 
   // the arrays of the tau = 1 scheme, or none of them
   static void use_t1(Ctx* c, LBArgs<MODE>& a, bool t1) {
-    a.p4 = t1 ? c->ptr<R4<Real>>(c->L.p4) : nullptr;
+    a.p4 = c->packed() ? c->ptr<R4<Real>>(c->L.p4) : nullptr;
     a.j2 = t1 ? c->ptr<R2<Real>>(c->L.j2) : nullptr;
     a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
     a.pull = c->state_in_pops;
   }
   static void use_t1(Ctx* c, IBArgs<Real>& a, bool t1) {
-    a.psi = t1 ? &c->ptr<R4<Real>>(c->L.p4)->z : c->ptr<Real>(c->L.psi);
-    a.psi_step = t1 ? 4 : 1;
+    a.psi = c->packed() ? &c->ptr<R4<Real>>(c->L.p4)->z : c->ptr<Real>(c->L.psi);
+    a.psi_step = c->packed() ? 4 : 1;
     a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
   }
 

@@ -19,8 +19,9 @@ struct LBArgs {
   Real* rho;        // rho - 1 (the deviation keeps its low bits in FP32)
   Real* phi;
   Real* psi;
-  // the tau = 1 scheme (NULL otherwise):
   R4<Real>* p4;     // [P] (rho - 1, phi, psi, j_x) of the streamed populations
+                    // (NULL with the pressure-tensor force: rho, phi, psi)
+  // the tau = 1 scheme (NULL otherwise):
   R2<Real>* j2;     // [P] (j_y, j_z)
   R4<Real>* M;      // [3][P] the stored state (see EqCell)
   int pull;         // the state is in the populations, not in M (set by an
@@ -79,10 +80,12 @@ __device__ __forceinline__ void moments_store(const LBArgs<MODE>& a, int n, cons
   using Real = typename Prec<MODE>::Real;
   if (a.p4) {
     a.p4[n] = R4<Real>{m.drho, m.phi, m.psi, m.j[0]};
-    R2<Real> t;
-    t.x = m.j[1];
-    t.y = m.j[2];
-    a.j2[n] = t;
+    if (a.j2) {
+      R2<Real> t;
+      t.x = m.j[1];
+      t.y = m.j[2];
+      a.j2[n] = t;
+    }
   } else {
     a.rho[n] = m.drho;
     a.phi[n] = m.phi;
@@ -278,6 +281,116 @@ __device__ __forceinline__ Real eq_poly(Real cu, Real uu) {
   return Real(3) * cu + Real(4.5) * cu * cu - Real(1.5) * uu;
 }
 
+// Collision of one cell with its populations (eq. LBE): the three sets are
+// pulled, collided and stored one after another, so only one is live in
+// registers at a time.  rho, phi, psi are the cell's moments, F its force,
+// mup and mus its potentials mu_phi and mu_psi'.
+template <class L, int MODE>
+__device__ __forceinline__ void collide_pops(const LBArgs<MODE>& a, const Nbr<L>& nb, typename Prec<MODE>::Real phi,
+                                             typename Prec<MODE>::Real psi, typename Prec<MODE>::Real rho,
+                                             const typename Prec<MODE>::Real* F, typename Prec<MODE>::Real mup,
+                                             typename Prec<MODE>::Real mus) {
+  using Real = typename Prec<MODE>::Real;
+  using Store = typename Prec<MODE>::Store;
+  using Rest = typename Prec<MODE>::Rest;
+  constexpr int Q = L::Q;
+  const Geo& G = a.G;
+  const int n = nb.self;
+  // pull of the order-parameter set `set` (0: g, 1: h) into v
+  auto load_set = [&](int set, Real* v) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      if (i == 0) {
+        v[0] = to_real(__ldg(a.rest_src + (set == 0 ? 0 : G.P32) + n));
+      } else {
+        const int o = set == 0 ? nb.off(i, plane_g<L>(i), plane_g<L>(L::opp(i)), G.P32)
+                               : nb.off(i, plane_h<L>(i), plane_h<L>(L::opp(i)), G.P32);
+        v[i] = to_real(__ldg(a.lo_src + o));
+      }
+    }
+  };
+  // f: pull, first moment, BGK + exact difference method (eq. LBE) for f_i - w_i
+  Real fv[Q];
+  Real drho = 0, jx = 0, jy = 0, jz = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    fv[i] = to_real(__ldg(a.lo_src + nb.off(i, plane_f<L>(i), plane_f<L>(L::opp(i)), G.P32)));
+  }
+#pragma unroll
+  for (int cz = 1; cz >= -1; --cz)  // in the order of Pull::moments (rest last)
+#pragma unroll
+    for (int k = 0; k < L::NCOL; ++k) {
+      const int i = col_dir<L>(k, cz);
+      if (i <= 0) continue;
+      drho += fv[i];
+      if (L::cx(i)) jx += L::cx(i) > 0 ? fv[i] : -fv[i];
+      if (L::cy(i)) jy += L::cy(i) > 0 ? fv[i] : -fv[i];
+      if (L::cz(i)) jz += L::cz(i) > 0 ? fv[i] : -fv[i];
+    }
+  drho += fv[0];
+  const Real irho = Real(1) / rho;
+  const Real j[3] = {jx, jy, jz};
+  Real u[3], du[3], v[3], us[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    u[d] = j[d] * irho;
+    du[d] = F[d] * irho;
+    v[d] = u[d] + Real(0.5) * du[d];
+    us[d] = u[d] + u[d] + du[d];  // u + (u + du)
+  }
+  const Real uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const Real vv = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+  const Real dus = du[0] * us[0] + du[1] * us[1] + du[2] * us[2];
+  const Real om = a.om;
+  if (a.forcing == TLB_FORCE_GUO) {
+    // Guo forcing: BGK towards f^eq(rho, v) plus (1 - om/2) w_i [3 (c_i - v) + 9 (c_i.v) c_i] . F
+    const Real vF = v[0] * F[0] + v[1] * F[1] + v[2] * F[2];
+    const Real sc = Real(1) - Real(0.5) * om;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const Real w = Real(L::w(i));
+      const Real cv = cdot<L>(i, v);
+      const Real cF = cdot<L>(i, F);
+      const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cv, vv)) +
+                      sc * w * (Real(3) * (cF - vF) + Real(9) * cv * cF);
+      a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const Real w = Real(L::w(i));
+      const Real cu = cdot<L>(i, u);
+      const Real cdu = cdot<L>(i, du);
+      const Real cus = cdot<L>(i, us);
+      const Real dP = Real(3) * cdu + Real(4.5) * cdu * cus - Real(1.5) * dus;
+      const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cu, uu)) + w * rho * dP;
+      a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
+    }
+  }
+  // g and h: BGK towards the order-parameter equilibria at v (eq. EDF); the
+  // rest population closes the zeroth moment
+  const Real w0 = Real(L::w(0));
+#pragma unroll
+  for (int set = 0; set < 2; ++set) {
+    const Real om_s = set == 0 ? a.om_phi : a.om_psi;
+    const Real Gm = set == 0 ? a.gphi * mup : a.gpsi * mus;
+    const Real ord = set == 0 ? phi : psi;
+    Real gv[Q];
+    load_set(set, gv);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const Real w = Real(L::w(i));
+      const Real cv = cdot<L>(i, v);
+      const Real pv = Real(3) * cv + Real(4.5) * cv * cv - Real(1.5) * vv;
+      const Real ge = w * (Real(3) * Gm + ord * pv);
+      const int pp = set == 0 ? plane_g<L>(i) : plane_h<L>(i);
+      a.lo_dst[pp * G.P32 + n] = from_real<Store>((Real(1) - om_s) * gv[i] + om_s * ge);
+    }
+    const Real ge0 = ord - Real(3) * Gm * (Real(1) - w0) - Real(1.5) * w0 * ord * vv;
+    a.rest_dst[(set == 0 ? 0 : G.P32) + n] = from_real<Rest>((Real(1) - om_s) * gv[0] + om_s * ge0);
+  }
+}
+
 // ------------------------------------------------- fused collide + stream
 // One block owns a TX x TY tile of (x, y) columns and sweeps a chunk of z
 // planes.  Shared memory holds a 5-plane ring of the moment fields rho - 1,
@@ -337,25 +450,18 @@ __device__ __forceinline__ void pressure_tensor(const FEParams<Real>& fe, Real d
 // pressure-tensor force; the others the general one.
 template <int FORM> constexpr bool form_t1() { return FORM == 5 || FORM == 6; }
 
-template <class L, int MODE, int TX, int TY, int FORM>
-__device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Blk& blk) {
-  constexpr bool PF = FORM == 1;  // the next population set prefetched
-  // form 7: the force from the explicit pressure tensor (see pt_of)
-  constexpr bool PT = FORM == 7;
+template <class L, int MODE, int TX, int TY>
+__device__ __forceinline__ void collide_pt_body(const LBArgs<MODE>& a, const Blk& blk) {
   using Real = typename Prec<MODE>::Real;
-  using Store = typename Prec<MODE>::Store;
-  using Rest = typename Prec<MODE>::Rest;
   constexpr int Q = L::Q;
   constexpr bool D3 = L::DIM == 3;
   constexpr int HY = D3 ? 2 : 0;
   constexpr int MX = TX + 4, MY = TY + 2 * HY;
   constexpr int UX = TX + 2, UY = TY + (D3 ? 2 : 0);
   constexpr int NT = TX * TY;
-  // per cell of the potentials' ring: mu~rho, mu_phi, mu_psi'; with the
-  // pressure tensor: p_xx p_yy p_zz p_xy p_xz p_yz, kappa_c (psi - I),
-  // mu_phi, mu_psi'
-  constexpr int NMU = PT ? 9 : 3;
-  constexpr int MUP = PT ? 7 : 1, MUS = PT ? 8 : 2;  // slots of mu_phi, mu_psi'
+  // per cell of the potentials' ring: p_xx p_yy p_zz p_xy p_xz p_yz, kappa_c
+  // (psi - I), mu_phi, mu_psi'
+  constexpr int NMU = 9, MUP = 7, MUS = 8;
   __shared__ Real smom[5][3][MY * MX];
   __shared__ Real smu[3][NMU][UY * UX];
 
@@ -413,7 +519,7 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
       Real Iv = a.I[(zp + gy) * G.nx + gx];
       Real mr, mp, ms;
       chem_potentials<Real>(a.fe, cen[0], cen[1], cen[2], lap[0], lap[1], lap[2], Iv, mr, mp, ms);
-      if constexpr (PT) {
+      {
         // gradients of rho - 1, phi, psi (radius 1, isotropic stencil)
         Real gr[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
 #pragma unroll
@@ -436,18 +542,10 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
         smu[slot][6][k] = a.fe.kc * (cen[2] - Iv);
         smu[slot][MUP][k] = mp;
         smu[slot][MUS][k] = ms;
-      } else {
-        smu[slot][0][k] = mr;
-        smu[slot][1][k] = mp;
-        smu[slot][2][k] = ms;
       }
     }
   };
 
-  // Collision of one cell.  rho, phi, psi come from the moment ring (k_moments
-  // summed them in the same order as Pull::moments); the three population
-  // sets are pulled, collided and stored one after another, so only one set
-  // is live in registers at a time.
   auto collide = [&](int zz) {
     if (!active) return;
     const Nbr<L> nb(G, x, y, zz);
@@ -458,7 +556,7 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
     const Real rho = Real(1) + drho_c;
     // gradients of the potentials' ring entries (radius 1, isotropic
     // stencil; the 1/cs^2 is applied below)
-    constexpr int NG = PT ? 7 : 3;
+    constexpr int NG = 7;
     Real gm[NG][3];
 #pragma unroll
     for (int q = 0; q < NG; ++q) gm[q][0] = gm[q][1] = gm[q][2] = Real(0);
@@ -480,126 +578,20 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
     const int cc = uy * UX + ux;
     const Real mup = smu[sc][MUP][cc], mus = smu[sc][MUS][cc];
     // force (+ f_IB inside the bricks the markers spread into):
-    //  potential form: f_FE = -rho grad mu~rho - phi grad mu_phi - psi grad mu_psi'
-    //  pressure-tensor form: f_FE = -div p' - psi grad(kappa_c (psi - I)), p' the
-    //  tensor of App. A without rho cs^2 (whose divergence cancels grad rho cs^2)
+    //  f_FE = -div p' - psi grad(kappa_c (psi - I)), p' the tensor of App. A
+    //  without rho cs^2 (whose divergence cancels grad rho cs^2)
     const bool ib = a.bflag[((zz >> 2) * a.nby + (y >> 2)) * a.nbx + (x >> 2)] != 0;
     Real F[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      if constexpr (PT) {
-        // row d of the symmetric tensor: (xx, xy, xz), (xy, yy, yz), (xz, yz, zz)
-        const int r0 = d == 0 ? 0 : (d == 1 ? 3 : 4), r1 = d == 0 ? 3 : (d == 1 ? 1 : 5),
-                  r2 = d == 0 ? 4 : (d == 1 ? 5 : 2);
-        F[d] = -Real(3) * (gm[r0][0] + gm[r1][1] + gm[r2][2] + psi * gm[6][d]);
-      } else {
-        F[d] = -Real(3) * (rho * gm[0][d] + phi * gm[1][d] + psi * gm[2][d]);
-      }
+      // row d of the symmetric tensor: (xx, xy, xz), (xy, yy, yz), (xz, yz, zz)
+      const int r0 = d == 0 ? 0 : (d == 1 ? 3 : 4), r1 = d == 0 ? 3 : (d == 1 ? 1 : 5),
+                r2 = d == 0 ? 4 : (d == 1 ? 5 : 2);
+      F[d] = -Real(3) * (gm[r0][0] + gm[r1][1] + gm[r2][2] + psi * gm[6][d]);
       if (ib) F[d] += a.fib[d * G.P32 + n];
     }
     if (!D3) F[1] = 0;
-    // pull of the order-parameter set `set` (0: g, 1: h) into v
-    auto load_set = [&](int set, Real* v) {
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        if (i == 0) {
-          v[0] = to_real(__ldg(a.rest_src + (set == 0 ? 0 : G.P32) + n));
-        } else {
-          const int o = set == 0 ? nb.off(i, plane_g<L>(i), plane_g<L>(L::opp(i)), G.P32)
-                                 : nb.off(i, plane_h<L>(i), plane_h<L>(L::opp(i)), G.P32);
-          v[i] = to_real(__ldg(a.lo_src + o));
-        }
-      }
-    };
-    // f: pull, first moment, BGK + exact difference method (eq. LBE) for f_i - w_i
-    Real fv[Q];
-    Real drho = 0, jx = 0, jy = 0, jz = 0;
-    // with PF the next set's loads are in flight while this one is computed
-    Real nextv[PF ? Q : 1];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      fv[i] = to_real(__ldg(a.lo_src + nb.off(i, plane_f<L>(i), plane_f<L>(L::opp(i)), G.P32)));
-    }
-    if constexpr (PF) load_set(0, nextv);
-#pragma unroll
-    for (int cz = 1; cz >= -1; --cz)  // in the order of Pull::moments (rest last)
-#pragma unroll
-      for (int k = 0; k < L::NCOL; ++k) {
-        const int i = col_dir<L>(k, cz);
-        if (i <= 0) continue;
-        drho += fv[i];
-        if (L::cx(i)) jx += L::cx(i) > 0 ? fv[i] : -fv[i];
-        if (L::cy(i)) jy += L::cy(i) > 0 ? fv[i] : -fv[i];
-        if (L::cz(i)) jz += L::cz(i) > 0 ? fv[i] : -fv[i];
-      }
-    drho += fv[0];
-    const Real irho = Real(1) / rho;
-    const Real j[3] = {jx, jy, jz};
-    Real u[3], du[3], v[3], us[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      u[d] = j[d] * irho;
-      du[d] = F[d] * irho;
-      v[d] = u[d] + Real(0.5) * du[d];
-      us[d] = u[d] + u[d] + du[d];  // u + (u + du)
-    }
-    const Real uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const Real vv = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    const Real dus = du[0] * us[0] + du[1] * us[1] + du[2] * us[2];
-    const Real om = a.om;
-    if (a.forcing == TLB_FORCE_GUO) {
-      // Guo forcing: BGK towards f^eq(rho, v) plus (1 - om/2) w_i [3 (c_i - v) + 9 (c_i.v) c_i] . F
-      const Real vF = v[0] * F[0] + v[1] * F[1] + v[2] * F[2];
-      const Real sc = Real(1) - Real(0.5) * om;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const Real w = Real(L::w(i));
-        const Real cv = cdot<L>(i, v);
-        const Real cF = cdot<L>(i, F);
-        const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cv, vv)) +
-                        sc * w * (Real(3) * (cF - vF) + Real(9) * cv * cF);
-        a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const Real w = Real(L::w(i));
-        const Real cu = cdot<L>(i, u);
-        const Real cdu = cdot<L>(i, du);
-        const Real cus = cdot<L>(i, us);
-        const Real dP = Real(3) * cdu + Real(4.5) * cdu * cus - Real(1.5) * dus;
-        const Real fn = (Real(1) - om) * fv[i] + om * w * (drho + rho * eq_poly(cu, uu)) + w * rho * dP;
-        a.lo_dst[plane_f<L>(i) * G.P32 + n] = from_real<Store>(fn);
-      }
-    }
-    // g and h: BGK towards the order-parameter equilibria at v (eq. EDF); the
-    // rest population closes the zeroth moment
-    const Real w0 = Real(L::w(0));
-#pragma unroll
-    for (int set = 0; set < 2; ++set) {
-      const Real om_s = set == 0 ? a.om_phi : a.om_psi;
-      const Real Gm = set == 0 ? a.gphi * mup : a.gpsi * mus;
-      const Real ord = set == 0 ? phi : psi;
-      Real gv[Q];
-      if constexpr (PF) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) gv[i] = nextv[i];
-        if (set == 0) load_set(1, nextv);
-      } else {
-        load_set(set, gv);
-      }
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        const Real w = Real(L::w(i));
-        const Real cv = cdot<L>(i, v);
-        const Real pv = Real(3) * cv + Real(4.5) * cv * cv - Real(1.5) * vv;
-        const Real ge = w * (Real(3) * Gm + ord * pv);
-        const int pp = set == 0 ? plane_g<L>(i) : plane_h<L>(i);
-        a.lo_dst[pp * G.P32 + n] = from_real<Store>((Real(1) - om_s) * gv[i] + om_s * ge);
-      }
-      const Real ge0 = ord - Real(3) * Gm * (Real(1) - w0) - Real(1.5) * w0 * ord * vv;
-      a.rest_dst[(set == 0 ? 0 : G.P32) + n] = from_real<Rest>((Real(1) - om_s) * gv[0] + om_s * ge0);
-    }
+    collide_pops<L, MODE>(a, nb, phi, psi, rho, F, mup, mus);
     if (ib)
 #pragma unroll
       for (int d = 0; d < 3; ++d) a.ftot[d * G.P32 + n] = F[d];
@@ -624,10 +616,11 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
   }
 }
 
-// The collide of forms 5 and 6 (tau = tau_phi = tau_psi = 1, exact
-// difference method): every post-collision population is an equilibrium of
-// the cell's moments, so nothing is pulled and what is stored is the 11
-// values those equilibria are made of (see EqCell).
+// The collide with the potential force.  T1 (forms 5 and 6; tau = tau_phi =
+// tau_psi = 1, exact difference method): every post-collision population is
+// an equilibrium of the cell's moments, so nothing is pulled and what is
+// stored is the 11 values those equilibria are made of (see EqCell).
+// Otherwise the cell's populations are pulled, collided and stored.
 //
 // A TX x TY tile of columns walks a.zc planes.  The moments of a plane (one
 // vector (rho - 1, phi, psi, j_x) per cell, tile plus a halo of 2) are copied
@@ -646,8 +639,8 @@ __device__ __forceinline__ void collide_gen_body(const LBArgs<MODE>& a, const Bl
 // of a stencil that lie in one plane are formed once for the three planes
 // that use them.  Laplacians are sums of differences from the centre of
 // their own plane, so FP32 keeps their low bits.
-template <class L, int MODE, int TX, int TY>
-__device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk& blk) {
+template <class L, int MODE, int TX, int TY, bool T1>
+__device__ __forceinline__ void collide_body_of(const LBArgs<MODE>& a, const Blk& blk) {
   using Real = typename Prec<MODE>::Real;
   constexpr bool D3 = L::DIM == 3;
   constexpr int HY = D3 ? 2 : 0;
@@ -743,17 +736,19 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
   };
 
   // force sums (times -12) of planes r - 1 and r, and what they need: the
-  // centre moments of planes r - 1 and r, the centre potentials of r - 1
+  // centre moments of planes r - 1 and r, the centre potentials of planes
+  // r - 1 and r - 2 (their difference from plane r's is taken at the end: the
+  // sums along z then hold in-plane differences only, at their own scale)
   Real A[3] = {0, 0, 0}, B[3] = {0, 0, 0};
   R4<Real> c1 = {0, 0, 0, 0}, c2 = {0, 0, 0, 0};
-  Real mup = 0, mus = 0;
+  Real h1[3] = {0, 0, 0}, h2[3] = {0, 0, 0};
   // (j_y, j_z) and the brick flag of the plane collided next
   R2<Real> jn;
   jn.x = jn.y = 0;
   bool ibn = false;
   auto ahead = [&](int p) {
     if (!active) return;
-    jn = a.j2[(p * G.ny + y) * G.nx + x];
+    if (T1) jn = a.j2[(p * G.ny + y) * G.nx + x];
     ibn = a.bflag[((p >> 2) * a.nby + (y >> 2)) * a.nbx + (x >> 2)] != 0;
   };
 
@@ -768,6 +763,14 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
       if (ibn) F[d] = radd(F[d], a.fib[d * G.P32 + n]);
     }
     if (!D3) F[1] = 0;
+    if (ibn)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) a.ftot[d * G.P32 + n] = F[d];
+    if (!(rho == rho) || !(phi == phi) || !(psi == psi)) atomicOr(a.status, (unsigned)ST_NAN);
+    if constexpr (!T1) {
+      collide_pops<L, MODE>(a, Nbr<L>(G, x, y, zz), phi, psi, rho, F, h1[1], h1[2]);
+      return;
+    }
     const Real irho = rcp_rn(rho);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -778,12 +781,8 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
     const Real vv = rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0])));
     R4<Real>* M = a.M + n;
     M[M_F * G.P32] = R4<Real>{drho, radd(u[0], du[0]), radd(u[1], du[1]), radd(u[2], du[2])};
-    M[M_ORD * G.P32] = R4<Real>{phi, rmul(Real(3), rmul(a.gphi, mup)), psi, rmul(Real(3), rmul(a.gpsi, mus))};
+    M[M_ORD * G.P32] = R4<Real>{phi, rmul(Real(3), rmul(a.gphi, h1[1])), psi, rmul(Real(3), rmul(a.gpsi, h1[2]))};
     M[M_V * G.P32] = R4<Real>{v[0], v[1], v[2], rmul(Real(-1.5), vv)};
-    if (ibn)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) a.ftot[d * G.P32 + n] = F[d];
-    if (!(rho == rho) || !(phi == phi) || !(psi == psi)) atomicOr(a.status, (unsigned)ST_NAN);
   };
 
   issue(z0 - 2, 0);
@@ -806,8 +805,8 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
       const R4<Real> c = s[o], xm = s[o - 1], xp = s[o + 1];
       const Real* cv = &c.x;
       const Real gx[3] = {xp.x - xm.x, xp.y - xm.y, xp.z - xm.z};
-      Real S[3] = {xm.x + xp.x, xm.y + xp.y, xm.z + xp.z};
-      Real gy[3] = {0, 0, 0}, mx[3], my[3] = {0, 0, 0}, T[3];
+      Real S[3] = {(xm.x - c.x) + (xp.x - c.x), (xm.y - c.y) + (xp.y - c.y), (xm.z - c.z) + (xp.z - c.z)};
+      Real gy[3] = {0, 0, 0}, mx[3], my[3] = {0, 0, 0};
       Real gxd[3] = {0, 0, 0};
       if constexpr (D3) {
         const R4<Real> ym = s[o - UX], yp = s[o + UX];
@@ -816,17 +815,14 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
           gy[k] = ypv[k] - ymv[k];
-          S[k] += ymv[k] + ypv[k];
+          S[k] += (ymv[k] - cv[k]) + (ypv[k] - cv[k]);
           const Real d0 = ppv[k] - mmv[k], d1 = pmv[k] - mpv[k];
           gxd[k] = d0 + d1;
           my[k] = rfma(Real(AE), gy[k], d0 - d1);
         }
       }
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        T[k] = rfma(Real(AE), cv[k], S[k]);
-        mx[k] = rfma(Real(AE), gx[k], gxd[k]);
-      }
+      for (int k = 0; k < 3; ++k) mx[k] = rfma(Real(AE), gx[k], gxd[k]);
       // weights rho, phi, psi of planes r - 1, r and r + 1 (the centre of
       // plane r + 1 = q - 1 is the one the potentials hold)
       const Real w1[3] = {Real(1) + c1.x, c1.y, c1.z}, w2[3] = {Real(1) + c2.x, c2.y, c2.z};
@@ -837,28 +833,29 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
         for (int k = 0; k < 3; ++k) {
           B[0] = rfma(w2[k], gx[k], B[0]);
           if (D3) B[1] = rfma(w2[k], gy[k], B[1]);
-          B[2] = rfma(-w2[k], T[k], B[2]);
+          B[2] = rfma(-w2[k], S[k], B[2]);
+          h1[k] = cv[k];
         }
       }
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         A[0] = rfma(w1[k], gx[k], A[0]);
         if (D3) A[1] = rfma(w1[k], gy[k], A[1]);
-        A[2] = rfma(w1[k], T[k], A[2]);
+        A[2] = rfma(w1[k], rfma(Real(6), cv[k] - h2[k], S[k]), A[2]);
         B[0] = rfma(w2[k], mx[k], B[0]);
         if (D3) B[1] = rfma(w2[k], my[k], B[1]);
         N[0] = rfma(w3[k], gx[k], N[0]);
         if (D3) N[1] = rfma(w3[k], gy[k], N[1]);
-        N[2] = rfma(-w3[k], T[k], N[2]);
+        N[2] = rfma(-w3[k], S[k], N[2]);
       }
       if (r > z0 && active) collide(r - 1, A, c1);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         A[d] = B[d];
         B[d] = N[d];
+        h2[d] = h1[d];
+        h1[d] = cv[d];
       }
-      mup = c.y;
-      mus = c.z;
     }
     if (r >= z0 && r < z1) ahead(r);  // collided next
     c1 = c2;
@@ -874,17 +871,16 @@ __device__ __forceinline__ void collide_t1_body(const LBArgs<MODE>& a, const Blk
   cp_async_wait<0>();
 }
 
-// The collide of a form: the tau = 1 body for forms 5 and 6, else the
-// general one.
+// The collide of a form.
 template <class L, int MODE, int TX, int TY, int FORM>
 __device__ __forceinline__ void collide_body(const LBArgs<MODE>& a, const Blk& blk) {
-  if constexpr (form_t1<FORM>())
-    collide_t1_body<L, MODE, TX, TY>(a, blk);
+  if constexpr (FORM == 7)
+    collide_pt_body<L, MODE, TX, TY>(a, blk);
   else
-    collide_gen_body<L, MODE, TX, TY, FORM>(a, blk);
+    collide_body_of<L, MODE, TX, TY, form_t1<FORM>()>(a, blk);
 }
 // Forms of the collide: threads per SM the register budget is set for
-// (0: 640; 1: 512 with the next set prefetched; 2: 768; 3: 1024; 4: 896;
+// (0: 640; 1: 512; 2: 768; 3: 1024; 4: 896; pressure tensor at 7: 640;
 // the tau = 1 collide at 5: 768 and 6: 1024).
 template <int FORM> constexpr int collide_threads() {
   return FORM == 1 ? 512 : (FORM == 2 || FORM == 5 ? 768 : (FORM == 3 || FORM == 6 ? 1024 : (FORM == 4 ? 896 : 640)));
