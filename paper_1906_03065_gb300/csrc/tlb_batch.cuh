@@ -158,7 +158,7 @@ struct BatchImpl : BatchBase {
       case PRE: return {mem ? (int)std::min<unsigned>(64, std::max(1u, cdiv(3ll * c->nn, NT))) : 0, 1, 1};
       case MOM:
         if (!variant_t1(b->tile_variant)) return {(int)cdiv(c->N, NT), 1, 1};
-        return {(int)cdiv(c->nx, recon_x<L>()), (int)cdiv(c->ny, recon_y<L>()), (int)cdiv(c->nz, I::RECON_ZC)};
+        return {(int)cdiv(c->nx, recon_x<L>()), (int)cdiv(c->ny, recon_y<L>()), (int)cdiv(c->nz, b->recon_zc)};
       case GEOM: return {mem ? (int)cdiv((long long)c->ne + c->nn, NT) : 0, 1, 1};
       case BCOUNT: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
       case NODEF: return {mem ? (int)cdiv(32ll * c->nn, NT) : 0, 1, 1};
@@ -337,6 +337,7 @@ struct BatchImpl : BatchBase {
         BA& a = t[j];
         a.lb = I::lbargs(c, t1 ? c->cur : c->cur ^ q);
         a.lb.zc = b->zc;
+        a.lb.zcm = b->recon_zc;
         I::use_t1(c, a.lb, t1);
         if (q == 0) a.lb.pull = 0;
         if (t1 && scratch) a.lb.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);

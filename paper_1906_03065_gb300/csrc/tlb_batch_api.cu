@@ -118,7 +118,6 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
   }
   s = cuda_check(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking), "batch capture stream");
   if (s != TLB_OK) { delete b; return s; }
-  int nzmax = 1;
   for (int i = 0; i < n_inst; ++i) {
     void* h = nullptr;
     s = tlb_create(&inst[i].params, inst[i].mems, inst[i].n_mem, b->base + bp.off[i], bp.bytes[i], cuda_stream, &h);
@@ -134,12 +133,10 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
     box_estimates(c, &bb, &sb);
     b->band_blocks.push_back(bb);
     b->spread_blocks.push_back(sb);
-    nzmax = std::max(nzmax, c->nz);
   }
-  b->zc = nzmax >= 64 ? 16 : std::min(nzmax, 8);
   // the tau = 1 collide wherever it applies; one force form per batch
-  b->tile_variant = 0;
-  for (int v : {13, 19, 0}) {
+  b->tile_variant = 3;
+  for (int v : {13, 19, 3}) {
     bool ok = true;
     for (Ctx* c : b->inst) ok = ok && c->variant_ok(v);
     if (ok) {
@@ -153,6 +150,10 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
       delete b;
       return TLB_ERR_ARG;
     }
+  // chunks of the plane sweeps over all instances together (the rebuild in
+  // the phases' 128-thread blocks)
+  b->zc = b->inst[0]->impl->collide_chunk(b->inst, b->tile_variant);
+  b->recon_zc = b->inst[0]->impl->recon_chunk(b->inst, b->dim == 3 ? 32 : 128, b->dim == 3 ? 4 : 1);
   for (int q = 0; q < 2; ++q) b->targs[q] = {bp.targs[q], (size_t)n_inst * Batch::ARGS_BYTES};
   b->vg = {bp.vg, (size_t)Batch::NPH * Batch::MAXOPS * n_inst * 16};
   b->res = {bp.res, (size_t)n_inst * 4 * 8};

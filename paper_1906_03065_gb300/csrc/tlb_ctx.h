@@ -35,6 +35,53 @@ inline std::vector<int> z_chunk_candidates(int nz) {
   return v;
 }
 
+// Length of the z chunks of a plane sweep.  A block of the sweep walks its
+// chunk plus `ahead` planes that only fill its rings and running sums, and
+// `resident` blocks share an SM; a plane of a block takes 1 + load * b in
+// units of what it takes alone when b blocks of the SM run beside each other
+// (load: 0 if they only hid each other's latency, large if they only queued
+// for the SM's arithmetic).  Short chunks repeat the `ahead` planes, long
+// ones leave SMs idle on small lattices or end in a nearly empty last wave:
+// the chunk taken is the one with the least sum over its waves.  `tiles`:
+// column tiles and planes of each lattice swept together.
+struct SweepCost {
+  int resident;
+  double ahead, load;
+};
+struct SweepTiles {
+  long long columns;
+  int nz;
+};
+inline int sweep_chunk(const std::vector<SweepTiles>& tiles, int nsm, const SweepCost& s) {
+  int nzmax = 1, best = 1;
+  for (const SweepTiles& t : tiles) nzmax = t.nz > nzmax ? t.nz : nzmax;
+  double tbest = 0;
+  for (int m = 1, last = 0; m <= nzmax; ++m) {
+    const int zc = (nzmax + m - 1) / m;
+    if (zc == last) continue;
+    last = zc;
+    long long n = 0;
+    for (const SweepTiles& t : tiles) n += t.columns * ((t.nz + zc - 1) / zc);
+    const long long cap = (long long)s.resident * nsm, rest = n % cap;
+    const double t = (zc + s.ahead) * ((double)(n / cap) * (1 + s.load * s.resident) +
+                                       (rest ? 1 + s.load * (double)((rest + nsm - 1) / nsm) : 0));
+    if (tbest == 0 || t < tbest) {
+      tbest = t;
+      best = zc;
+    }
+  }
+  return best;
+}
+// The collide and the moments rebuild.  The numbers fit timings of every
+// chunk length on 64^2 and 240x120 (FP64, FP32) and 41x37x35 to 192x128x128
+// lattices; the chunk taken was within 8% of the fastest one on each, where a
+// fixed one (32 planes from nz = 64, else 8) lost 15% at 128^3 (71 against 61
+// us), a factor 2 at 64^3 (43 against 18) and 7 at 64^2 FP64 (225 against 30).
+inline SweepCost collide_cost(int resident, int threads, bool f64, bool t1) {
+  return {resident, t1 ? 5.0 : 3.0, (f64 ? 0.47 : (t1 ? 0.15 : 0.5)) * threads / 128};
+}
+inline SweepCost recon_cost(int resident, int threads, bool f64) { return {resident, 3.0, (f64 ? 0.8 : 0.6) * threads / 128}; }
+
 struct Ctx;
 
 struct ImplBase {
@@ -59,6 +106,10 @@ struct ImplBase {
   // write the populations that the state in M stands for into the current
   // population buffer if it is stale (no-op otherwise)
   virtual tlb_status sync_pops(Ctx* c) = 0;
+  // chunk lengths of the plane sweeps for lattices swept together (the
+  // default collide variant; the moments rebuild in blocks of bt threads)
+  virtual int collide_chunk(const std::vector<Ctx*>& cs, int variant) = 0;
+  virtual int recon_chunk(const std::vector<Ctx*>& cs, int tx, int ty) = 0;
 };
 
 // CUDA events bracketing the phases of a step when profiling.
@@ -151,6 +202,7 @@ struct Ctx {
   int nn = 0, ne = 0, NV = 0, ncap = 0, nedge = 0;
   int nbx = 0, nby = 0, nbz = 0, nbricks = 0;
   int tiles_zc = 16;
+  int recon_zc = 16;     // the same of the moments rebuild
   int tile_variant = 0;  // collide tile shape and form (see collide_variant)
   PhaseEvents* prof = nullptr;  // non-null while tlb_profile_steps runs
   double prof_ms[4] = {0, 0, 0, 0};
@@ -231,7 +283,7 @@ struct Batch {
   cudaGraphExec_t graph = nullptr;
   bool graph_dirty = true;
   long graph_launches = 0;  // kernels in one launch of the step graph
-  int tile_variant = 0, zc = 16;
+  int tile_variant = 0, zc = 16, recon_zc = 16;
   long launches = 0;
   BatchBase* impl = nullptr;
 

@@ -18,7 +18,7 @@ struct Impl : ImplBase {
   using Rest = typename Prec<MODE>::Rest;
 
   // tiles of the rebuilding moments sweep
-  static constexpr int RECON_X = L::DIM == 3 ? 32 : 64, RECON_Y = L::DIM == 3 ? 4 : 1, RECON_ZC = 16;
+  static constexpr int RECON_X = L::DIM == 3 ? 32 : 64, RECON_Y = L::DIM == 3 ? 4 : 1;
 
   static Geo geo(const Ctx* c) {
     Geo g;
@@ -73,7 +73,7 @@ struct Impl : ImplBase {
     a.gphi = (Real)c->p.gamma_phi;
     a.gpsi = (Real)c->p.gamma_psi;
     a.zc = c->tiles_zc;
-    a.zcm = RECON_ZC;
+    a.zcm = c->recon_zc;
     a.forcing = c->p.forcing;
     a.status = c->ptr<unsigned>(c->L.status);
     return a;
@@ -273,6 +273,26 @@ struct Impl : ImplBase {
     c->state_in_pops = true;
     c->pops_stale = false;
     return TLB_OK;
+  }
+
+  static std::vector<SweepTiles> sweep_tiles(const std::vector<Ctx*>& cs, int tx, int ty) {
+    std::vector<SweepTiles> t;
+    for (const Ctx* c : cs) t.push_back({(long long)blocks(c->nx, tx) * blocks(c->ny, ty), c->nz});
+    return t;
+  }
+  int collide_chunk(const std::vector<Ctx*>& cs, int variant) override {
+    constexpr bool f64 = MODE == TLB_F64;
+    int zc = 1;
+    collide_variant<L>(variant, [&](auto tx, auto ty, auto fm) {
+      constexpr int TX = decltype(tx)::value, TY = decltype(ty)::value, FM = decltype(fm)::value;
+      zc = sweep_chunk(sweep_tiles(cs, TX, TY), cs[0]->nsm,
+                       collide_cost(collide_minb<MODE, FM, TX, TY>(), TX * TY, f64, form_t1<FM>()));
+      return TLB_OK;
+    });
+    return zc;
+  }
+  int recon_chunk(const std::vector<Ctx*>& cs, int tx, int ty) override {
+    return sweep_chunk(sweep_tiles(cs, tx, ty), cs[0]->nsm, recon_cost(768 / (tx * ty), tx * ty, MODE == TLB_F64));
   }
 
   tlb_status sync_pops(Ctx* c) override {

@@ -880,10 +880,11 @@ __device__ __forceinline__ void collide_body(const LBArgs<MODE>& a, const Blk& b
     collide_body_of<L, MODE, TX, TY, form_t1<FORM>()>(a, blk);
 }
 // Forms of the collide: threads per SM the register budget is set for
-// (0: 640; 1: 512; 2: 768; 3: 1024; 4: 896; pressure tensor at 7: 640;
-// the tau = 1 collide at 5: 768 and 6: 1024).
+// (0: 640; 1: 512; 2: 768; 3: 1024; 4: 896; the tau = 1 collide at 5: 640 and
+// 6: 768; the pressure tensor at 7: 640).  The tau = 1 collide holds about 90
+// values per thread: at 768 threads per SM it spilled 52 bytes.
 template <int FORM> constexpr int collide_threads() {
-  return FORM == 1 ? 512 : (FORM == 2 || FORM == 5 ? 768 : (FORM == 3 || FORM == 6 ? 1024 : (FORM == 4 ? 896 : 640)));
+  return FORM == 1 ? 512 : (FORM == 2 || FORM == 6 ? 768 : (FORM == 3 ? 1024 : (FORM == 4 ? 896 : 640)));
 }
 // threads of a collide block: one per cell of the TX x TY tile
 template <int FORM, int TX, int TY> constexpr int collide_block() { return TX * TY; }
