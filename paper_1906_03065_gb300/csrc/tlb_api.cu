@@ -386,6 +386,7 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
     if (r0 != TLB_OK) { delete c; return r0; }
   }
   c->tiles_zc = c->impl->collide_chunk({c}, c->tile_variant);
+  c->scat_split = scatter_split((c->features() + 31) / 32, params->dc, c->nsm);
   c->recon_zc = c->impl->recon_chunk({c}, params->dim == 3 ? 32 : 64, params->dim == 3 ? 4 : 1);
   // zero everything, then set the non-zero initial values
   tlb_status r = cuda_check(cudaMemsetAsync(c->base, 0, c->L.total, st), "memset arena");

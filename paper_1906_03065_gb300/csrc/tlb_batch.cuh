@@ -163,8 +163,7 @@ struct BatchImpl : BatchBase {
       case BCOUNT: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
       case NODEF: return {mem ? (int)cdiv(32ll * c->nn, NT) : 0, 1, 1};
       case SCAT: {
-        const long long nfeat = (long long)c->ne + (c->NV == 3 ? c->nedge : 0) + c->nn;
-        return {mem ? SCAT_SPLIT * (int)cdiv(nfeat, 32 * scatter_warps<typename Prec<MODE>::Real>()) : 0, 1, 1};
+        return {mem ? b->scat_split * (int)cdiv(c->features(), 32 * scatter_warps<typename Prec<MODE>::Real>()) : 0, 1, 1};
       }
       case BCOMP: return {mem ? (int)cdiv(c->nbricks, NT) : 0, 1, 1};
       case BAND: return {mem ? b->band_blocks[i] : 0, 1, 1};
@@ -343,6 +342,7 @@ struct BatchImpl : BatchBase {
         if (t1 && scratch) a.lb.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
         a.ib = I::ibargs(c);
         I::use_t1(c, a.ib, t1);
+        a.ib.split = b->scat_split;
         a.rp = I::resptrs(c, b->ptr<unsigned long long>(b->res) + 4 * (size_t)b->act[j]);
       }
       TLB_CUDA(cudaMemcpyAsync(b->ptr<char>(b->targs[q]), t.data(), (size_t)n * sizeof(BA), cudaMemcpyHostToDevice,

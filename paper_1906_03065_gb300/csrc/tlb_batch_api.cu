@@ -154,6 +154,13 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
   // the phases' 128-thread blocks)
   b->zc = b->inst[0]->impl->collide_chunk(b->inst, b->tile_variant);
   b->recon_zc = b->inst[0]->impl->recon_chunk(b->inst, b->dim == 3 ? 32 : 128, b->dim == 3 ? 4 : 1);
+  long long warps = 0;
+  double dcmax = 0;
+  for (Ctx* c : b->inst) {
+    warps += (c->features() + 31) / 32;
+    dcmax = std::max(dcmax, c->p.dc);
+  }
+  b->scat_split = scatter_split(warps, dcmax, b->inst[0]->nsm);
   for (int q = 0; q < 2; ++q) b->targs[q] = {bp.targs[q], (size_t)n_inst * Batch::ARGS_BYTES};
   b->vg = {bp.vg, (size_t)Batch::NPH * Batch::MAXOPS * n_inst * 16};
   b->res = {bp.res, (size_t)n_inst * 4 * 8};

@@ -82,6 +82,14 @@ inline SweepCost collide_cost(int resident, int threads, bool f64, bool t1) {
 }
 inline SweepCost recon_cost(int resident, int threads, bool f64) { return {resident, 3.0, (f64 ? 0.8 : 0.6) * threads / 128}; }
 
+// Warps that share one group of 32 features in the distance scatter: as many
+// as bring its warps to 16 per SM, at most one per round of slices (4 slices
+// each, 2 dc + 3 per feature or so); for `warps` groups swept together.
+inline int scatter_split(long long warps, double dc, int nsm) {
+  const long long rounds = ((long long)(2 * dc) + 3 + 3) / 4, want = (16ll * nsm + warps / 2) / (warps > 0 ? warps : 1);
+  return (int)(want < 1 ? 1 : (want > rounds ? rounds : want));
+}
+
 struct Ctx;
 
 struct ImplBase {
@@ -203,6 +211,8 @@ struct Ctx {
   int nbx = 0, nby = 0, nbz = 0, nbricks = 0;
   int tiles_zc = 16;
   int recon_zc = 16;     // the same of the moments rebuild
+  int scat_split = 1;    // see scatter_split
+  long long features() const { return (long long)ne + nedge + nn; }  // of the distance scatter
   int tile_variant = 0;  // collide tile shape and form (see collide_variant)
   PhaseEvents* prof = nullptr;  // non-null while tlb_profile_steps runs
   double prof_ms[4] = {0, 0, 0, 0};
@@ -283,7 +293,7 @@ struct Batch {
   cudaGraphExec_t graph = nullptr;
   bool graph_dirty = true;
   long graph_launches = 0;  // kernels in one launch of the step graph
-  int tile_variant = 0, zc = 16, recon_zc = 16;
+  int tile_variant = 0, zc = 16, recon_zc = 16, scat_split = 1;
   long launches = 0;
   BatchBase* impl = nullptr;
 

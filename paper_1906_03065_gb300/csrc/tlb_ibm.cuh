@@ -34,6 +34,7 @@ struct IBArgs {
   const Real* skc;       // 3D: per triangle G0i[0], 2 G0i[1], G0i[2], det G0i, A0 (working precision)
   const Real* capr;      // per capsule ks, kb, G, C (working precision), [4][ncaps]
   int ncaps;
+  int split;             // virtual blocks sharing one block of features (distance scatter)
   const int* inc_off;    // node -> incident elements (CSR, ascending)
   const int* inc;
   const int* adj;        // 3D: triangle across edge q (q: vertex q -> q+1)
@@ -367,101 +368,6 @@ __device__ __forceinline__ unsigned long long dist_code(double d) {
   return (unsigned long long)(d * 17179869184.0);
 }
 
-// Squared distance from a point to a triangle (or a segment), without
-// branches: the projection onto the plane when it falls inside the
-// triangle, else the nearest of the three clamped edge projections.  The
-// per-face quantities are set up once; a point costs about fifty
-// arithmetic instructions and no divergence.
-template <class Real>
-struct FaceDist {
-  V3<Real> A, B, ab, ac, bc;
-  Real d00, d01, d11, i00, i11, ibc, iden;
-  bool tri;
-  static constexpr int NC = 22;  // constants kept in shared memory
-  static constexpr int NCP = 24; // row stride of the shared copy (16-byte rows for FP32)
-  __device__ __forceinline__ FaceDist() {}
-  __device__ __forceinline__ void store(Real* p) const {
-    const Real v[NC] = {A.x,  A.y,  A.z,  B.x,  B.y,  B.z,  ab.x, ab.y, ab.z, ac.x, ac.y,
-                        ac.z, bc.x, bc.y, bc.z, d00,  d01,  d11,  i00,  i11,  ibc,  iden};
-    for (int i = 0; i < NC; ++i) p[i] = v[i];
-  }
-  __device__ __forceinline__ static FaceDist load(const Real* p, bool is_tri) {
-    if constexpr (sizeof(Real) == 4) {  // six 16-byte loads of the padded row
-      float v[NCP];
-#pragma unroll
-      for (int i = 0; i < NCP / 4; ++i) {
-        const float4 q = reinterpret_cast<const float4*>(p)[i];
-        v[4 * i] = q.x;
-        v[4 * i + 1] = q.y;
-        v[4 * i + 2] = q.z;
-        v[4 * i + 3] = q.w;
-      }
-      FaceDist f;
-      f.A = mk<Real>(v[0], v[1], v[2]);
-      f.B = mk<Real>(v[3], v[4], v[5]);
-      f.ab = mk<Real>(v[6], v[7], v[8]);
-      f.ac = mk<Real>(v[9], v[10], v[11]);
-      f.bc = mk<Real>(v[12], v[13], v[14]);
-      f.d00 = v[15];
-      f.d01 = v[16];
-      f.d11 = v[17];
-      f.i00 = v[18];
-      f.i11 = v[19];
-      f.ibc = v[20];
-      f.iden = v[21];
-      f.tri = is_tri;
-      return f;
-    }
-    FaceDist f;
-    f.A = mk<Real>(p[0], p[1], p[2]);
-    f.B = mk<Real>(p[3], p[4], p[5]);
-    f.ab = mk<Real>(p[6], p[7], p[8]);
-    f.ac = mk<Real>(p[9], p[10], p[11]);
-    f.bc = mk<Real>(p[12], p[13], p[14]);
-    f.d00 = p[15];
-    f.d01 = p[16];
-    f.d11 = p[17];
-    f.i00 = p[18];
-    f.i11 = p[19];
-    f.ibc = p[20];
-    f.iden = p[21];
-    f.tri = is_tri;
-    return f;
-  }
-  __device__ __forceinline__ FaceDist(V3<Real> a, V3<Real> b, V3<Real> c, bool is_tri) : A(a), B(b), tri(is_tri) {
-    ab = b - a;
-    ac = c - a;
-    bc = c - b;
-    d00 = dot(ab, ab);
-    d01 = dot(ab, ac);
-    d11 = dot(ac, ac);
-    const Real dbc = dot(bc, bc), den = d00 * d11 - d01 * d01;
-    i00 = d00 > Real(0) ? rcp_rn(d00) : Real(0);  // degenerate edge: its first end
-    i11 = d11 > Real(0) ? rcp_rn(d11) : Real(0);
-    ibc = dbc > Real(0) ? rcp_rn(dbc) : Real(0);
-    iden = den > Real(0) ? rcp_rn(den) : Real(0);  // degenerate face: edges only
-  }
-  __device__ __forceinline__ Real dist2(V3<Real> x) const {
-    const V3<Real> ap = x - A;
-    const Real d20 = dot(ap, ab);
-    const Real t0 = fmin(Real(1), fmax(Real(0), d20 * i00));
-    const V3<Real> e0 = ap - t0 * ab;
-    Real best = dot(e0, e0);
-    if (!tri) return best;
-    const Real d21 = dot(ap, ac);
-    const Real t1 = fmin(Real(1), fmax(Real(0), d21 * i11));
-    const V3<Real> e1 = ap - t1 * ac;
-    const V3<Real> bp = x - B;
-    const Real t2 = fmin(Real(1), fmax(Real(0), dot(bp, bc) * ibc));
-    const V3<Real> e2 = bp - t2 * bc;
-    best = fmin(best, fmin(dot(e1, e1), dot(e2, e2)));
-    const Real v = (d11 * d20 - d01 * d21) * iden, w = (d00 * d21 - d01 * d20) * iden;
-    const V3<Real> q = ap - v * ab - w * ac;
-    const bool inside = iden > Real(0) && v >= Real(0) && w >= Real(0) && v + w <= Real(1);
-    return inside ? dot(q, q) : best;
-  }
-};
-
 // ------------------------------------------------------------ distance scatter
 // Every cell within dc of the membrane must receive the key (distance,
 // element) of its nearest element; keys are combined with atomicMin.  The
@@ -471,16 +377,26 @@ struct FaceDist {
 // edge, the cone of the face normals around a vertex (in 2D: segment normal,
 // and the fan of the two segment normals at a marker).  Each feature sweeps
 // the cells x = P + t m, P on the feature, m in its cone (either sign),
-// |t| < dc, and offers every cell the exact distance to the faces that
-// contain the feature.  The sweep runs slice by slice along an axis k in
-// which all cone generators have a component of one sign; on slice x_k = c
-// the region lies in the convex hull of the points where the rays from the
-// feature's corners along the generators meet the slice, whose bounding box
-// is enumerated.  Distances are compared on a grid of 2^-34 lattice units,
-// ties going to the lowest element index.
+// |t| < dc.  The sweep runs slice by slice along an axis k in which all cone
+// generators have a component of one sign; on slice x_k = c the region lies
+// in the convex hull of the points where the rays from the feature's corners
+// along the generators meet the slice, whose bounding box is enumerated.
+// Distances are compared on a grid of 2^-34 lattice units, ties going to the
+// lowest element index.
+//
+// A feature offers its lowest-index face at the cell's distance to the
+// feature itself: to the face's plane where the cell projects into the face,
+// to the edge where it projects between the edge's ends (ends included, with
+// the distance clamped to them), to the vertex.  Where P lies on the feature
+// that is |x - P|; elsewhere it is a larger distance, or nothing is offered
+// and the feature that holds P offers it.  (The boxes are widened by 1e-3
+// cells and the ends of an edge likewise, far above the rounding of either
+// test, so a cell on the border of two features is offered by one of them.)
+// So a cell costs three dot products for a face, two for an edge and one for
+// a vertex, where the exact distance to the offered face took seven.
 constexpr int MAXG = 12;  // generators (and faces) per feature
 constexpr int SCAT_W = 4;       // slices per lane per round
-constexpr int SCAT_SPLIT = 4;   // warps sharing one group of 32 features (round r goes to r % SCAT_SPLIT)
+constexpr int SCAT_TAB = 1024;  // cells laid out at a time
 // warps per block (every lane sweeps one feature): FP64 halves them to keep
 // the shared memory under the static limit
 template <class Real> constexpr int scatter_warps() { return sizeof(Real) == 4 ? 4 : 2; }
@@ -492,24 +408,20 @@ struct ScatterWarp {
   Real gk[32][MAXG];            // 1 / generator component along the slice axis
   Real ga[32][MAXG];            // generator components along the two other axes
   Real gb[32][MAXG];
-  alignas(16) Real fd[32][FaceDist<Real>::NCP];  // distance constants of the offered face
-  int4 sl[32][SCAT_W];          // the round's slices: a0, b0, width, cumulative cells
+  R4<Real> rec[32][3];          // what the distance needs (see offer below)
+  int4 sl[32][SCAT_W];          // the round's slices: a0, b0, width, first cell
   int4 ft[32][2];               // origin cell (wrapped) and packed axes; face, first slice
+  unsigned char tab[SCAT_TAB];  // slice (lane * SCAT_W + h) of each cell of the round
 };
 
 // One lane per feature, geometry in Real relative to an integer origin (the
 // lattice cell below the first corner), so the FP32 build sweeps in single
-// precision without losing accuracy; slice boxes are widened by 1e-3 cells
-// to stay conservative under rounding.  The warp then shares out the cells:
+// precision without losing accuracy.  The warp then shares out the cells:
 // per round every lane sizes SCAT_W slices of its feature, a warp prefix sum
-// lays all their cells end to end, and the lanes take them round-robin.
-// SCAT_SPLIT virtual blocks set up the same features and take turns over
-// the rounds (the set-up is short; the rounds are not).
-// A feature offers only its lowest-index face: if the nearest point P of a
-// cell lies on the feature, every face containing the feature is at exactly
-// |x - P|, so that face carries the key the tie rule selects; faces offered
-// for cells whose nearest point lies elsewhere are at their exact (larger or
-// equal) distance and cannot win wrongly.
+// lays all their cells end to end, every lane enters its slices in a table
+// over them, and the lanes take the cells round-robin.  `split` virtual
+// blocks set up the same features and take turns over the rounds (the set-up
+// is short; the rounds are not; see scatter_split).
 template <class Real>
 __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const Blk& blk) {
   constexpr int SW = scatter_warps<Real>();
@@ -518,7 +430,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
   if (w >= SW) return;
   ScatterWarp<Real>& sm = smw[w];
   const int nfeat = a.ne + (a.NV == 3 ? a.nedge : 0) + a.nn;
-  const int grp = blk.x / SCAT_SPLIT, phase = blk.x % SCAT_SPLIT;
+  const int grp = blk.x / a.split, phase = blk.x % a.split;
   const int f = (grp * SW + w) * 32 + lane;
   if (__ballot_sync(0xffffffffu, f < nfeat) == 0) return;
   // ---- the lane's feature: corners, cone generators (the normals of the
@@ -602,14 +514,47 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
     }
     c0 = (int)ceil(bmin - dc - eps);
     nsl = (int)floor(bmax + dc + eps) - c0 + 1;
-    V3<Real> vq[3];
-    for (int q = 0; q < 3; ++q) {
-      const int m = a.E[a.NV * tmin + min(q, a.NV - 1)];
-      vq[q] = mk<Real>(node_off(a, m, 0, o[0]), node_off(a, m, 1, o[1]), node_off(a, m, 2, o[2]));
+    // first corner A, then by kind: the face's normal and the vectors whose
+    // products with x - A are the barycentric coordinates of the projection
+    // (a segment: one), or the edge and the vector that gives its parameter
+    const Real A[3] = {sm.cb[lane][0], sm.cb[lane][1], sm.cb[lane][2]};
+    Real p[3] = {0, 0, 0}, q[3] = {0, 0, 0}, r[3] = {0, 0, 0};
+    if (kind == 0) {
+      const Real* e = a.ecst + 16 * f;
+      const Real d00 = e[9], d01 = e[10], d11 = e[11], iden = e[15];
+      for (int d = 0; d < 3; ++d) {
+        p[d] = a.en[3 * f + d];
+        q[d] = a.NV == 2 ? e[d] * e[12] : (d11 * e[d] - d01 * e[3 + d]) * iden;
+        r[d] = a.NV == 2 ? Real(0) : (d00 * e[3 + d] - d01 * e[d]) * iden;
+      }
+    } else if (kind == 1) {
+      Real l2 = 0;
+      for (int d = 0; d < 3; ++d) {
+        p[d] = sm.cb[lane][3 + d] - A[d];
+        l2 += p[d] * p[d];
+      }
+      const Real il2 = l2 > Real(0) ? rcp_rn(l2) : Real(0);  // degenerate edge: its first end
+      for (int d = 0; d < 3; ++d) q[d] = p[d] * il2;
     }
-    FaceDist<Real>(vq[0], vq[1], vq[2], a.NV == 3).store(sm.fd[lane]);
+    sm.rec[lane][0] = R4<Real>{A[0], A[1], A[2], r[0]};
+    sm.rec[lane][1] = R4<Real>{p[0], p[1], p[2], r[1]};
+    sm.rec[lane][2] = R4<Real>{q[0], q[1], q[2], r[2]};
     const int ow[3] = {wrap_coord(o[0], a.G.nx), wrap_coord(o[1], a.G.ny), a.G.wall ? o[2] : wrap_coord(o[2], a.G.nz)};
-    sm.ft[lane][0] = make_int4(ow[0], ow[1], ow[2], k | (oa << 2) | (ob << 4));
+    // no cell the feature can offer lies across a periodic side or a wall
+    const int mg = (int)ceil(dc) + 2;
+    const int n3[3] = {a.G.nx, a.G.ny, a.G.nz};
+    bool inner = true;
+    for (int d = 0; d < 3; ++d) {
+      if (a.dim == 2 && d == 1) continue;
+      Real lo = 0, hi = 0;
+      for (int j = 0; j < nB; ++j) {
+        lo = fmin(lo, sm.cb[lane][3 * j + d]);
+        hi = fmax(hi, sm.cb[lane][3 * j + d]);
+      }
+      inner &= ow[d] + (int)floor(lo) - mg >= 0 && ow[d] + (int)ceil(hi) + mg < n3[d];
+    }
+    // (a wide or grazing cone's rectangle can reach beyond dc)
+    sm.ft[lane][0] = make_int4(ow[0], ow[1], ow[2], k | (oa << 2) | (ob << 4) | (kind << 6) | (inner ? 256 : 0));
     sm.ft[lane][1] = make_int4(tmin, c0, 0, 0);
   }
   // bounding rectangle of the cone's cross-section in slice c: origin (a0,
@@ -642,19 +587,18 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       if (wa > 1024 || wb > 1024) atomicOr(a.status, (unsigned)ST_OVERFLOW);  // bounded work, flagged
       else cnt = wa * wb;
     }
-    if (cnt == 0) wa = 1;
   };
   const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)((nsl + SCAT_W - 1) / SCAT_W));
-  const Real dc2 = dc * dc;
-  for (int r = phase; r < rounds; r += SCAT_SPLIT) {
-    int tot = 0;
+  for (int r = phase; r < rounds; r += a.split) {
+    int cnt[SCAT_W], tot = 0;
 #pragma unroll
     for (int h = 0; h < SCAT_W; ++h) {
       const int sidx = r * SCAT_W + h;
-      int a0 = 0, b0 = 0, wa = 1, cnt = 0;
-      if (sidx < nsl) slice_rect(c0 + sidx, a0, b0, wa, cnt);
-      tot += cnt;
+      int a0 = 0, b0 = 0, wa = 1;
+      cnt[h] = 0;
+      if (sidx < nsl) slice_rect(c0 + sidx, a0, b0, wa, cnt[h]);
       sm.sl[lane][h] = make_int4(a0, b0, wa, tot);
+      tot += cnt[h];
     }
     int incl = tot;
 #pragma unroll
@@ -662,49 +606,71 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       const int v = __shfl_up_sync(0xffffffffu, incl, sh);
       if (lane >= sh) incl += v;
     }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    __syncwarp();
-    for (int j0 = 0; j0 < total; j0 += 32) {
-      const int i = j0 + lane;
-      // lane holding cell i: the first lane whose inclusive prefix exceeds i
-      int L = 0;
+    const int total = __shfl_sync(0xffffffffu, incl, 31), first = incl - tot;
 #pragma unroll
-      for (int step = 16; step >= 1; step >>= 1) {
-        const int v = __shfl_sync(0xffffffffu, incl, L + step - 1);
-        if (v <= i) L += step;
+    for (int h = 0; h < SCAT_W; ++h) sm.sl[lane][h].w += first;
+    for (int base = 0; base < total; base += SCAT_TAB) {
+      __syncwarp();
+      int s = first - base;
+#pragma unroll
+      for (int h = 0; h < SCAT_W; ++h) {
+        const int e = s + cnt[h];
+        for (int i = max(s, 0); i < min(e, SCAT_TAB); ++i) sm.tab[i] = (unsigned char)(lane * SCAT_W + h);
+        s = e;
       }
-      const int base = __shfl_sync(0xffffffffu, incl, L) - __shfl_sync(0xffffffffu, tot, L);
-      if (i >= total) continue;
-      int jj = i - base;
-      // its slice: the first whose cumulative count exceeds jj
-      int4 e = sm.sl[L][0];
-      int h = 0, prev = 0;
-#pragma unroll
-      for (int q = 1; q < SCAT_W; ++q) {
-        if (jj >= e.w) {
-          prev = e.w;
-          e = sm.sl[L][q];
-          h = q;
+      __syncwarp();
+      const int n = min(total - base, SCAT_TAB);
+      for (int i = lane; i < n; i += 32) {
+        const int id = sm.tab[i], L = id / SCAT_W, h = id % SCAT_W;
+        const int4 e = sm.sl[L][h], F0 = sm.ft[L][0], F1 = sm.ft[L][1];
+        const int jj = base + i - e.w;
+        // jj / wa: jj < 2^20 and wa <= 1024 keep the product within 2^-13 of the
+        // true (jj + 1/2) / wa, whose fraction is at least 2^-11 from an
+        // integer, so the truncation is exact
+        const int qb = (int)(((float)jj + 0.5f) * __frcp_rn((float)e.z));
+        const int rk = F1.y + r * SCAT_W + h, ra = e.x + (jj - qb * e.z), rb = a.dim == 3 ? e.y + qb : 0;
+        // axes (k, a, b): 3D k = 0: (x, y, z); 1: (y, x, z); 2: (z, x, y); 2D the
+        // plane (x, z) with b along the empty y
+        const int kk = F0.w & 3, kind_c = (F0.w >> 6) & 3;
+        int rx, ry, rz;
+        if (a.dim == 3) {
+          rx = kk == 0 ? rk : ra;
+          ry = kk == 0 ? ra : (kk == 1 ? rk : rb);
+          rz = kk == 2 ? rk : rb;
+        } else {
+          rx = kk == 0 ? rk : ra;
+          ry = 0;
+          rz = kk == 0 ? ra : rk;
         }
+        const R4<Real> A = sm.rec[L][0], p = sm.rec[L][1], q = sm.rec[L][2];
+        const Real ax = (Real)rx - A.x, ay = (Real)ry - A.y, az = (Real)rz - A.z;
+        Real dist;
+        if (kind_c == 0) {
+          const Real v = ax * q.x + ay * q.y + az * q.z, u = ax * A.w + ay * p.w + az * q.w;
+          if (!(v >= Real(0) && u >= Real(0) && v + u <= Real(1))) continue;
+          dist = fabs(ax * p.x + ay * p.y + az * p.z);
+        } else {
+          Real t = 0;
+          if (kind_c == 1) {
+            t = ax * q.x + ay * q.y + az * q.z;
+            if (!(t >= -eps && t <= Real(1) + eps)) continue;
+            t = fmin(Real(1), fmax(Real(0), t));
+          }
+          const Real x = ax - t * p.x, y = ay - t * p.y, z = az - t * p.z;
+          dist = sqrt(x * x + y * y + z * z);
+        }
+        if (!(dist < dc)) continue;
+        long long cell;
+        if (F0.w & 256) {  // (within dc of the feature, so inside the lattice)
+          cell = ((long long)(F0.z + rz) * a.G.ny + (F0.y + ry)) * a.G.nx + (F0.x + rx);
+        } else {
+          const int pc[3] = {F0.x + rx, F0.y + ry, F0.z + rz};
+          cell = cell_of(a, pc);
+          if (cell < 0) continue;
+        }
+        const unsigned long long key = (dist_code(dist) << 24) | (unsigned long long)F1.x;
+        atomicMin(a.key + cell, key);  // no return value: a fire-and-forget reduction
       }
-      jj -= prev;
-      // jj / wa: jj < 2^20 and wa <= 1024 keep the product within 2^-13 of the
-      // true (jj + 1/2) / wa, whose fraction is at least 2^-11 from an
-      // integer, so the truncation is exact
-      const int qb = (int)(((float)jj + 0.5f) * __frcp_rn((float)e.z));
-      const int4 F0 = sm.ft[L][0], F1 = sm.ft[L][1];
-      const int kk = F0.w & 3, ka = (F0.w >> 2) & 3, kb = (F0.w >> 4) & 3;
-      int rr[3];
-      rr[kk] = F1.y + r * SCAT_W + h;
-      rr[ka] = e.x + (jj - qb * e.z);
-      rr[kb] = a.dim == 3 ? e.y + qb : 0;
-      const int pc[3] = {F0.x + rr[0], F0.y + rr[1], F0.z + rr[2]};
-      const long long cell = cell_of(a, pc);
-      if (cell < 0) continue;
-      const Real d2 = FaceDist<Real>::load(sm.fd[L], a.NV == 3).dist2(mk<Real>((Real)rr[0], (Real)rr[1], (Real)rr[2]));
-      if (!(d2 < dc2)) continue;
-      const unsigned long long key = (dist_code(sqrt(d2)) << 24) | (unsigned long long)F1.x;
-      atomicMin(a.key + cell, key);  // no return value: a fire-and-forget reduction
     }
     __syncwarp();  // the next round rewrites the slice table
   }

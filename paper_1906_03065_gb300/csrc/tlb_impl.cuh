@@ -117,6 +117,7 @@ struct Impl : ImplBase {
     a.skc = c->ptr<Real>(c->L.skc);
     a.capr = c->ptr<Real>(c->L.capr);
     a.ncaps = c->ncap;
+    a.split = c->scat_split;
     a.ncpl = c->ptr<unsigned long long>(c->L.ncpl);
     a.F = c->ptr<Real>(c->L.F);
     a.box = c->ptr<int>(c->L.box);
@@ -160,9 +161,8 @@ struct Impl : ImplBase {
   static tlb_status ibm_positions(Ctx* c, IBArgs<Real>& a, cudaStream_t s, bool snap = false) {
     k_geometry<Real><<<blocks((long long)c->ne + c->nn, 128), 128, 0, s>>>(a, snap ? 1 : 0);
     TLB_LAUNCHED(c, "k_geometry");
-    const long long nfeat = (long long)c->ne + c->nedge + c->nn;
     constexpr int sw = scatter_warps<Real>();
-    const unsigned nvb = SCAT_SPLIT * blocks(nfeat, 32 * sw);
+    const unsigned nvb = (unsigned)a.split * blocks(c->features(), 32 * sw);
     k_dist_scatter<Real><<<std::min(nvb, 4u * (unsigned)c->nsm), 32 * sw, 0, s>>>(a, (int)nvb);
     TLB_LAUNCHED(c, "k_dist_scatter");
     return TLB_OK;
