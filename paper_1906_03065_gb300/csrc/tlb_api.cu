@@ -291,8 +291,8 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.ring, NV * ne * 4);
   take(L.en, 3 * ne * R);
   take(L.vn, 3 * nn * R);
-  take(L.erel, 3 * NV * ne * R);
-  take(L.eorg, 3 * ne * 4);
+  take(L.erel, 4 * ne * R);
+  take(L.eorg, 4 * ne * 4);
   take(L.ecst, 16 * ne * R);
   take(L.xo, 3 * nn * 4);
   take(L.xr, 3 * nn * R);

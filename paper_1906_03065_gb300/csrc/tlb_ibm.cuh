@@ -45,9 +45,10 @@ struct IBArgs {
   // per-step work
   Real* en;              // [ne][3] unit outward normal
   Real* vn;              // [nn][3] angle-weighted vertex pseudo-normal
-  Real* erel;            // [ne][NV][3] vertices relative to the element's origin
-  int* eorg;             // [ne][3] element origin: floor of its first vertex
-  Real* ecst;            // [ne][16] edge vectors ab, ac, bc, Gram entries d00 d01 d11 and
+  // per element, read as whole vectors by the band:
+  R4<Real>* erel;        // [ne] first vertex relative to the element's origin
+  int4* eorg;            // [ne] element origin: floor of its first vertex
+  R4<Real>* ecst;        // [ne][4] edge vectors ab, ac, bc, Gram entries d00 d01 d11 and
                          // the reciprocals of d00, d11, |bc|^2 and the Gram determinant
   unsigned long long* ncpl;  // [nn][3] coupling force per marker, fixed point (CPL_SCALE)
   Real* F;               // [nn][3] node force
@@ -134,11 +135,12 @@ __device__ __forceinline__ void split_coord(double x, int* xo, Real* xr) {
 // the edge constants from ecst, so a cell needs no division and no
 // double-precision arithmetic.
 template <class Real>
-__device__ __forceinline__ V3<Real> elem_closest(const IBArgs<Real>& a, int e, const int* p, Real* beta, int* feat) {
-  const Real* r = a.erel + 3 * a.NV * e;
-  const int* o = a.eorg + 3 * e;
-  const Real* k = a.ecst + 16 * e;
-  const V3<Real> A = mk<Real>(r[0] + (Real)(o[0] - p[0]), r[1] + (Real)(o[1] - p[1]), r[2] + (Real)(o[2] - p[2]));
+__device__ __forceinline__ V3<Real> elem_closest(const IBArgs<Real>& a, int e, const int4& o, const int* p, Real* beta,
+                                                 int* feat) {
+  const R4<Real> r = ldg4(a.erel + e), k0 = ldg4(a.ecst + 4 * e), k1 = ldg4(a.ecst + 4 * e + 1),
+                 k2 = ldg4(a.ecst + 4 * e + 2), k3 = ldg4(a.ecst + 4 * e + 3);
+  const Real k[16] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w, k2.x, k2.y, k2.z, k2.w, k3.x, k3.y, k3.z, k3.w};
+  const V3<Real> A = mk<Real>(r.x + (Real)(o.x - p[0]), r.y + (Real)(o.y - p[1]), r.z + (Real)(o.z - p[2]));
   const V3<Real> ab = mk<Real>(k[0], k[1], k[2]);
   const V3<Real> ap = mk<Real>(-A.x, -A.y, -A.z);
   const Real d20 = dot(ap, ab);
@@ -224,14 +226,13 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
     a.en[3 * t + 2] = n.z;
     const int* Et = a.E + a.NV * t;
     Real rv[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    int org[3];
     for (int d = 0; d < 3; ++d) {
-      const int o = a.xo[3 * Et[0] + d];
-      a.eorg[3 * t + d] = o;
-      for (int q = 0; q < a.NV; ++q) {
-        rv[q][d] = node_off(a, Et[q], d, o);
-        a.erel[3 * (a.NV * t + q) + d] = rv[q][d];
-      }
+      org[d] = a.xo[3 * Et[0] + d];
+      for (int q = 0; q < a.NV; ++q) rv[q][d] = node_off(a, Et[q], d, org[d]);
     }
+    a.eorg[t] = make_int4(org[0], org[1], org[2], 0);
+    a.erel[t] = R4<Real>{rv[0][0], rv[0][1], rv[0][2], 0};
     // edge constants of the band's closest-point search (a segment keeps
     // ac = bc = 0)
     const V3<Real> A = mk<Real>(rv[0][0], rv[0][1], rv[0][2]), Bv = mk<Real>(rv[1][0], rv[1][1], rv[1][2]);
@@ -239,11 +240,12 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
     const V3<Real> ab = Bv - A, ac = a.NV == 3 ? Cv - A : mk<Real>(0, 0, 0), bc = a.NV == 3 ? Cv - Bv : mk<Real>(0, 0, 0);
     const Real d00 = dot(ab, ab), d01 = dot(ab, ac), d11 = dot(ac, ac), dbc = dot(bc, bc);
     const Real den = d00 * d11 - d01 * d01;
-    Real* k = a.ecst + 16 * t;
-    const Real kv[16] = {ab.x, ab.y, ab.z, ac.x, ac.y, ac.z, bc.x, bc.y, bc.z, d00, d01, d11,
-                         d00 > Real(0) ? rcp_rn(d00) : Real(0), d11 > Real(0) ? rcp_rn(d11) : Real(0),
-                         dbc > Real(0) ? rcp_rn(dbc) : Real(0), den > Real(0) ? rcp_rn(den) : Real(0)};
-    for (int q = 0; q < 16; ++q) k[q] = kv[q];
+    R4<Real>* k = a.ecst + 4 * t;
+    k[0] = R4<Real>{ab.x, ab.y, ab.z, ac.x};
+    k[1] = R4<Real>{ac.y, ac.z, bc.x, bc.y};
+    k[2] = R4<Real>{bc.z, d00, d01, d11};
+    k[3] = R4<Real>{d00 > Real(0) ? rcp_rn(d00) : Real(0), d11 > Real(0) ? rcp_rn(d11) : Real(0),
+                    dbc > Real(0) ? rcp_rn(dbc) : Real(0), den > Real(0) ? rcp_rn(den) : Real(0)};
     return;
   }
   int k = t - a.ne;
@@ -341,26 +343,6 @@ __device__ __forceinline__ unsigned long long scaled_floor_u64(float v, int s) {
   else e = 1;
   const int sh = e - 150 + s;  // v = m 2^(e - 150)
   return sh >= 0 ? m << sh : (sh > -24 ? m >> -sh : 0ull);
-}
-// rint(v 2^s), ties to even; saturates at +-2^62:
-__device__ __forceinline__ long long scaled_rint_s64(float v, int s) {
-  const unsigned b = __float_as_uint(v);
-  int e = (int)((b >> 23) & 0xFFu);
-  unsigned long long m = b & 0x7FFFFFu;
-  if (e) m |= 0x800000u;
-  else e = 1;
-  const int sh = e - 150 + s;
-  unsigned long long r;
-  if (sh >= 0) {
-    r = sh <= 38 ? m << sh : (1ull << 62);
-  } else if (sh >= -24) {
-    const int k = -sh;
-    const unsigned long long q = m >> k, rem = m - (q << k), half = 1ull << (k - 1);
-    r = q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull);
-  } else {
-    r = 0;
-  }
-  return (b >> 31) ? -(long long)r : (long long)r;
 }
 // distance part of a scatter key: the distance on a grid of 2^-34
 __device__ __forceinline__ unsigned long long dist_code(float d) { return scaled_floor_u64(d, 34); }
@@ -520,7 +502,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
     const Real A[3] = {sm.cb[lane][0], sm.cb[lane][1], sm.cb[lane][2]};
     Real p[3] = {0, 0, 0}, q[3] = {0, 0, 0}, r[3] = {0, 0, 0};
     if (kind == 0) {
-      const Real* e = a.ecst + 16 * f;
+      const Real* e = &a.ecst[4 * f].x;
       const Real d00 = e[9], d01 = e[10], d11 = e[11], iden = e[15];
       for (int d = 0; d < 3; ++d) {
         p[d] = a.en[3 * f + d];
@@ -704,7 +686,17 @@ __device__ __forceinline__ Real feature_sign(const IBArgs<Real>& a, int e, int f
 // Fixed-point scale of the coupling sums: integer additions make the
 // per-element totals independent of the order of the contributions.
 #define CPL_SCALE 1125899906842624.0  // 2^50
-__device__ __forceinline__ long long cpl_fixed(float v) { return scaled_rint_s64(v, 50); }
+// rint(v 2^50) as hi 2^26 + lo with |lo| <= 2^25: hi = rint(v 2^24), lo the
+// rest, which is exact (v - hi 2^-24 is a multiple of v's last place below
+// 2^-25) but for its own rounding, so no 64-bit conversion is needed (slow
+// on this GPU).  The parts of a warp's lanes add up in 32 bits while every
+// |v| < CPL_SMALL; hi saturates at +-2^31.
+constexpr float CPL_SMALL = 3.9f;
+__device__ __forceinline__ void cpl_split(float v, int* hi, int* lo) {
+  *hi = __float2int_rn(v * 0x1p24f);
+  *lo = __float2int_rn(fmaf((float)*hi, -0x1p-24f, v) * 0x1p50f);
+}
+__device__ __forceinline__ long long cpl_join(int hi, int lo) { return (long long)hi * (1 << 26) + lo; }
 __device__ __forceinline__ long long cpl_fixed(double v) { return llrint(v * CPL_SCALE); }
 
 // Band cells of the marker box (one thread per cell, x fastest): signed
@@ -729,7 +721,7 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
   const int wx = bhi[0] - bx0 + 1, wy = bhi[1] - by0 + 1, wz = bhi[2] - bz0 + 1;
   const long long total = (long long)wx * wy * wz;
   const bool full[3] = {wx == a.G.nx, a.dim == 3 && wy == a.G.ny, !a.G.wall && wz == a.G.nz};
-  const Real al = a.alpha, Iin = a.Iin, Iout = a.Iout;
+  const Real ial = rcp_rn(a.alpha), Iin = a.Iin, Iout = a.Iout;
   // the box origin wrapped into the lattice: cells are indexed from it, the
   // geometry uses the unwrapped coordinates
   const int ox = wrap_coord(bx0, a.G.nx), oy = wrap_coord(by0, a.G.ny), oz = a.G.wall ? bz0 : wrap_coord(bz0, a.G.nz);
@@ -779,23 +771,25 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
           // (the element origin, floor of its first vertex, is within a cell
           // of it: the nearest image is the same)
           int pi[3] = {pc[0], pc[1], pc[2]};
+          const int4 eo = a.eorg[e];
           if (full[0] | full[1] | full[2]) {
-            const int* eo = a.eorg + 3 * e;
-            if (full[0]) pi[0] += a.G.nx * __float2int_rn((float)(eo[0] - pi[0]) / (float)a.G.nx);
-            if (full[1]) pi[1] += a.G.ny * __float2int_rn((float)(eo[1] - pi[1]) / (float)a.G.ny);
-            if (full[2]) pi[2] += a.G.nz * __float2int_rn((float)(eo[2] - pi[2]) / (float)a.G.nz);
+            if (full[0]) pi[0] += a.G.nx * __float2int_rn((float)(eo.x - pi[0]) / (float)a.G.nx);
+            if (full[1]) pi[1] += a.G.ny * __float2int_rn((float)(eo.y - pi[1]) / (float)a.G.ny);
+            if (full[2]) pi[2] += a.G.nz * __float2int_rn((float)(eo.z - pi[2]) / (float)a.G.nz);
           }
-          V3<Real> P = elem_closest(a, e, pi, beta, &feat);
+          V3<Real> P = elem_closest(a, e, eo, pi, beta, &feat);
           V3<Real> xmP = mk<Real>(-P.x, -P.y, -P.z);
           Real dist = sqrt(dot(xmP, xmP));
           Real s = feature_sign(a, e, feat, xmP);
           Real d = s * dist;
-          Real I = Real(0.5) * (Real(1) + tanh(d / (Real(2) * al)));
+          // with E = exp(-|d|/alpha): I = (1 + tanh(d/(2 alpha)))/2 is 1/(1 + E)
+          // inside and E/(1 + E) outside, sech^2(d/(2 alpha)) = 4 E/(1 + E)^2
+          const Real E = exp(-dist * ial), iE = rcp_rn(Real(1) + E);
+          const Real I = d > Real(0) ? iE : E * iE;
           a.dsel[c] = d;
           a.own[c] = e;
           a.I[c] = I;
-          Real ch = cosh(d / (Real(2) * al));
-          Real coef = a.kc * (psic - I) / (ch * ch) / (Real(4) * al);
+          const Real coef = a.kc * (psic - I) * (E * iE) * (iE * ial);
           V3<Real> dir;
           if (dist > Real(1e-12)) dir = (-s / dist) * xmP;
           else dir = mk<Real>(a.en[3 * e], a.en[3 * e + 1], a.en[3 * e + 2]);
@@ -814,17 +808,50 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
       const unsigned grp = __match_any_sync(active, e);
       const int leader = __ffs(grp) - 1;
       const int lane = threadIdx.x & 31;
-      long long v[9], sum[9];
+      long long sum[9];
+      if constexpr (std::is_same<Real, float>::value) {
+        bool small = true;
+        int hi[9], lo[9], sh[9], sl[9];
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        v[i] = cpl_fixed(acc[i / 3][i % 3]);
-        sum[i] = 0;
-      }
-      // sum over the group (integers: any order gives the same total)
-      for (unsigned m = grp; m; m &= m - 1) {
-        const int src = __ffs(m) - 1;
+        for (int i = 0; i < 9; ++i) {
+          const float v = acc[i / 3][i % 3];
+          small &= fabsf(v) < CPL_SMALL;
+          cpl_split(v, hi + i, lo + i);
+          sh[i] = sl[i] = 0;
+          sum[i] = 0;
+        }
+        if (__all_sync(active, small)) {
+          // sum over the group (integers: any order gives the same total)
+          for (unsigned m = grp; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) sum[i] += __shfl_sync(grp, v[i], src);
+            for (int i = 0; i < 9; ++i) {
+              sh[i] += __shfl_sync(grp, hi[i], src);
+              sl[i] += __shfl_sync(grp, lo[i], src);
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 9; ++i) sum[i] = cpl_join(sh[i], sl[i]);
+        } else {
+          for (unsigned m = grp; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+              sum[i] += cpl_join(__shfl_sync(grp, hi[i], src), __shfl_sync(grp, lo[i], src));
+          }
+        }
+      } else {
+        long long v[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          v[i] = cpl_fixed((double)acc[i / 3][i % 3]);
+          sum[i] = 0;
+        }
+        for (unsigned m = grp; m; m &= m - 1) {
+          const int src = __ffs(m) - 1;
+#pragma unroll
+          for (int i = 0; i < 9; ++i) sum[i] += __shfl_sync(grp, v[i], src);
+        }
       }
       if (lane == leader) {  // straight to the element's nodes
 #pragma unroll

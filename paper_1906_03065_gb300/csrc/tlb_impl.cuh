@@ -109,9 +109,9 @@ struct Impl : ImplBase {
     a.edges = c->ptr<int>(c->L.edges);
     a.en = c->ptr<Real>(c->L.en);
     a.vn = c->ptr<Real>(c->L.vn);
-    a.erel = c->ptr<Real>(c->L.erel);
-    a.eorg = c->ptr<int>(c->L.eorg);
-    a.ecst = c->ptr<Real>(c->L.ecst);
+    a.erel = c->ptr<R4<Real>>(c->L.erel);
+    a.eorg = c->ptr<int4>(c->L.eorg);
+    a.ecst = c->ptr<R4<Real>>(c->L.ecst);
     a.xo = c->ptr<int>(c->L.xo);
     a.xr = c->ptr<Real>(c->L.xr);
     a.skc = c->ptr<Real>(c->L.skc);
