@@ -287,10 +287,9 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.inc, NV * ne * 4);
   take(L.adj, 3 * ne * 4);
   take(L.edges, 4 * (size_t)c.nedge * 4);
-  take(L.ring_off, (nn + 1) * 4);
-  take(L.ring, NV * ne * 4);
   take(L.en, 3 * ne * R);
   take(L.vn, 3 * nn * R);
+  take(L.nadj, 4 * nn * R);
   take(L.erel, 4 * ne * R);
   take(L.eorg, 4 * ne * 4);
   take(L.ecst, 16 * ne * R);
@@ -380,6 +379,7 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
       r0 = cuda_check(cudaStreamCreateWithPriority(&c->side2, cudaStreamNonBlocking, hi_prio), "side stream");
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_bins, cudaEventDisableTiming), "event");
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "event");
+    if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_geom, cudaEventDisableTiming), "event");
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming), "event");
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_coll, cudaEventDisableTiming), "event");
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_interp, cudaEventDisableTiming), "event");
@@ -476,20 +476,17 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
       inc_off[v + 1] = inc_off[v] + (int)inc[v].size();
       incl.insert(incl.end(), inc[v].begin(), inc[v].end());
     }
-    // distinct 1-ring neighbours of every node, in the order of its incident
-    // elements (ascending) and of their vertices
-    std::vector<int> ring_off(c->nn + 1, 0), ring;
+    // incident elements and distinct 1-ring neighbours of a node, at most
     int max_inc = 0, max_ring = 0;
     for (int v = 0; v < c->nn; ++v) {
-      const size_t r0 = ring.size();
+      std::vector<int> ring;
       for (int e : inc[v])
         for (int q = 0; q < c->NV; ++q) {
           const int u = E[(size_t)c->NV * e + q];
-          if (u != v && std::find(ring.begin() + r0, ring.end(), u) == ring.end()) ring.push_back(u);
+          if (u != v && std::find(ring.begin(), ring.end(), u) == ring.end()) ring.push_back(u);
         }
-      ring_off[v + 1] = (int)ring.size();
       max_inc = std::max(max_inc, (int)inc[v].size());
-      max_ring = std::max(max_ring, (int)(ring.size() - r0));
+      max_ring = std::max(max_ring, (int)ring.size());
     }
     if (c->NV == 3 && (max_inc > 16 || max_ring > 15)) {
       set_error("membrane: a node has more than 16 incident triangles or 15 neighbours");
@@ -531,8 +528,6 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
     u = u != TLB_OK ? u : up(c->L.inc_off, inc_off.data(), inc_off.size() * 4);
     u = u != TLB_OK ? u : up(c->L.inc, incl.data(), incl.size() * 4);
     u = u != TLB_OK ? u : up(c->L.adj, adj.data(), adj.size() * 4);
-    u = u != TLB_OK ? u : up(c->L.ring_off, ring_off.data(), ring_off.size() * 4);
-    if (!ring.empty()) u = u != TLB_OK ? u : up(c->L.ring, ring.data(), ring.size() * 4);
     if ((int)edges.size() != 4 * c->nedge) {
       set_error("membrane is not a closed surface (every edge must belong to two triangles)");
       delete c;

@@ -159,9 +159,9 @@ struct BatchImpl : BatchBase {
       case MOM:
         if (!variant_t1(b->tile_variant)) return {(int)cdiv(c->N, NT), 1, 1};
         return {(int)cdiv(c->nx, recon_x<L>()), (int)cdiv(c->ny, recon_y<L>()), (int)cdiv(c->nz, b->recon_zc)};
-      case GEOM: return {mem ? (int)cdiv((long long)c->ne + c->nn, NT) : 0, 1, 1};
+      case GEOM: return {mem ? (int)cdiv(geometry_threads(c->ne, c->nn), NT) : 0, 1, 1};
       case BCOUNT: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
-      case NODEF: return {mem ? (int)cdiv(32ll * c->nn, NT) : 0, 1, 1};
+      case NODEF: return {mem ? (int)cdiv(16ll * c->nn, NT) : 0, 1, 1};
       case SCAT: {
         return {mem ? b->scat_split * (int)cdiv(c->features(), 32 * scatter_warps<typename Prec<MODE>::Real>()) : 0, 1, 1};
       }

@@ -141,8 +141,8 @@ struct Layout {
   Region lo[2], rest[2];
   Region rho, phi, psi, p4, j2, M, I, dsel, own, key, fib, ftot, mu, rb;
   // membranes
-  Region X, E, ecap, ncap, cap_par, ds0, rprev, rnext, A0, G0i, inc_off, inc, adj, edges, ring_off, ring;
-  Region en, vn, erel, eorg, ecst, xo, xr, skc, capr, ncpl, F, box;
+  Region X, E, ecap, ncap, cap_par, ds0, rprev, rnext, A0, G0i, inc_off, inc, adj, edges;
+  Region en, vn, nadj, erel, eorg, ecst, xo, xr, skc, capr, ncpl, F, box;
   Region bcnt, bprev, bcur, boff, blist, bact, ctr, bflag;
   // misc
   Region status, part, meas;
@@ -196,8 +196,8 @@ struct Ctx {
   cudaStream_t stream = nullptr;
   cudaStream_t side = nullptr;   // membrane work that overlaps the moments: geometry
                                  // and the distance scatter
-  cudaStream_t side2 = nullptr;  // elastic forces and brick binning, beside `side`
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_bins = nullptr, ev_coll = nullptr, ev_interp = nullptr;
+  cudaStream_t side2 = nullptr;  // brick binning and elastic forces, beside `side`
+  cudaEvent_t ev_fork = nullptr, ev_geom = nullptr, ev_join = nullptr, ev_bins = nullptr, ev_coll = nullptr, ev_interp = nullptr;
   int nsm = 1;  // streaming multiprocessors of the device
   int cur = 0;  // population buffer holding the current state
   long t = 0;
@@ -250,6 +250,7 @@ struct Ctx {
     if (side) cudaStreamSynchronize(side);
     if (side2) cudaStreamSynchronize(side2);
     if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_geom) cudaEventDestroy(ev_geom);
     if (ev_join) cudaEventDestroy(ev_join);
     if (ev_bins) cudaEventDestroy(ev_bins);
     if (ev_coll) cudaEventDestroy(ev_coll);

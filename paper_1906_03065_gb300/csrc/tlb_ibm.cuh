@@ -38,13 +38,13 @@ struct IBArgs {
   const int* inc_off;    // node -> incident elements (CSR, ascending)
   const int* inc;
   const int* adj;        // 3D: triangle across edge q (q: vertex q -> q+1)
-  const int* ring_off;   // node -> distinct 1-ring neighbours (CSR, in the order
-  const int* ring;       // of the incident elements and their vertices)
   int nedge;             // 3D: unique edges
   const int* edges;      // 3D: [nedge][4] vertex a, vertex b, face left, face right
   // per-step work
   Real* en;              // [ne][3] unit outward normal
   Real* vn;              // [nn][3] angle-weighted vertex pseudo-normal
+  R4<Real>* nadj;        // [nn] 3D: derivatives of the marker's bending energy with
+                         // respect to its K (three) and A (see geometry_body)
   // per element, read as whole vectors by the band:
   R4<Real>* erel;        // [ne] first vertex relative to the element's origin
   int4* eorg;            // [ne] element origin: floor of its first vertex
@@ -211,11 +211,23 @@ __device__ __forceinline__ V3<Real> face_normal(const IBArgs<Real>& a, int e) {
   return (Real(1) / sqrt(dot(cr, cr))) * cr;
 }
 
-// One launch for the geometry of the step: threads [0, ne) store the unit
-// outward face normals; threads [ne, ne + nn) store the vertex
-// pseudo-normals, the angle-weighted sum of the incident face normals
-// (Baerentzen and Aanaes 2005; in 2D the sum of the two segment normals),
-// computing those normals themselves.
+// The geometry of the step in one launch.  Threads [0, ne) store the unit
+// outward face normals and what the band reads of each face.  Then 16 lanes
+// per marker, one incident face each, store the vertex pseudo-normal, the
+// angle-weighted sum of the incident face normals (Baerentzen and Aanaes
+// 2005; in 2D the sum of the two segment normals), and in 3D the marker's
+// part of the Helfrich energy: with E_v = kb |K|^2 / (8 A), K = sum_T (cot_k
+// (x_v - x_j) + cot_j (x_v - x_k)) and A the mixed Voronoi area (Meyer et al.
+// 2003), the derivatives dE_v/dK = kb K / (4 A) and dE_v/dA = -kb |K|^2 /
+// (8 A^2), which the force of every marker around it needs (see
+// node_forces_body).  Lane sums are combined by a fixed shuffle tree.
+template <class Real>
+__device__ __forceinline__ Real group_sum(Real v) {  // over the 16 lanes of a marker
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+TLB_HD int geometry_threads(int ne, int nn) { return (ne + 31) / 32 * 32 + 16 * nn; }
 template <class Real>
 __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& blk) {
   int t = blk.x * blockDim.x + threadIdx.x;
@@ -248,27 +260,47 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
                     dbc > Real(0) ? rcp_rn(dbc) : Real(0), den > Real(0) ? rcp_rn(den) : Real(0)};
     return;
   }
-  int k = t - a.ne;
-  if (k >= a.nn) return;
-  V3<Real> s = mk<Real>(0, 0, 0);
-  for (int j = a.inc_off[k]; j < a.inc_off[k + 1]; ++j) {
-    int e = a.inc[j];
-    V3<Real> n = face_normal(a, e);
-    Real wgt = 1;
-    if (a.NV == 3) {
-      int q0 = a.E[3 * e], q1 = a.E[3 * e + 1], q2 = a.E[3 * e + 2];
-      int u = q0 == k ? q1 : (q1 == k ? q2 : q0);
-      int v = q0 == k ? q2 : (q1 == k ? q0 : q1);
-      V3<Real> eu = node_dv(a, u, k);
-      V3<Real> ev = node_dv(a, v, k);
-      Real c = dot(eu, ev) / sqrt(dot(eu, eu) * dot(ev, ev));
-      wgt = acos(fmin(Real(1), fmax(Real(-1), c)));
+  if (t < (a.ne + 31) / 32 * 32) return;  // (markers start at a whole warp)
+  const int g = t - (a.ne + 31) / 32 * 32, lane = g & 15;
+  const bool valid = (g >> 4) < a.nn;
+  const int k = valid ? g >> 4 : a.nn - 1;  // every lane takes part in the sums
+  const int i0 = a.inc_off[k], ninc = valid ? a.inc_off[k + 1] - i0 : 0;
+  V3<Real> s = mk<Real>(0, 0, 0), K = s;
+  Real A = 0;
+  for (int j = lane; j < ninc; j += 16) {
+    const int e = a.inc[i0 + j];
+    if (a.NV == 2) {
+      s = s + face_normal(a, e);
+      continue;
     }
-    s = s + wgt * n;
+    const int q0 = a.E[3 * e], q1 = a.E[3 * e + 1], q2 = a.E[3 * e + 2];
+    const int u = q0 == k ? q1 : (q1 == k ? q2 : q0);
+    const int v = q0 == k ? q2 : (q1 == k ? q0 : q1);
+    const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = ev - eu;
+    const V3<Real> cr = cross(eu, ev);
+    const Real A2 = sqrt(dot(cr, cr)), iA2 = Real(1) / A2;
+    const Real duu = dot(eu, eu), dvv = dot(ev, ev), dk = dot(eu, ev), du = -dot(eu, w), dv = dot(ev, w);
+    const Real c = dk / sqrt(duu * dvv);
+    s = s + (acos(fmin(Real(1), fmax(Real(-1), c))) * iA2) * cr;
+    const Real cu = du * iA2, cv = dv * iA2;
+    K = K - cv * eu - cu * ev;
+    if (dk < 0) A += Real(0.25) * A2;
+    else if (du < 0 || dv < 0) A += Real(0.125) * A2;
+    else A += Real(0.125) * (duu * cv + dvv * cu);
   }
+  s = mk<Real>(group_sum(s.x), group_sum(s.y), group_sum(s.z));
+  if (a.NV == 3) {
+    K = mk<Real>(group_sum(K.x), group_sum(K.y), group_sum(K.z));
+    A = group_sum(A);
+  }
+  if (!valid || lane != 0) return;
   a.vn[3 * k] = s.x;
   a.vn[3 * k + 1] = s.y;
   a.vn[3 * k + 2] = s.z;
+  if (a.NV == 3) {
+    const Real kA = Real(0.25) * a.capr[a.ncaps + a.ncap[k]] / A;
+    a.nadj[k] = R4<Real>{kA * K.x, kA * K.y, kA * K.z, Real(-0.5) * kA * dot(K, K) / A};
+  }
 }
 template <class Real>
 __global__ void k_geometry(const __grid_constant__ IBArgs<Real> a, int snap) {
@@ -932,230 +964,136 @@ __global__ void k_fill(const __grid_constant__ IBArgs<Real> a) {
 }
 
 // ------------------------------------------------------------ elastic forces
-constexpr int NODEF_WARPS = 4;  // warps per block of the node-force kernel (at most)
-
-// Forward-mode dual number with derivatives with respect to one node.
-template <class T>
-struct D3 {
-  T v, d0, d1, d2;
-};
-template <class T> TLB_HD D3<T> dc(T v) { return {v, 0, 0, 0}; }
-template <class T> TLB_HD D3<T> operator+(D3<T> a, D3<T> b) { return {a.v + b.v, a.d0 + b.d0, a.d1 + b.d1, a.d2 + b.d2}; }
-template <class T> TLB_HD D3<T> operator-(D3<T> a, D3<T> b) { return {a.v - b.v, a.d0 - b.d0, a.d1 - b.d1, a.d2 - b.d2}; }
-template <class T> TLB_HD D3<T> operator*(D3<T> a, D3<T> b) {
-  return {a.v * b.v, a.d0 * b.v + a.v * b.d0, a.d1 * b.v + a.v * b.d1, a.d2 * b.v + a.v * b.d2};
-}
-template <class T> TLB_HD D3<T> operator*(T s, D3<T> a) { return {s * a.v, s * a.d0, s * a.d1, s * a.d2}; }
-template <class T> TLB_HD D3<T> operator/(D3<T> a, D3<T> b) {
-  T ib = T(1) / b.v;
-  T q = a.v * ib;
-  return {q, (a.d0 - q * b.d0) * ib, (a.d1 - q * b.d1) * ib, (a.d2 - q * b.d2) * ib};
-}
-template <class T> TLB_HD D3<T> dsqrt(D3<T> a) {
-  T s = sqrt(a.v);
-  T h = T(0.5) / s;
-  return {s, a.d0 * h, a.d1 * h, a.d2 * h};
-}
-template <class T> using DV = V3<D3<T>>;
-template <class T> TLB_HD DV<T> dsub(DV<T> a, DV<T> b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
-template <class T> TLB_HD D3<T> ddot(DV<T> a, DV<T> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-template <class T> TLB_HD DV<T> dcross(DV<T> a, DV<T> b) {
-  return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
-}
-
-// Position of node j relative to the seed node k, differentiated with
-// respect to X_k (the seed carries derivative -1 in every other node's frame:
-// we place the origin at X_k so only the seed itself moves).
+// Elastic node forces, 16 lanes per marker, summed by a fixed shuffle tree.
+// They depend on the marker positions only; the coupling force joins them in
+// k_spread.
+//
+// 3D: lane j takes incident face j = (k, u, v), whose energy as a function of
+// X_k is its Skalak energy A0 W, W = (G/4)(I1^2 + 2 I1 - 2 I2 + C I2^2) with
+// I1 = tr(G0^-1 g) - 2, I2 = det(G0^-1 g) - 1 of the edge metric g, plus its
+// share of the three vertices' bending energies.  The bending energies are
+// functions of the sums K_v and A_v, whose derivatives (nadj) are known from
+// the geometry pass, so face (k, u, v) contributes the derivative of
+//   cot_v P_v + cot_u P_u + cot_k P_k,   P_v = (x_k - x_u).(K'_k - K'_u) +
+//   |x_k - x_u|^2 (A'_k + A'_u)/8 and cyclically
+// (an obtuse face's areas are A2/4 or A2/8 times the A' instead, A2 twice its
+// area), with cot_i = d_i / A2.  (Each marker used to differentiate the
+// energies of its whole 1-ring, 42 face terms in dual numbers, for 18 that
+// depend on it.)
+// 2D: lanes 0 and 1 the two segments (eq. DiscreteSE), lanes 2..4 the bending
+// at the previous marker, this one and the next (eqs. DiscreteBE,
+// DiscreteTheta, DiscreteArcLength).
 template <class Real>
-__device__ __forceinline__ DV<Real> dnode(const IBArgs<Real>& a, int j, int k) {
-  DV<Real> r;
-  r.x = dc<Real>(node_dx(a, j, k, 0));
-  r.y = dc<Real>(node_dx(a, j, k, 1));
-  r.z = dc<Real>(node_dx(a, j, k, 2));
-  if (j == k) { r.x.d0 = 1; r.y.d1 = 1; r.z.d2 = 1; }
-  return r;
+__device__ __forceinline__ V3<Real> ring_force(const IBArgs<Real>& a, int k, int lane) {
+  const int cap = a.ncap[k];
+  const Real ks = a.capr[cap], kb = a.capr[a.ncaps + cap];
+  if (lane < 2) {
+    const int e = a.inc[a.inc_off[k] + lane];
+    const int p = a.E[2 * e], q = a.E[2 * e + 1];
+    const Real tx = node_dx(a, q, p, 0), tz = node_dx(a, q, p, 2);
+    const Real L = sqrt(tx * tx + tz * tz);
+    const Real T = ks * (L / (Real)a.ds0[e] - Real(1)) / L;
+    const Real sgn = (p == k) ? Real(1) : Real(-1);  // -dE/dX_p = +T t ; -dE/dX_q = -T t
+    return mk<Real>(sgn * T * tx, Real(0), sgn * T * tz);
+  }
+  const int m = lane == 2 ? a.rprev[k] : (lane == 3 ? k : a.rnext[k]);
+  const int mp = a.rnext[m], mq = a.rprev[m];
+  const Real ax = node_dx(a, mp, m, 0), az = node_dx(a, mp, m, 2);
+  const Real bx = node_dx(a, m, mq, 0), bz = node_dx(a, m, mq, 2);
+  const Real la = sqrt(ax * ax + az * az), lb = sqrt(bx * bx + bz * bz);
+  const Real ab = ax * bx + az * bz;
+  const Real cr = ax * bz - az * bx;
+  // theta1 = arccos(a.b / |a||b|), evaluated as atan2(|a x b|, a.b)
+  const Real th = atan2(fabs(cr), ab);
+  const Real sn = fabs(cr) / (la * lb);
+  const Real ratio = th < Real(1e-4) ? Real(1) + th * th / Real(6) : th / sn;
+  const Real dsp = la + lb;
+  const Real k1 = Real(0.25) * kb * (Real(-8) * ratio / dsp);
+  const Real dth = Real(2) * th;
+  const Real k2 = Real(0.25) * kb * (dth / dsp) * (dth / dsp);
+  const Real iab = Real(1) / (la * lb);
+  const Real dya_x = bx * iab - ab * ax * iab / (la * la), dya_z = bz * iab - ab * az * iab / (la * la);
+  const Real dyb_x = ax * iab - ab * bx * iab / (lb * lb), dyb_z = az * iab - ab * bz * iab / (lb * lb);
+  Real gx = 0, gz = 0;
+  if (k == mp) { gx += k1 * dya_x - k2 * ax / la; gz += k1 * dya_z - k2 * az / la; }
+  if (k == m) {
+    gx += k1 * (dyb_x - dya_x) - k2 * (bx / lb - ax / la);
+    gz += k1 * (dyb_z - dya_z) - k2 * (bz / lb - az / la);
+  }
+  if (k == mq) { gx += -k1 * dyb_x + k2 * bx / lb; gz += -k1 * dyb_z + k2 * bz / lb; }
+  return mk<Real>(-gx, Real(0), -gz);
 }
-
-// Skalak energy of triangle t (shear modulus G, area ratio C):
-// W = (G/4)(I1^2 + 2 I1 - 2 I2 + C I2^2), I1 = tr(G0^-1 g) - 2, I2 = det(G0^-1 g) - 1.
 template <class Real>
-__device__ __forceinline__ D3<Real> skalak_dual(const IBArgs<Real>& a, int t, int k) {
-  int p = a.E[3 * t], q = a.E[3 * t + 1], r = a.E[3 * t + 2];
-  DV<Real> xp = dnode(a, p, k), xq = dnode(a, q, k), xr = dnode(a, r, k);
-  DV<Real> e1 = dsub(xq, xp), e2 = dsub(xr, xp);
-  D3<Real> g11 = ddot(e1, e1), g12 = ddot(e1, e2), g22 = ddot(e2, e2);
-  const Real* K = a.skc + 5 * t;
-  D3<Real> tr = K[0] * g11 + K[1] * g12 + K[2] * g22;
-  D3<Real> det = K[3] * (g11 * g22 - g12 * g12);
-  D3<Real> I1 = tr - dc<Real>(2), I2 = det - dc<Real>(1);
-  int cap = a.ecap[t];
-  Real G = a.capr[2 * a.ncaps + cap], C = a.capr[3 * a.ncaps + cap];
-  D3<Real> w = (G * Real(0.25)) * (I1 * I1 + Real(2) * I1 - Real(2) * I2 + C * (I2 * I2));
-  return K[4] * w;
+__device__ __forceinline__ V3<Real> face_force(const IBArgs<Real>& a, int k, int e) {
+  const int q0 = a.E[3 * e], q1 = a.E[3 * e + 1], q2 = a.E[3 * e + 2];
+  const int u = q0 == k ? q1 : (q1 == k ? q2 : q0);
+  const int v = q0 == k ? q2 : (q1 == k ? q0 : q1);
+  const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = ev - eu;
+  const R4<Real> Nk = a.nadj[k], Nu = a.nadj[u], Nv = a.nadj[v];
+  const Real duu = dot(eu, eu), dvv = dot(ev, ev), dk = dot(eu, ev), dww = dot(w, w);
+  // bending
+  const V3<Real> cr = cross(eu, ev);
+  const Real A2 = sqrt(dot(cr, cr)), iA2 = Real(1) / A2;
+  const Real du = -dot(eu, w), dv = dot(ev, w);
+  const Real ck = dk * iA2, cu = du * iA2, cv = dv * iA2;
+  const V3<Real> Ku = mk<Real>(Nk.x - Nu.x, Nk.y - Nu.y, Nk.z - Nu.z), Kv = mk<Real>(Nk.x - Nv.x, Nk.y - Nv.y, Nk.z - Nv.z);
+  const V3<Real> Kw = mk<Real>(Nu.x - Nv.x, Nu.y - Nv.y, Nu.z - Nv.z);
+  Real Pv = -dot(eu, Ku), Pu = -dot(ev, Kv), Pk = -dot(w, Kw), S = 0;  // S: factor of A2
+  V3<Real> g = cv * Ku + cu * Kv;  // the cotangents times dP
+  if (dk < 0 || du < 0 || dv < 0) {
+    S = (dk < 0 ? Real(0.25) : Real(0.125)) * Nk.w + (du < 0 ? Real(0.25) : Real(0.125)) * Nu.w +
+        (dv < 0 ? Real(0.25) : Real(0.125)) * Nv.w;
+  } else {
+    const Real au = Real(0.125) * (Nk.w + Nu.w), av = Real(0.125) * (Nk.w + Nv.w);
+    Pv += duu * au;
+    Pu += dvv * av;
+    Pk += dww * Real(0.125) * (Nu.w + Nv.w);
+    g = g - (Real(2) * cv * au) * eu - (Real(2) * cu * av) * ev;
+  }
+  // d(d_k) = -(eu + ev), d(d_u) = w, d(d_v) = -w, dA2 = n x w
+  const V3<Real> dA = iA2 * cross(cr, w);
+  g = g + (iA2 * (Pu - Pv)) * w - (iA2 * Pk) * (eu + ev) + (S - iA2 * (cv * Pv + cu * Pu + ck * Pk)) * dA;
+  // Skalak: with the metric of the edges from the face's first vertex,
+  // dE = D1 dI1 + D2 dI2
+  const Real* c = a.skc + 5 * e;
+  const int cap = a.ecap[e];
+  const Real G = a.capr[2 * a.ncaps + cap], C = a.capr[3 * a.ncaps + cap];
+  // e1, e2 of the face in terms of (eu, ev): first vertex k: (eu, ev); v: (-ev,
+  // -w) (to k and u); u: (w, -eu) (to v and k)
+  const V3<Real> e1 = q0 == k ? eu : (q1 == k ? Real(-1) * ev : w);
+  const V3<Real> e2 = q0 == k ? ev : (q1 == k ? Real(-1) * w : Real(-1) * eu);
+  const Real g11 = q0 == k ? duu : (q1 == k ? dvv : dww), g22 = q0 == k ? dvv : (q1 == k ? dww : duu);
+  const Real g12 = dot(e1, e2);
+  const Real I1 = c[0] * g11 + c[1] * g12 + c[2] * g22 - Real(2), I2 = c[3] * (g11 * g22 - g12 * g12) - Real(1);
+  const Real q = c[4] * G * Real(0.5);
+  const Real D1 = q * (I1 + Real(1)), D2 = q * (C * I2 - Real(1)) * c[3];
+  const Real h11 = Real(2) * (D1 * c[0] + D2 * g22), h22 = Real(2) * (D1 * c[2] + D2 * g11), h12 = D1 * c[1] - Real(2) * D2 * g12;
+  const V3<Real> f1 = h11 * e1 + h12 * e2, f2 = h22 * e2 + h12 * e1;  // dE/de1, dE/de2
+  const V3<Real> sk = q0 == k ? Real(-1) * (f1 + f2) : (q1 == k ? f1 : f2);
+  return Real(-1) * (g + sk);
 }
-
-// Helfrich energy of vertex v: kb |sum_T (cot_k (x_v - x_j) + cot_j (x_v - x_k))|^2 / (8 A_v)
-// with A_v the mixed Voronoi area (Meyer et al. 2003).  One term: the
-// contributions of face t of v to the sums K and A, differentiated with
-// respect to X_k.
-template <class Real>
-__device__ __forceinline__ void helfrich_term(const IBArgs<Real>& a, int v, int t, int k, DV<Real>& Kc, D3<Real>& Ac) {
-  int q0 = a.E[3 * t], q1 = a.E[3 * t + 1], q2 = a.E[3 * t + 2];
-  int j = q0 == v ? q1 : (q1 == v ? q2 : q0);
-  int kk = q0 == v ? q2 : (q1 == v ? q0 : q1);
-  DV<Real> xv = dnode(a, v, k), xj = dnode(a, j, k), xk = dnode(a, kk, k);
-  DV<Real> vj = dsub(xv, xj), vk = dsub(xv, xk);
-  DV<Real> kj = dsub(xk, xj), jk = dsub(xj, xk);
-  DV<Real> c1 = dcross(vj, kj), c2 = dcross(vk, jk);
-  D3<Real> cotj = ddot(vj, kj) / dsqrt(ddot(c1, c1));
-  D3<Real> cotk = ddot(vk, jk) / dsqrt(ddot(c2, c2));
-  Kc.x = cotk * vj.x + cotj * vk.x;
-  Kc.y = cotk * vj.y + cotj * vk.y;
-  Kc.z = cotk * vj.z + cotj * vk.z;
-  DV<Real> ej = dsub(xj, xv), ek = dsub(xk, xv);
-  DV<Real> cr = dcross(ej, ek);
-  D3<Real> area = Real(0.5) * dsqrt(ddot(cr, cr));
-  Real dv = ddot(ej, ek).v, dj = ddot(vj, kj).v, dk = ddot(vk, jk).v;
-  if (dv < 0) Ac = Real(0.5) * area;
-  else if (dj < 0 || dk < 0) Ac = Real(0.25) * area;
-  else Ac = Real(0.125) * (ddot(vj, vj) * cotk + ddot(vk, vk) * cotj);
-}
-
-// Elastic node forces, one warp per marker (2D stretching + bending; 3D
-// Skalak + Helfrich, differentiated with forward-mode duals with respect to
-// the marker).  In 3D lane t takes the Skalak term of incident face t, and
-// the Helfrich terms of the marker and its 1-ring vertices are shared out
-// as (vertex, face) pairs, 32 at a time: each lane stages its pair's
-// contributions to K and A, the lane of each vertex adds them in face order
-// and forms the vertex's energy.  Lane sums are combined by a fixed shuffle
-// tree.  They depend on the marker positions only; the coupling force joins
-// them in k_spread.
 template <class Real>
 __device__ __forceinline__ void node_forces_body(const IBArgs<Real>& a, const Blk& blk) {
-  __shared__ Real hstage[NODEF_WARPS][32 * 16];  // one chunk of Helfrich pairs per warp
-  const int k = (blk.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (k >= a.nn) return;
-  Real F[3] = {0, 0, 0};
-  if (a.NV == 2) {
-    if (lane == 0) {
-      // 2D ring: segment l joins node l -> next(l) (eq. DiscreteSE), bending
-      // at nodes prev, k, next (eqs. DiscreteBE, DiscreteTheta, DiscreteArcLength).
-      const int cap = a.ncap[k];
-      const Real ks = a.capr[cap], kb = a.capr[a.ncaps + cap];
-      for (int side = 0; side < 2; ++side) {
-        int e = a.inc[a.inc_off[k] + side];
-        int p = a.E[2 * e], q = a.E[2 * e + 1];
-        Real tx = node_dx(a, q, p, 0), tz = node_dx(a, q, p, 2);
-        Real L = sqrt(tx * tx + tz * tz);
-        Real T = ks * (L / (Real)a.ds0[e] - Real(1)) / L;
-        Real sgn = (p == k) ? Real(1) : Real(-1);  // -dE/dX_p = +T t ; -dE/dX_q = -T t
-        F[0] += sgn * T * tx;
-        F[2] += sgn * T * tz;
-      }
-      int ms[3] = {a.rprev[k], k, a.rnext[k]};
-      for (int mi = 0; mi < 3; ++mi) {
-        int m = ms[mi], mp = a.rnext[m], mq = a.rprev[m];
-        Real ax = node_dx(a, mp, m, 0), az = node_dx(a, mp, m, 2);
-        Real bx = node_dx(a, m, mq, 0), bz = node_dx(a, m, mq, 2);
-        Real la = sqrt(ax * ax + az * az), lb = sqrt(bx * bx + bz * bz);
-        Real ab = ax * bx + az * bz;
-        Real cr = ax * bz - az * bx;
-        // theta1 = arccos(a.b / |a||b|), evaluated as atan2(|a x b|, a.b)
-        Real th = atan2(fabs(cr), ab);
-        Real sn = fabs(cr) / (la * lb);
-        Real ratio = th < Real(1e-4) ? Real(1) + th * th / Real(6) : th / sn;
-        Real dsp = la + lb;
-        Real k1 = Real(0.25) * kb * (Real(-8) * ratio / dsp);
-        Real dth = Real(2) * th;
-        Real k2 = Real(0.25) * kb * (dth / dsp) * (dth / dsp);
-        Real iab = Real(1) / (la * lb);
-        Real dya_x = bx * iab - ab * ax * iab / (la * la), dya_z = bz * iab - ab * az * iab / (la * la);
-        Real dyb_x = ax * iab - ab * bx * iab / (lb * lb), dyb_z = az * iab - ab * bz * iab / (lb * lb);
-        Real gx = 0, gz = 0;
-        if (k == mp) { gx += k1 * dya_x - k2 * ax / la; gz += k1 * dya_z - k2 * az / la; }
-        if (k == m) {
-          gx += k1 * (dyb_x - dya_x) - k2 * (bx / lb - ax / la);
-          gz += k1 * (dyb_z - dya_z) - k2 * (bz / lb - az / la);
-        }
-        if (k == mq) { gx += -k1 * dyb_x + k2 * bx / lb; gz += -k1 * dyb_z + k2 * bz / lb; }
-        F[0] -= gx;
-        F[2] -= gz;
-      }
-    }
-  } else {
-    const int i0 = a.inc_off[k], ninc = a.inc_off[k + 1] - i0;
-    if (lane < 16 && lane < ninc) {
-      D3<Real> e = skalak_dual(a, a.inc[i0 + lane], k);
-      F[0] -= e.d0; F[1] -= e.d1; F[2] -= e.d2;
-    }
-    // Helfrich vertex slots: 0 the marker, 1.. its distinct 1-ring
-    // neighbours in the order of the incident faces and their vertices
-    const int r0 = a.ring_off[k], nV = min(a.ring_off[k + 1] - r0 + 1, 16);
-    int vs = 0, fs = 0, ds = 0;
-    if (lane < nV) {
-      vs = lane == 0 ? k : a.ring[r0 + lane - 1];
-      fs = a.inc_off[vs];
-      ds = a.inc_off[vs + 1] - fs;
-    }
-    int incl = ds;
-#pragma unroll
-    for (int sh = 1; sh < 32; sh <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, sh);
-      if (lane >= sh) incl += v;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    Real* stg = hstage[threadIdx.x >> 5];
-    DV<Real> K = {dc<Real>(0), dc<Real>(0), dc<Real>(0)};
-    D3<Real> A = dc<Real>(0);
-    for (int p0 = 0; p0 < total; p0 += 32) {
-      const int p = p0 + lane;
-      int S = 0;  // slot of pair p: the first whose inclusive prefix exceeds p
-#pragma unroll
-      for (int step = 16; step >= 1; step >>= 1) {
-        const int v = __shfl_sync(0xffffffffu, incl, S + step - 1);
-        if (v <= p) S += step;
-      }
-      const int vS = __shfl_sync(0xffffffffu, vs, S), fS = __shfl_sync(0xffffffffu, fs, S);
-      const int eS = __shfl_sync(0xffffffffu, incl, S) - __shfl_sync(0xffffffffu, ds, S);
-      if (p < total) {
-        DV<Real> Kc;
-        D3<Real> Ac;
-        helfrich_term(a, vS, a.inc[fS + p - eS], k, Kc, Ac);
-        const Real c[16] = {Kc.x.v, Kc.x.d0, Kc.x.d1, Kc.x.d2, Kc.y.v, Kc.y.d0, Kc.y.d1, Kc.y.d2,
-                            Kc.z.v, Kc.z.d0, Kc.z.d1, Kc.z.d2, Ac.v,   Ac.d0,   Ac.d1,   Ac.d2};
-#pragma unroll
-        for (int q = 0; q < 16; ++q) stg[lane * 16 + q] = c[q];
-      }
-      __syncwarp();
-      if (lane < nV) {  // this slot's pairs of the chunk, in face order
-        const int lo = max(incl - ds, p0), hi = min(incl, p0 + 32);
-        for (int q = lo; q < hi; ++q) {
-          const Real* c = stg + (q - p0) * 16;
-          K.x = K.x + D3<Real>{c[0], c[1], c[2], c[3]};
-          K.y = K.y + D3<Real>{c[4], c[5], c[6], c[7]};
-          K.z = K.z + D3<Real>{c[8], c[9], c[10], c[11]};
-          A = A + D3<Real>{c[12], c[13], c[14], c[15]};
-        }
-      }
-      __syncwarp();
-    }
-    if (lane < nV) {
-      const Real kb = a.capr[a.ncaps + a.ncap[vs]];
-      D3<Real> h = (kb * Real(0.125)) * (ddot(K, K) / A);
-      F[0] -= h.d0; F[1] -= h.d1; F[2] -= h.d2;
+  const int t = blk.x * blockDim.x + threadIdx.x, lane = t & 15;
+  const bool valid = (t >> 4) < a.nn;
+  const int k = valid ? t >> 4 : a.nn - 1;
+  V3<Real> F = mk<Real>(0, 0, 0);
+  if (valid) {
+    if (a.NV == 2) {
+      if (lane < 5) F = ring_force(a, k, lane);
+    } else {
+      const int i0 = a.inc_off[k], ninc = a.inc_off[k + 1] - i0;
+      for (int j = lane; j < ninc; j += 16) F = F + face_force(a, k, a.inc[i0 + j]);
     }
   }
-  for (int d = 0; d < 3; ++d)
-    for (int o = 16; o > 0; o >>= 1) F[d] += __shfl_xor_sync(0xffffffffu, F[d], o);
-  if (lane == 0) {
-    if (a.dim == 2) F[1] = 0;
-    for (int d = 0; d < 3; ++d) a.F[3 * k + d] = F[d];
-  }
+  F = mk<Real>(group_sum(F.x), group_sum(F.y), group_sum(F.z));
+  if (!valid || lane != 0) return;
+  a.F[3 * k] = F.x;
+  a.F[3 * k + 1] = a.dim == 2 ? Real(0) : F.y;
+  a.F[3 * k + 2] = F.z;
 }
 template <class Real>
 __global__ void k_node_forces(const __grid_constant__ IBArgs<Real> a) {
-  if (blockIdx.x == 0 && threadIdx.x < 2) a.ctr[threadIdx.x] = 0;  // the brick compaction's counters
   node_forces_body(a, hw_blk());
 }
 
@@ -1221,6 +1159,7 @@ __device__ __forceinline__ void brick_count_body(const IBArgs<Real>& a, const Bl
 }
 template <class Real>
 __global__ void k_brick_count(const __grid_constant__ IBArgs<Real> a) {
+  if (blockIdx.x == 0 && threadIdx.x < 2) a.ctr[threadIdx.x] = 0;  // the brick compaction's counters
   brick_count_body(a, hw_blk());
 }
 

@@ -103,12 +103,11 @@ struct Impl : ImplBase {
     a.inc_off = c->ptr<int>(c->L.inc_off);
     a.inc = c->ptr<int>(c->L.inc);
     a.adj = c->ptr<int>(c->L.adj);
-    a.ring_off = c->ptr<int>(c->L.ring_off);
-    a.ring = c->ptr<int>(c->L.ring);
     a.nedge = c->nedge;
     a.edges = c->ptr<int>(c->L.edges);
     a.en = c->ptr<Real>(c->L.en);
     a.vn = c->ptr<Real>(c->L.vn);
+    a.nadj = c->ptr<R4<Real>>(c->L.nadj);
     a.erel = c->ptr<R4<Real>>(c->L.erel);
     a.eorg = c->ptr<int4>(c->L.eorg);
     a.ecst = c->ptr<R4<Real>>(c->L.ecst);
@@ -157,10 +156,12 @@ struct Impl : ImplBase {
   // brick binning in ibm_bins).  It runs on the side stream while the
   // moments of the step are computed.
   // With snap the geometry kernel also takes the marker box's snapshot (the
-  // advection's accumulator) and resets it.
-  static tlb_status ibm_positions(Ctx* c, IBArgs<Real>& a, cudaStream_t s, bool snap = false) {
-    k_geometry<Real><<<blocks((long long)c->ne + c->nn, 128), 128, 0, s>>>(a, snap ? 1 : 0);
+  // advection's accumulator) and resets it; `done` is recorded after it.
+  static tlb_status ibm_positions(Ctx* c, IBArgs<Real>& a, cudaStream_t s, bool snap = false,
+                                  cudaEvent_t done = nullptr) {
+    k_geometry<Real><<<blocks(geometry_threads(c->ne, c->nn), 128), 128, 0, s>>>(a, snap ? 1 : 0);
     TLB_LAUNCHED(c, "k_geometry");
+    if (done) TLB_CUDA(cudaEventRecord(done, s));
     constexpr int sw = scatter_warps<Real>();
     const unsigned nvb = (unsigned)a.split * blocks(c->features(), 32 * sw);
     k_dist_scatter<Real><<<std::min(nvb, 4u * (unsigned)c->nsm), 32 * sw, 0, s>>>(a, (int)nvb);
@@ -182,17 +183,19 @@ struct Impl : ImplBase {
     return TLB_OK;
   }
 
-  // Elastic forces and the binning of markers into spreading bricks (the
-  // bins are consumed and reset by k_spread of the same step).
-  static tlb_status ibm_bins(Ctx* c, IBArgs<Real>& a, cudaStream_t s) {
-    k_node_forces<Real><<<blocks((long long)c->nn * 32, 128), 128, 0, s>>>(a);  // (clears ctr)
-    TLB_LAUNCHED(c, "k_node_forces");
-    k_brick_count<Real><<<blocks(c->nn, 128), 128, 0, s>>>(a);
+  // The binning of markers into spreading bricks (the bins are consumed and
+  // reset by k_spread of the same step) and, once the geometry is done, the
+  // elastic forces.
+  static tlb_status ibm_bins(Ctx* c, IBArgs<Real>& a, cudaStream_t s, cudaEvent_t geometry) {
+    k_brick_count<Real><<<blocks(c->nn, 128), 128, 0, s>>>(a);  // (clears ctr)
     TLB_LAUNCHED(c, "k_brick_count");
     k_brick_compact<Real><<<blocks(c->nbricks, 256), 256, 0, s>>>(a);
     TLB_LAUNCHED(c, "k_brick_compact");
     k_brick_fill<Real><<<blocks(c->nn, 128), 128, 0, s>>>(a);
     TLB_LAUNCHED(c, "k_brick_fill");
+    TLB_CUDA(cudaStreamWaitEvent(s, geometry, 0));
+    k_node_forces<Real><<<blocks((long long)c->nn * 16, 128), 128, 0, s>>>(a);
+    TLB_LAUNCHED(c, "k_node_forces");
     return TLB_OK;
   }
 
@@ -583,8 +586,8 @@ struct Impl : ImplBase {
         // the previous advection (a graph's first step follows the whole
         // previous launch on the caller's stream instead)
         if (pipe && !(c->capturing && k == 0)) TLB_CUDA(cudaStreamWaitEvent(c->side2, c->ev_interp, 0));
-        if ((st = ibm_positions(c, ia, c->side, box_on_side)) != TLB_OK) return st;
-        if ((st = ibm_bins(c, ia, c->side2)) != TLB_OK) return st;
+        if ((st = ibm_positions(c, ia, c->side, box_on_side, c->ev_geom)) != TLB_OK) return st;
+        if ((st = ibm_bins(c, ia, c->side2, c->ev_geom)) != TLB_OK) return st;
         TLB_CUDA(cudaEventRecord(c->ev_bins, c->side2));
       }
       if ((st = launch_moments(c, la, s)) != TLB_OK) return st;
