@@ -287,8 +287,8 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.inc, NV * ne * 4);
   take(L.adj, 3 * ne * 4);
   take(L.edges, 4 * (size_t)c.nedge * 4);
-  take(L.en, 3 * ne * R);
-  take(L.vn, 3 * nn * R);
+  take(L.en, 4 * ne * R);
+  take(L.vn, 4 * nn * R);
   take(L.nadj, 4 * nn * R);
   take(L.erel, 4 * ne * R);
   take(L.eorg, 4 * ne * 4);
@@ -385,8 +385,9 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
     if (r0 == TLB_OK) r0 = cuda_check(cudaEventCreateWithFlags(&c->ev_interp, cudaEventDisableTiming), "event");
     if (r0 != TLB_OK) { delete c; return r0; }
   }
+  box_estimates(c, &c->band_blocks, &c->spread_blocks);
   c->tiles_zc = c->impl->collide_chunk({c}, c->tile_variant);
-  c->scat_split = scatter_split((c->features() + 31) / 32, params->dc, c->nsm);
+  c->scat_split = scatter_split((c->features() + 31) / 32, params->dc, c->nsm, 1);
   c->recon_zc = c->impl->recon_chunk({c}, params->dim == 3 ? 32 : 64, params->dim == 3 ? 4 : 1);
   // zero everything, then set the non-zero initial values
   tlb_status r = cuda_check(cudaMemsetAsync(c->base, 0, c->L.total, st), "memset arena");

@@ -166,10 +166,10 @@ struct BatchImpl : BatchBase {
         return {mem ? b->scat_split * (int)cdiv(c->features(), 32 * scatter_warps<typename Prec<MODE>::Real>()) : 0, 1, 1};
       }
       case BCOMP: return {mem ? (int)cdiv(c->nbricks, NT) : 0, 1, 1};
-      case BAND: return {mem ? b->band_blocks[i] : 0, 1, 1};
+      case BAND: return {mem ? c->band_blocks : 0, 1, 1};
       case BFILL: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
       case FILL: return {mem ? (int)cdiv(32ll * c->nx * c->ny, NT) : 0, 1, 1};
-      case SPREAD: return {mem ? b->spread_blocks[i] : 0, 1, 1};
+      case SPREAD: return {mem ? c->spread_blocks : 0, 1, 1};
       case COLL: {
         const int tx = tile_x(b->tile_variant), ty = tile_y(b->tile_variant);
         return {(int)cdiv(c->nx, tx), (int)cdiv(c->ny, ty), (int)cdiv(c->nz, b->zc)};

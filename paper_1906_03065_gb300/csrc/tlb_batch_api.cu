@@ -52,29 +52,6 @@ static tlb_status batch_plan(const tlb_instance_desc* inst, int n, BatchPlan& bp
   return TLB_OK;
 }
 
-// Virtual blocks of the box-sized operations (profile band, spreading): the
-// work scales with the marker box, estimated from the initial markers.
-static void box_estimates(const Ctx* c, int* band_blocks, int* spread_blocks) {
-  if (c->nn == 0) { *band_blocks = *spread_blocks = 0; return; }
-  double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-  for (const HostMem& m : c->mems)
-    for (int l = 0; l < m.nn; ++l)
-      for (int d = 0; d < 3; ++d) {
-        lo[d] = std::min(lo[d], m.X0[3 * l + d]);
-        hi[d] = std::max(hi[d], m.X0[3 * l + d]);
-      }
-  const int n[3] = {c->nx, c->ny, c->nz};
-  const double margin = 2.0 * (ceil(c->p.dc) + 2.0) + 2.0;
-  double cells = 1, bricks = 1;
-  for (int d = 0; d < 3; ++d) {
-    cells *= std::min((double)n[d], hi[d] - lo[d] + margin);
-    bricks *= std::min(ceil(n[d] / 4.0), ceil((hi[d] - lo[d] + 4.0) / 4.0) + 1.0);
-  }
-  // about two box cells per thread of a 128-thread block
-  *band_blocks = (int)std::max(1.0, std::min(65536.0, ceil(cells / 256.0)));
-  *spread_blocks = (int)std::max(1.0, std::min((double)c->nbricks, bricks));
-}
-
 extern "C" {
 
 tlb_status tlb_batch_state_bytes(const tlb_instance_desc* inst, int n_inst, size_t* bytes) {
@@ -129,10 +106,6 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
     Ctx* c = (Ctx*)h;
     b->inst.push_back(c);
     b->act.push_back(i);
-    int bb = 0, sb = 0;
-    box_estimates(c, &bb, &sb);
-    b->band_blocks.push_back(bb);
-    b->spread_blocks.push_back(sb);
   }
   // the tau = 1 collide wherever it applies; one force form per batch
   b->tile_variant = 3;
@@ -160,7 +133,7 @@ tlb_status tlb_batch_create(const tlb_instance_desc* inst, int n_inst, void* are
     warps += (c->features() + 31) / 32;
     dcmax = std::max(dcmax, c->p.dc);
   }
-  b->scat_split = scatter_split(warps, dcmax, b->inst[0]->nsm);
+  b->scat_split = scatter_split(warps, dcmax, b->inst[0]->nsm, 4);
   for (int q = 0; q < 2; ++q) b->targs[q] = {bp.targs[q], (size_t)n_inst * Batch::ARGS_BYTES};
   b->vg = {bp.vg, (size_t)Batch::NPH * Batch::MAXOPS * n_inst * 16};
   b->res = {bp.res, (size_t)n_inst * 4 * 8};

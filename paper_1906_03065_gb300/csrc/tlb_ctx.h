@@ -3,8 +3,10 @@
 // tlb_create; no other device memory is ever allocated.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -83,10 +85,12 @@ inline SweepCost collide_cost(int resident, int threads, bool f64, bool t1) {
 inline SweepCost recon_cost(int resident, int threads, bool f64) { return {resident, 3.0, (f64 ? 0.8 : 0.6) * threads / 128}; }
 
 // Warps that share one group of 32 features in the distance scatter: as many
-// as bring its warps to 16 per SM, at most one per round of slices (4 slices
-// each, 2 dc + 3 per feature or so); for `warps` groups swept together.
-inline int scatter_split(long long warps, double dc, int nsm) {
-  const long long rounds = ((long long)(2 * dc) + 3 + 3) / 4, want = (16ll * nsm + warps / 2) / (warps > 0 ? warps : 1);
+// as bring its warps to 16 per SM (a batch: four times that, so that the last
+// of its waves over the resident blocks costs little), at most one per round
+// of slices (4 slices each, 2 dc + 3 per feature or so); for `warps` groups
+// swept together.
+inline int scatter_split(long long warps, double dc, int nsm, int waves) {
+  const long long rounds = ((long long)(2 * dc) + 3 + 3) / 4, want = (16ll * waves * nsm + warps / 2) / (warps > 0 ? warps : 1);
   return (int)(want < 1 ? 1 : (want > rounds ? rounds : want));
 }
 
@@ -212,6 +216,7 @@ struct Ctx {
   int tiles_zc = 16;
   int recon_zc = 16;     // the same of the moments rebuild
   int scat_split = 1;    // see scatter_split
+  int band_blocks = 0, spread_blocks = 0;  // see box_estimates
   long long features() const { return (long long)ne + nedge + nn; }  // of the distance scatter
   int tile_variant = 0;  // collide tile shape and form (see collide_variant)
   PhaseEvents* prof = nullptr;  // non-null while tlb_profile_steps runs
@@ -260,6 +265,29 @@ struct Ctx {
   }
 };
 
+// Blocks of the box-sized operations (profile band, spreading): the
+// work scales with the marker box, estimated from the initial markers.
+inline void box_estimates(const Ctx* c, int* band_blocks, int* spread_blocks) {
+  if (c->nn == 0) { *band_blocks = *spread_blocks = 0; return; }
+  double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+  for (const HostMem& m : c->mems)
+    for (int l = 0; l < m.nn; ++l)
+      for (int d = 0; d < 3; ++d) {
+        lo[d] = std::min(lo[d], m.X0[3 * l + d]);
+        hi[d] = std::max(hi[d], m.X0[3 * l + d]);
+      }
+  const int n[3] = {c->nx, c->ny, c->nz};
+  const double margin = 2.0 * (ceil(c->p.dc) + 2.0) + 2.0;
+  double cells = 1, bricks = 1;
+  for (int d = 0; d < 3; ++d) {
+    cells *= std::min((double)n[d], hi[d] - lo[d] + margin);
+    bricks *= std::min(ceil(n[d] / 4.0), ceil((hi[d] - lo[d] + 4.0) / 4.0) + 1.0);
+  }
+  // about two box cells per thread of a 128-thread block
+  *band_blocks = (int)std::max(1.0, std::min(65536.0, ceil(cells / 256.0)));
+  *spread_blocks = (int)std::max(1.0, std::min((double)c->nbricks, bricks));
+}
+
 struct Batch;
 
 struct BatchBase {
@@ -289,7 +317,6 @@ struct Batch {
   char* base = nullptr;
   size_t bytes = 0;
   Region targs[2], vg, res;
-  std::vector<int> band_blocks, spread_blocks;  // virtual grids of the box-sized ops
   int ph_ent[NPH] = {0}, ph_total[NPH] = {0}, ph_grid[NPH] = {0};
   cudaGraphExec_t graph = nullptr;
   bool graph_dirty = true;

@@ -41,8 +41,8 @@ struct IBArgs {
   int nedge;             // 3D: unique edges
   const int* edges;      // 3D: [nedge][4] vertex a, vertex b, face left, face right
   // per-step work
-  Real* en;              // [ne][3] unit outward normal
-  Real* vn;              // [nn][3] angle-weighted vertex pseudo-normal
+  R4<Real>* en;          // [ne] unit outward normal
+  R4<Real>* vn;          // [nn] angle-weighted vertex pseudo-normal
   R4<Real>* nadj;        // [nn] 3D: derivatives of the marker's bending energy with
                          // respect to its K (three) and A (see geometry_body)
   // per element, read as whole vectors by the band:
@@ -233,9 +233,7 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
   int t = blk.x * blockDim.x + threadIdx.x;
   if (t < a.ne) {
     V3<Real> n = face_normal(a, t);
-    a.en[3 * t] = n.x;
-    a.en[3 * t + 1] = n.y;
-    a.en[3 * t + 2] = n.z;
+    a.en[t] = R4<Real>{n.x, n.y, n.z, 0};
     const int* Et = a.E + a.NV * t;
     Real rv[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     int org[3];
@@ -294,9 +292,7 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
     A = group_sum(A);
   }
   if (!valid || lane != 0) return;
-  a.vn[3 * k] = s.x;
-  a.vn[3 * k + 1] = s.y;
-  a.vn[3 * k + 2] = s.z;
+  a.vn[k] = R4<Real>{s.x, s.y, s.z, 0};
   if (a.NV == 3) {
     const Real kA = Real(0.25) * a.capr[a.ncaps + a.ncap[k]] / A;
     a.nadj[k] = R4<Real>{kA * K.x, kA * K.y, kA * K.z, Real(-0.5) * kA * dot(K, K) / A};
@@ -363,21 +359,10 @@ __device__ __forceinline__ long long cell_of(const IBArgs<Real>& a, const int* p
   return ((long long)z * a.G.ny + y) * a.G.nx + x;
 }
 
-// Fixed-point conversions from the bits of an FP32 value, equal to the
-// conversions of the exactly scaled number (v * 2^s) that the FP64 path
-// makes, without FP64 arithmetic (a slow pipe on this GPU).
-// floor(v 2^s) for finite v >= 0, v 2^s < 2^63:
-__device__ __forceinline__ unsigned long long scaled_floor_u64(float v, int s) {
-  const unsigned b = __float_as_uint(v);
-  int e = (int)((b >> 23) & 0xFFu);
-  unsigned long long m = b & 0x7FFFFFu;
-  if (e) m |= 0x800000u;
-  else e = 1;
-  const int sh = e - 150 + s;  // v = m 2^(e - 150)
-  return sh >= 0 ? m << sh : (sh > -24 ? m >> -sh : 0ull);
-}
-// distance part of a scatter key: the distance on a grid of 2^-34
-__device__ __forceinline__ unsigned long long dist_code(float d) { return scaled_floor_u64(d, 34); }
+// Distance part of a scatter key (d >= 0): the distance on a grid of 2^-34;
+// in FP32 the bits of d, which order as d does (from d = 2^-10 up every FP32
+// value is on that grid).
+__device__ __forceinline__ unsigned long long dist_code(float d) { return __float_as_uint(d); }
 __device__ __forceinline__ unsigned long long dist_code(double d) {
   return (unsigned long long)(d * 17179869184.0);
 }
@@ -450,6 +435,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
   // ---- the lane's feature: corners, cone generators (the normals of the
   // faces containing it), slice axis and range, offered face
   int kind = 0, nB = 0, nG = 0, i0 = 0, corners[3] = {0, 0, 0};
+  int4 ed = make_int4(0, 0, 0, 0);  // an edge: its ends and faces
   if (f < nfeat) {
     if (f < a.ne) {  // face (3D) or segment (2D)
       nB = a.NV;
@@ -457,9 +443,9 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       for (int q = 0; q < a.NV; ++q) corners[q] = a.E[a.NV * f + q];
     } else if (a.NV == 3 && f < a.ne + a.nedge) {  // edge
       kind = 1;
-      const int* ed = a.edges + 4 * (f - a.ne);
-      corners[0] = ed[0];
-      corners[1] = ed[1];
+      ed = __ldg(reinterpret_cast<const int4*>(a.edges) + (f - a.ne));
+      corners[0] = ed.x;
+      corners[1] = ed.y;
       nB = 2;
       nG = 2;
     } else {  // vertex
@@ -471,21 +457,26 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       nG = min(a.inc_off[v + 1] - i0, MAXG);
     }
   }
-  auto face_of = [&](int j) { return kind == 0 ? f : (kind == 1 ? a.edges[4 * (f - a.ne) + 2 + j] : a.inc[i0 + j]); };
   bool ok = nG > 0;
   int o[3] = {0, 0, 0}, tmin = 0x7fffffff;
   Real S[3] = {0, 0, 0};
   if (ok) {
     for (int d = 0; d < 3; ++d) o[d] = a.xo[3 * corners[0] + d];
     if (a.dim == 2) o[1] = 0;
+    // the generators, kept as they come (components x, y, z) until the slice
+    // axis is known; the read-only loads of an unrolled group are all in flight
+#pragma unroll 4
     for (int j = 0; j < nG; ++j) {
-      const int t = face_of(j);
+      const int t = kind == 0 ? f : (kind == 1 ? (j ? ed.w : ed.z) : __ldg(a.inc + i0 + j));
+      const R4<Real> n = ldg4(a.en + t);
       tmin = min(tmin, t);
-      for (int d = 0; d < 3; ++d) {
-        const Real g = a.en[3 * t + d];
-        S[d] += g;
-        ok &= fabs(g) <= Real(1.001);
-      }
+      S[0] += n.x;
+      S[1] += n.y;
+      S[2] += n.z;
+      ok &= fabs(n.x) <= Real(1.001) && fabs(n.y) <= Real(1.001) && fabs(n.z) <= Real(1.001);
+      sm.gk[lane][j] = n.x;
+      sm.ga[lane][j] = n.y;
+      sm.gb[lane][j] = n.z;
     }
     for (int q = 0; q < nB; ++q)
       for (int d = 0; d < 3; ++d) {
@@ -511,14 +502,17 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
   bool wide = false;
   if (ok) {
     Real gmin = Real(1e30f);
+    Real n0[3] = {0, 0, 0};  // a face's normal
     for (int j = 0; j < nG; ++j) {
-      const int t = face_of(j);
-      const Real gkj = a.en[3 * t + k];
+      const Real n[3] = {sm.gk[lane][j], sm.ga[lane][j], sm.gb[lane][j]};
+      const Real gkj = k == 0 ? n[0] : (k == 1 ? n[1] : n[2]);
       gmin = fmin(gmin, gkj * (S[k] >= 0 ? Real(1) : Real(-1)));
       // (the rectangles are widened by eps, far above the rounding of a product)
       sm.gk[lane][j] = rcp_rn(gkj);
-      sm.ga[lane][j] = a.en[3 * t + oa];
-      sm.gb[lane][j] = a.en[3 * t + ob];
+      sm.ga[lane][j] = oa == 0 ? n[0] : (oa == 1 ? n[1] : n[2]);
+      sm.gb[lane][j] = ob == 0 ? n[0] : (ob == 1 ? n[1] : n[2]);
+      if (j == 0)
+        for (int d = 0; d < 3; ++d) n0[d] = n[d];
     }
     wide = gmin < Real(0.25);  // a generator nearly parallel to the slices
     Real bmin = 1e30f, bmax = -1e30f;
@@ -537,7 +531,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       const Real* e = &a.ecst[4 * f].x;
       const Real d00 = e[9], d01 = e[10], d11 = e[11], iden = e[15];
       for (int d = 0; d < 3; ++d) {
-        p[d] = a.en[3 * f + d];
+        p[d] = n0[d];
         q[d] = a.NV == 2 ? e[d] * e[12] : (d11 * e[d] - d01 * e[3 + d]) * iden;
         r[d] = a.NV == 2 ? Real(0) : (d00 * e[3 + d] - d01 * e[d]) * iden;
       }
@@ -634,18 +628,20 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       }
       __syncwarp();
       const int n = min(total - base, SCAT_TAB);
-      for (int i = lane; i < n; i += 32) {
+      // one cell of the round: its index and key; false if nothing is offered
+      auto probe = [&](int i, long long& cell, unsigned long long& key) {
         const int id = sm.tab[i], L = id / SCAT_W, h = id % SCAT_W;
         const int4 e = sm.sl[L][h], F0 = sm.ft[L][0], F1 = sm.ft[L][1];
         const int jj = base + i - e.w;
-        // jj / wa: jj < 2^20 and wa <= 1024 keep the product within 2^-13 of the
-        // true (jj + 1/2) / wa, whose fraction is at least 2^-11 from an
-        // integer, so the truncation is exact
-        const int qb = (int)(((float)jj + 0.5f) * __frcp_rn((float)e.z));
+        // jj / wa with an approximate reciprocal: jj < 2^20, so the product is
+        // within 0.2 / wa of (jj + 1/2) / wa, which lies at least 1 / (2 wa)
+        // from an integer: the truncation is exact
+        const int qb = (int)(((float)jj + 0.5f) * __fdividef(1.0f, (float)e.z));
         const int rk = F1.y + r * SCAT_W + h, ra = e.x + (jj - qb * e.z), rb = a.dim == 3 ? e.y + qb : 0;
         // axes (k, a, b): 3D k = 0: (x, y, z); 1: (y, x, z); 2: (z, x, y); 2D the
         // plane (x, z) with b along the empty y
-        const int kk = F0.w & 3, kind_c = (F0.w >> 6) & 3;
+        const int kk = F0.w & 3;
+        const bool face = (F0.w & 192) == 0;
         int rx, ry, rz;
         if (a.dim == 3) {
           rx = kk == 0 ? rk : ra;
@@ -656,34 +652,29 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
           ry = 0;
           rz = kk == 0 ? ra : rk;
         }
+        // one expression for the three kinds (an edge's u and a vertex's v and
+        // p are zero), so that two cells are computed side by side
         const R4<Real> A = sm.rec[L][0], p = sm.rec[L][1], q = sm.rec[L][2];
         const Real ax = (Real)rx - A.x, ay = (Real)ry - A.y, az = (Real)rz - A.z;
-        Real dist;
-        if (kind_c == 0) {
-          const Real v = ax * q.x + ay * q.y + az * q.z, u = ax * A.w + ay * p.w + az * q.w;
-          if (!(v >= Real(0) && u >= Real(0) && v + u <= Real(1))) continue;
-          dist = fabs(ax * p.x + ay * p.y + az * p.z);
-        } else {
-          Real t = 0;
-          if (kind_c == 1) {
-            t = ax * q.x + ay * q.y + az * q.z;
-            if (!(t >= -eps && t <= Real(1) + eps)) continue;
-            t = fmin(Real(1), fmax(Real(0), t));
-          }
-          const Real x = ax - t * p.x, y = ay - t * p.y, z = az - t * p.z;
-          dist = sqrt(x * x + y * y + z * z);
-        }
-        if (!(dist < dc)) continue;
-        long long cell;
-        if (F0.w & 256) {  // (within dc of the feature, so inside the lattice)
-          cell = ((long long)(F0.z + rz) * a.G.ny + (F0.y + ry)) * a.G.nx + (F0.x + rx);
-        } else {
-          const int pc[3] = {F0.x + rx, F0.y + ry, F0.z + rz};
-          cell = cell_of(a, pc);
-          if (cell < 0) continue;
-        }
-        const unsigned long long key = (dist_code(dist) << 24) | (unsigned long long)F1.x;
-        atomicMin(a.key + cell, key);  // no return value: a fire-and-forget reduction
+        const Real v = ax * q.x + ay * q.y + az * q.z, u = ax * A.w + ay * p.w + az * q.w;
+        const Real t = fmin(Real(1), fmax(Real(0), v));
+        const Real x = ax - t * p.x, y = ay - t * p.y, z = az - t * p.z;
+        const Real dist = face ? fabs(ax * p.x + ay * p.y + az * p.z) : sqrt(x * x + y * y + z * z);
+        const bool on = face ? (v >= Real(0) && u >= Real(0) && v + u <= Real(1)) : (v >= -eps && v <= Real(1) + eps);
+        const int pc[3] = {F0.x + rx, F0.y + ry, F0.z + rz};
+        cell = ((long long)pc[2] * a.G.ny + pc[1]) * a.G.nx + pc[0];
+        // (inner features: what they offer lies within dc of them, in the lattice)
+        if (!(F0.w & 256)) cell = cell_of(a, pc);
+        key = (dist_code(dist) << 24) | (unsigned long long)F1.x;
+        return on && dist < dc && cell >= 0;
+      };
+      for (int i = lane; i < n; i += 64) {  // two cells at a time
+        long long c0i, c1i;
+        unsigned long long k0, k1;
+        const bool v0 = probe(i, c0i, k0), v1 = probe(min(i + 32, n - 1), c1i, k1) && i + 32 < n;
+        // no return value: fire-and-forget reductions
+        if (v0) atomicMin(a.key + c0i, k0);
+        if (v1) atomicMin(a.key + c1i, k1);
       }
     }
     __syncwarp();  // the next round rewrites the slice table
@@ -699,17 +690,14 @@ __global__ void __launch_bounds__(scatter_warps<Real>() * 32) k_dist_scatter(con
 // element normal; edge: sum of the two adjacent normals; vertex: vertex
 // pseudo-normal): +1 inside (d > 0 in eq. Iprofile), -1 outside.
 template <class Real>
-__device__ __forceinline__ Real feature_sign(const IBArgs<Real>& a, int e, int feat, V3<Real> xmP) {
-  V3<Real> N;
-  if (feat == 0) {
-    N = mk<Real>(a.en[3 * e], a.en[3 * e + 1], a.en[3 * e + 2]);
-  } else if (a.NV == 3 && feat <= 3) {
-    int f = a.adj[3 * e + (feat - 1)];
-    N = mk<Real>(a.en[3 * e] + a.en[3 * f], a.en[3 * e + 1] + a.en[3 * f + 1], a.en[3 * e + 2] + a.en[3 * f + 2]);
-  } else {
-    int q = feat - 4;
-    int k = a.E[a.NV * e + q];
-    N = mk<Real>(a.vn[3 * k], a.vn[3 * k + 1], a.vn[3 * k + 2]);
+__device__ __forceinline__ Real feature_sign(const IBArgs<Real>& a, int e, const R4<Real>& n, int feat, V3<Real> xmP) {
+  V3<Real> N = mk<Real>(n.x, n.y, n.z);
+  if (a.NV == 3 && feat >= 1 && feat <= 3) {
+    const R4<Real> m = ldg4(a.en + __ldg(a.adj + 3 * e + (feat - 1)));
+    N = mk<Real>(n.x + m.x, n.y + m.y, n.z + m.z);
+  } else if (feat > 0) {
+    const R4<Real> m = ldg4(a.vn + __ldg(a.E + a.NV * e + feat - 4));
+    N = mk<Real>(m.x, m.y, m.z);
   }
   // x - P points outward for a cell outside
   return dot(xmP, N) > Real(0) ? Real(-1) : Real(1);
@@ -803,7 +791,8 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
           // (the element origin, floor of its first vertex, is within a cell
           // of it: the nearest image is the same)
           int pi[3] = {pc[0], pc[1], pc[2]};
-          const int4 eo = a.eorg[e];
+          const int4 eo = __ldg(a.eorg + e);
+          const R4<Real> en = ldg4(a.en + e);
           if (full[0] | full[1] | full[2]) {
             if (full[0]) pi[0] += a.G.nx * __float2int_rn((float)(eo.x - pi[0]) / (float)a.G.nx);
             if (full[1]) pi[1] += a.G.ny * __float2int_rn((float)(eo.y - pi[1]) / (float)a.G.ny);
@@ -812,7 +801,7 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
           V3<Real> P = elem_closest(a, e, eo, pi, beta, &feat);
           V3<Real> xmP = mk<Real>(-P.x, -P.y, -P.z);
           Real dist = sqrt(dot(xmP, xmP));
-          Real s = feature_sign(a, e, feat, xmP);
+          Real s = feature_sign(a, e, en, feat, xmP);
           Real d = s * dist;
           // with E = exp(-|d|/alpha): I = (1 + tanh(d/(2 alpha)))/2 is 1/(1 + E)
           // inside and E/(1 + E) outside, sech^2(d/(2 alpha)) = 4 E/(1 + E)^2
@@ -824,7 +813,7 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
           const Real coef = a.kc * (psic - I) * (E * iE) * (iE * ial);
           V3<Real> dir;
           if (dist > Real(1e-12)) dir = (-s / dist) * xmP;
-          else dir = mk<Real>(a.en[3 * e], a.en[3 * e + 1], a.en[3 * e + 2]);
+          else dir = mk<Real>(en.x, en.y, en.z);
 #pragma unroll
           for (int q = 0; q < 3; ++q) {  // beta[2] = 0 for segments
             acc[q][0] = coef * beta[q] * dir.x;

@@ -105,8 +105,8 @@ struct Impl : ImplBase {
     a.adj = c->ptr<int>(c->L.adj);
     a.nedge = c->nedge;
     a.edges = c->ptr<int>(c->L.edges);
-    a.en = c->ptr<Real>(c->L.en);
-    a.vn = c->ptr<Real>(c->L.vn);
+    a.en = c->ptr<R4<Real>>(c->L.en);
+    a.vn = c->ptr<R4<Real>>(c->L.vn);
     a.nadj = c->ptr<R4<Real>>(c->L.nadj);
     a.erel = c->ptr<R4<Real>>(c->L.erel);
     a.eorg = c->ptr<int4>(c->L.eorg);
@@ -202,7 +202,8 @@ struct Impl : ImplBase {
   // Profile I of the band and the coupling sums (needs psi(t)); the rest of
   // the box (column fill).
   static tlb_status launch_band(Ctx* c, IBArgs<Real>& a, cudaStream_t s) {
-    k_band<Real><<<8 * c->nsm, 256, 0, s>>>(a);
+    // one cell of the marker box per thread, as the markers started
+    k_band<Real><<<std::max(1, 2 * c->band_blocks), 128, 0, s>>>(a);
     TLB_LAUNCHED(c, "k_band");
     return TLB_OK;
   }
