@@ -141,7 +141,8 @@ struct BatchImpl : BatchBase {
       case 0: return {PRE, MOM, GEOM, BCOUNT};  // depend on X(t) and the populations only
       case 1: return {NODEF, SCAT, BCOMP};      // need the normals and the brick counts
       case 2: return {BAND, BFILL};             // need the keys, psi(t) and the brick offsets
-      case 3: return {SPREAD, FILL};            // need the band and the coupling sums
+      case 3: return {SPREAD};                  // need the band and the coupling sums
+      case Batch::PH_FRESH: return {SPREAD, FILL};
       case 4: return {COLL};
       case 5: return {INTERP};
       default: return {RESID};
@@ -237,7 +238,8 @@ struct BatchImpl : BatchBase {
         case 0: per_sm = occupancy_grid<6, OpPre<MODE>, OpMoments<L, MODE>, OpGeometry<MODE>, OpBrickCount<MODE>>(NT); break;
         case 1: per_sm = occupancy_grid<5, OpNodeForces<MODE>, OpScatter<MODE>, OpBrickCompact<MODE>>(NT); break;
         case 2: per_sm = occupancy_grid<8, OpBand<MODE>, OpBrickFill<MODE>>(NT); break;
-        case 3: per_sm = occupancy_grid<8, OpSpread<MODE>, OpFill<MODE>>(NT); break;
+        case 3: per_sm = occupancy_grid<8, OpSpread<MODE>>(NT); break;
+        case Batch::PH_FRESH: per_sm = occupancy_grid<8, OpSpread<MODE>, OpFill<MODE>>(NT); break;
         case 4: per_sm = collide_occupancy(b->tile_variant); break;
         case 5: per_sm = occupancy_grid<8, OpInterp<L, MODE>>(NT); break;
         default: per_sm = occupancy_grid<4, OpResidual<L, MODE>>(NT); break;
@@ -301,7 +303,8 @@ struct BatchImpl : BatchBase {
         k_phase<NT, 5, BA, OpNodeForces<MODE>, OpScatter<MODE>, OpBrickCompact<MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot);
         break;
       case 2: k_phase<NT, 8, BA, OpBand<MODE>, OpBrickFill<MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
-      case 3: k_phase<NT, 8, BA, OpSpread<MODE>, OpFill<MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
+      case 3: k_phase<NT, 8, BA, OpSpread<MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
+      case Batch::PH_FRESH: k_phase<NT, 8, BA, OpSpread<MODE>, OpFill<MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
       case 4: return launch_collide(b, A, vg, s);
       case 5: k_phase<NT, 8, BA, OpInterp<L, MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
       default: k_phase<NT, 4, BA, OpResidual<L, MODE>><<<g, NT, 0, s>>>(A, vg, n, ne, tot); break;
@@ -310,11 +313,13 @@ struct BatchImpl : BatchBase {
     return cuda_check(cudaGetLastError(), "k_phase");
   }
 
-  // One step of every active instance with the argument table of parity q.
-  tlb_status launch_step(Batch* b, int q, cudaStream_t s) {
+  // One step of every active instance with argument table q; `fresh`: after
+  // markers were set from outside (between such steps the band keeps the cells
+  // beyond dc, see band_body).
+  tlb_status launch_step(Batch* b, int q, cudaStream_t s, bool fresh = false) {
     const BA* A = b->ptr<BA>(b->targs[q]);
     for (int ph = 0; ph < 6; ++ph) {
-      tlb_status st = launch_phase(b, ph, A, s);
+      tlb_status st = launch_phase(b, fresh && ph == 3 ? Batch::PH_FRESH : ph, A, s);
       if (st != TLB_OK) return st;
     }
     return TLB_OK;
@@ -385,6 +390,7 @@ struct BatchImpl : BatchBase {
       b->launches++;
       TLB_CUDA(cudaGetLastError());
       c->box_stale = false;
+      b->fresh = true;
     }
     return TLB_OK;
   }
@@ -436,17 +442,22 @@ struct BatchImpl : BatchBase {
     tlb_status st = prepare(b);
     if (st != TLB_OK) return st;
     long left = n;
-    if (variant_t1(b->tile_variant) && any_pull(b)) {
-      if ((st = launch_step(b, 1, b->stream)) != TLB_OK) return st;
-      --left;
+    // a first step that the graph's steps differ from
+    const bool pull = variant_t1(b->tile_variant) && any_pull(b);
+    if (pull || b->fresh) {
+      if ((st = launch_step(b, pull ? 1 : 0, b->stream, b->fresh)) != TLB_OK) return st;
+      b->fresh = false;
+      advanced(b, 1);
+      if (--left > 0 && !variant_t1(b->tile_variant) && (st = upload_tables(b)) != TLB_OK) return st;
     }
+    const long rest = left;
     // the graph's two steps leave every buffer parity as it was
     for (; left >= 2; left -= 2) {
       TLB_CUDA(cudaGraphLaunch(b->graph, b->stream));
       b->launches += b->graph_launches;
     }
     if (left && (st = launch_step(b, 0, b->stream)) != TLB_OK) return st;
-    advanced(b, n);
+    if (rest > 0) advanced(b, rest);
     return TLB_OK;
   }
 
@@ -462,7 +473,7 @@ struct BatchImpl : BatchBase {
       const BA* A = b->ptr<BA>(b->targs[t1 ? (k == 0 && any_pull(b)) : (k & 1)]);
       for (int ph = 0; ph < 6 && st == TLB_OK; ++ph) {
         cudaEventRecord(ev[ph], b->stream);
-        st = launch_phase(b, ph, A, b->stream);
+        st = launch_phase(b, ph == 3 && k == 0 && b->fresh ? Batch::PH_FRESH : ph, A, b->stream);
       }
       cudaEventRecord(ev[6], b->stream);
       cudaEventSynchronize(ev[6]);
@@ -474,6 +485,7 @@ struct BatchImpl : BatchBase {
     }
     for (int k = 0; k < 7; ++k) cudaEventDestroy(ev[k]);
     if (st != TLB_OK) return st;
+    b->fresh = false;
     advanced(b, n);
     return TLB_OK;
   }

@@ -306,7 +306,9 @@ struct BatchBase {
 // together (see tlb_batch.cuh).  The instances live in sub-arenas of the
 // batch arena, followed by the batch's own tables.
 struct Batch {
-  static constexpr int NPH = 7;      // six phases of a step + the residual
+  // six phases of a step, the residual, and phase 3 of a step after markers
+  // were set from outside (with the column fill)
+  static constexpr int NPH = 8, PH_FRESH = 7;
   static constexpr int MAXOPS = 4;   // kernel bodies per phase
   static constexpr size_t ARGS_BYTES = 1024;  // bound on one instance's argument record
   std::vector<Ctx*> inst;
@@ -320,6 +322,7 @@ struct Batch {
   int ph_ent[NPH] = {0}, ph_total[NPH] = {0}, ph_grid[NPH] = {0};
   cudaGraphExec_t graph = nullptr;
   bool graph_dirty = true;
+  bool fresh = false;  // the next step follows markers set from outside
   long graph_launches = 0;  // kernels in one launch of the step graph
   int tile_variant = 0, zc = 16, recon_zc = 16, scat_split = 1;
   long launches = 0;
