@@ -310,17 +310,17 @@ tlb_status tlb_autotune(void* ctx, int* tile_variant, int* z_chunk);
  * on the choice beyond rounding. */
 tlb_status tlb_set_tile(void* ctx, int tile_variant, int z_chunk);
 
-/* Step graphs on (on != 0) or off (the default).  With graphs on, tlb_step
- * and tlb_run issue runs of 8 steps as one CUDA graph launch, captured once
- * per population buffer and collide variant from the same kernels the
- * direct launches use (the results are identical bit for bit); the first
- * step after markers were set from outside, the first step after
- * populations were written with moment storage, the steps of
- * tlb_profile_steps and a remainder below 8 steps run as direct launches.
- * Turning graphs off releases the captured graphs.  On the 128^3 capsule
- * the replay measured slower than direct launches (the captured side-stream
- * kernels lose their stream priority), hence off by default.  Not in the
- * paper: a launch mechanism of this implementation. */
+/* Step graphs.  tlb_step and tlb_run issue runs of 8 steps of a lattice with
+ * membranes as one CUDA graph launch, captured once per population buffer and
+ * collide variant from the same kernels the direct launches use (the results
+ * are identical bit for bit; the kernels keep their streams' priorities); the
+ * first step after markers were set from outside or after populations were
+ * written, the steps of tlb_profile_steps, calls while the context stream is
+ * being captured and a remainder below 8 steps run as direct launches.  By
+ * default a graph is captured in a call of 32 steps or more; on != 0 asks for
+ * it in any call of 8 steps or more, on = 0 turns graphs off and releases the
+ * captured ones.  Not in the paper: a launch mechanism of this
+ * implementation. */
 tlb_status tlb_set_graphs(void* ctx, int on);
 
 /* Number of CUDA kernel launches enqueued by the last tlb_step call (a

@@ -719,7 +719,7 @@ tlb_status tlb_set_graphs(void* ctx, int on) {
     TLB_CUDA(cudaStreamSynchronize(c->stream));
     c->drop_graphs();
   }
-  c->graphs = on != 0;
+  c->graphs = c->graphs_asked = on != 0;
   return TLB_OK;
 }
 
