@@ -1178,7 +1178,7 @@ __global__ void k_ws_move(double* __restrict__ X, int nn, const float* __restric
   double T[3], n[3], r = 0, len = 0;
   for (int q = 0; q < 3; ++q) {
     T[q] = tot[q] / nn;
-    n[q] = vn[3 * l + q];
+    n[q] = vn[4 * l + q];  // (one vector of four per marker)
     len += n[q] * n[q];
   }
   len = sqrt(len);
