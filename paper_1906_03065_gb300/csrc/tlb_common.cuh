@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/tlb.h"
 
 #define TLB_HD __host__ __device__ __forceinline__
@@ -111,6 +113,20 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_real<__nv_bfloat16>(fl
 template <class S, class R>
 __device__ __forceinline__ R as_stored(R v) {
   return to_real(from_real<S>(v));
+}
+
+// The same of two values: with 16-bit storage one conversion for both.
+template <class S, class R>
+__device__ __forceinline__ void as_stored2(R& a, R& b) {
+  if constexpr (std::is_same<S, __half>::value) {
+    const float2 v = __half22float2(__floats2half2_rn(a, b));
+    a = v.x;
+    b = v.y;
+  } else if constexpr (std::is_same<S, __nv_bfloat16>::value) {
+    const float2 v = __bfloat1622float2(__floats2bfloat162_rn(a, b));
+    a = v.x;
+    b = v.y;
+  }
 }
 
 // Two consecutive Real values (one 8 or 16-byte load).
@@ -328,10 +344,13 @@ __device__ __forceinline__ double rfma(double a, double b, double c) { return __
 // its storage type holds it: with 16-bit storage every rebuilt population is
 // rounded, so the state is that of stored populations, bit for bit.
 // They are kept as three 16-byte vectors per cell (32 in double precision),
-// one plane array each: (rho - 1, w), (phi, 3 Gamma_phi mu_phi, psi,
-// 3 Gamma_psi mu_psi'), (v, -1.5 v^2).  A cell is then moved by three
-// vector copies instead of eleven, and what every reader would form again
-// (3 Gamma mu, -1.5 v^2) is stored once, in the otherwise idle twelfth slot.
+// one plane array each: (rho - 1, q), (phi, 3 Gamma_phi mu_phi, psi,
+// 3 Gamma_psi mu_psi'), (v, 1/rho) with q = rho w = j + F.  A cell is then
+// moved by three vector copies instead of eleven.  The momentum q, rounded
+// once, is the linear part of every f_i; w would be rounded three times on its
+// way back to it (in FP32 that made the velocity's error a quarter larger than
+// with stored populations).  3 Gamma mu and 1/rho spare the readers their
+// products and the division.
 enum { M_F = 0, M_ORD = 1, M_V = 2, M_COUNT = 3 };
 
 // Four values of one cell side by side: one 16-byte access (two in double
@@ -358,18 +377,18 @@ template <class L, int MODE>
 struct EqCell {
   using Real = typename Prec<MODE>::Real;
   using Store = typename Prec<MODE>::Store;
-  Real drho, rho, w[3], w15, ord[2], gm3[2], v[3], v15;
-  // rho - 1 and w only (what f_i needs)
-  __device__ __forceinline__ void set_f(const R4<Real>& A) {
-    drho = A.x;
-    w[0] = A.y;
-    w[1] = A.z;
-    w[2] = A.w;
-    rho = Real(1) + drho;
-    w15 = rmul(Real(-1.5), rfma(w[2], w[2], rfma(w[1], w[1], rmul(w[0], w[0]))));
+  Real ds, k, q[3], ord[2], gm3[2], v[3], v15;
+  // rho - 1, q and 1/rho only (what f_i needs)
+  __device__ __forceinline__ void set_f(const R4<Real>& A, Real irho) {
+    q[0] = A.y;
+    q[1] = A.z;
+    q[2] = A.w;
+    const Real qq = rfma(q[2], q[2], rfma(q[1], q[1], rmul(q[0], q[0])));
+    k = rmul(Real(4.5), irho);
+    ds = rfma(rmul(Real(-1.5), irho), qq, A.x);
   }
   __device__ __forceinline__ void set(const R4<Real>& A, const R4<Real>& B, const R4<Real>& C) {
-    set_f(A);
+    set_f(A, C.w);
     ord[0] = B.x;
     gm3[0] = B.y;
     ord[1] = B.z;
@@ -377,31 +396,31 @@ struct EqCell {
     v[0] = C.x;
     v[1] = C.y;
     v[2] = C.z;
-    v15 = C.w;
+    v15 = rmul(Real(-1.5), rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0]))));
   }
   __device__ __forceinline__ void load(const R4<Real>* M, int P32, int c) {
     set(M[M_F * P32 + c], M[M_ORD * P32 + c], M[M_V * P32 + c]);
   }
+  // f_i - w_i = w_i (rho - 1 + 3 c.q + (4.5 (c.q)^2 - 1.5 q^2) / rho)
+  __device__ __forceinline__ Real f(int i) const { return f_or_back(i, false); }
+  // the same of direction i, or of its opposite where `back` (c.q changes sign)
+  __device__ __forceinline__ Real f_or_back(int i, bool back) const {
+    if (i == 0) return as_stored<Store>(rmul(Real(L::w(0)), ds));
+    const Real c = cdot<L>(i, q), cq = back ? -c : c;
+    return as_stored<Store>(rmul(Real(L::w(i)), rfma(cq, rfma(k, cq, Real(3)), ds)));
+  }
   // 3 c.u + 4.5 (c.u)^2 - 1.5 u^2
   static __device__ __forceinline__ Real poly(int i, const Real* u, Real u15) {
-    if (i == 0) return u15;
     const Real cu = cdot<L>(i, u);
     return rfma(cu, rfma(Real(4.5), cu, Real(3)), u15);
   }
-  // f_i - w_i = w_i (drho + rho p(w))
-  __device__ __forceinline__ Real f(int i) const {
-    return as_stored<Store>(rmul(Real(L::w(i)), rfma(rho, poly(i, w, w15), drho)));
-  }
-  // the same of direction i, or of its opposite where `back` (c.u changes sign)
-  __device__ __forceinline__ Real f_or_back(int i, bool back) const {
-    const Real c = cdot<L>(i, w), cu = back ? -c : c;
-    const Real p = i == 0 ? w15 : rfma(cu, rfma(Real(4.5), cu, Real(3)), w15);
-    return as_stored<Store>(rmul(Real(L::w(i)), rfma(rho, p, drho)));
-  }
-  // g_i (s = 0) or h_i (s = 1): w_i (3 Gamma mu + ord p(c.v)) for i != 0; the
-  // rest population closes the zeroth moment
-  __device__ __forceinline__ Real o(int s, Real p, int i) const {
-    return as_stored<Store>(rmul(Real(L::w(i)), rfma(ord[s], p, gm3[s])));
+  // g_i and h_i for i != 0: w_i (3 Gamma mu + ord p(c.v)); the rest population
+  // closes the zeroth moment
+  __device__ __forceinline__ void gh(int i, Real* g, Real* h) const {
+    const Real p = poly(i, v, v15);
+    *g = rmul(Real(L::w(i)), rfma(ord[0], p, gm3[0]));
+    *h = rmul(Real(L::w(i)), rfma(ord[1], p, gm3[1]));
+    as_stored2<Store>(*g, *h);
   }
   __device__ __forceinline__ Real rest(int s) const {
     return radd(rfma(gm3[s], Real(L::w(0)) - Real(1), ord[s]), rmul(rmul(Real(L::w(0)), ord[s]), v15));

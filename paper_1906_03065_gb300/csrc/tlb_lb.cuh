@@ -195,8 +195,9 @@ __device__ __forceinline__ void moments_recon_body(const LBArgs<MODE>& a, const 
         const int i = col_dir<L>(k, cz);
         if (i < 0) continue;
         const int o = L::opp(i);
-        const Real p = EqCell<L, MODE>::poly(o, e.v, e.v15);
-        add(t, i, e.f(o), e.o(0, p, o), e.o(1, p, o));
+        Real g, h;
+        e.gh(o, &g, &h);
+        add(t, i, e.f(o), g, h);
       }
     };
     if (!ghost) {
@@ -216,8 +217,9 @@ __device__ __forceinline__ void moments_recon_body(const LBArgs<MODE>& a, const 
             rest_mid[1] = e.rest(0);
             rest_mid[2] = e.rest(1);
           } else {
-            const Real p = EqCell<L, MODE>::poly(i, e.v, e.v15);
-            add(cz > 0 ? up : (cz == 0 ? mid : lo), i, e.f(i), e.o(0, p, i), e.o(1, p, i));
+            Real g, h;
+            e.gh(i, &g, &h);
+            add(cz > 0 ? up : (cz == 0 ? mid : lo), i, e.f(i), g, h);
           }
         }
       }
@@ -268,10 +270,11 @@ __global__ void k_materialize(Geo G, const R4<typename Prec<MODE>::Real>* M, typ
   rest[G.P + n] = from_real<Rest>(e.rest(1));
 #pragma unroll
   for (int i = 1; i < L::Q; ++i) {
-    const Real p = EqCell<L, MODE>::poly(i, e.v, e.v15);
+    Real g, h;
+    e.gh(i, &g, &h);
     lo[(long long)plane_f<L>(i) * G.P + n] = from_real<Store>(e.f(i));
-    lo[(long long)plane_g<L>(i) * G.P + n] = from_real<Store>(e.o(0, p, i));
-    lo[(long long)plane_h<L>(i) * G.P + n] = from_real<Store>(e.o(1, p, i));
+    lo[(long long)plane_g<L>(i) * G.P + n] = from_real<Store>(g);
+    lo[(long long)plane_h<L>(i) * G.P + n] = from_real<Store>(h);
   }
 }
 
@@ -756,7 +759,7 @@ __device__ __forceinline__ void collide_body_of(const LBArgs<MODE>& a, const Blk
     const int n = (zz * G.ny + y) * G.nx + x;
     const Real drho = c.x, phi = c.y, psi = c.z, rho = Real(1) + drho;
     const Real j[3] = {c.w, jn.x, jn.y};
-    Real F[3], u[3], du[3], v[3];
+    Real F[3], v[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       F[d] = rmul(Real(-1.0 / 12), F12[d]);
@@ -773,16 +776,11 @@ __device__ __forceinline__ void collide_body_of(const LBArgs<MODE>& a, const Blk
     }
     const Real irho = rcp_rn(rho);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      u[d] = rmul(j[d], irho);
-      du[d] = rmul(F[d], irho);
-      v[d] = rfma(Real(0.5), du[d], u[d]);
-    }
-    const Real vv = rfma(v[2], v[2], rfma(v[1], v[1], rmul(v[0], v[0])));
+    for (int d = 0; d < 3; ++d) v[d] = rmul(rfma(Real(0.5), F[d], j[d]), irho);
     R4<Real>* M = a.M + n;
-    M[M_F * G.P32] = R4<Real>{drho, radd(u[0], du[0]), radd(u[1], du[1]), radd(u[2], du[2])};
+    M[M_F * G.P32] = R4<Real>{drho, radd(j[0], F[0]), radd(j[1], F[1]), radd(j[2], F[2])};
     M[M_ORD * G.P32] = R4<Real>{phi, rmul(Real(3), rmul(a.gphi, h1[1])), psi, rmul(Real(3), rmul(a.gpsi, h1[2]))};
-    M[M_V * G.P32] = R4<Real>{v[0], v[1], v[2], rmul(Real(-1.5), vv)};
+    M[M_V * G.P32] = R4<Real>{v[0], v[1], v[2], irho};
   };
 
   issue(z0 - 2, 0);
