@@ -290,6 +290,7 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.en, 4 * ne * R);
   take(L.vn, 4 * nn * R);
   take(L.nadj, 4 * nn * R);
+  take(L.wts, 12 * nn * R);
   take(L.erel, 4 * ne * R);
   take(L.eorg, 4 * ne * 4);
   take(L.ecst, 16 * ne * R);

@@ -170,7 +170,7 @@ struct BatchImpl : BatchBase {
       case BAND: return {mem ? c->band_blocks : 0, 1, 1};
       case BFILL: return {mem ? (int)cdiv(c->nn, NT) : 0, 1, 1};
       case FILL: return {mem ? (int)cdiv(32ll * c->nx * c->ny, NT) : 0, 1, 1};
-      case SPREAD: return {mem ? c->spread_blocks : 0, 1, 1};
+      case SPREAD: return {mem ? (int)cdiv(c->spread_blocks, NT / 32) : 0, 1, 1};
       case COLL: {
         const int tx = tile_x(b->tile_variant), ty = tile_y(b->tile_variant);
         return {(int)cdiv(c->nx, tx), (int)cdiv(c->ny, ty), (int)cdiv(c->nz, b->zc)};

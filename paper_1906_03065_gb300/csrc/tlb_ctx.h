@@ -146,7 +146,7 @@ struct Layout {
   Region rho, phi, psi, p4, j2, M, I, dsel, own, key, fib, ftot, mu, rb;
   // membranes
   Region X, E, ecap, ncap, cap_par, ds0, rprev, rnext, A0, G0i, inc_off, inc, adj, edges;
-  Region en, vn, nadj, erel, eorg, ecst, xo, xr, skc, capr, ncpl, F, box;
+  Region en, vn, nadj, wts, erel, eorg, ecst, xo, xr, skc, capr, ncpl, F, box;
   Region bcnt, bprev, bcur, boff, blist, bact, ctr, bflag;
   // misc
   Region status, part, meas;

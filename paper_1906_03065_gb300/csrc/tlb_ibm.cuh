@@ -43,6 +43,8 @@ struct IBArgs {
   // per-step work
   R4<Real>* en;          // [ne] unit outward normal
   R4<Real>* vn;          // [nn] angle-weighted vertex pseudo-normal
+  Real* wts;             // [nn][3][4] kernel weights (eq. DiscreteDirac) at the support
+                         // cells floor(X) - 1 .. floor(X) + 2 along each axis
   R4<Real>* nadj;        // [nn] 3D: derivatives of the marker's bending energy with
                          // respect to its K (three) and A (see geometry_body)
   // per element, read as whole vectors by the band:
@@ -194,6 +196,16 @@ __device__ __forceinline__ V3<Real> elem_closest(const IBArgs<Real>& a, int e, c
   return P0;
 }
 
+// ------------------------------------------------------------ delta kernel
+// eq. DiscreteDirac along one axis.
+template <class Real>
+__device__ __forceinline__ Real peskin(Real r) {
+  Real x = fabs(r);
+  if (x <= Real(1)) return (Real(3) - Real(2) * x + sqrt(fmax(Real(0), Real(1) + Real(4) * x - Real(4) * x * x))) * Real(0.125);
+  if (x <= Real(2)) return (Real(5) - Real(2) * x - sqrt(fmax(Real(0), Real(-7) + Real(12) * x - Real(4) * x * x))) * Real(0.125);
+  return Real(0);
+}
+
 // ------------------------------------------------------------ geometry pass
 // Face normal of element e, computed from the marker positions.
 template <class Real>
@@ -263,6 +275,12 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
   const bool valid = (g >> 4) < a.nn;
   const int k = valid ? g >> 4 : a.nn - 1;  // every lane takes part in the sums
   const int i0 = a.inc_off[k], ninc = valid ? a.inc_off[k + 1] - i0 : 0;
+  // the marker's kernel weights at its 4 support cells along each axis, one
+  // per lane (read by the spreading and by the interpolation)
+  if (valid && lane < 12) {
+    const int d = lane >> 2, c = a.xo[3 * k + d] - 1 + (lane & 3);
+    a.wts[12 * k + lane] = d == 1 && a.dim == 2 ? Real(0) : peskin(-node_off(a, k, d, c));
+  }
   V3<Real> s = mk<Real>(0, 0, 0), K = s;
   Real A = 0;
   for (int j = lane; j < ninc; j += 16) {
@@ -1102,14 +1120,6 @@ __device__ __forceinline__ void coupling_of(const IBArgs<Real>& a, int k, Real* 
 }
 
 // ------------------------------------------------------------ spreading
-template <class Real>
-__device__ __forceinline__ Real peskin(Real r) {
-  Real x = fabs(r);
-  if (x <= Real(1)) return (Real(3) - Real(2) * x + sqrt(fmax(Real(0), Real(1) + Real(4) * x - Real(4) * x * x))) * Real(0.125);
-  if (x <= Real(2)) return (Real(5) - Real(2) * x - sqrt(fmax(Real(0), Real(-7) + Real(12) * x - Real(4) * x * x))) * Real(0.125);
-  return Real(0);
-}
-
 // Distinct bricks touched along one axis by the 4 support cells starting at base.
 __device__ __forceinline__ int axis_bricks(int base, int n, int* out) {
   int m = 0;
@@ -1194,89 +1204,86 @@ __global__ void k_brick_fill(const __grid_constant__ IBArgs<Real> a) {
 // markers in ascending marker order (the list is sorted first, so the result
 // does not depend on the order of the atomic slot claims).  Bricks that held
 // markers in the previous step are visited too, so their cells return to zero.
+// One warp per brick: its work is a chain of dependent loads (brick, list,
+// markers), so many small chains beside each other beat a block with barriers
+// per brick (24 2D lattices of 240x120, batched: 17.9 -> 10.3 us).
+constexpr int SPREAD_WARPS = 4;  // per block (at most)
 template <class Real>
 __device__ __forceinline__ void spread_body(const IBArgs<Real>& a, const Blk& blk) {
-  constexpr int CH = 128;  // markers staged at a time
-  __shared__ int list[512], sorted[512];
-  __shared__ Real sW[CH][12];  // per marker: delta_h at the brick's 4 cells along x, y, z
-  __shared__ Real sF[CH][3];
+  constexpr int CH = 32;  // markers staged at a time, one per lane
+  __shared__ int s_list[SPREAD_WARPS][2][512];
+  __shared__ Real s_w[SPREAD_WARPS][CH][13];  // delta_h at the brick's 4 cells along x, y, z
+  __shared__ Real s_f[SPREAD_WARPS][CH][3];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int *list = s_list[w][0], *sorted = s_list[w][1];
   const int nact = min(a.ctr[0], a.nbricks);
-  const int BY = a.dim == 3 ? BRICK : 1;
-  for (int ib = blk.x; ib < nact; ib += blk.gx) {
+  // the lane's cells of the brick: 3D (x, y, z) and (x, y, z + 2), 2D one of 16
+  const int lx = lane & 3, ly = a.dim == 3 ? (lane >> 2) & 3 : 0, lz = a.dim == 3 ? lane >> 4 : (lane >> 2) & 3;
+  const int ncell = a.dim == 3 ? 2 : (lane < 16 ? 1 : 0);
+  for (int ib = blk.x * nw + w; ib < nact; ib += blk.gx * nw) {
     const int b = a.bact[ib];
     if (b < 0 || b >= a.nbricks) continue;
-    const int cnt = a.bcnt[b];
-    const int off = a.boff[b];
-    const int m = min(cnt, 512);
-    if (cnt > 512 && threadIdx.x == 0) atomicOr(a.status, (unsigned)ST_OVERFLOW);
-    for (int j = threadIdx.x; j < m; j += blockDim.x) list[j] = a.blist[off + j];
-    __syncthreads();
+    const int cnt = a.bcnt[b], off = a.boff[b], m = min(cnt, 512);
+    if (cnt > 512 && lane == 0) atomicOr(a.status, (unsigned)ST_OVERFLOW);
+    for (int j = lane; j < m; j += 32) list[j] = a.blist[off + j];
+    __syncwarp();
     // rank sort (marker indices are distinct), so the sum runs in marker order
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      int v = list[j], r = 0;
+    for (int j = lane; j < m; j += 32) {
+      const int v = list[j];
+      int r = 0;
       for (int i = 0; i < m; ++i) r += list[i] < v;
       sorted[r] = v;
     }
-    __syncthreads();
-    const int bx = b % a.nbx, by = (b / a.nbx) % a.nby, bz = b / (a.nbx * a.nby);
-    const int ox = bx * BRICK, oy = by * BRICK, oz = bz * BRICK;
-    const int lx = threadIdx.x % BRICK, ly = (threadIdx.x / BRICK) % BY, lz = threadIdx.x / (BRICK * BY);
-    const int cx = ox + lx, cy = oy + ly, cz = oz + lz;
-    const bool ok = threadIdx.x < BRICK * BY * BRICK && cx < a.G.nx && cy < a.G.ny && cz < a.G.nz;
-    Real f[3] = {0, 0, 0};
+    __syncwarp();
+    const int o[3] = {b % a.nbx * BRICK, a.dim == 3 ? b / a.nbx % a.nby * BRICK : 0, b / (a.nbx * a.nby) * BRICK};
+    Real f[2][3] = {{0, 0, 0}, {0, 0, 0}};
     for (int j0 = 0; j0 < m; j0 += CH) {
       const int mc = min(CH, m - j0);
-      // marker positions relative to the brick corner (nearest periodic
-      // image) and the kernel weights of the brick's cells along each axis
-      for (int j = threadIdx.x; j < mc; j += blockDim.x) {
-        int l = sorted[j0 + j];
-        Real r3[3];
-        if constexpr (std::is_same<Real, float>::value) {
-          // integer part wrapped to [-n/2, n/2) (the image nearest the brick)
-          auto img = [](int k, int n) { return wrap_coord(k + n / 2, n) - n / 2; };
-          r3[0] = (float)img(a.xo[3 * l] - ox, a.G.nx) + a.xr[3 * l];
-          r3[1] = a.dim == 3 ? (float)img(a.xo[3 * l + 1] - oy, a.G.ny) + a.xr[3 * l + 1] : 0.0f;
-          r3[2] = (float)(a.G.wall ? a.xo[3 * l + 2] - oz : img(a.xo[3 * l + 2] - oz, a.G.nz)) + a.xr[3 * l + 2];
-        } else {
-          double rx = a.X[3 * l] - ox, ry = a.X[3 * l + 1] - oy, rz = a.X[3 * l + 2] - oz;
-          rx -= a.G.nx * floor(rx / a.G.nx + 0.5);
-          if (a.dim == 3) ry -= a.G.ny * floor(ry / a.G.ny + 0.5); else ry = 0;
-          if (!a.G.wall) rz -= a.G.nz * floor(rz / a.G.nz + 0.5);
-          r3[0] = (Real)rx;
-          r3[1] = (Real)ry;
-          r3[2] = (Real)rz;
+      if (lane < mc) {
+        const int l = sorted[j0 + lane];
+        // brick cell c along axis d is support cell c + sh (nearest periodic
+        // image of the marker); outside the support the kernel is zero
+        auto img = [](int k, int n) { return wrap_coord(k + n / 2, n) - n / 2; };
+        const int n3[3] = {a.G.nx, a.G.ny, a.G.nz};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const int rel = a.xo[3 * l + d] - o[d];
+          const int sh = 1 - (d == 2 && a.G.wall ? rel : img(rel, n3[d]));
+#pragma unroll
+          for (int c = 0; c < BRICK; ++c)
+            s_w[w][lane][4 * d + c] = (unsigned)(c + sh) < 4u ? a.wts[12 * l + 4 * d + c + sh] : Real(0);
         }
-        // delta_h vanishes outside |r| < 2 (peskin returns 0 there)
-  #pragma unroll
-        for (int d = 0; d < 3; ++d)
-  #pragma unroll
-          for (int o = 0; o < BRICK; ++o) sW[j][4 * d + o] = peskin((Real)o - r3[d]);
         Real cp[3];
         coupling_of(a, l, cp);  // F_mem = F_s + F_b + F_c (eq. MembraneForces)
-        for (int d = 0; d < 3; ++d) sF[j][d] = a.F[3 * l + d] + cp[d];
+        for (int d = 0; d < 3; ++d) s_f[w][lane][d] = a.F[3 * l + d] + cp[d];
       }
-      __syncthreads();
-      if (ok) {  // summed in marker order across the chunks
-        for (int j = 0; j < mc; ++j) {
-          Real wgt = sW[j][lx] * sW[j][8 + lz];
-          if (a.dim == 3) wgt *= sW[j][4 + ly];
-          if (wgt == Real(0)) continue;  // outside the support
-          for (int d = 0; d < 3; ++d) f[d] += wgt * sF[j][d];
+      __syncwarp();
+      for (int j = 0; j < mc; ++j) {  // in marker order across the chunks
+        const Real* W = s_w[w][j];
+        const Real* F = s_f[w][j];
+        const Real xy = a.dim == 3 ? W[lx] * W[4 + ly] : W[lx];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const Real wgt = xy * W[8 + ((lz + 2 * h) & 3)];
+          for (int d = 0; d < 3; ++d) f[h][d] += wgt * F[d];
         }
       }
-      __syncthreads();
+      __syncwarp();
     }
-    if (ok) {
-      long long c = ((long long)cz * a.G.ny + cy) * a.G.nx + cx;
-      for (int d = 0; d < 3; ++d) a.fib[d * a.G.P + c] = f[d];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int cx = o[0] + lx, cy = o[1] + ly, cz = o[2] + lz + 2 * h;
+      if (h < ncell && cx < a.G.nx && cy < a.G.ny && cz < a.G.nz) {
+        const long long c = ((long long)cz * a.G.ny + cy) * a.G.nx + cx;
+        for (int d = 0; d < 3; ++d) a.fib[d * a.G.P + c] = f[h][d];
+      }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
       a.bprev[b] = cnt;
       a.bcnt[b] = 0;
       a.bcur[b] = 0;
     }
-    __syncthreads();
+    __syncwarp();
   }
 }
 template <class Real>
@@ -1298,11 +1305,7 @@ __device__ __forceinline__ void interp_advect_body(const IBArgs<typename Prec<MO
   const Geo G = a.G;
   const int bb[3] = {a.xo[3 * l] - 1, a.xo[3 * l + 1] - 1, a.xo[3 * l + 2] - 1};
   // delta_h along each axis at the 4 support offsets: lane 4 d + o
-  Real wax = 0;
-  if (lane < 12) {
-    const int d = lane >> 2, o = lane & 3;
-    if (d != 1 || a.dim == 3) wax = peskin(-node_off(a, l, d, bb[d] + o));
-  }
+  const Real wax = lane < 12 ? a.wts[12 * l + lane] : Real(0);
   const int ncell = a.dim == 3 ? 64 : 16;
   // the lane's two support cells: weights and addresses first, so that all
   // their loads are in flight together (a cell of weight 0 reads cell 0)

@@ -108,6 +108,7 @@ struct Impl : ImplBase {
     a.en = c->ptr<R4<Real>>(c->L.en);
     a.vn = c->ptr<R4<Real>>(c->L.vn);
     a.nadj = c->ptr<R4<Real>>(c->L.nadj);
+    a.wts = c->ptr<Real>(c->L.wts);
     a.erel = c->ptr<R4<Real>>(c->L.erel);
     a.eorg = c->ptr<int4>(c->L.eorg);
     a.ecst = c->ptr<R4<Real>>(c->L.ecst);
@@ -218,7 +219,8 @@ struct Impl : ImplBase {
   }
 
   static tlb_status ibm_spread(Ctx* c, IBArgs<Real>& a, cudaStream_t s) {
-    k_spread<Real><<<min(c->nbricks, 8 * c->nsm), 64, 0, s>>>(a);
+    constexpr int nt = 64;  // (two bricks at a time)
+    k_spread<Real><<<min((int)blocks(c->nbricks, nt / 32), 8 * c->nsm), nt, 0, s>>>(a);
     TLB_LAUNCHED(c, "k_spread");
     return TLB_OK;
   }
