@@ -92,6 +92,13 @@ template <class T> TLB_HD V3<T> cross(V3<T> a, V3<T> b) {
   return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
 
+// dot(a, b) with explicit roundings (see rmul): the small strains and
+// curvatures left over from sums of larger terms then come out the same in
+// every kernel the code is inlined into.
+template <class T> __device__ __forceinline__ T rdot(V3<T> a, V3<T> b) {
+  return rfma(a.z, b.z, rfma(a.y, b.y, rmul(a.x, b.x)));
+}
+
 // Correctly rounded reciprocal (the value of 1 / x, without the division).
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
@@ -292,14 +299,15 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
     const int q0 = a.E[3 * e], q1 = a.E[3 * e + 1], q2 = a.E[3 * e + 2];
     const int u = q0 == k ? q1 : (q1 == k ? q2 : q0);
     const int v = q0 == k ? q2 : (q1 == k ? q0 : q1);
-    const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = ev - eu;
+    const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = node_dv(a, v, u);
     const V3<Real> cr = cross(eu, ev);
     const Real A2 = sqrt(dot(cr, cr)), iA2 = Real(1) / A2;
-    const Real duu = dot(eu, eu), dvv = dot(ev, ev), dk = dot(eu, ev), du = -dot(eu, w), dv = dot(ev, w);
+    const Real duu = rdot(eu, eu), dvv = rdot(ev, ev), dk = rdot(eu, ev), du = -rdot(eu, w), dv = rdot(ev, w);
     const Real c = dk / sqrt(duu * dvv);
     s = s + (acos(fmin(Real(1), fmax(Real(-1), c))) * iA2) * cr;
-    const Real cu = du * iA2, cv = dv * iA2;
-    K = K - cv * eu - cu * ev;
+    const Real cu = rmul(du, iA2), cv = rmul(dv, iA2);
+    K = mk<Real>(rfma(-cu, ev.x, rfma(-cv, eu.x, K.x)), rfma(-cu, ev.y, rfma(-cv, eu.y, K.y)),
+                 rfma(-cu, ev.z, rfma(-cv, eu.z, K.z)));
     if (dk < 0) A += Real(0.25) * A2;
     else if (du < 0 || dv < 0) A += Real(0.125) * A2;
     else A += Real(0.125) * (duu * cv + dvv * cu);
@@ -1035,13 +1043,13 @@ __device__ __forceinline__ V3<Real> face_force(const IBArgs<Real>& a, int k, int
   const int q0 = a.E[3 * e], q1 = a.E[3 * e + 1], q2 = a.E[3 * e + 2];
   const int u = q0 == k ? q1 : (q1 == k ? q2 : q0);
   const int v = q0 == k ? q2 : (q1 == k ? q0 : q1);
-  const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = ev - eu;
+  const V3<Real> eu = node_dv(a, u, k), ev = node_dv(a, v, k), w = node_dv(a, v, u);
   const R4<Real> Nk = a.nadj[k], Nu = a.nadj[u], Nv = a.nadj[v];
-  const Real duu = dot(eu, eu), dvv = dot(ev, ev), dk = dot(eu, ev), dww = dot(w, w);
+  const Real duu = rdot(eu, eu), dvv = rdot(ev, ev), dk = rdot(eu, ev), dww = rdot(w, w);
   // bending
   const V3<Real> cr = cross(eu, ev);
   const Real A2 = sqrt(dot(cr, cr)), iA2 = Real(1) / A2;
-  const Real du = -dot(eu, w), dv = dot(ev, w);
+  const Real du = -rdot(eu, w), dv = rdot(ev, w);
   const Real ck = dk * iA2, cu = du * iA2, cv = dv * iA2;
   const V3<Real> Ku = mk<Real>(Nk.x - Nu.x, Nk.y - Nu.y, Nk.z - Nu.z), Kv = mk<Real>(Nk.x - Nv.x, Nk.y - Nv.y, Nk.z - Nv.z);
   const V3<Real> Kw = mk<Real>(Nu.x - Nv.x, Nu.y - Nv.y, Nu.z - Nv.z);
@@ -1070,8 +1078,9 @@ __device__ __forceinline__ V3<Real> face_force(const IBArgs<Real>& a, int k, int
   const V3<Real> e1 = q0 == k ? eu : (q1 == k ? Real(-1) * ev : w);
   const V3<Real> e2 = q0 == k ? ev : (q1 == k ? Real(-1) * w : Real(-1) * eu);
   const Real g11 = q0 == k ? duu : (q1 == k ? dvv : dww), g22 = q0 == k ? dvv : (q1 == k ? dww : duu);
-  const Real g12 = dot(e1, e2);
-  const Real I1 = c[0] * g11 + c[1] * g12 + c[2] * g22 - Real(2), I2 = c[3] * (g11 * g22 - g12 * g12) - Real(1);
+  const Real g12 = rdot(e1, e2);
+  const Real I1 = rfma(c[2], g22, rfma(c[1], g12, rfma(c[0], g11, Real(-2))));
+  const Real I2 = rfma(c[3], rfma(g11, g22, -rmul(g12, g12)), Real(-1));
   const Real q = c[4] * G * Real(0.5);
   const Real D1 = q * (I1 + Real(1)), D2 = q * (C * I2 - Real(1)) * c[3];
   const Real h11 = Real(2) * (D1 * c[0] + D2 * g22), h22 = Real(2) * (D1 * c[2] + D2 * g11), h12 = D1 * c[1] - Real(2) * D2 * g12;
