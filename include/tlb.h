@@ -296,7 +296,7 @@ tlb_status tlb_profile_steps(void* ctx, long n_steps, tlb_profile* out);
  * two with an even nx.  Variants 19..21 are tiles 0..2 of the general
  * collide with the
  * pressure-tensor force.  They are tried only where they apply, and a new
- * context starts on variant 13 there (19 with the pressure-tensor force,
+ * context starts on variant 14 there (19 with the pressure-tensor force,
  * else 3), with a z chunk set by the lattice's size.
  * Synchronises the stream.  Not in the paper: an autotuner for this
  * implementation's launch shape. */

@@ -353,10 +353,12 @@ tlb_status tlb_create(const tlb_params* params, const tlb_membrane_desc* mems, i
   c->base = (char*)arena;
   c->bytes = bytes;
   c->stream = (cudaStream_t)cuda_stream;
-  // the tau = 1 collide (no population pull) wherever it applies, else the
-  // general one with registers for all it holds (96^3 FP32: 88 us against 95
-  // at 640 threads per SM)
-  c->tile_variant = params->force_form == TLB_FE_PRESSURE_TENSOR ? 19 : (c->t1_ok() ? 13 : 3);
+  // the tau = 1 collide (no population pull) wherever it applies, on 32 x 8
+  // tiles (less halo than 32 x 4: 128^3 58 -> 55 us, 192 x 128 x 128 79 -> 70,
+  // 64^3 and below equal; 32 x 16: 57, 73 and slower below), else the general
+  // one with registers for all it holds (96^3 FP32: 88 us against 95 at 640
+  // threads per SM)
+  c->tile_variant = params->force_form == TLB_FE_PRESSURE_TENSOR ? 19 : (c->t1_ok() ? 14 : 3);
   switch (params->dim * 10 + params->storage) {
     case 20: c->impl = make_impl_d2q9_f64(); break;
     case 21: c->impl = make_impl_d2q9_f32(); break;
