@@ -4,7 +4,7 @@
 Workload: the 128^3 D3Q19 capsule workload (walls in z, flat C1/C2
 interface at z = 64, icosphere level-4 capsule of radius 20 with Skalak and
 Helfrich membrane mechanics, FP32 storage), stepped with the library's CUDA
-kernels.  The state (about 1.1 GB) is far larger than L2, so no explicit L2
+kernels.  A step reads and writes over 160 MB, more than L2 holds, so no L2
 flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -46,17 +46,37 @@ def step_bytes(store: int, real: int = 4, q: int = 19) -> int:
 
 def kernel_bytes(store: int, real: int = 4, q: int = 19, t1: bool = True):
     """Algorithmic DRAM bytes per cell of the two lattice kernels of a step
-    (each array element read or written once; store = bytes of a stored
-    population, real = of a moment field):
-      k_moments: pulls the populations, writes rho - 1, phi, psi and, for
-        the tau = 1 collide, j;
+    that keeps the populations (each array element read or written once;
+    store = bytes of a stored population, real = of a moment field):
+      k_moments: pulls the populations, writes rho - 1, phi, psi and, for a
+        tau = 1 collide, j;
       k_collide: reads rho - 1, phi, psi and I, writes the populations;
-        the general form also pulls the populations, the tau = 1 form
-        reads j instead."""
+        the general form also pulls the populations, a tau = 1 form reads j
+        instead.
+    The default tau = 1 step keeps the moment state: state_kernel_bytes."""
     pops = pop_bytes(store, real, q)
     mom = (6 if t1 else 3) * real
     coll = pops + 4 * real + (3 * real if t1 else pops)
     return {"k_moments": pops + mom, "k_collide": coll}
+
+
+def state_kernel_bytes(real: int = 4):
+    """Algorithmic DRAM bytes per cell of the lattice kernels of a tau = 1
+    step, which keeps 12 values per cell (in the arithmetic type for every
+    storage type) instead of the populations: k_moments_recon reads them and
+    writes rho - 1, phi, psi, j; k_collide reads those and I and writes them."""
+    return {"k_moments_recon": (12 + 6) * real, "k_collide": (6 + 1 + 12) * real}
+
+
+def lattice_kernels(storage: str, t1: bool):
+    """(name, phase, bytes per cell) of the two lattice kernels of a step."""
+    kb = state_kernel_bytes() if t1 else kernel_bytes(4 if storage == "f32" else 2, t1=False)
+    return [(name, "ms_collide" if name == "k_collide" else "ms_moments", b) for name, b in kb.items()]
+
+
+def moved_bytes(storage: str, t1: bool) -> int:
+    """Bytes per cell that the two lattice kernels of a step read and write."""
+    return sum(b for _, _, b in lattice_kernels(storage, t1))
 
 
 def _peaks():
@@ -67,7 +87,7 @@ def _peaks():
 
 
 # sources each profiled kernel is compiled from
-KERNEL_SOURCES = {"k_collide": ("tlb_lb.cuh", "tlb_common.cuh"), "k_moments": ("tlb_lb.cuh", "tlb_common.cuh")}
+KERNEL_SOURCES = {k: ("tlb_lb.cuh", "tlb_common.cuh") for k in ("k_collide", "k_moments", "k_moments_recon")}
 
 
 def _src_hash(kernel: str = "k_collide"):
@@ -281,23 +301,26 @@ def main():
     peaks = _peaks()
     peak = peaks["hbm_gbs"] if peaks else 6800.0
     t1 = tile_variant >= 13
-    kb = kernel_bytes(4 if args.storage == "f32" else 2, t1=t1)
     kern = {}
-    for name, ms in (("k_moments", pr.ms_moments), ("k_collide", pr.ms_collide)):
-        t = ms / nprof / 1e3
-        ach = kb[name] * N / t / 1e9
-        kern[name] = {"bytes_per_cell": kb[name], "bytes_per_launch": kb[name] * N, "ms": t * 1e3,
+    for name, phase, kb in lattice_kernels(args.storage, t1):
+        t = getattr(pr, phase) / nprof / 1e3
+        ach = kb * N / t / 1e9
+        kern[name] = {"bytes_per_cell": kb, "bytes_per_launch": kb * N, "ms": t * 1e3,
                       "achieved": ach, "frac": ach / peak,
                       "traffic": _traffic(name if args.storage == "f32" else f"{name}_{args.storage}")}
     dom = max(kern, key=lambda k: kern[k]["ms"])
     sb = step_bytes(4 if args.storage == "f32" else 2)
-    step_eff = sb * N * args.steps / (ms_max / 1e3) / 1e9
+    mb = moved_bytes(args.storage, t1)
+    step_rate = N * args.steps / (ms_max / 1e3) / 1e9
     roofline = {"bound": "hbm", "achieved": kern[dom]["achieved"], "peak": peak, "unit": "GB/s",
                 "frac": kern[dom]["frac"], "traffic": kern[dom]["traffic"],
                 "kernel": dom, "peak_source": "measured" if peaks else "fallback",
                 "bytes_per_launch": kern[dom]["bytes_per_launch"],
-                "whole_step_frac": step_eff / peak, "whole_step_bytes_per_cell": sb,
-                "collide_form": "tau=1 equilibrium store" if t1 else "general (populations pulled)",
+                "whole_step_frac": mb * step_rate / peak, "whole_step_bytes_per_cell": mb,
+                # the same step in units of a population update (every
+                # population read and written once), which it does not move
+                "population_update_bytes_per_cell": sb, "population_update_frac": sb * step_rate / peak,
+                "collide_form": "tau=1 moment state" if t1 else "general (populations pulled)",
                 "kernels": kern,
                 "phase_ms_per_step": {"moments": pr.ms_moments / nprof, "ibm": pr.ms_ibm / nprof,
                                       "collide": pr.ms_collide / nprof, "interp": pr.ms_interp / nprof}}
@@ -338,8 +361,8 @@ def main():
     h2d = (Ch.nbytes + Uh.nbytes) / Ke
     d2h = (c3.nbytes + X.nbytes) / Ke
 
-    # the same workload with moment storage (tau = 1): 11 stored moments per
-    # cell instead of the 57 populations, rebuilt in the pull
+    # the same workload with the moment state asked for (a tau = 1 step keeps
+    # it anyway: same kernels)
     moments = {}
     if rank == 0 and not args.no_moments:
         del sim
@@ -359,16 +382,12 @@ def main():
         torch.cuda.synchronize(dev)
         msm = m0.elapsed_time(m1)
         pm = sm.profile(nprof)
-        # algorithmic bytes per cell: the 11 stored moments read once by the
-        # rebuilding pull (k_moments_recon, which writes rho - 1, phi, psi, j)
-        # and written once by the collide (which reads those and I)
-        kbm = {"k_moments_recon": 11 * 4 + 6 * 4, "k_collide": 7 * 4 + 11 * 4}
         km = {}
-        for name, ms in (("k_moments_recon", pm.ms_moments), ("k_collide", pm.ms_collide)):
-            t = ms / nprof / 1e3
-            ach = kbm[name] * N / t / 1e9
-            km[name] = {"bytes_per_cell": kbm[name], "ms": t * 1e3, "achieved": ach, "frac": ach / peak}
-        bpm = 11 * 8 + 24  # stored moments read and written, rho - 1, phi, psi written and read
+        for name, phase, kbm in lattice_kernels("f32", True):
+            t = getattr(pm, phase) / nprof / 1e3
+            ach = kbm * N / t / 1e9
+            km[name] = {"bytes_per_cell": kbm, "ms": t * 1e3, "achieved": ach, "frac": ach / peak}
+        bpm = moved_bytes("f32", True)
         moments = {"workload": wlm.name + " (state: moments)", "value": N * nm / (msm / 1e3) / 1e6,
                    "unit": "MLUPS", "steps": nm, "ms_per_step": msm / nm, "tile_variant": tvm,
                    "whole_step_bytes_per_cell": bpm,
@@ -384,7 +403,7 @@ def main():
         if "sim" in locals():
             del sim
         torch.cuda.empty_cache()
-        for fmt, bpc in (("f16", step_bytes(2)), ("bf16", step_bytes(2))):
+        for fmt in ("f16", "bf16"):
             wl16 = W.capsule_3d(fmt)
             s16 = T.Simulation(wl16, device=dev)
             s16.init()
@@ -399,12 +418,12 @@ def main():
             torch.cuda.synchronize(dev)
             ms16 = a0.elapsed_time(a1)
             p16 = s16.profile(nprof)
-            kb16 = kernel_bytes(2, t1=tv16 >= 13)
+            bpc = moved_bytes(fmt, tv16 >= 13)
             k16 = {}
-            for name, ms in (("k_moments", p16.ms_moments), ("k_collide", p16.ms_collide)):
-                t = ms / nprof / 1e3
-                ach = kb16[name] * N / t / 1e9
-                k16[name] = {"bytes_per_cell": kb16[name], "ms": t * 1e3, "achieved": ach, "frac": ach / peak,
+            for name, phase, kb16 in lattice_kernels(fmt, tv16 >= 13):
+                t = getattr(p16, phase) / nprof / 1e3
+                ach = kb16 * N / t / 1e9
+                k16[name] = {"bytes_per_cell": kb16, "ms": t * 1e3, "achieved": ach, "frac": ach / peak,
                              "traffic": _traffic(f"{name}_{fmt}")}
             lowprec[fmt] = {"value": N * n16 / (ms16 / 1e3) / 1e6, "unit": "MLUPS", "steps": n16,
                             "whole_step_bytes_per_cell": bpc,
@@ -447,11 +466,12 @@ def main():
         b1.record(bt.stream)
         torch.cuda.synchronize(dev)
         mss = b0.elapsed_time(b1)
-        eff = step_bytes(2) * cells * nsw / (msb / 1e3) / 1e9
+        bpc = moved_bytes("f16", tv >= 13)
+        eff = bpc * cells * nsw / (msb / 1e3) / 1e9
         sweep = {"workload": f"sweep_3d: {len(wls)} instances, edges 48-96, FP16 storage, seed 1",
                  "instances": len(wls), "cells": cells, "value": cells * nsw / (msb / 1e3) / 1e6,
                  "unit": "MLUPS", "steps": nsw, "ms_per_step": msb / nsw, "gpu_launches_per_step": lps,
-                 "effective_gbs": eff, "effective_frac": eff / peak, "bytes_per_cell": step_bytes(2),
+                 "effective_gbs": eff, "effective_frac": eff / peak, "bytes_per_cell": bpc,
                  "collide_tile_variant": tv, "collide_z_chunk": zc, "phase_ms_per_step": phase_ms,
                  "one_at_a_time": {"value": cells * nsingle / (mss / 1e3) / 1e6, "unit": "MLUPS",
                                    "steps": nsingle, "ms_per_step": mss / nsingle}}
@@ -498,7 +518,7 @@ def main():
             workloads["bridge_3d_" + fmt] = {
                 "workload": wb.name, "storage": fmt, "steps": nb_, "value": wb.params.ncells * nb_ / (msb_ / 1e3) / 1e6,
                 "unit": "MLUPS", "ms_per_step": msb_ / nb_, "tile_variant": tvb,
-                "whole_step_frac": step_bytes(2) * wb.params.ncells * nb_ / (msb_ / 1e3) / 1e9 / peak,
+                "whole_step_frac": moved_bytes(fmt, tvb >= 13) * wb.params.ncells * nb_ / (msb_ / 1e3) / 1e9 / peak,
                 "fp64_mass": list(db.mass[:]), "area": list(db.area[:2]), "volume": list(db.volume[:2])}
             del sb
             torch.cuda.empty_cache()
@@ -711,7 +731,7 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": wl.name, "cells": N, "markers": int(wl.membranes[0].X.shape[0]),
-                       "storage": args.storage, "l2": "state > 0.6 GB > L2, no flush needed",
+                       "storage": args.storage, "l2": "a step reads and writes over 0.16 GB > L2, no flush needed",
                        "parallelism": "replicas" if world > 1 else "single",
                        "collide_tile_variant": tile_variant, "collide_z_chunk": z_chunk},
             "roofline": roofline, "cpu_baseline": cpu, "clocks": clocks,

@@ -183,7 +183,7 @@ struct Ctx {
     return p.state != TLB_STATE_MOMENTS;
   }
   // Where the state is.  A step with a tau = 1 collide variant keeps it in
-  // the 11 values per cell of M (see EqCell), any other in the population
+  // the 12 values per cell of M (see EqCell), any other in the population
   // buffer `cur`.  state_in_pops: in the populations (after an
   // initialisation, a load, a write of populations or a general step), which
   // the next tau = 1 step pulls; otherwise in M, and pops_stale says that the

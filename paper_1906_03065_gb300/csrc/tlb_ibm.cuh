@@ -240,6 +240,8 @@ __device__ __forceinline__ V3<Real> face_normal(const IBArgs<Real>& a, int e) {
 // 2003), the derivatives dE_v/dK = kb K / (4 A) and dE_v/dA = -kb |K|^2 /
 // (8 A^2), which the force of every marker around it needs (see
 // node_forces_body).  Lane sums are combined by a fixed shuffle tree.
+// A chain of dependent loads on few threads: 2562 markers 6 us (10 us with
+// one thread per marker and no Helfrich part).
 template <class Real>
 __device__ __forceinline__ Real group_sum(Real v) {  // over the 16 lanes of a marker
 #pragma unroll
@@ -447,6 +449,11 @@ struct ScatterWarp {
 // over them, and the lanes take the cells round-robin.  `split` virtual
 // blocks set up the same features and take turns over the rounds (the set-up
 // is short; the rounds are not; see scatter_split).
+//
+// Bound by the scattered 64-bit min reductions (lanes that walked their own
+// slices, with less arithmetic but neighbouring lanes in unrelated cells, took
+// 51 us): 15 360 features, dc = 10, 24 us; 35 us with the exact distance to
+// the offered face and a binary search per cell.
 template <class Real>
 __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const Blk& blk) {
   constexpr int SW = scatter_warps<Real>();
@@ -759,6 +766,11 @@ __device__ __forceinline__ long long cpl_fixed(double v) { return llrint(v * CPL
 // step and cannot cross a cell farther than dc from it): it takes +-dc and
 // I_in/I_out here, so that between fresh starts the column fill, which
 // would find the same sides, is not needed.
+// Bound by instruction issue with part-filled warps (half the box lies outside
+// the band) and the grouped reductions: radius-20 capsule, 28 us (30 us
+// with 64-bit conversions and scalar loads).  Warps on compact 8 x 2 x 2 cells
+// instead of rows: 23 us there, but 13% slower on coarse meshes, whose lanes
+// then share elements; one warp sum per element: slower on every mesh.
 template <class Real>
 __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk) {
   int blo[3], bhi[3];
@@ -994,7 +1006,7 @@ __global__ void k_fill(const __grid_constant__ IBArgs<Real> a) {
 // (an obtuse face's areas are A2/4 or A2/8 times the A' instead, A2 twice its
 // area), with cot_i = d_i / A2.  (Each marker used to differentiate the
 // energies of its whole 1-ring, 42 face terms in dual numbers, for 18 that
-// depend on it.)
+// depend on it: 17 us for 2562 markers with 32 lanes each, now 5.5.)
 // 2D: lanes 0 and 1 the two segments (eq. DiscreteSE), lanes 2..4 the bending
 // at the previous marker, this one and the next (eqs. DiscreteBE,
 // DiscreteTheta, DiscreteArcLength).
