@@ -281,21 +281,19 @@ tlb_status tlb_profile_steps(void* ctx, long n_steps, tlb_profile* out);
 
 /* Choose the tile shape and z chunk of the collide plane sweep by timing
  * the collide kernel on the current state (CUDA events; the state is not
- * advanced).  Writes the chosen variant v = 3 form + tile (tile 0: 32x4,
- * 1: 32x8, 2: 64x4 in 3D; 0: 32, 1: 64, 2: 128 columns in 2D; form 0:
- * registers for 640 threads per SM, 1: 512, 2: 768, 3: 1024; v = 12: tile 0
- * at 896) and planes per chunk
- * when the pointers are non-NULL.  Variants 13..18 (tiles 0..2 at 640,
+ * advanced).  Writes the chosen variant v and planes per chunk when the
+ * pointers are non-NULL.  Variants 0..12 are the general collide on tile
+ * v % 3 (0: 32x4, 1: 32x8, 2: 64x4 in 3D; 0: 32, 1: 64, 2: 128 columns in
+ * 2D); of the equal ones 3..5 are tried.  Variants 13..18 (tiles 0..2 at 640,
  * then at 768 threads per SM) are the collide for tau = tau_phi = tau_psi
  * = 1 with TLB_FORCE_EDM, the paper's setting (Sec. 3.1): there every
  * post-collision population is an equilibrium of the cell's moments (eq.
- * LBE), so that collide pulls no population and stores only the 11 values
+ * LBE), so that collide pulls no population and stores only the 12 values
  * per cell they are made of (see TLB_STATE_POPULATIONS).  Variants 22..27
  * name those six again and need an even nx; 28..31 are the tau = 1 collide
  * on 32x16 tiles (3D) at 640, 768, 640 and 768 threads per SM, the last
  * two with an even nx.  Variants 19..21 are tiles 0..2 of the general
- * collide with the
- * pressure-tensor force.  They are tried only where they apply, and a new
+ * collide with the pressure-tensor force.  They are tried only where they apply, and a new
  * context starts on variant 14 there (19 with the pressure-tensor force,
  * else 3), with a z chunk set by the lattice's size.
  * Synchronises the stream.  Not in the paper: an autotuner for this

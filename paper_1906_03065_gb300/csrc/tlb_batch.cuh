@@ -534,7 +534,7 @@ struct BatchImpl : BatchBase {
     }
     for (int v = 0; v < COLLIDE_NVAR && st == TLB_OK; ++v)
       for (size_t zi = 0; zi < zcs.size() && st == TLB_OK; ++zi) {
-        if (!all_ok(v) || variant_t1(v) != t1 || variant_pair(v)) continue;
+        if (!all_ok(v) || variant_t1(v) != t1 || variant_again(v)) continue;
         b->tile_variant = v;
         b->zc = zcs[zi];
         b->graph_dirty = true;

@@ -12,15 +12,17 @@
 
 #include "../../include/tlb.h"
 
-// Collide variants: 3 tile shapes x 4 register forms, v = 3 form + tile,
-// the smallest tile in a fifth form (v = 12), and the 3 tiles in the two
-// forms of the tau = 1 collide (v = 13..18, see variant_t1); 22..27 name
-// those again, 28..31 a fourth tile.
+// Collide variants: the 3 tile shapes of the general collide (v = 0..12, tile
+// v % 3), the 3 tiles in the two forms of the tau = 1 collide (v = 13..18, see
+// variant_t1); 22..27 name those again, 28..31 a fourth tile.
 constexpr int COLLIDE_NVAR = 32;
 constexpr bool variant_t1(int v) { return (v >= 13 && v <= 18) || v >= 22; }
 // variants 22..27 and 30, 31 need an even nx (two-cell forms of the tau = 1
 // collide; they run the one-cell kernels)
 constexpr bool variant_pair(int v) { return (v >= 22 && v <= 27) || v == 30 || v == 31; }
+// variants that run the kernel of another one (3..5 for the general collide):
+// an autotuner need not time them
+constexpr bool variant_again(int v) { return variant_pair(v) || (v <= 12 && (v < 3 || v > 5)); }
 // variants 19..21: the general collide with the pressure-tensor force
 constexpr bool variant_pt(int v) { return v >= 19 && v <= 21; }
 

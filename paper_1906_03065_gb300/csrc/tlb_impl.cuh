@@ -420,7 +420,7 @@ struct Impl : ImplBase {
     const std::vector<int> zcs = z_chunk_candidates(c->nz);
     for (int v = 0; v < COLLIDE_NVAR; ++v)
       for (const int zcv : zcs) {
-        if (!c->variant_ok(v) || variant_t1(v) != t1 || variant_pair(v)) continue;
+        if (!c->variant_ok(v) || variant_t1(v) != t1 || variant_again(v)) continue;
         c->tile_variant = v;
         c->tiles_zc = zcv;
         la.zc = c->tiles_zc;
@@ -587,7 +587,6 @@ struct Impl : ImplBase {
 
   tlb_status step_direct(Ctx* c, long n) {
     cudaStream_t s = c->stream;
-    const long long N = c->N;
     tlb_status st;
     // Pipelined: the interpolation and advection of a step runs on the side
     // stream beside the next step's moments (which read the populations

@@ -453,8 +453,8 @@ __device__ __forceinline__ void pressure_tensor(const FEParams<Real>& fe, Real d
 }
 
 // Forms 5 and 6 are the collide at tau = tau_phi = tau_psi = 1 with the exact
-// difference method (collide_t1_body), form 7 the general one with the
-// pressure-tensor force; the others the general one.
+// difference method, form 7 the general one with the pressure-tensor force,
+// form 1 the general one.
 template <int FORM> constexpr bool form_t1() { return FORM == 5 || FORM == 6; }
 
 template <class L, int MODE, int TX, int TY>
@@ -881,13 +881,14 @@ __device__ __forceinline__ void collide_body(const LBArgs<MODE>& a, const Blk& b
   else
     collide_body_of<L, MODE, TX, TY, form_t1<FORM>()>(a, blk);
 }
-// Forms of the collide: threads per SM the register budget is set for
-// (0: 640; 1: 512; 2: 768; 3: 1024; 4: 896; the tau = 1 collide at 5: 640 and
-// 6: 768; the pressure tensor at 7: 640).  The tau = 1 collide holds about 90
+// Forms of the collide: threads per SM the register budget is set for (1, the
+// general collide: 512; the tau = 1 collide at 5: 640 and 6: 768; the
+// pressure tensor at 7: 640).  The general collide holds its cell's
+// populations, so fewer threads with their values in registers win: step of
+// 128^3 FP32 0.360 ms on 32 x 4 tiles, against 0.394 at 640, 0.422 at 768 and
+// over 0.48 at 896 and 1024 (spills).  The tau = 1 collide holds about 90
 // values per thread: at 768 threads per SM it spilled 52 bytes.
-template <int FORM> constexpr int collide_threads() {
-  return FORM == 1 ? 512 : (FORM == 2 || FORM == 6 ? 768 : (FORM == 3 ? 1024 : (FORM == 4 ? 896 : 640)));
-}
+template <int FORM> constexpr int collide_threads() { return FORM == 1 ? 512 : (FORM == 6 ? 768 : 640); }
 // threads of a collide block: one per cell of the TX x TY tile
 template <int FORM, int TX, int TY> constexpr int collide_block() { return TX * TY; }
 
@@ -904,28 +905,19 @@ __global__ void __launch_bounds__(collide_block<FORM, TX, TY>(), collide_minb<MO
 }
 
 // Calls fn(tile x, tile y, form) with the variant's compile-time values
-// (3D tiles 32x4, 32x8, 64x4; 2D rows of 32, 64, 128; variant 12 is the
-// smallest tile in form 4; variants 13-18 the three tiles in the tau = 1
-// forms 5 and 6; variants 19-21 the three tiles of form 7, the general
-// collide with the pressure-tensor force).
+// (3D tiles 32x4, 32x8, 64x4; 2D rows of 32, 64, 128): variants 0..12 the
+// three tiles of the general collide in turn, all in form 1 (each of the three
+// has several numbers; see variant_again); 13..18 the tiles in the tau = 1
+// forms 5 and 6; 19..21 in form 7, the general collide with the
+// pressure-tensor force.
 template <int V> using CIdx = std::integral_constant<int, V>;
 template <class L, class Fn>
 __host__ tlb_status collide_variant(int v, Fn&& fn) {
   constexpr bool D3 = L::DIM == 3;
   constexpr int X1 = D3 ? 32 : 64, Y1 = D3 ? 8 : 1, X2 = D3 ? 64 : 128, Y0 = D3 ? 4 : 1;
   switch (v) {
-    case 1: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<0>{});
-    case 2: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<0>{});
-    case 3: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<1>{});
-    case 4: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<1>{});
-    case 5: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<1>{});
-    case 6: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<2>{});
-    case 7: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<2>{});
-    case 8: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<2>{});
-    case 9: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<3>{});
-    case 10: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<3>{});
-    case 11: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<3>{});
-    case 12: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<4>{});  // (the larger tiles at 896 repeat 768)
+    case 1: case 4: case 7: case 10: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<1>{});
+    case 2: case 5: case 8: case 11: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<1>{});
     case 13: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<5>{});
     case 14: return fn(CIdx<X1>{}, CIdx<Y1>{}, CIdx<5>{});
     case 15: return fn(CIdx<X2>{}, CIdx<Y0>{}, CIdx<5>{});
@@ -947,7 +939,7 @@ __host__ tlb_status collide_variant(int v, Fn&& fn) {
     case 30: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<5>{});
     case 29:
     case 31: return fn(CIdx<32>{}, CIdx<D3 ? 16 : 1>{}, CIdx<6>{});
-    default: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<0>{});
+    default: return fn(CIdx<32>{}, CIdx<Y0>{}, CIdx<1>{});  // 0, 3, 6, 9, 12
   }
 }
 
