@@ -270,14 +270,15 @@ struct Impl : ImplBase {
     TLB_LAUNCHED(c, "k_init_eq");
     TLB_CUDA(cudaMemsetAsync(c->ptr<char>(c->L.ftot), 0, c->L.ftot.bytes, s));
     // the initial state is the first reference of the equilibrium residual
+    // (of these populations: what M held before is not written over them)
+    c->state_in_pops = true;
+    c->pops_stale = false;
     tlb_status rs = residual_launch(c);
     if (rs != TLB_OK) return rs;
     TLB_CUDA(cudaStreamSynchronize(s));
     c->t = 0;
     c->t_snap = 0;
     c->initialised = true;
-    c->state_in_pops = true;
-    c->pops_stale = false;
     return TLB_OK;
   }
 
@@ -355,14 +356,15 @@ struct Impl : ImplBase {
                                                           c->ptr<Store>(c->L.lo[c->cur]),
                                                           c->ptr<Rest>(c->L.rest[c->cur]));
     TLB_LAUNCHED(c, "k_init_eq");
+    // (of these populations: what M held before is not written over them)
+    c->state_in_pops = true;
+    c->pops_stale = false;
     tlb_status rs = residual_launch(c);
     if (rs != TLB_OK) return rs;
     TLB_CUDA(cudaStreamSynchronize(s));
     c->t = 0;
     c->t_snap = 0;
     c->initialised = true;
-    c->state_in_pops = true;
-    c->pops_stale = false;
     return TLB_OK;
   }
 
