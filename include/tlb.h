@@ -313,12 +313,21 @@ tlb_status tlb_set_tile(void* ctx, int tile_variant, int z_chunk);
  * collide variant from the same kernels the direct launches use (the results
  * are identical bit for bit; the kernels keep their streams' priorities); the
  * first step after markers were set from outside or after populations were
- * written, the steps of tlb_profile_steps, calls while the context stream is
- * being captured and a remainder below 8 steps run as direct launches.  By
+ * written, the steps of tlb_profile_steps and a remainder below 8 steps run as
+ * direct launches.  By
  * default a graph is captured in a call of 32 steps or more; on != 0 asks for
  * it in any call of 8 steps or more, on = 0 turns graphs off and releases the
- * captured ones.  Not in the paper: a launch mechanism of this
- * implementation. */
+ * captured ones.
+ * tlb_step may also be called while the caller captures the context's stream.
+ * Nothing runs then and the state stays as it is; each replay of the caller's
+ * graph takes those steps from the state it finds, as a direct call would, and
+ * other calls may stand between replays (the collide variant stays the
+ * captured one).  Two things are the caller's: the step counter advances once,
+ * in the captured call, and steps of the general collide swap the population
+ * buffers, so a captured call takes an even number of them and finds its
+ * buffer after an even number.  Calls that read back or synchronise (tlb_run,
+ * tlb_read_*, tlb_residual, the batch calls) cannot be captured.  Not in the
+ * paper: a launch mechanism of this implementation. */
 tlb_status tlb_set_graphs(void* ctx, int on);
 
 /* Number of CUDA kernel launches enqueued by the last tlb_step call (a
@@ -373,7 +382,8 @@ tlb_status tlb_batch_set_active(void* batch, const int* flags);
 
 /* Advance every active instance n_steps steps (enqueued on the stream; the
  * host synchronises only while uploading the argument tables).
- * TLB_ERR_STATE if an active instance is not initialised. */
+ * TLB_ERR_STATE if an active instance is not initialised or the stream is
+ * being captured. */
 tlb_status tlb_batch_step(void* batch, long n_steps);
 
 /* Run to equilibrium: advance the active instances in chunks of

@@ -311,6 +311,7 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.ctr, 4 * 4);
   take(L.bflag, nb);
   take(L.status, 64);
+  take(L.in_M, 4);
   take(L.part, 3 * 1024 * 8);
   take(L.meas, 32 * 8);
   take(L.snap, 2 * P * 8);

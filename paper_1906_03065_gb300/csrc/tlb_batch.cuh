@@ -343,7 +343,10 @@ struct BatchImpl : BatchBase {
         a.lb.zc = b->zc;
         a.lb.zcm = b->recon_zc;
         I::use_t1(c, a.lb, t1);
-        if (q == 0) a.lb.pull = 0;
+        if (q == 0) {
+          a.lb.pull = 0;
+          a.lb.in_M = nullptr;
+        }
         if (t1 && scratch) a.lb.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
         a.ib = I::ibargs(c);
         I::use_t1(c, a.ib, t1);
@@ -357,25 +360,34 @@ struct BatchImpl : BatchBase {
     return TLB_OK;
   }
 
-  // some active instance's state is in its populations
+  // some active instance's state is in its populations, or may be
+  static bool pulls(const Ctx* c) { return c->state_in_pops || c->asks(); }
   static bool any_pull(const Batch* b) {
     for (int i : b->act)
-      if (b->inst[i]->state_in_pops) return true;
+      if (pulls(b->inst[i])) return true;
     return false;
   }
   // after n steps: where the state is, and the step counts
-  static void advanced(Batch* b, long n) {
+  static tlb_status advanced(Batch* b, long n) {
     const bool t1 = variant_t1(b->tile_variant);
     for (int i : b->act) {
       Ctx* c = b->inst[i];
       if (t1) {
-        c->state_in_pops = false;
+        if (pulls(c))
+          if (tlb_status st = I::entered_M(c, b->stream); st != TLB_OK) return st;
         c->pops_stale = true;
       } else if (n & 1) {
         c->cur ^= 1;
       }
       c->t += n;
     }
+    return TLB_OK;
+  }
+  // No graph can hold a batch call: its argument tables are uploaded in each.
+  static tlb_status refuse_capture(const Batch* b) {
+    if (!I::caller_captures(b->stream)) return TLB_OK;
+    set_error("batch: not while its stream is being captured");
+    return TLB_ERR_STATE;
   }
 
   // Markers overwritten since the last step: rebuild the box accumulator
@@ -439,7 +451,8 @@ struct BatchImpl : BatchBase {
 
   tlb_status step(Batch* b, long n) override {
     if (b->act.empty() || n == 0) return TLB_OK;
-    tlb_status st = prepare(b);
+    tlb_status st = refuse_capture(b);
+    if (st == TLB_OK) st = prepare(b);
     if (st != TLB_OK) return st;
     long left = n;
     // a first step that the graph's steps differ from
@@ -447,7 +460,7 @@ struct BatchImpl : BatchBase {
     if (pull || b->fresh) {
       if ((st = launch_step(b, pull ? 1 : 0, b->stream, b->fresh)) != TLB_OK) return st;
       b->fresh = false;
-      advanced(b, 1);
+      if ((st = advanced(b, 1)) != TLB_OK) return st;
       if (--left > 0 && !variant_t1(b->tile_variant) && (st = upload_tables(b)) != TLB_OK) return st;
     }
     const long rest = left;
@@ -457,14 +470,14 @@ struct BatchImpl : BatchBase {
       b->launches += b->graph_launches;
     }
     if (left && (st = launch_step(b, 0, b->stream)) != TLB_OK) return st;
-    if (rest > 0) advanced(b, rest);
-    return TLB_OK;
+    return rest > 0 ? advanced(b, rest) : TLB_OK;
   }
 
   tlb_status profile(Batch* b, long n, double* ms) override {
     for (int ph = 0; ph < 6; ++ph) ms[ph] = 0;
     if (b->act.empty() || n == 0) return TLB_OK;
-    tlb_status st = prepare(b);
+    tlb_status st = refuse_capture(b);
+    if (st == TLB_OK) st = prepare(b);
     if (st != TLB_OK) return st;
     cudaEvent_t ev[7];
     for (int k = 0; k < 7; ++k) TLB_CUDA(cudaEventCreate(&ev[k]));
@@ -486,8 +499,7 @@ struct BatchImpl : BatchBase {
     for (int k = 0; k < 7; ++k) cudaEventDestroy(ev[k]);
     if (st != TLB_OK) return st;
     b->fresh = false;
-    advanced(b, n);
-    return TLB_OK;
+    return advanced(b, n);
   }
 
   tlb_status residual(Batch* b) override {
@@ -505,6 +517,7 @@ struct BatchImpl : BatchBase {
   // other, so repeats leave the state unchanged).
   tlb_status autotune(Batch* b, int* variant, int* zc) override {
     if (b->act.empty()) return TLB_OK;
+    if (tlb_status rs = refuse_capture(b); rs != TLB_OK) return rs;
     cudaEvent_t e0, e1;
     TLB_CUDA(cudaEventCreate(&e0));
     TLB_CUDA(cudaEventCreate(&e1));

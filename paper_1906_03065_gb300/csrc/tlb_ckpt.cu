@@ -188,14 +188,13 @@ tlb_status tlb_load(void* ctx, const void* host_blob, size_t bytes) {
     off += sz[k];
   }
   TLB_CUDA(cudaMemsetAsync(c->ptr<char>(c->L.status), 0, c->L.status.bytes, c->stream));
+  if (tlb_status st = c->impl->pops_written(c); st != TLB_OK) return st;
   TLB_CUDA(cudaStreamSynchronize(c->stream));
   c->cur = 0;
   c->t = h.t;
   c->t_snap = h.t_snap;
   c->initialised = true;
   c->box_stale = true;
-  c->state_in_pops = true;
-  c->pops_stale = false;
   return TLB_OK;
 }
 

@@ -120,6 +120,8 @@ struct ImplBase {
   // write the populations that the state in M stands for into the current
   // population buffer if it is stale (no-op otherwise)
   virtual tlb_status sync_pops(Ctx* c) = 0;
+  // the population buffer holds the state from here on
+  virtual tlb_status pops_written(Ctx* c) = 0;
   // chunk lengths of the plane sweeps for lattices swept together (the
   // default collide variant; the moments rebuild in blocks of bt threads)
   virtual int collide_chunk(const std::vector<Ctx*>& cs, int variant) = 0;
@@ -152,6 +154,7 @@ struct Layout {
   Region bcnt, bprev, bcur, boff, blist, bact, ctr, bflag;
   // misc
   Region status, part, meas;
+  Region in_M;
   // equilibrium residual: reference phi, psi and marker positions, maxima
   Region snap, xsnap, res;
   size_t total = 0;
@@ -192,6 +195,13 @@ struct Ctx {
   // population buffer does not show it yet (sync_pops writes it there).
   bool state_in_pops = true;
   bool pops_stale = false;
+  // The device word L.in_M says the same (0: in the populations) and is kept
+  // beside the flag.  Once the caller has captured steps into a graph of its
+  // own (`outside`), replays move the state without the host: kernels then
+  // read the word, except within a step call after its first step (`known`).
+  bool outside = false;
+  bool known = false;
+  bool asks() const { return outside && !known; }
   int Q = 0;
   int nx = 0, ny = 0, nz = 0;  // internal sizes (2D: nx, 1, ny)
   long long N = 0, P = 0;

@@ -38,6 +38,7 @@ struct Impl : ImplBase {
     a.j2 = t1 ? c->ptr<R2<Real>>(c->L.j2) : nullptr;
     a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
     a.pull = c->state_in_pops;
+    a.in_M = t1 && c->asks() ? c->ptr<int>(c->L.in_M) : nullptr;
   }
   static void use_t1(Ctx* c, IBArgs<Real>& a, bool t1) {
     a.psi = c->packed() ? &c->ptr<R4<Real>>(c->L.p4)->z : c->ptr<Real>(c->L.psi);
@@ -271,9 +272,8 @@ struct Impl : ImplBase {
     TLB_CUDA(cudaMemsetAsync(c->ptr<char>(c->L.ftot), 0, c->L.ftot.bytes, s));
     // the initial state is the first reference of the equilibrium residual
     // (of these populations: what M held before is not written over them)
-    c->state_in_pops = true;
-    c->pops_stale = false;
-    tlb_status rs = residual_launch(c);
+    tlb_status rs = pops_written(c);
+    if (rs == TLB_OK) rs = residual_launch(c);
     if (rs != TLB_OK) return rs;
     TLB_CUDA(cudaStreamSynchronize(s));
     c->t = 0;
@@ -303,18 +303,41 @@ struct Impl : ImplBase {
   }
 
   tlb_status sync_pops(Ctx* c) override {
-    if (c->state_in_pops || !c->pops_stale) return TLB_OK;
+    if (!c->asks() && (c->state_in_pops || !c->pops_stale)) return TLB_OK;
     k_materialize<L, MODE><<<blocks(c->N, 256), 256, 0, c->stream>>>(
-        geo(c), c->ptr<R4<Real>>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]));
+        geo(c), c->ptr<R4<Real>>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]),
+        c->asks() ? c->ptr<int>(c->L.in_M) : nullptr);
     TLB_LAUNCHED(c, "k_materialize");
+    // (captured, it has not run; the flag of a context that asks is not used)
+    if (!caller_captures(c->stream)) c->pops_stale = false;
+    return TLB_OK;
+  }
+
+  // the state is in the populations / in M from here on
+  tlb_status pops_written(Ctx* c) override {
+    TLB_CUDA(cudaMemsetAsync(c->ptr<int>(c->L.in_M), 0, sizeof(int), c->stream));
+    c->state_in_pops = true;
     c->pops_stale = false;
     return TLB_OK;
+  }
+  static tlb_status entered_M(Ctx* c, cudaStream_t s) {
+    TLB_CUDA(cudaMemsetAsync(c->ptr<int>(c->L.in_M), 1, sizeof(int), s));
+    c->state_in_pops = false;
+    return TLB_OK;
+  }
+  // The caller is capturing the stream.  (A query that fails, as on the
+  // legacy default stream beside another capture, is left to the launches.)
+  static bool caller_captures(cudaStream_t s) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return false;
   }
 
   // the moments of the streamed populations: rebuilt from the state in M, or
   // pulled from the population buffer
   static tlb_status launch_moments(Ctx* c, const LBArgs<MODE>& la, cudaStream_t s) {
-    if (la.M && !la.pull) {
+    if (la.M && (la.in_M || !la.pull)) {
       const dim3 grid(blocks(c->nx, RECON_X), blocks(c->ny, RECON_Y), blocks(c->nz, la.zcm));
       k_moments_recon<L, MODE, RECON_X, RECON_Y><<<grid, RECON_X * RECON_Y, 0, s>>>(la);
       TLB_LAUNCHED(c, "k_moments_recon");
@@ -357,9 +380,8 @@ struct Impl : ImplBase {
                                                           c->ptr<Rest>(c->L.rest[c->cur]));
     TLB_LAUNCHED(c, "k_init_eq");
     // (of these populations: what M held before is not written over them)
-    c->state_in_pops = true;
-    c->pops_stale = false;
-    tlb_status rs = residual_launch(c);
+    tlb_status rs = pops_written(c);
+    if (rs == TLB_OK) rs = residual_launch(c);
     if (rs != TLB_OK) return rs;
     TLB_CUDA(cudaStreamSynchronize(s));
     c->t = 0;
@@ -469,6 +491,36 @@ struct Impl : ImplBase {
   // n steps; runs of GRAPH_STEPS steps replay a captured graph where the
   // steps qualify (see graph_ready)
   tlb_status step(Ctx* c, long n) override {
+    if (n > 0 && caller_captures(c->stream)) return step_captured(c, n);
+    c->known = false;
+    const tlb_status st = step_calls(c, n);
+    c->known = false;
+    return st;
+  }
+
+  // A call inside a capture of the caller's stream.  Nothing runs now, and
+  // each replay continues from the state it finds, which other calls may have
+  // moved in between: the first tau = 1 step asks the device where the state
+  // is, the first step rebuilds the marker box (with the profile, as after
+  // markers set from outside), and what the host holds about the state is put
+  // back.  The step counter advances once, and an odd number of general steps
+  // leaves the state in the other population buffer.
+  tlb_status step_captured(Ctx* c, long n) {
+    const bool sp0 = c->state_in_pops, ps0 = c->pops_stale, stale0 = c->box_stale;
+    c->outside = true;
+    c->known = false;
+    c->box_stale = c->nn > 0;
+    c->capturing = true;
+    const tlb_status st = step_direct(c, n);
+    c->capturing = false;
+    c->known = false;
+    c->state_in_pops = sp0;
+    c->pops_stale = ps0;
+    c->box_stale = stale0;
+    return st;
+  }
+
+  tlb_status step_calls(Ctx* c, long n) {
     if (c->nn == 0 || !graphs_usable(c, n)) return step_direct(c, n);
     while (n > 0) {
       if (n >= Ctx::GRAPH_STEPS && graph_ready(c) && have_graph(c)) {
@@ -486,17 +538,12 @@ struct Impl : ImplBase {
     return TLB_OK;
   }
 
-  // Graphs serve this call: not while the caller's stream is being captured
-  // or phases are timed; and unless tlb_set_graphs asked for them, only where
-  // a graph exists already or the call is long enough to pay for its capture
-  // (about 0.5 ms, against 15 to 25 us saved per step).
+  // Graphs serve this call: not while phases are timed; and unless
+  // tlb_set_graphs asked for them, only where a graph exists already or the
+  // call is long enough to pay for its capture (about 0.5 ms, against 15 to 25
+  // us saved per step).
   bool graphs_usable(Ctx* c, long n) const {
     if (!c->graphs || c->prof || n < Ctx::GRAPH_STEPS) return false;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-      (void)cudaGetLastError();
-      return false;
-    }
     return c->graphs_asked || graph_current(c) || n >= 4 * Ctx::GRAPH_STEPS;
   }
   bool graph_current(const Ctx* c) const {
@@ -509,13 +556,14 @@ struct Impl : ImplBase {
   // box is rebuilt first) and the state where the collide variant keeps it
   // (the first tau = 1 step after populations were written pulls them).
   bool graph_ready(Ctx* c) const {
-    return c->graphs && !c->box_stale && c->state_in_pops == !variant_t1(c->tile_variant);
+    return c->graphs && !c->box_stale && !c->asks() && c->state_in_pops == !variant_t1(c->tile_variant);
   }
 
   // the state into the populations, for a step of a general variant
   static tlb_status enter_pops(Ctx* c) {
+    if (c->state_in_pops && !c->asks()) return TLB_OK;
     tlb_status st = c->impl->sync_pops(c);
-    if (st == TLB_OK) c->state_in_pops = true;
+    if (st == TLB_OK) st = c->impl->pops_written(c);
     return st;
   }
 
@@ -597,6 +645,8 @@ struct Impl : ImplBase {
     const bool pipe = c->nn > 0 && !c->prof;
     const bool t1 = variant_t1(c->tile_variant);
     if (!t1 && (st = enter_pops(c)) != TLB_OK) return st;
+    // (the last record may stand for a node of the caller's capture)
+    if (pipe && c->outside && !c->capturing) TLB_CUDA(cudaEventRecord(c->ev_interp, s));
     for (long k = 0; k < n; ++k) {
       LBArgs<MODE> la = lbargs(c, c->cur);
       IBArgs<Real> ia = ibargs(c);
@@ -654,11 +704,12 @@ struct Impl : ImplBase {
       if ((st = mark(c, 4)) != TLB_OK) return st;
       if ((st = collect(c)) != TLB_OK) return st;
       if (t1) {  // the state is M from here on
-        c->state_in_pops = false;
+        if ((la.pull || la.in_M) && (st = entered_M(c, s)) != TLB_OK) return st;
         c->pops_stale = true;
       } else {
         c->cur = 1 - c->cur;
       }
+      c->known = true;
       c->t += 1;
     }
     if (pipe && n > 0) TLB_CUDA(cudaStreamWaitEvent(s, c->ev_interp, 0));  // all of it on the caller's stream
@@ -748,10 +799,9 @@ struct Impl : ImplBase {
     }
     TLB_CUDA(cudaMemcpyAsync(c->ptr<Store>(c->L.lo[c->cur]), lo.data(), lo.size() * sizeof(Store), cudaMemcpyHostToDevice, s));
     TLB_CUDA(cudaMemcpyAsync(c->ptr<Rest>(c->L.rest[c->cur]), rest.data(), rest.size() * sizeof(Rest), cudaMemcpyHostToDevice, s));
+    if (tlb_status st = pops_written(c); st != TLB_OK) return st;
     TLB_CUDA(cudaStreamSynchronize(s));
     c->initialised = true;
-    c->state_in_pops = true;
-    c->pops_stale = false;
     return TLB_OK;
   }
 

@@ -26,6 +26,7 @@ struct LBArgs {
   R4<Real>* M;      // [3][P] the stored state (see EqCell)
   int pull;         // the state is in the populations, not in M (set by an
                     // initialisation, a load or a write): pull them this once
+  const int* in_M;  // not NULL: this device word decides instead (0: pull)
   const Real* I;
   const Real* fib;  // [3][P] immersed-boundary force density
   Real* ftot;       // [3][P] total force of the step (read by the interpolation)
@@ -136,7 +137,7 @@ __device__ __forceinline__ void moments_recon_body(const LBArgs<MODE>& a, const 
   const int x0 = blk.x * TX, y0 = blk.y * TY, z0 = blk.z * a.zcm, z1 = min(z0 + a.zcm, G.nz);
   const int x = x0 + tx, y = y0 + ty;
   const bool active = x < G.nx && y < G.ny;
-  if (a.pull) {  // once after an initialisation or a write of populations
+  if (a.in_M ? *a.in_M == 0 : a.pull) {  // once after an initialisation or a write of populations
     if (active)
       for (int zz = z0; zz < z1; ++zz) {
         Pull<L, MODE> p;
@@ -259,14 +260,15 @@ __global__ void __launch_bounds__(TX* TY, 768 / (TX * TY)) k_moments_recon(const
 
 // The populations a cell's stored state stands for, written post-collision
 // into the population buffers (for the readers of the population state).
+// in_M not NULL: only if the state is in M.
 template <class L, int MODE>
 __global__ void k_materialize(Geo G, const R4<typename Prec<MODE>::Real>* M, typename Prec<MODE>::Store* lo,
-                              typename Prec<MODE>::Rest* rest) {
+                              typename Prec<MODE>::Rest* rest, const int* in_M) {
   using Real = typename Prec<MODE>::Real;
   using Store = typename Prec<MODE>::Store;
   using Rest = typename Prec<MODE>::Rest;
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= G.N) return;
+  if (n >= G.N || (in_M && *in_M == 0)) return;
   EqCell<L, MODE> e;
   e.load(M, G.P32, (int)n);
   lo[(long long)plane_f<L>(0) * G.P + n] = from_real<Store>(e.f(0));
