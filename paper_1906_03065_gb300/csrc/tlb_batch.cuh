@@ -398,7 +398,7 @@ struct BatchImpl : BatchBase {
       if (!c->box_stale || c->nn == 0) continue;
       IBArgs<Real> a = I::ibargs(c);
       TLB_CUDA(cudaMemsetAsync(a.box, 0x7F, 6 * sizeof(int), b->stream));
-      k_box<Real><<<cdiv(c->nn, 128), 128, 0, b->stream>>>(a);
+      k_fresh<Real><<<I::fresh_blocks(c), 128, 0, b->stream>>>(a);
       b->launches++;
       TLB_CUDA(cudaGetLastError());
       c->box_stale = false;

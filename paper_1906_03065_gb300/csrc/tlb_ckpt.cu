@@ -3,8 +3,8 @@
 //
 // A checkpoint holds exactly the state a continued run reads: the current
 // population buffer (populations are stored post-collision), the profile I
-// (cells that leave the moving marker box keep their last value), the
-// marker positions, the residual's reference state and the step counters.
+// (for readers; the next step forms it anew from the markers), the marker
+// positions, the residual's reference state and the step counters.
 // Everything else is rebuilt within the next step: moments, potentials,
 // forces, keys, bricks; the marker box is recomputed from the markers, which
 // gives the same integers as the accumulator the advection leaves.

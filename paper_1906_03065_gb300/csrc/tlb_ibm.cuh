@@ -343,8 +343,9 @@ __global__ void k_geometry(const __grid_constant__ IBArgs<Real> a, int snap) {
 
 // Marker bounding box.  The advection kernel accumulates floor(min X) and
 // -ceil(max X) per axis with integer atomicMin into box[0..5] (reset to a
-// large value after use); k_box does the same from scratch at set-up, and
-// both store the split X = xo + xr of the positions.
+// large value after use); k_fresh does the same from scratch where markers
+// or the state were set from outside, and both store the split X = xo + xr of
+// the positions.
 template <class Real>
 __device__ __forceinline__ void box_body(const IBArgs<Real>& a, const Blk& blk) {
   int k = blk.x * blockDim.x + threadIdx.x;
@@ -356,9 +357,17 @@ __device__ __forceinline__ void box_body(const IBArgs<Real>& a, const Blk& blk) 
     split_coord(a.X[3 * k + d], a.xo + 3 * k + d, a.xr + 3 * k + d);
   }
 }
+// With the new box, the profile of a lattice without membranes: the band and
+// the column fill of the step write the new box only, and cells that were
+// band cells somewhere else must not keep that (see band_body).
 template <class Real>
-__global__ void k_box(const __grid_constant__ IBArgs<Real> a) {
+__global__ void k_fresh(const __grid_constant__ IBArgs<Real> a) {
   box_body(a, hw_blk());
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.G.N; i += (long long)gridDim.x * blockDim.x) {
+    a.own[i] = -1;
+    a.dsel[i] = -a.dc;
+    a.I[i] = a.Iout;
+  }
 }
 
 // The box of cells the profile visits: the step's marker box widened by
@@ -764,8 +773,8 @@ __device__ __forceinline__ long long cpl_fixed(double v) { return llrint(v * CPL
 // band cell in the previous step and is not one now lies beyond dc on the
 // side of its last distance (the membrane moves less than half a cell per
 // step and cannot cross a cell farther than dc from it): it takes +-dc and
-// I_in/I_out here, so that between fresh starts the column fill, which
-// would find the same sides, is not needed.
+// I_in/I_out here, so that between fresh starts (k_fresh) the column fill,
+// which would find the same sides, is not needed.
 // Bound by instruction issue with part-filled warps (half the box lies outside
 // the band) and the grouped reductions: radius-20 capsule, 28 us (30 us
 // with 64-bit conversions and scalar loads).  Warps on compact 8 x 2 x 2 cells

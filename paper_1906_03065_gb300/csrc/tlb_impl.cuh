@@ -171,14 +171,18 @@ struct Impl : ImplBase {
     return TLB_OK;
   }
 
+  static unsigned fresh_blocks(const Ctx* c) {
+    return std::max(blocks(c->nn, 128), std::min(blocks(c->N, 128), 8u * (unsigned)c->nsm));
+  }
+
   // The step's marker box: recompute the accumulator if the markers were
   // overwritten, copy it to the snapshot every kernel of the step reads, and
   // reset it for the advection of this step.
   static tlb_status snapshot_box(Ctx* c, IBArgs<Real>& a, cudaStream_t s, bool fresh) {
     if (fresh) {
       TLB_CUDA(cudaMemsetAsync(a.box, 0x7F, 6 * sizeof(int), s));
-      k_box<Real><<<blocks(c->nn, 128), 128, 0, s>>>(a);
-      TLB_LAUNCHED(c, "k_box");
+      k_fresh<Real><<<fresh_blocks(c), 128, 0, s>>>(a);
+      TLB_LAUNCHED(c, "k_fresh");
     }
     TLB_CUDA(cudaMemcpyAsync((void*)a.boxc, a.box, 6 * sizeof(int), cudaMemcpyDeviceToDevice, s));
     TLB_CUDA(cudaMemsetAsync(a.box, 0x7F, 6 * sizeof(int), s));
