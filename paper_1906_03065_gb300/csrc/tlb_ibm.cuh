@@ -41,7 +41,8 @@ struct IBArgs {
   int nedge;             // 3D: unique edges
   const int* edges;      // 3D: [nedge][4] vertex a, vertex b, face left, face right
   // per-step work
-  R4<Real>* en;          // [ne] unit outward normal
+  R4<Real>* en;          // [ne] unit outward normal; reach of a thin face's border
+                         // (see dist_scatter_body), else 0
   R4<Real>* vn;          // [nn] angle-weighted vertex pseudo-normal
   Real* wts;             // [nn][3][4] kernel weights (eq. DiscreteDirac) at the support
                          // cells floor(X) - 1 .. floor(X) + 2 along each axis
@@ -230,6 +231,24 @@ __device__ __forceinline__ V3<Real> face_normal(const IBArgs<Real>& a, int e) {
   return (Real(1) / sqrt(dot(cr, cr))) * cr;
 }
 
+// Half a unit of the last place, relative.
+__device__ __forceinline__ float eps_of(float) { return 0x1p-24f; }
+__device__ __forceinline__ double eps_of(double) { return 0x1p-53; }
+
+// A face whose first angle (between ab and ac) lies within 3.6 degrees of 0 or
+// 180, from the Gram entries and determinant of ab and ac.  The determinant,
+// d00 d11 sin^2, carries an error of a few eps d00 d11, so the barycentric
+// coordinates that it gives lose eps / sin^2; below sin = 5e-4 in FP32 it may
+// come out as zero or less.  Through the cross product of ab and ac they lose
+// eps / sin.
+constexpr float FLAT_SIN2 = 0x1p-15f;  // sin^2 up to which a face is its edges for the closest
+                                       // point: within sin / 2 of its size, where the
+                                       // coordinates lose eps / sin^2 (FP32: 2e-3)
+template <class Real>
+__device__ __forceinline__ bool thin_face(Real d00, Real d11, Real den) {
+  return !(den >= rmul(rmul(d00, d11), Real(1.0 / 256)));
+}
+
 // The geometry of the step in one launch.  Threads [0, ne) store the unit
 // outward face normals and what the band reads of each face.  Then 16 lanes
 // per marker, one incident face each, store the vertex pseudo-normal, the
@@ -254,7 +273,6 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
   int t = blk.x * blockDim.x + threadIdx.x;
   if (t < a.ne) {
     V3<Real> n = face_normal(a, t);
-    a.en[t] = R4<Real>{n.x, n.y, n.z, 0};
     const int* Et = a.E + a.NV * t;
     Real rv[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     int org[3];
@@ -271,12 +289,19 @@ __device__ __forceinline__ void geometry_body(const IBArgs<Real>& a, const Blk& 
     const V3<Real> ab = Bv - A, ac = a.NV == 3 ? Cv - A : mk<Real>(0, 0, 0), bc = a.NV == 3 ? Cv - Bv : mk<Real>(0, 0, 0);
     const Real d00 = dot(ab, ab), d01 = dot(ab, ac), d11 = dot(ac, ac), dbc = dot(bc, bc);
     const Real den = d00 * d11 - d01 * d01;
+    Real reach = 0;
+    if (a.NV == 3 && thin_face(d00, d11, den)) {
+      const V3<Real> N = cross(ab, ac);
+      const Real len = a.dc + sqrt(fmax(d00, d11));
+      reach = fmin(a.dc, Real(8) * eps_of(Real(0)) * len * sqrt(rmul(d00, d11) / dot(N, N)));
+    }
+    a.en[t] = R4<Real>{n.x, n.y, n.z, reach};
     R4<Real>* k = a.ecst + 4 * t;
     k[0] = R4<Real>{ab.x, ab.y, ab.z, ac.x};
     k[1] = R4<Real>{ac.y, ac.z, bc.x, bc.y};
     k[2] = R4<Real>{bc.z, d00, d01, d11};
     k[3] = R4<Real>{d00 > Real(0) ? rcp_rn(d00) : Real(0), d11 > Real(0) ? rcp_rn(d11) : Real(0),
-                    dbc > Real(0) ? rcp_rn(dbc) : Real(0), den > Real(0) ? rcp_rn(den) : Real(0)};
+                    dbc > Real(0) ? rcp_rn(dbc) : Real(0), den > rmul(rmul(d00, d11), FLAT_SIN2) ? rcp_rn(den) : Real(0)};
     return;
   }
   if (t < (a.ne + 31) / 32 * 32) return;  // (markers start at a whole warp)
@@ -425,9 +450,16 @@ __device__ __forceinline__ unsigned long long dist_code(double d) {
 // to the edge where it projects between the edge's ends (ends included, with
 // the distance clamped to them), to the vertex.  Where P lies on the feature
 // that is |x - P|; elsewhere it is a larger distance, or nothing is offered
-// and the feature that holds P offers it.  (The boxes are widened by 1e-3
-// cells and the ends of an edge likewise, far above the rounding of either
-// test, so a cell on the border of two features is offered by one of them.)
+// and the feature that holds P offers it.  The boxes are widened by 1e-3
+// cells and the ends of an edge likewise, above the rounding of either test,
+// so a cell on the border of two features is offered by one of them.  The
+// error of a face's normal moves a cell t away by some eps (t + size) / sin in
+// the face's plane, sin of its first angle: in FP32 at t = 16 by 1e-3 cells
+// from half a degree down.  So thin faces take their coordinates from the
+// cross product, a face without area offers nothing, and the edges and
+// vertices of a thin face widen their boxes to its reach 8 eps (dc + size) /
+// sin where that exceeds 1e-3.  (Without, I was off by up to 0.1 on meshes
+// with needle faces.)
 // So a cell costs three dot products for a face, two for an edge and one for
 // a vertex, where the exact distance to the offered face took seven.
 constexpr int MAXG = 12;  // generators (and faces) per feature
@@ -502,6 +534,8 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
   bool ok = nG > 0;
   int o[3] = {0, 0, 0}, tmin = 0x7fffffff;
   Real S[3] = {0, 0, 0};
+  const Real eps = Real(1e-3);
+  Real reach = 0;  // of the faces that contain the feature; > 0: thin ones among them
   if (ok) {
     for (int d = 0; d < 3; ++d) o[d] = a.xo[3 * corners[0] + d];
     if (a.dim == 2) o[1] = 0;
@@ -515,6 +549,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       S[0] += n.x;
       S[1] += n.y;
       S[2] += n.z;
+      reach = fmax(reach, n.w);
       ok &= fabs(n.x) <= Real(1.001) && fabs(n.y) <= Real(1.001) && fabs(n.z) <= Real(1.001);
       sm.gk[lane][j] = n.x;
       sm.ga[lane][j] = n.y;
@@ -539,7 +574,7 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
   int oa, ob;
   if (a.dim == 3) { oa = k == 0 ? 1 : 0; ob = k == 2 ? 1 : 2; }
   else { oa = k == 0 ? 2 : 0; ob = 1; }
-  const Real dc = a.dc, eps = Real(1e-3);
+  const Real dc = a.dc, widen = kind == 0 ? eps : fmax(eps, reach);  // of the slices' boxes
   int c0 = 0, nsl = 0;
   bool wide = false;
   if (ok) {
@@ -562,8 +597,8 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
       bmin = fmin(bmin, sm.cb[lane][3 * q + k]);
       bmax = fmax(bmax, sm.cb[lane][3 * q + k]);
     }
-    c0 = (int)ceil(bmin - dc - eps);
-    nsl = (int)floor(bmax + dc + eps) - c0 + 1;
+    c0 = (int)ceil(bmin - dc - widen);
+    nsl = (int)floor(bmax + dc + widen) - c0 + 1;
     // first corner A, then by kind: the face's normal and the vectors whose
     // products with x - A are the barycentric coordinates of the projection
     // (a segment: one), or the edge and the vector that gives its parameter
@@ -576,6 +611,18 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
         p[d] = n0[d];
         q[d] = a.NV == 2 ? e[d] * e[12] : (d11 * e[d] - d01 * e[3 + d]) * iden;
         r[d] = a.NV == 2 ? Real(0) : (d00 * e[3 + d] - d01 * e[d]) * iden;
+      }
+      if (reach > Real(0)) {
+        const V3<Real> ab = mk<Real>(e[0], e[1], e[2]), ac = mk<Real>(e[3], e[4], e[5]), N = cross(ab, ac);
+        const Real inn = Real(1) / dot(N, N);
+        const V3<Real> Q = inn * cross(ac, N), T = inn * cross(N, ab);
+        q[0] = Q.x;
+        q[1] = Q.y;
+        q[2] = Q.z;
+        r[0] = T.x;
+        r[1] = T.y;
+        r[2] = T.z;
+        if (!(dot(N, N) > Real(0))) nsl = 0;
       }
     } else if (kind == 1) {
       Real l2 = 0;
@@ -625,11 +672,11 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
         lo1 = fmin(lo1, bb - dc); hi1 = fmax(hi1, bb + dc);
       }
     }
-    a0 = (int)ceil(lo0 - eps);
-    const int a1 = (int)floor(hi0 + eps);
+    a0 = (int)ceil(lo0 - widen);
+    const int a1 = (int)floor(hi0 + widen);
     int b1 = 0;
     b0 = 0;
-    if (a.dim == 3) { b0 = (int)ceil(lo1 - eps); b1 = (int)floor(hi1 + eps); }
+    if (a.dim == 3) { b0 = (int)ceil(lo1 - widen); b1 = (int)floor(hi1 + widen); }
     const int wb = b1 - b0 + 1;
     wa = a1 - a0 + 1;
     cnt = 0;
