@@ -104,6 +104,14 @@ template <class T> __device__ __forceinline__ T rdot(V3<T> a, V3<T> b) {
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
 
+// rcp_rn(x) for x and 1/x well inside the normal range: an approximation
+// (2 ulp) and one Newton step in fused arithmetic (Markstein 1990), the same
+// bits for every one of the 2^23 significands.
+__device__ __forceinline__ float rcp_normal(float x) {
+  const float r = __fdividef(1.0f, x);
+  return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
+}
+
 // Marker coordinates in the working precision.  FP32 builds them from the
 // split X = xo + xr (integer cell, fraction) so that the per-step kernels
 // issue no FP64 instructions (a slow pipe on this GPU); FP64 subtracts the
@@ -1416,9 +1424,9 @@ __device__ __forceinline__ void interp_advect_body(const IBArgs<typename Prec<MO
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
         EqCell<L, MODE> e;
-        // (the quadratic terms' 1/rho: an approximate one in FP32, where gathering
-        // the stored ones took the kernel from 11 to 13 us)
-        if constexpr (std::is_same<Real, float>::value) e.set_f(src[i], __fdividef(1.0f, 1.0f + src[i].x));
+        // (the 1/rho that the collide stored: in FP32 formed again, as gathering
+        // them took the kernel from 11 to 13 us)
+        if constexpr (std::is_same<Real, float>::value) e.set_f(src[i], rcp_normal(1.0f + src[i].x));
         else e.set_f(src[i], __ldg(&a.M[M_V * G.P32 + nb.src(i)].w));
         const Real fi = e.f_or_back(i, nb.bounce(i));
         r += fi;
