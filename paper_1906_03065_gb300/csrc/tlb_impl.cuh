@@ -271,7 +271,7 @@ struct Impl : ImplBase {
     TLB_LAUNCHED(c, "k_mu_global");
     k_init_eq<L, MODE><<<blocks(N, 256), 256, 0, s>>>(G, rho, phi, psi, uf, mu, la.gphi, la.gpsi,
                                                        c->ptr<Store>(c->L.lo[c->cur]),
-                                                       c->ptr<Rest>(c->L.rest[c->cur]));
+                                                       c->ptr<Rest>(c->L.rest[c->cur]), la.p4);
     TLB_LAUNCHED(c, "k_init_eq");
     TLB_CUDA(cudaMemsetAsync(c->ptr<char>(c->L.ftot), 0, c->L.ftot.bytes, s));
     // the initial state is the first reference of the equilibrium residual
@@ -381,7 +381,7 @@ struct Impl : ImplBase {
     TLB_LAUNCHED(c, "k_mu_global");
     k_init_eq<L, MODE><<<blocks(c->N, 256), 256, 0, s>>>(G, rho, phi, psi, uf, mu, la.gphi, la.gpsi,
                                                           c->ptr<Store>(c->L.lo[c->cur]),
-                                                          c->ptr<Rest>(c->L.rest[c->cur]));
+                                                          c->ptr<Rest>(c->L.rest[c->cur]), la.p4);
     TLB_LAUNCHED(c, "k_init_eq");
     // (of these populations: what M held before is not written over them)
     tlb_status rs = pops_written(c);

@@ -977,17 +977,19 @@ __global__ void k_mu_global(Geo G, FEParams<typename Prec<MODE>::Real> fe, const
 // stored post-collision:
 // the value of direction i at cell y is the equilibrium f_i at y + c_i (or,
 // across a wall, f_{opp(i)} at y), which the next pull brings back to place.
+// p4 not NULL: phi and psi there too, for readers of the moment field.
 template <class L, int MODE>
 __global__ void k_init_eq(Geo G, const typename Prec<MODE>::Real* rho, const typename Prec<MODE>::Real* phi,
                           const typename Prec<MODE>::Real* psi, const typename Prec<MODE>::Real* u,
                           const typename Prec<MODE>::Real* mu, typename Prec<MODE>::Real gphi,
                           typename Prec<MODE>::Real gpsi, typename Prec<MODE>::Store* lo,
-                          typename Prec<MODE>::Rest* rest) {
+                          typename Prec<MODE>::Rest* rest, R4<typename Prec<MODE>::Real>* p4) {
   using Real = typename Prec<MODE>::Real;
   using Store = typename Prec<MODE>::Store;
   using Rest = typename Prec<MODE>::Rest;
   long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= G.N) return;
+  if (p4) p4[n] = R4<Real>{rho[n], phi[n], psi[n], 0};
   int x, y, z;
   cell_xyz(G, n, x, y, z);
   for (int i = 0; i < L::Q; ++i) {

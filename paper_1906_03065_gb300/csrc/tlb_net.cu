@@ -1140,12 +1140,13 @@ __global__ void k_weights(const float* __restrict__ W, int taps, int Ci, int Co,
 
 // Network input of one sample from a context's fields: phi0, psi0, the
 // broadcast features, zeros.
-__global__ void k_make_input(const float* __restrict__ phi, const float* __restrict__ psi, long long V, float f0,
-                             float f1, float f2, float f3, float f4, bf16* __restrict__ x) {
+// (phi and psi of cell v at phi[v * step], psi[v * step])
+__global__ void k_make_input(const float* __restrict__ phi, const float* __restrict__ psi, int step, long long V,
+                             float f0, float f1, float f2, float f3, float f4, bf16* __restrict__ x) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   __align__(16) bf16 c[16];
-  const float fv[7] = {phi[v], psi[v], f0, f1, f2, f3, f4};
+  const float fv[7] = {phi[v * step], psi[v * step], f0, f1, f2, f3, f4};
   for (int k = 0; k < 16; ++k) c[k] = __float2bfloat16_rn(k < 7 ? fv[k] : 0.f);
   reinterpret_cast<uint4*>(x + v * 16)[0] = reinterpret_cast<uint4*>(c)[0];
   reinterpret_cast<uint4*>(x + v * 16)[1] = reinterpret_cast<uint4*>(c)[1];
@@ -2052,9 +2053,15 @@ tlb_status tlb_net_input(void* net, void* ctx, const double* feats, void* x_dev)
   if (!n || !feats || !x_dev) { set_error("net/feats/x is NULL"); return TLB_ERR_ARG; }
   tlb_status s = check_ctx(n, c);
   if (s != TLB_OK) return s;
-  k_make_input<<<nb(c->N, 256), 256, 0, n->stream>>>(c->ptr<float>(c->L.phi), c->ptr<float>(c->L.psi), c->N,
-                                                     (float)feats[0], (float)feats[1], (float)feats[2],
-                                                     (float)feats[3], (float)feats[4], (bf16*)x_dev);
+  // the fields of the start, or those the last step started from (where the
+  // moments pass writes them)
+  const bool packed = c->packed();
+  const float* p4 = c->ptr<float>(c->L.p4);
+  const float* phi = packed ? p4 + 1 : c->ptr<float>(c->L.phi);
+  const float* psi = packed ? p4 + 2 : c->ptr<float>(c->L.psi);
+  k_make_input<<<nb(c->N, 256), 256, 0, n->stream>>>(phi, psi, packed ? 4 : 1, c->N, (float)feats[0],
+                                                     (float)feats[1], (float)feats[2], (float)feats[3],
+                                                     (float)feats[4], (bf16*)x_dev);
   NET_LAUNCHED(n, "k_make_input");
   return TLB_OK;
 }
@@ -2080,7 +2087,7 @@ tlb_status tlb_net_warm_start(void* net, void* ctx, const double* feats) {
   float* phi = c->ptr<float>(c->L.phi);
   float* psi = c->ptr<float>(c->L.psi);
   float* I = c->ptr<float>(c->L.I);
-  k_make_input<<<nb(c->N, 256), 256, 0, st>>>(phi, psi, c->N, (float)feats[0], (float)feats[1], (float)feats[2],
+  k_make_input<<<nb(c->N, 256), 256, 0, st>>>(phi, psi, 1, c->N, (float)feats[0], (float)feats[1], (float)feats[2],
                                               (float)feats[3], (float)feats[4], x);
   NET_LAUNCHED(n, "k_make_input");
   if ((s = forward(n, 1)) != TLB_OK) return s;

@@ -63,3 +63,48 @@ def test_markers_move_with_the_readable_populations(storage):
                 ref += wt[:, None] * v[:, q[:, 2], q[:, 1], q[:, 0]].T
     assert np.abs(U).max() < 0.5
     assert np.abs(U - ref).max() < 2e-7
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("general", [False, True])
+def test_network_input_of_a_stepped_context(storage, general):
+    """The network's input tensor holds the phi and psi that the last step
+    started from (bf16, to half a unit beside FP32 rounding), those of the
+    start before any step, and those of the new start after another one."""
+    import torch
+    from paper_1906_03065_gb300 import Simulation, WarmStartNet
+    n = 48
+    p = W.Params(dim=3, nx=n, ny=n, nz=n, wall_last=1, storage=storage, alpha=1.0, dc=8.0, interface_pos=24.0,
+                 tau=0.8 if general else 1.0)
+    m = W.icosphere(2, 8.0, (24.2, 24.1, 23.7))
+    m.G, m.kb = 0.01, 0.005
+    s = Simulation(W.Workload("cap", p, [m]))
+    C0, u0 = W.random_fields(p, seed=8)
+    s.init(C0, u0)
+    net = WarmStartNet(n, 16, 4, 1)
+
+    def check(phi, psi):
+        x = net.input(s, np.zeros(5))
+        torch.cuda.synchronize()
+        x = x.float().cpu().numpy().astype(float)
+        for k, ref in ((0, phi), (1, psi)):
+            assert np.all(np.abs(x[:, k] - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-6), k
+
+    def order(s):
+        return s.field("phi"), s.field("psi")
+
+    check(C0[0] - C0[1], C0[2])
+    s.step(2)
+    ref = order(s)
+    s.step(1)
+    check(*ref)
+    ref = order(s)
+    s.step(1)
+    check(*ref)
+    s.step(39)
+    ref = order(s)
+    s.step(1)
+    check(*ref)
+    C1, u1 = W.random_fields(p, seed=9)
+    s.init(C1, u1)
+    check(C1[0] - C1[1], C1[2])
