@@ -315,7 +315,9 @@ tlb_status tlb_set_tile(void* ctx, int tile_variant, int z_chunk);
  * first step after markers were set from outside or after populations were
  * written, the steps of tlb_profile_steps and a remainder below 8 steps run as
  * direct launches.  By
- * default a graph is captured in a call of 32 steps or more; on != 0 asks for
+ * default a graph is captured in a call of 32 steps or more (of 64 or more
+ * with a general collide on 2^25 cells x velocities or more, about 120^3, where
+ * it saves less); on != 0 asks for
  * it in any call of 8 steps or more, on = 0 turns graphs off and releases the
  * captured ones.
  * tlb_step may also be called while the caller captures the context's stream.

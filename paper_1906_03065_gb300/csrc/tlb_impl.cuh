@@ -544,11 +544,16 @@ struct Impl : ImplBase {
 
   // Graphs serve this call: not while phases are timed; and unless
   // tlb_set_graphs asked for them, only where a graph exists already or the
-  // call is long enough to pay for its capture (about 0.5 ms, against 15 to 25
-  // us saved per step).
+  // call is long enough to pay for its capture: 0.32 ms, against 10 to 20 us
+  // saved per step (32^3 to 128^3 at tau = 1, all of 2D), so from 32 steps on.
+  // Where the general collide hides the launches, 7 us are saved (128^3 and
+  // 160^3; 10 at 96^3, which comes out even at 32 steps): from 64 steps on.  A
+  // first call of 32 or 50 steps of the 128^3 general collide: 374 us per step
+  // direct, 378 and 375 with the capture; 100 steps: 373 against 370.
   bool graphs_usable(Ctx* c, long n) const {
     if (!c->graphs || c->prof || n < Ctx::GRAPH_STEPS) return false;
-    return c->graphs_asked || graph_current(c) || n >= 4 * Ctx::GRAPH_STEPS;
+    const bool hidden = !variant_t1(c->tile_variant) && c->N * c->Q >= (1ll << 25);
+    return c->graphs_asked || graph_current(c) || n >= (hidden ? 8 : 4) * Ctx::GRAPH_STEPS;
   }
   bool graph_current(const Ctx* c) const {
     const int k = c->cur;
