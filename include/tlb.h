@@ -308,17 +308,16 @@ tlb_status tlb_autotune(void* ctx, int* tile_variant, int* z_chunk);
  * on the choice beyond rounding. */
 tlb_status tlb_set_tile(void* ctx, int tile_variant, int z_chunk);
 
-/* Step graphs.  tlb_step and tlb_run issue runs of 8 steps of a lattice with
- * membranes as one CUDA graph launch, captured once per population buffer and
- * collide variant from the same kernels the direct launches use (the results
- * are identical bit for bit; the kernels keep their streams' priorities); the
- * first step after markers were set from outside or after populations were
- * written, the steps of tlb_profile_steps and a remainder below 8 steps run as
- * direct launches.  By
- * default a graph is captured in a call of 32 steps or more (of 64 or more
- * with a general collide on 2^25 cells x velocities or more, about 120^3, where
- * it saves less); on != 0 asks for
- * it in any call of 8 steps or more, on = 0 turns graphs off and releases the
+/* Step graphs.  tlb_step and tlb_run can issue runs of 8 steps as one CUDA
+ * graph launch, captured once per population buffer and collide variant from
+ * the same kernels the direct launches use (the results are identical bit for
+ * bit; the kernels keep their streams' priorities); the first step after
+ * markers were set from outside or after populations were written, the steps
+ * of tlb_profile_steps and a remainder below 8 steps run as direct launches.
+ * By default a graph is captured in a call of 32 steps or more on a lattice
+ * with membranes (of 64 or more with a general collide on 2^25 cells x
+ * velocities or more, about 120^3, where it saves less); on != 0 asks for it in
+ * any call of 8 steps or more, on = 0 turns graphs off and releases the
  * captured ones.
  * tlb_step may also be called while the caller captures the context's stream.
  * Nothing runs then and the state stays as it is; each replay of the caller's

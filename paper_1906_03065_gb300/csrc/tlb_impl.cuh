@@ -525,7 +525,7 @@ struct Impl : ImplBase {
   }
 
   tlb_status step_calls(Ctx* c, long n) {
-    if (c->nn == 0 || !graphs_usable(c, n)) return step_direct(c, n);
+    if (!graphs_usable(c, n)) return step_direct(c, n);
     while (n > 0) {
       if (n >= Ctx::GRAPH_STEPS && graph_ready(c) && have_graph(c)) {
         tlb_status st = replay(c);
@@ -549,11 +549,13 @@ struct Impl : ImplBase {
   // Where the general collide hides the launches, 7 us are saved (128^3 and
   // 160^3; 10 at 96^3, which comes out even at 32 steps): from 64 steps on.  A
   // first call of 32 or 50 steps of the 128^3 general collide: 374 us per step
-  // direct, 378 and 375 with the capture; 100 steps: 373 against 370.
+  // direct, 378 and 375 with the capture; 100 steps: 373 against 370.  Without
+  // membranes two launches a step hardly wait: only where asked for.
   bool graphs_usable(Ctx* c, long n) const {
     if (!c->graphs || c->prof || n < Ctx::GRAPH_STEPS) return false;
     const bool hidden = !variant_t1(c->tile_variant) && c->N * c->Q >= (1ll << 25);
-    return c->graphs_asked || graph_current(c) || n >= (hidden ? 8 : 4) * Ctx::GRAPH_STEPS;
+    if (c->graphs_asked) return true;
+    return c->nn > 0 && (graph_current(c) || n >= (hidden ? 8 : 4) * Ctx::GRAPH_STEPS);
   }
   bool graph_current(const Ctx* c) const {
     const int k = c->cur;

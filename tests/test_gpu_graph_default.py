@@ -43,3 +43,21 @@ def test_default_calls_equal_direct_launches(name):
         runs.append((s.field("C1"), s.field("C3"), s.field("u"), s.nodes(0)))
     for x, y in zip(*runs):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("storage,tau", [("f32", 1.0), ("bf16", 1.0), ("f32", 0.8)])
+def test_graphs_asked_for_without_membranes(storage, tau):
+    from paper_1906_03065_gb300 import Simulation
+    p = W.Params(dim=3, nx=33, ny=20, nz=18, wall_last=1, storage=storage, alpha=1.0, interface_pos=9.0, tau=tau)
+    C0, u0 = W.random_fields(p, seed=2)
+    runs = []
+    for on in (False, True):
+        s = Simulation(W.Workload("fluid", p, [])).init(C0, u0)
+        s.set_graphs(on)
+        for n in (8, 9, 40, 3, 16):
+            s.step(n)
+        s.set_pops(s.pops())
+        s.step(17)
+        runs.append((s.launches(), s.pops()))
+    assert runs[0][0] == runs[1][0]
+    assert np.array_equal(runs[0][1], runs[1][1])
