@@ -257,13 +257,13 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
     take(L.lo[b], (size_t)(3 * c.Q - 2) * P * c.ts.store);
     take(L.rest[b], 2 * P * c.ts.rest);
   }
-  take(L.rho, P * R);
+  if (!c.packed()) take(L.rho, P * R);
   take(L.phi, P * R);
   take(L.psi, P * R);
-  const size_t t1 = c.t1_ok() ? 1 : 0;  // the tau = 1 scheme's momenta and state
   take(L.p4, c.packed() ? 4 * P * R : 0);
-  take(L.j2, t1 * 2 * P * R);
-  take(L.M, t1 * 12 * P * R);
+  // (offsets in the idle population buffer, see Ctx::idle)
+  L.M = {0, 12 * P * R};
+  L.j2 = {L.M.bytes, 2 * P * R};
   take(L.I, P * R);
   take(L.dsel, P * R);
   take(L.own, P * 4);
@@ -272,6 +272,8 @@ static void plan(const tlb_params* p, const std::vector<HostMem>& mems, Ctx& c) 
   take(L.ftot, 3 * P * R);
   take(L.mu, 3 * P * R);
   take(L.rb, 6 * P * 8);
+  // (with packed moments rho serves an initialisation only, which reads nothing back)
+  if (c.packed()) L.rho = {L.rb.off, P * R};
   const size_t nn = c.nn, ne = c.ne, NV = c.NV;
   take(L.X, 3 * nn * 8);
   take(L.E, NV * ne * 4);

@@ -329,9 +329,8 @@ struct BatchImpl : BatchBase {
   // the population buffer cur ^ q of each instance.  Tau = 1 collide: both
   // read and write the state M; in table 1 the instances whose state is in
   // the populations pull it (the first step after an initialisation), in
-  // table 0 none does.  With `scratch` the collide writes into the idle
-  // population buffer (timing of collide variants).
-  tlb_status upload_tables(Batch* b, bool scratch = false) {
+  // table 0 none does.
+  tlb_status upload_tables(Batch* b) {
     const int n = (int)b->act.size();
     const bool t1 = variant_t1(b->tile_variant);
     for (int q = 0; q < 2; ++q) {
@@ -347,7 +346,6 @@ struct BatchImpl : BatchBase {
           a.lb.pull = 0;
           a.lb.in_M = nullptr;
         }
-        if (t1 && scratch) a.lb.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
         a.ib = I::ibargs(c);
         I::use_t1(c, a.ib, t1);
         a.ib.split = b->scat_split;
@@ -538,8 +536,8 @@ struct BatchImpl : BatchBase {
     const bool t1 = all_ok(13);
     for (int i : b->act) {
       Ctx* c = b->inst[i];
-      if (!t1)
-        if (tlb_status es = I::enter_pops(c); es != TLB_OK) return es;
+      // (the timed collides write the idle population buffer)
+      if (tlb_status es = I::enter_pops(c); es != TLB_OK) return es;
       LBArgs<MODE> la = I::lbargs(c, c->cur);
       I::use_t1(c, la, t1);
       if (tlb_status ms = I::launch_moments(c, la, b->stream); ms != TLB_OK) return ms;
@@ -552,7 +550,7 @@ struct BatchImpl : BatchBase {
         b->zc = zcs[zi];
         b->graph_dirty = true;
         st = plan_phases(b);
-        if (st == TLB_OK) st = upload_tables(b, true);
+        if (st == TLB_OK) st = upload_tables(b);
         if (st == TLB_OK) st = launch_collide(b, b->ptr<BA>(b->targs[0]), vg_of(b, 4), b->stream);
         float tmin = 1e30f;
         for (int r = 0; r < 2 && st == TLB_OK; ++r) {

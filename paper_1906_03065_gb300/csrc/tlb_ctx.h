@@ -256,6 +256,12 @@ struct Ctx {
   }
 
   template <class T> T* ptr(const Region& r) const { return reinterpret_cast<T*>(base + r.off); }
+  // The tau = 1 scheme's state and momenta, M and j2, lie in the population
+  // buffer that its steps leave idle (they take 14 planes of the arithmetic
+  // type, the buffer holds 3Q - 2 of the storage type: at least 1.7 times as
+  // much).  A general step writes its populations there and others use it as
+  // scratch, all after the state has entered the current buffer.
+  template <class T> T* idle(const Region& r) const { return reinterpret_cast<T*>(base + L.lo[1 - cur].off + r.off); }
 
   ~Ctx() {
     if (gexec[0] || gexec[1]) cudaEventSynchronize(ev_interp);  // (recorded after every replay)

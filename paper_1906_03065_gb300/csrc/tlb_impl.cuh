@@ -35,15 +35,15 @@ struct Impl : ImplBase {
   // the arrays of the tau = 1 scheme, or none of them
   static void use_t1(Ctx* c, LBArgs<MODE>& a, bool t1) {
     a.p4 = c->packed() ? c->ptr<R4<Real>>(c->L.p4) : nullptr;
-    a.j2 = t1 ? c->ptr<R2<Real>>(c->L.j2) : nullptr;
-    a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
+    a.j2 = t1 ? c->idle<R2<Real>>(c->L.j2) : nullptr;
+    a.M = t1 ? c->idle<R4<Real>>(c->L.M) : nullptr;
     a.pull = c->state_in_pops;
     a.in_M = t1 && c->asks() ? c->ptr<int>(c->L.in_M) : nullptr;
   }
   static void use_t1(Ctx* c, IBArgs<Real>& a, bool t1) {
     a.psi = c->packed() ? &c->ptr<R4<Real>>(c->L.p4)->z : c->ptr<Real>(c->L.psi);
     a.psi_step = c->packed() ? 4 : 1;
-    a.M = t1 ? c->ptr<R4<Real>>(c->L.M) : nullptr;
+    a.M = t1 ? c->idle<R4<Real>>(c->L.M) : nullptr;
   }
 
   static LBArgs<MODE> lbargs(Ctx* c, int src) {
@@ -309,7 +309,7 @@ struct Impl : ImplBase {
   tlb_status sync_pops(Ctx* c) override {
     if (!c->asks() && (c->state_in_pops || !c->pops_stale)) return TLB_OK;
     k_materialize<L, MODE><<<blocks(c->N, 256), 256, 0, c->stream>>>(
-        geo(c), c->ptr<R4<Real>>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]),
+        geo(c), c->idle<R4<Real>>(c->L.M), c->ptr<Store>(c->L.lo[c->cur]), c->ptr<Rest>(c->L.rest[c->cur]),
         c->asks() ? c->ptr<int>(c->L.in_M) : nullptr);
     TLB_LAUNCHED(c, "k_materialize");
     // (captured, it has not run; the flag of a context that asks is not used)
@@ -432,14 +432,11 @@ struct Impl : ImplBase {
     // the candidates: the tau = 1 variants where they apply (a general one
     // pulls and stores several times their bytes), else the general ones
     const bool t1 = c->t1_ok();
-    if (!t1)
-      if (tlb_status st = enter_pops(c); st != TLB_OK) return st;
+    // (the timed collides write the idle population buffer)
+    if (tlb_status st = enter_pops(c); st != TLB_OK) return st;
     LBArgs<MODE> la = lbargs(c, c->cur);
     use_t1(c, la, t1);
     if (tlb_status st = launch_moments(c, la, s); st != TLB_OK) return st;
-    // the timed collides store into the idle population buffer, not into the
-    // state
-    if (t1) la.M = c->ptr<R4<Real>>(c->L.lo[1 - c->cur]);
     cudaEvent_t e0, e1;
     TLB_CUDA(cudaEventCreate(&e0));
     TLB_CUDA(cudaEventCreate(&e1));
@@ -818,7 +815,7 @@ struct Impl : ImplBase {
 
   // Contact angles (tlb_measure.cuh).  Scratch: phi in the read-back
   // buffer; marker values, edge angles and the per-capsule results in the
-  // population buffer that the next step writes (idle between steps).
+  // idle population buffer (the state goes to the other one).
   tlb_status contact_angle(Ctx* c, double* out) override {
     cudaStream_t s = c->stream;
     const long long N = c->N;
@@ -826,7 +823,7 @@ struct Impl : ImplBase {
     const size_t need = (size_t)(4 * c->nn + nedge + 4 * c->ncap) * sizeof(double) + (size_t)nedge * sizeof(int);
     if (c->ncap == 0) return TLB_OK;
     if (need > c->L.lo[1 - c->cur].bytes) { set_error("contact_angle: scratch too small"); return TLB_ERR_ARG; }
-    if (tlb_status st = sync_pops(c); st != TLB_OK) return st;
+    if (tlb_status st = enter_pops(c); st != TLB_OK) return st;
     double* phi = c->ptr<double>(c->L.rb);
     k_fields<L, MODE><<<blocks(N, 256), 256, 0, s>>>(geo(c), c->ptr<Store>(c->L.lo[c->cur]),
                                                       c->ptr<Rest>(c->L.rest[c->cur]), TLB_FIELD_PHI, phi);
