@@ -575,6 +575,16 @@ struct Impl : ImplBase {
     return st;
   }
 
+  // The calls around a capture of the library's own (stream creation,
+  // synchronisation, instantiation) would invalidate a capture of another
+  // stream that the program has under way in the global mode.  They concern
+  // this context's streams only, so the thread takes the relaxed mode meanwhile.
+  struct OwnCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OwnCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OwnCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  };
+
   // The graph of the current buffer, captured first if missing or captured
   // with another collide variant.  Its kernels keep the priorities of the
   // streams they were captured from (the membrane chain's blocks go first
@@ -582,6 +592,7 @@ struct Impl : ImplBase {
   // directly from here on.
   bool have_graph(Ctx* c) {
     if (graph_current(c)) return true;
+    const OwnCapture own;
     const int k = c->cur;
     if (!c->gstream && cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking) != cudaSuccess) return no_graphs(c);
     cudaStream_t user = c->stream;
