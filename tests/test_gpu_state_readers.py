@@ -65,6 +65,51 @@ def test_markers_move_with_the_readable_populations(storage):
     assert np.abs(U - ref).max() < 2e-7
 
 
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_moment_state_equals_the_population_scheme(storage):
+    """From populations written by the caller, one step of the tau = 1 collide
+    (state in 12 values per cell, pulled this once) and a second one (rebuilt
+    from them) give the populations of the general collide, which stores and
+    pulls them: the collisions round differently in FP32 (a few units of 6e-8
+    of values up to 1), and each of the two roundings to the storage type may
+    then fall on either side."""
+    import oracle
+    from paper_1906_03065_gb300 import Simulation
+    oracle.build()
+    wl = W.small_3d(storage)
+    o = oracle.Oracle(wl, init=False)
+    C0, u0 = W.random_fields(wl.params, seed=4)
+    c, w = o.lattice()
+    a, b = Simulation(wl).init(C0, u0), Simulation(wl).init(C0, u0)
+    b.set_tile(3, 8)
+    rng = np.random.default_rng(5)
+    P = a.pops() + 1e-3 * rng.standard_normal((3, o.Q, o.N)) * w[None, :, None]
+    eps = {"f32": 0.0, "f16": 2.0 ** -10, "bf16": 2.0 ** -7}[storage]
+    for s in (a, b):
+        s.set_pops(P)
+    a.step(1)
+    b.step(1)
+    Pa, Pb = a.pops(), b.pops()
+    stored = np.abs(Pb)
+    stored[0] -= w[:, None]
+    stored = np.abs(stored)
+    stored[1:, 0] = 0.0  # the rest populations of the order parameters are FP32
+    assert np.all(np.abs(Pa - Pb) <= eps * stored + 1e-6)
+    assert np.abs(a.nodes(0) - b.nodes(0)).max() < (1e-6 if storage == "f32" else 2e-3)
+    # the second step from the same stored state in both schemes
+    blob = a.save()
+    b.load(blob)
+    assert np.array_equal(b.pops(), Pa)
+    a.step(1)
+    b.step(1)
+    Pa, Pb = a.pops(), b.pops()
+    stored = np.abs(np.stack([Pb[0] - w[:, None], Pb[1], Pb[2]]))
+    stored[1:, 0] = 0.0
+    assert np.all(np.abs(Pa - Pb) <= eps * stored + 1e-6)
+    da, db = a.diagnostics(), b.diagnostics()
+    assert np.allclose(da.mass[:], db.mass[:], rtol=0, atol=(1e-6 + eps * 0.05) * o.N)
+
+
 @pytest.mark.parametrize("storage", ["f32", "bf16"])
 @pytest.mark.parametrize("general", [False, True])
 def test_network_input_of_a_stepped_context(storage, general):
