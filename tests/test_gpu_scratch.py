@@ -76,3 +76,20 @@ def test_batch_autotune_between_steps():
     for i in range(2):
         assert np.array_equal(a[i].field("I"), b[i].field("I"))
         assert np.abs(a[i].pops() - b[i].pops()).max() < 1e-6
+
+
+def test_contact_angle_of_a_dense_ring():
+    """A ring whose scratch does not fit past the state: the state moves over."""
+    from paper_1906_03065_gb300 import Simulation
+    wl = W.small_2d("f64", nx=24, ny=24, nodes=1200, radius=6.0, centre=(12.2, 11.9))
+    wl.params.interface_pos = 12.0
+    wl.membranes[0].kb = 0.0
+    a, b = Simulation(wl).init(), Simulation(wl).init()
+    for s in (a, b):
+        s.step(3)
+    assert a.contact_angle()[0, 3] == 2
+    for s in (a, b):
+        s.step(4)
+    assert np.array_equal(a.pops(), b.pops())
+    assert np.array_equal(a.nodes(0), b.nodes(0))
+    assert np.isfinite(a.pops()).all()
