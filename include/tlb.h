@@ -116,13 +116,13 @@ enum { TLB_FORCE_EDM = 0, TLB_FORCE_GUO = 1 };
 /* State between steps (tlb_params.state): the 3Q post-collision populations,
  * in the storage type.  At tau = tau_phi = tau_psi = 1 with TLB_FORCE_EDM
  * (the paper's setting, Sec. 3.1) and the potential force every one of them
- * is an equilibrium (eq. EDF) of its cell, so 11 values per cell stand for
- * all of them: rho - 1, u + du, phi, Gamma_phi mu_phi, psi, Gamma_psi mu_psi'
- * and v (eq. LBE at tau = 1).  Steps of the tau = 1 collide variants (the
- * default there, see tlb_autotune) keep those and rebuild every population,
- * rounded to the storage type, where it streams from: 96 bytes of state
- * traffic per cell update against 456 in FP32 and 236 in FP16, and the same
- * populations.  Initial states and populations written by the caller are
+ * is an equilibrium (eq. EDF) of its cell, so a few values per cell stand for
+ * all of them (eq. LBE at tau = 1).  Steps of the tau = 1 collide variants (the
+ * default there, see tlb_autotune) keep 12 in the arithmetic type -- rho - 1,
+ * q = j + F, phi, 3 Gamma_phi mu_phi, psi, 3 Gamma_psi mu_psi', v and 1/rho --
+ * and rebuild every population, rounded to the storage type, where it streams
+ * from: 96 bytes of state traffic per cell update against 456 in FP32 and 236
+ * in FP16.  The stored populations and the rebuilt ones are the same bits.  Initial states and populations written by the caller are
  * pulled as populations by the next step; reads of populations or fields
  * see the populations the state stands for.
  * TLB_STATE_POPULATIONS -- any collide variant;

@@ -730,9 +730,11 @@ __device__ __forceinline__ void dist_scatter_body(const IBArgs<Real>& a, const B
         const int id = sm.tab[i], L = id / SCAT_W, h = id % SCAT_W;
         const int4 e = sm.sl[L][h], F0 = sm.ft[L][0], F1 = sm.ft[L][1];
         const int jj = base + i - e.w;
-        // jj / wa with an approximate reciprocal: jj < 2^20, so the product is
-        // within 0.2 / wa of (jj + 1/2) / wa, which lies at least 1 / (2 wa)
-        // from an integer: the truncation is exact
+        // jj / wa with an approximate reciprocal (__fdividef: 2 ulp, 2^-22
+        // relative; the product adds 2^-24): jj < 2^20, as slice_rect holds both
+        // sides to 1024, so the result is within (0.25 + 0.0625) / wa of (jj + 1/2)
+        // / wa, which lies at least 1 / (2 wa) from an integer: the truncation is
+        // exact
         const int qb = (int)(((float)jj + 0.5f) * __fdividef(1.0f, (float)e.z));
         const int rk = F1.y + r * SCAT_W + h, ra = e.x + (jj - qb * e.z), rb = a.dim == 3 ? e.y + qb : 0;
         // axes (k, a, b): 3D k = 0: (x, y, z); 1: (y, x, z); 2: (z, x, y); 2D the
