@@ -809,26 +809,17 @@ __device__ __forceinline__ Real feature_sign(const IBArgs<Real>& a, int e, const
 // rest, which is exact (v - hi 2^-24 is a multiple of v's last place below
 // 2^-25) but for its own rounding, so no 64-bit conversion is needed (slow
 // on this GPU).  The parts of a warp's lanes add up in 32 bits while every
-// |v| < CPL_SMALL; beyond it the value is converted whole.
-constexpr float CPL_SMALL = 3.9f;
+// |v| < CPL_SMALL, and in 64 bits while hi holds it (|v| < CPL_SPLIT).
+constexpr float CPL_SMALL = 3.9f, CPL_SPLIT = 120.0f;
 __device__ __forceinline__ void cpl_split(float v, int* hi, int* lo) {
   *hi = __float2int_rn(v * 0x1p24f);
   *lo = __float2int_rn(fmaf((float)*hi, -0x1p-24f, v) * 0x1p50f);
 }
 __device__ __forceinline__ long long cpl_join(int hi, int lo) { return (long long)hi * (1 << 26) + lo; }
-// The same of any v, from its bits: saturates at +-2^62 (|v| = 4096; a NaN too,
-// so that it shows in the markers).
+// The same of any v with the slow conversion: saturates at +-2^62 (|v| = 4096;
+// a NaN too, so that it shows in the markers).
 __device__ __forceinline__ long long cpl_whole(float v) {
-  const unsigned b = __float_as_uint(v), a = b & 0x7FFFFFFFu;
-  long long r = 1ll << 62;
-  if (a < __float_as_uint(CPL_SMALL)) {
-    int hi, lo;
-    cpl_split(__uint_as_float(a), &hi, &lo);
-    r = cpl_join(hi, lo);
-  } else if (a < __float_as_uint(4096.0f)) {  // a multiple of 2^-50: 2^1 <= |v| < 2^12
-    r = (long long)((a & 0x7FFFFFu) | 0x800000u) << ((int)(a >> 23) - 100);
-  }
-  return b >> 31 ? -r : r;
+  return __float2ll_rn(fmaxf(-4096.0f, fminf(4096.0f, v)) * 0x1p50f);
 }
 __device__ __forceinline__ long long cpl_fixed(double v) { return llrint(v * CPL_SCALE); }
 
@@ -957,6 +948,7 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
           small &= fabsf(v) < CPL_SMALL;
           cpl_split(v, hi + i, lo + i);
           sh[i] = sl[i] = 0;
+          sum[i] = 0;
         }
         if (__all_sync(active, small)) {
           // sum over the group (integers: any order gives the same total)
@@ -971,11 +963,21 @@ __device__ __forceinline__ void band_body(const IBArgs<Real>& a, const Blk& blk)
 #pragma unroll
           for (int i = 0; i < 9; ++i) sum[i] = cpl_join(sh[i], sl[i]);
         } else {
+          // (what hi cannot hold goes straight to the marker; converting all
+          // lanes' values whole instead took the band of a 240x120 ring from 9
+          // to 12 us, though no value was that large)
 #pragma unroll
           for (int i = 0; i < 9; ++i) {
-            const long long v = cpl_whole(acc[i / 3][i % 3]);
-            sum[i] = 0;
-            for (unsigned m = grp; m; m &= m - 1) sum[i] += __shfl_sync(grp, v, __ffs(m) - 1);
+            const float v = acc[i / 3][i % 3];
+            if (fabsf(v) < CPL_SPLIT) continue;
+            if (i / 3 < a.NV) atomicAdd(a.ncpl + 3 * a.E[a.NV * e + i / 3] + i % 3, (unsigned long long)cpl_whole(v));
+            hi[i] = lo[i] = 0;
+          }
+          for (unsigned m = grp; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+              sum[i] += cpl_join(__shfl_sync(grp, hi[i], src), __shfl_sync(grp, lo[i], src));
           }
         }
       } else {
